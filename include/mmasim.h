@@ -103,9 +103,11 @@ typedef struct {
                                    in Sections 2.2 and 6.3; FP32-accumulator FDPA models only) */
     const float* row_scale;     /* device, M floats or NULL */
     const float* col_scale;     /* device, N floats or NULL: D = fl32(fl32(row_scale[i]*col_scale[j]) * d) */
-    int32_t flags;              /* MMASIM_GEMM_FORCE_GENERIC: skip the tuned kernels (used to cross-check them) */
+    int32_t flags;              /* MMASIM_GEMM_FORCE_GENERIC: skip the tuned kernels; MMASIM_GEMM_LARGE_TILES: skip those for
+                                   small tiles where a large-tile kernel serves the call (both are used to cross-check) */
 } mmasim_gemm_opts;
 #define MMASIM_GEMM_FORCE_GENERIC 1
+#define MMASIM_GEMM_LARGE_TILES 2
 
 /* Registry lookup (Tables 3-7).  Returns NULL and sets the error message if the triple is not in the paper. */
 mmasim_model* mmasim_create_model(int arch, int in_fmt, int acc_fmt);

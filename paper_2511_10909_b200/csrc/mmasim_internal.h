@@ -87,6 +87,10 @@ int launch_generic(const DevModel& m, const GemmArgs& g, cudaStream_t stream);
 // mmasim_tfdpa_fast.cu
 bool fast_tfdpa_supported(const DevModel& m, const GemmArgs& g);
 int launch_fast_tfdpa(const DevModel& m, const GemmArgs& g, cudaStream_t stream);
+// the small-tile kernels (mmasim_direct.cuh): any K, any row stride; DIRECT_NONE: the large kernel is the better one
+enum DirectSize : int { DIRECT_NONE = 0, DIRECT_8x16, DIRECT_16x16, DIRECT_32x32 };
+DirectSize direct_size(const DevModel& m, const GemmArgs& g);
+int launch_direct(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStream_t stream);
 int launch_gemm_noalloc(const DevModel& m, const GemmArgs& g, cudaStream_t stream);   // status code; sets the error message
 // mmasim_fp_fast.cu
 bool fast_fp_supported(const DevModel& m, const GemmArgs& g);

@@ -4,6 +4,15 @@
 
 namespace mmasim {
 
+namespace direct {      // mmasim_direct_*.cu
+cudaError_t launch_lut8(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStream_t stream);
+cudaError_t launch_f16(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStream_t stream);
+cudaError_t launch_bf16(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStream_t stream);
+cudaError_t launch_tf32(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStream_t stream);
+cudaError_t launch_tr(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStream_t stream);
+cudaError_t launch_e(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStream_t stream);
+}  // namespace direct
+
 namespace {
 
 bool is8(int f) { return f == EF_E4M3 || f == EF_E5M2 || f == EF_E3M2 || f == EF_E2M3 || f == EF_E2M1; }
@@ -67,6 +76,60 @@ bool fast_tfdpa_supported(const DevModel& m, const GemmArgs& g) {
     if (g.M > 65535ll * fast::BM) return false;                             // grid.y
     if (g.N > 0x7FFFFFFFll - 128 || g.K > 0x7FFFFFFFll - 64) return false;   // 32-bit tile origins and k offsets in the kernels
     return true;
+}
+
+namespace {
+bool rows16(const DevModel& m, const GemmArgs& g) {                          // every row starts on a 16-byte boundary
+    const int bytes = fmt_desc(m.fmt_a).storage_bits / 8;
+    return (g.lda * bytes) % 16 == 0 && (g.ldb * bytes) % 16 == 0;
+}
+}  // namespace
+
+// Small tiles, or the large kernel?  What an SM does per chunk of 32 elements of K decides: CTAs on the fullest SM times the time
+// of one, plus the latency of a chunk when there are few.  In units of a 16 x 16 tile's chunk (0.33 - 0.55 us by family), measured
+// on full grids (4096 x 4096 x 256) and on single waves: 8 x 16 tiles 0.6, 32 x 32 tiles `mid`, tiles of the large kernel `large`
+// (its decode pass and two more launches: about 6 us, fifteen units of one chunk).  Examples, small against large in us, on both
+// sides of the line: Hopper FP16 128 x 2048 x 2048 128 / 337, 2352 x 192 x 3328 320 / 771, 1000 x 1111 x 992 245 / 254,
+// 1024^3 225 / 175, 2048 x 2048 x 512 449 / 340.
+DirectSize direct_size(const DevModel& m, const GemmArgs& g) {
+    const int kind = kind_of(m);
+    if (!kind || g.dot_mode || m.literal_emax) return DIRECT_NONE;
+    if ((kind == KIND_TR || kind == KIND_E) && g.k_chunk) return DIRECT_NONE;
+    if (g.M > 65535ll * 8 || g.N > 0x7FFFFFFFll - 128 || g.K > 0x7FFFFFFFll - 256) return DIRECT_NONE;     // grid.y, 32-bit k
+    constexpr int64_t SMS = 148;
+    auto fullest = [&](int bm, int bn) { return double((((g.M + bm - 1) / bm) * ((g.N + bn - 1) / bn) + SMS - 1) / SMS); };
+    const bool f13 = kind == 1 + fast::EK_LUT8 && m.F == 13, bits8 = kind == 1 + fast::EK_LUT8;
+    const double mid = bits8 ? 2.1 : (kind == KIND_E ? 3.4 : (kind == KIND_TR ? 2.7 : (m.L >= 16 ? 2.7 : 3.2)));
+    const double large = f13 ? 13.5 : (bits8 ? 9.5 : (kind == KIND_E ? 22.0 : (kind == KIND_TR ? 18.0 : (m.L >= 16 ? 14.0 : 20.0))));
+    const double c8 = 0.5 + 0.6 * fullest(8, 16), c16 = 0.6 + fullest(16, 16), c32 = 0.6 + mid * fullest(32, 32);
+    const double chunks = double((g.K + fast::KC - 1) / fast::KC);
+    const double big = fast_tfdpa_supported(m, g) ? large * fullest(fast::BM, f13 && m.acc != ACC_F16 && !g.k_chunk ? 128 : fast::BN) + 15.0 / chunks : 1e30;
+    if (big <= c8 && big <= c16 && big <= c32) return DIRECT_NONE;
+    return c8 <= c16 && c8 <= c32 ? DIRECT_8x16 : (c16 <= c32 ? DIRECT_16x16 : DIRECT_32x32);
+}
+
+int launch_direct(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStream_t stream) {
+    cudaError_t err = cudaErrorInvalidValue;
+    const int kind = kind_of(m);
+    if (kind == KIND_TR) {
+        set_kernel_name(m.family == FAM_GTR ? "gtrfdpa" : "trfdpa");
+        err = direct::launch_tr(m, g, size, stream);
+    } else if (kind == KIND_E) {
+        set_kernel_name("efdpa");
+        err = direct::launch_e(m, g, size, stream);
+    } else switch (kind - 1) {
+        case fast::EK_LUT8: set_kernel_name("tfdpa_lut8"); err = direct::launch_lut8(m, g, size, stream); break;
+        case fast::EK_F16: set_kernel_name("tfdpa_f16"); err = direct::launch_f16(m, g, size, stream); break;
+        case fast::EK_BF16: set_kernel_name("tfdpa_bf16"); err = direct::launch_bf16(m, g, size, stream); break;
+        case fast::EK_TF32: set_kernel_name("tfdpa_tf32"); err = direct::launch_tf32(m, g, size, stream); break;
+        default: break;
+    }
+    if (!rows16(m, g)) set_kernel_name("generic");      // the any-shape route: rows at any address
+    if (err != cudaSuccess) {
+        set_error("small-tile FDPA kernel launch failed: %s", cudaGetErrorString(err));
+        return MMASIM_ERR_CUDA;
+    }
+    return MMASIM_OK;
 }
 
 // The counter of bulk-copy timeouts: one word per device in a device variable of the library (nothing is allocated).

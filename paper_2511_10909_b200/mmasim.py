@@ -20,7 +20,7 @@ FMT = {n: i for i, n in enumerate(
 ACC = {"fp32": 0, "fp16": 1, "fp64": 2}
 FAMILY = ["fma", "ftz", "e", "t", "st", "gst", "tr", "gtr"]
 RHO = ["", "RZ-FP32", "RZ-E8M13", "RNE-FP32", "RNE-FP16"]
-FORCE_GENERIC = 1
+FORCE_GENERIC, LARGE_TILES = 1, 2
 
 
 class MmasimError(RuntimeError):
@@ -168,14 +168,13 @@ def _acc_dtype(model: Model):
     return {8: torch.int64, 4: torch.int32, 2: torch.int16}[model.acc_bytes]
 
 
-def _make_opts(sfa=None, sfb=None, k_chunk=0, row_scale=None, col_scale=None, force_generic=False,
-               lda=0, ldb=0, ldc=0, ldd=0):
+def _make_opts(sfa=None, sfb=None, k_chunk=0, row_scale=None, col_scale=None, flags=0, lda=0, ldb=0, ldc=0, ldd=0):
     o = _GemmOpts()
     o.lda, o.ldb, o.ldc, o.ldd = lda, ldb, ldc, ldd
     o.sfa, o.sfb = sfa, sfb
     o.k_chunk = k_chunk
     o.row_scale, o.col_scale = row_scale, col_scale
-    o.flags = FORCE_GENERIC if force_generic else 0
+    o.flags = flags
     return o
 
 
@@ -208,13 +207,14 @@ def _vector(t, name, n, bytes_per, device):
 
 
 def gemm(model: Model, A, B, C=None, out=None, *, M=None, N=None, K=None, sfa=None, sfb=None, k_chunk=0,
-         row_scale=None, col_scale=None, force_generic=False, stream=None):
+         row_scale=None, col_scale=None, force_generic=False, large_tiles=False, stream=None):
     """D = Phi(A, B, C) on CUDA tensors of raw words.
 
     A: M x K, B: N x K (each row is one column of the paper's K x N matrix), C/D: M x N words of the accumulator
     type (integer tensors of the element width; FP4 of the GST models packed two per byte, so A is M x K/2 uint8).
     Row-strided views are accepted (the row stride becomes the leading dimension lda / ldb / ldc / ldd of
     mmasim_gemm_ex); the inner dimension must be contiguous.  Returns D (allocated with torch if ``out`` is None).
+    ``force_generic`` and ``large_tiles`` pick kernels for cross-checks (the flags of mmasim_gemm_opts).
     """
     import torch
     if not A.is_cuda:
@@ -240,12 +240,12 @@ def gemm(model: Model, A, B, C=None, out=None, *, M=None, N=None, K=None, sfa=No
     _vector(row_scale, "row_scale", M, 4, dev)
     _vector(col_scale, "col_scale", N, 4, dev)
     strided = (lda, ldb) != (K, K) or (C is not None and ldc != N) or ldd != N
-    plain = sfa is None and not k_chunk and row_scale is None and not force_generic and not strided
+    flags = (FORCE_GENERIC if force_generic else 0) | (LARGE_TILES if large_tiles else 0)
+    plain = sfa is None and not k_chunk and row_scale is None and not flags and not strided
     if plain:
         _check(_lib.mmasim_gemm(model._h, M, N, K, _ptr(A), _ptr(B), _ptr(C), _ptr(out), _stream(stream)))
     else:
-        o = _make_opts(_ptr(sfa), _ptr(sfb), k_chunk, _ptr(row_scale), _ptr(col_scale), force_generic,
-                       lda, ldb, ldc, ldd)
+        o = _make_opts(_ptr(sfa), _ptr(sfb), k_chunk, _ptr(row_scale), _ptr(col_scale), flags, lda, ldb, ldc, ldd)
         _check(_lib.mmasim_gemm_ex(model._h, M, N, K, _ptr(A), _ptr(B), _ptr(C), _ptr(out), byref(o), _stream(stream)))
     return out
 
@@ -265,7 +265,7 @@ def gemm_noalloc(model: Model, A, B, C, out, *, k_chunk=0, row_scale=None, col_s
     ldd = _matrix(out, "out", M, N, model.acc_bytes * 8, dev)
     _vector(row_scale, "row_scale", M, 4, dev)
     _vector(col_scale, "col_scale", N, 4, dev)
-    o = _make_opts(None, None, k_chunk, _ptr(row_scale), _ptr(col_scale), False, lda, ldb, ldc, ldd)
+    o = _make_opts(None, None, k_chunk, _ptr(row_scale), _ptr(col_scale), 0, lda, ldb, ldc, ldd)
     _check(_lib.mmasim_gemm_noalloc(model._h, M, N, K, _ptr(A), _ptr(B), _ptr(C), _ptr(out), byref(o), _stream(stream)))
     return out
 
@@ -314,7 +314,7 @@ def gemm_host(model: Model, A, B, C=None, *, K=None, sfa=None, sfb=None, k_chunk
         out = np.empty((M, N), dtype={8: np.uint64, 4: np.uint32, 2: np.uint16}[model.acc_bytes])
     ld = lambda x: 0 if x is None else x.strides[0] // x.itemsize
     p = lambda x: None if x is None else c_void_p(x.ctypes.data)
-    o = _make_opts(p(sfa), p(sfb), k_chunk, p(row_scale), p(col_scale), False,
+    o = _make_opts(p(sfa), p(sfb), k_chunk, p(row_scale), p(col_scale), 0,
                    ld(A) * per_word, ld(B) * per_word, ld(C), ld(out))
     _check(_lib.mmasim_gemm_host(model._h, M, N, K, p(A), p(B), p(C), p(out), byref(o)))
     return out
