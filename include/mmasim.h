@@ -103,8 +103,9 @@ typedef struct {
                                    in Sections 2.2 and 6.3; FP32-accumulator FDPA models only) */
     const float* row_scale;     /* device, M floats or NULL */
     const float* col_scale;     /* device, N floats or NULL: D = fl32(fl32(row_scale[i]*col_scale[j]) * d) */
-    int32_t flags;              /* MMASIM_GEMM_FORCE_GENERIC: skip the tuned kernels; MMASIM_GEMM_LARGE_TILES: skip those for
-                                   small tiles where a large-tile kernel serves the call (both are used to cross-check) */
+    int32_t flags;              /* MMASIM_GEMM_FORCE_GENERIC: skip the tuned kernels; MMASIM_GEMM_LARGE_TILES: skip the
+                                   small-tile and matrix-instruction kernels where a large-tile one serves the call (both are
+                                   used to cross-check) */
 } mmasim_gemm_opts;
 #define MMASIM_GEMM_FORCE_GENERIC 1
 #define MMASIM_GEMM_LARGE_TILES 2
@@ -263,7 +264,8 @@ int mmasim_error_stats(int acc_fmt, int64_t n, const void* D, const double* ref,
  *                     multiply-add lanes are counted): whether the FP32 and the integer pipe issue side by side. */
 int mmasim_int_peak(int kind, int64_t blocks, int64_t iters, void* sink, int32_t* ops_per_round, void* stream);
 
-/* Name of the kernel variant the last mmasim_gemm* call on this thread dispatched to ("generic", ...). */
+/* Whose arithmetic the last mmasim_gemm* call on this thread ran: the kernel family ("tfdpa_f16", "gstfdpa", ...; the same name for
+ * its large-tile, small-tile and matrix-instruction kernels), or "generic". */
 const char* mmasim_last_kernel(void);
 
 /* The tuned fused-summation kernels bring decoded operand blocks into shared memory with bulk copies and wait for each

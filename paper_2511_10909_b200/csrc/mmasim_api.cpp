@@ -60,6 +60,7 @@ int check_k(const DevModel& m, int64_t K) {
 int run_gemm(const mmasim_model* model, const GemmArgs& g, int flags, cudaStream_t stream) {
     const DevModel& m = model->dev;
     if (!(flags & MMASIM_GEMM_FORCE_GENERIC) && !m.literal_emax) {
+        if (!(flags & MMASIM_GEMM_LARGE_TILES) && umma_supported(m, g)) return launch_umma(m, g, stream);
         const DirectSize size = (flags & MMASIM_GEMM_LARGE_TILES) && fast_tfdpa_supported(m, g) ? DIRECT_NONE : direct_size(m, g);
         if (size != DIRECT_NONE) return launch_direct(m, g, size, stream);
         if (fast_tfdpa_supported(m, g)) return launch_fast_tfdpa(m, g, stream);

@@ -8,6 +8,15 @@
 
 namespace mmasim {
 
+// Whether the CTA's tile is the emulation's to compute (GemmArgs::least_a): called by whole warps, the same answer in all.
+__device__ __forceinline__ bool tile_wanted(const GemmArgs& g, int64_t row0, int rows, int64_t col0, int cols) {
+    if (!g.least_a) return true;
+    int a = 1 << 20, b = 1 << 20;
+    for (int64_t i = row0 + threadIdx.x % 32; i < min(row0 + rows, g.M); i += 32) a = min(a, g.least_a[i]);
+    for (int64_t j = col0 + threadIdx.x % 32; j < min(col0 + cols, g.N); j += 32) b = min(b, g.least_b[j]);
+    return __reduce_min_sync(0xFFFFFFFFu, a) + __reduce_min_sync(0xFFFFFFFFu, b) < -126;
+}
+
 // ---------------------------------------------------------------------------------------------------------
 // Decoded element: one 32-bit word.
 //   bits  0..11  integer significand (hidden bit included for normal numbers), at most 11 bits here

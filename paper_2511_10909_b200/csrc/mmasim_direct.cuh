@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(32 * (WR * WC + PW), min_ctas(TM * CN, L, WR *
     const int tid = int(threadIdx.x) - 32 * NC;         // (of a staging thread)
     const int wr = warp / WC, wc = warp % WC, gq = lane >> 2, tq = lane & 3;
     const int64_t row0 = int64_t(blockIdx.y) * BM, col0 = int64_t(blockIdx.x) * BN;
+    if (T && !tile_wanted(g, row0, BM, col0, BN)) return;
     auto row_at = [&](int r) { return wr * 8 * TM + 8 * r + gq; };                       // inside the CTA tile
     auto col_at = [&](int c) { return wc * 8 * CN + 8 * (c >> 1) + 2 * tq + (c & 1); };
     const FmtDesc fa = fmt_desc(m.fmt_a), fb = fmt_desc(m.fmt_b);

@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(NT, 2) gst_kernel(DevModel m, GemmArgs g) {
     const int tid = threadIdx.x;
     const int tx = tid % 16, ty = tid / 16;
     const int64_t row0 = int64_t(blockIdx.y) * BM, col0 = int64_t(blockIdx.x) * BN;
+    if (!tile_wanted(g, row0, BM, col0, BN)) return;
 
     uint32_t cw[TM][TN];                            // the accumulator of each output: a finite FP32 word
     uint32_t sp_nan = 0u, sp_pinf = 0u, sp_ninf = 0u;   // sticky special values (bit r * TN + c)
