@@ -1,4 +1,4 @@
-"""Builds libmmasim.so in-tree with nvcc for sm_100a (no JIT cache, no pip install)."""
+"""Builds libmmasim.so (nvcc, sm_100a) and the Python call path _mmasim_py.so (g++, against torch) in-tree."""
 from __future__ import annotations
 
 import os
@@ -8,6 +8,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmmasim.so")
+PY_EXT = os.path.join(HERE, "_mmasim_py.so")
 SOURCES = ["mmasim_api.cpp", "mmasim_registry.cpp", "mmasim_generic.cu", "mmasim_tfdpa_fast.cu",
            "mmasim_tfdpa_fast_lut8.cu", "mmasim_tfdpa_fast_f16.cu", "mmasim_tfdpa_fast_bf16.cu", "mmasim_direct_8.cu", "mmasim_direct_16.cu", "mmasim_direct_32.cu", "mmasim_direct_amd.cu", "mmasim_trfdpa_f64.cu", "mmasim_efdpa_f64.cu", "mmasim_fp_fast.cu", "mmasim_gst_fast.cu", "mmasim_umma.cu",
            "mmasim_dot_stream.cu", "mmasim_peak.cu", "mmasim_hw_mma.cu", "mmasim_hw_umma.cu", "mmasim_stats.cu"]
@@ -24,11 +25,22 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not (os.path.exists(LIB) and os.path.exists(PY_EXT)):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS] + [__file__]
+    t = min(os.path.getmtime(LIB), os.path.getmtime(PY_EXT))
+    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS + ["mmasim_py.cpp"]] + [__file__]
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def _py_ext_cmd() -> list[str]:
+    import sysconfig
+    import torch
+    root = os.path.dirname(torch.__file__)
+    inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"), "/usr/local/cuda/include",
+           sysconfig.get_paths()["include"]]
+    return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            *(f"-I{d}" for d in inc), os.path.join(CSRC, "mmasim_py.cpp"), "-o", PY_EXT, "-L" + os.path.join(root, "lib"),
+            "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -44,12 +56,13 @@ def build(force: bool = False, verbose: bool = False) -> str:
             cmd.insert(1, "-Xptxas=-v")
         procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
         objs.append(obj)
+    procs.append(("mmasim_py.cpp", subprocess.Popen(_py_ext_cmd(), stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
     for src, p in procs:
         out, _ = p.communicate()
         if verbose or p.returncode:
             sys.stderr.write(out)
         if p.returncode:
-            raise RuntimeError(f"nvcc failed on {src}")
+            raise RuntimeError(f"compiling {src} failed:\n{out}")
     link = [_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", LIB, *objs, "-lcudart"]
     subprocess.run(link, check=True)
     return LIB

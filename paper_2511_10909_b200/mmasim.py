@@ -1,6 +1,7 @@
-"""ctypes binding of libmmasim.so: argument marshalling only, every step of the path runs in the CUDA kernels.
+"""Binding of libmmasim.so: argument marshalling only, every step of the path runs in the CUDA kernels.
 
-PyTorch is used for device memory and streams.  There is no CPU fallback: if the shared library is missing the
+ctypes for most entry points; ordinary calls of gemm and dot_batch go through a small extension module (csrc/mmasim_py.cpp)
+that checks the tensors, allocates the output and calls the library without Python in between.  PyTorch is used for device memory and streams.  There is no CPU fallback: if the shared library is missing the
 import fails, and every compute call needs CUDA tensors.
 """
 from __future__ import annotations
@@ -88,6 +89,25 @@ def _load():
 _lib = _load()
 
 
+_fast = None
+
+
+def _load_fast():
+    """The extension module, loaded with the first call on tensors (it needs torch's libraries in the process)."""
+    global _fast
+    import importlib.util
+    import torch  # noqa: F401
+    path = os.path.join(_HERE, "_mmasim_py.so")
+    if not os.path.exists(path):
+        raise ImportError(f"{path} is missing: build it with `python -m paper_2511_10909_b200.build`")
+    spec = importlib.util.spec_from_file_location("_mmasim_py", path)
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    mod.bind(*(ctypes.cast(f, c_void_p).value for f in (_lib.mmasim_gemm_ex, _lib.mmasim_dot_batch, _lib.mmasim_model_info)))
+    _fast = mod
+    return mod
+
+
 def library_path() -> str:
     return _LIB_PATH
 
@@ -117,7 +137,7 @@ class Model:
         h = _lib.mmasim_create_model_ex(ARCH[arch], FMT[in_fmt], FMT[self.b_fmt], ACC[acc], ov)
         if not h:
             raise MmasimError(2, _lib.mmasim_last_error().decode())
-        self._h = c_void_p(h)
+        self._h, self._addr = c_void_p(h), h
         info = _Info()
         _check(_lib.mmasim_model_info(self._h, byref(info)))
         self.family = FAMILY[info.family]
@@ -159,8 +179,9 @@ def _ptr(t):
 
 def _stream(stream):
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return c_void_p(s.cuda_stream)
+    if stream is None:
+        return c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    return c_void_p(stream.cuda_stream)
 
 
 def _acc_dtype(model: Model):
@@ -216,6 +237,11 @@ def gemm(model: Model, A, B, C=None, out=None, *, M=None, N=None, K=None, sfa=No
     mmasim_gemm_ex); the inner dimension must be contiguous.  Returns D (allocated with torch if ``out`` is None).
     ``force_generic`` and ``large_tiles`` pick kernels for cross-checks (the flags of mmasim_gemm_opts).
     """
+    if stream is None and M is None and N is None:
+        D = (_fast or _load_fast()).gemm(model._addr, A, B, C, out, K, sfa, sfb, k_chunk, row_scale, col_scale,
+                                         (FORCE_GENERIC if force_generic else 0) | (LARGE_TILES if large_tiles else 0))
+        if D is not None:
+            return D
     import torch
     if not A.is_cuda:
         raise MmasimError(1, "mmasim.gemm needs CUDA tensors (no CPU fallback); use gemm_host for host buffers")
@@ -272,6 +298,10 @@ def gemm_noalloc(model: Model, A, B, C, out, *, k_chunk=0, row_scale=None, col_s
 
 def dot_batch(model: Model, A, B, C=None, out=None, *, stream=None):
     """d_t = Phi(a_t, b_t, c_t) for the n rows of A and B (contiguous n x K CUDA tensors of raw words)."""
+    if stream is None:
+        D = (_fast or _load_fast()).dot_batch(model._addr, A, B, C, out)
+        if D is not None:
+            return D
     import torch
     if not A.is_cuda:
         raise MmasimError(1, "mmasim.dot_batch needs CUDA tensors (no CPU fallback)")
