@@ -1,15 +1,18 @@
 // Streaming kernels for mmasim_dot_batch: n independent dot-product-accumulates d_t = Phi(a_t, b_t, c_t) (Equation 4),
 // the shape of the paper's probe vectors (Section 3.1).  One thread owns one dot product; nothing is shared between
 // dots, so the kernels are bound by HBM traffic (2 * K * element bytes + 8 bytes per dot).
-//   T-FDPA (Algorithm 7) for FP16 / BF16 / TF32 inputs, L in {4, 8, 16}, F in 23..25, rho in {RZ-FP32, RNE-FP16}
+//   T-FDPA (Algorithm 7) for FP16 / BF16 / TF32 inputs, L in {4, 8, 16}, F in 23..25, rho in {RZ-FP32, RNE-FP16}, and for E4M3 / E5M2
+//   inputs, L in {4, 8, 16, 32}, F = 13 (on the FP32 pipe) and F = 25
+//   TR-FDPA (Algorithm 10) for FP16 / BF16 / TF32 inputs, L in {4, 8}
 //   Phi_FTZ-AddMul (Algorithm 2) for FP16 / BF16 inputs, P in {2, 4}
 // Two ways to bring the rows in:
-//   staged - rows of 8, 16, 32, 64 or 128 bytes: the CTA's 128 rows of A and of B are one contiguous range each, copied
+//   staged - rows of 4, 8, 16, 32, 64 or 128 bytes: the CTA's 128 rows of A and of B are one contiguous range each, copied
 //            to shared memory with 16-byte asynchronous copies (consecutive threads, consecutive chunks: every
 //            sector of a request is used), chunks XOR-swizzled so that each thread then reads its own row without bank
 //            conflicts; several CTAs per SM keep the copies of one tile under the arithmetic of another
 //   direct - any other row length: each thread reads its row with 16-byte loads
-// Everything else (8-bit inputs, other families, odd shapes) uses the generic kernels.
+// Everything else (FP6 / FP4, mixed inputs, other families, odd shapes) uses the generic kernels, which take 2^20 dots of length 32 in
+// 312 us (Hopper E4M3) and 385 us (CDNA3 FP16).
 #include <cuda_fp16.h>
 #include "mmasim_tfdpa_fast.cuh"
 
@@ -33,6 +36,7 @@ struct GlobalRows {                      // row pointers into global memory
     __device__ __forceinline__ uint2 ld8(bool second, int byte_off) const {
         return *reinterpret_cast<const uint2*>((second ? b : a) + byte_off);
     }
+    __device__ __forceinline__ uint32_t ld4(bool second, int byte_off) const { return *reinterpret_cast<const uint32_t*>((second ? b : a) + byte_off); }
 };
 struct StagedRows {                      // this thread's rows inside the staged tile (shared memory, swizzled chunks)
     const unsigned char* a;              // start of the row's chunk group
@@ -44,20 +48,25 @@ struct StagedRows {                      // this thread's rows inside the staged
     __device__ __forceinline__ uint2 ld8(bool second, int byte_off) const {
         return *reinterpret_cast<const uint2*>((second ? b : a) + (((byte_off >> 4) ^ swz) << 4) + (byte_off & 8));
     }
+    __device__ __forceinline__ uint32_t ld4(bool second, int byte_off) const {
+        return *reinterpret_cast<const uint32_t*>((second ? b : a) + (((byte_off >> 4) ^ swz) << 4) + (byte_off & 12));
+    }
 };
 
-// L consecutive elements (L * BYTES is 8, 16, 32 or 64 bytes) as raw 32-bit words (two elements per word for the
-// 16-bit formats).
+// L consecutive elements (L * BYTES is 4, 8, 16, 32 or 64 bytes) as raw 32-bit words.
 template <int BYTES, int L, class Rows>
 __device__ __forceinline__ void load_raw(const Rows& rows, bool second, int elem_index, uint32_t (&raw)[L * BYTES / 4]) {
-    if (L * BYTES == 8) {
+    if (L * BYTES == 4) {
+        raw[0] = rows.ld4(second, elem_index * BYTES);
+    } else if (L * BYTES == 8) {
         const uint2 v = rows.ld8(second, elem_index * BYTES);
-        raw[0] = v.x; raw[1] = v.y;
+        raw[0] = v.x; raw[L * BYTES >= 8 ? 1 : 0] = v.y;
     } else {
 #pragma unroll
         for (int q = 0; q < L * BYTES / 16; ++q) {
             const uint4 v = rows.ld16(second, elem_index * BYTES + 16 * q);
-            raw[4 * q] = v.x; raw[4 * q + 1] = v.y; raw[4 * q + 2] = v.z; raw[4 * q + 3] = v.w;
+            constexpr int TOP = L * BYTES / 4 - 1;
+            raw[min(4 * q, TOP)] = v.x; raw[min(4 * q + 1, TOP)] = v.y; raw[min(4 * q + 2, TOP)] = v.z; raw[min(4 * q + 3, TOP)] = v.w;
         }
     }
 }
@@ -69,7 +78,7 @@ __device__ __forceinline__ void load_raw(const Rows& rows, bool second, int elem
 __device__ __forceinline__ void stage_issue(unsigned char* stage, const void* A, const void* B, int64_t t0, int nrows,
                                             int row_bytes) {
     const int tid = threadIdx.x;
-    const int lcpr = row_bytes >= 16 ? 31 - __clz(row_bytes >> 4) : 0;      // log2(chunks per row); rows of 8 bytes: two rows per chunk
+    const int lcpr = row_bytes >= 16 ? 31 - __clz(row_bytes >> 4) : 0;      // log2(chunks per row); rows of 4 or 8 bytes: several rows per chunk
     const int cmask = (1 << lcpr) - 1;
     const int lrpl = 3 - lcpr;                                              // log2(rows per 128-byte line)
     const int bytes = nrows * row_bytes;
@@ -88,9 +97,10 @@ __device__ __forceinline__ void stage_issue(unsigned char* stage, const void* A,
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(da), "l"(ga + (int64_t(g) << 4)) : "memory");
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(db), "l"(gb + (int64_t(g) << 4)) : "memory");
     }
-    if ((bytes & 8) && tid == 0) {                                          // 8-byte rows, odd row count: the last row
-        *reinterpret_cast<uint2*>(sa + bytes - 8) = *reinterpret_cast<const uint2*>(ga + bytes - 8);
-        *reinterpret_cast<uint2*>(sb + bytes - 8) = *reinterpret_cast<const uint2*>(gb + bytes - 8);
+    if (tid < ((bytes >> 2) & 3)) {                                         // short rows: the last ones, by words
+        const int at = (bytes & ~15) + 4 * tid;
+        *reinterpret_cast<uint32_t*>(sa + at) = *reinterpret_cast<const uint32_t*>(ga + at);
+        *reinterpret_cast<uint32_t*>(sb + at) = *reinterpret_cast<const uint32_t*>(gb + at);
     }
 }
 
@@ -133,6 +143,55 @@ __device__ __forceinline__ double trunc_scaled(double p, double scale, int sign_
     return __hiloint2double(__double2hiint(n) | (sign_word & int(0x80000000u)), __double2loint(n));
 }
 
+constexpr int NO_EXP = -100000;
+// Step 1 of a block: its exact products, and the return value, the largest exponent sum (NO_EXP: no nonzero product).
+template <int EK, int L, class Rows>
+__device__ __forceinline__ int products(const Rows& rows, int k0, float (&pf)[EK == EK_F16 ? L : 1], double (&pd)[EK == EK_F16 ? 1 : L]) {
+    using E = Elem<EK>;
+    constexpr int NRAW = L * E::BYTES / 4;
+            uint32_t ra[NRAW], rb[NRAW];
+            load_raw<E::BYTES, L>(rows, false, k0, ra);
+            load_raw<E::BYTES, L>(rows, true, k0, rb);
+            // Step 1: exact products (as FP32 for FP16 inputs, whose products stay inside the FP32 range; as FP64
+            // otherwise) and the largest exponent sum Exp(a) + Exp(b), with Exp = max(field, 1) - bias, over the products
+            // that are not zero (a zero term has no exponent): lanes of a zero product are masked to 0 before the maximum.
+            int e_prod;
+            if (E::BYTES == 2) {
+                constexpr uint32_t EXPM = ((1u << E::EBITS) - 1u) << E::MBITS, ONE = 1u << E::MBITS;
+                uint32_t mx = 0u;
+    #pragma unroll
+                for (int q = 0; q < NRAW; ++q) {
+                    const uint32_t ea = __vmaxu2(ra[q] & (EXPM * 0x10001u), ONE * 0x10001u);
+                    const uint32_t eb = __vmaxu2(rb[q] & (EXPM * 0x10001u), ONE * 0x10001u);
+                    // 1 per lane where both elements are nonzero, widened to a lane mask
+                    const uint32_t live = __vminu2(__vminu2(ra[q] & 0x7FFF7FFFu, rb[q] & 0x7FFF7FFFu), 0x00010001u) * 0xFFFFu;
+                    mx = __vmaxu2(mx, (ea + eb) & live);      // field sums stay below 2^16: no carry between the lanes
+                    if (EK == EK_F16) {
+                        const float2 fa = __half22float2(*reinterpret_cast<const __half2*>(&ra[q]));
+                        const float2 fb = __half22float2(*reinterpret_cast<const __half2*>(&rb[q]));
+                        pf[2 * q < L ? 2 * q : 0] = __fmul_rn(fa.x, fb.x);
+                        pf[2 * q + 1 < L ? 2 * q + 1 : 0] = __fmul_rn(fa.y, fb.y);
+                    } else {
+                        pd[2 * q < L ? 2 * q : 0] = __dmul_rn(double(__uint_as_float(ra[q] << 16)), double(__uint_as_float(rb[q] << 16)));
+                        pd[2 * q + 1 < L ? 2 * q + 1 : 0] = __dmul_rn(double(__uint_as_float(ra[q] & 0xFFFF0000u)), double(__uint_as_float(rb[q] & 0xFFFF0000u)));
+                    }
+                }
+                const uint32_t m1 = max(mx & 0xFFFFu, mx >> 16);
+                e_prod = m1 ? int(m1 >> E::MBITS) - 2 * E::BIAS : NO_EXP;
+            } else {
+                uint32_t mx = 0u;
+    #pragma unroll
+                for (int k = 0; k < L; ++k) {
+                    const uint32_t xa = ra[k] & 0x7FFFE000u, xb = rb[k] & 0x7FFFE000u;
+                    const uint32_t es = max(xa >> 23, 1u) + max(xb >> 23, 1u);
+                    mx = max(mx, (xa && xb) ? es : 0u);
+                    pd[EK == EK_F16 ? 0 : k] = __dmul_rn(double(__uint_as_float(ra[k] & 0xFFFFE000u)), double(__uint_as_float(rb[k] & 0xFFFFE000u)));
+                }
+                e_prod = mx ? int(mx) - 2 * E::BIAS : NO_EXP;
+            }
+    return e_prod;
+}
+
 // T-FDPA (Algorithm 7) on the FP64 pipe, the chain of Algorithm 5 for one dot product.  A double holds every quantity
 // of a block exactly: products of two 11-bit (8-bit) significands, their scaling by 2^(F - e_max) (a power of two, no
 // underflow in the FP64 range), the truncated terms (< 2^27) and their sum (< 2^32).  Infinities and NaNs need no
@@ -141,53 +200,11 @@ __device__ __forceinline__ double trunc_scaled(double p, double scale, int sign_
 // word when the sum is not finite.  Only e_max stays on the integer pipe (two terms per instruction, 16-bit lanes).
 template <int EK, int L, int RHO, class Rows>
 __device__ __forceinline__ uint32_t tfdpa_dot(const Rows& rows, int K, int F, uint32_t cw) {
-    using E = Elem<EK>;
     constexpr bool ACC16 = RHO == RHO_RNE_FP16;
-    constexpr int NRAW = L * E::BYTES / 4;
     for (int k0 = 0; k0 < K; k0 += L) {
-        uint32_t ra[NRAW], rb[NRAW];
-        load_raw<E::BYTES, L>(rows, false, k0, ra);
-        load_raw<E::BYTES, L>(rows, true, k0, rb);
-        // Step 1: exact products (as FP32 for FP16 inputs, whose products stay inside the FP32 range; as FP64
-        // otherwise) and the largest exponent sum Exp(a) + Exp(b), with Exp = max(field, 1) - bias, over the products
-        // that are not zero (a zero term has no exponent): lanes of a zero product are masked to 0 before the maximum.
-        float pf[E::BYTES == 2 && EK == EK_F16 ? L : 1];
+        float pf[EK == EK_F16 ? L : 1];
         double pd[EK == EK_F16 ? 1 : L];
-        constexpr int NO_EXP = -100000;
-        int e_prod;
-        if (E::BYTES == 2) {
-            constexpr uint32_t EXPM = ((1u << E::EBITS) - 1u) << E::MBITS, ONE = 1u << E::MBITS;
-            uint32_t mx = 0u;
-#pragma unroll
-            for (int q = 0; q < NRAW; ++q) {
-                const uint32_t ea = __vmaxu2(ra[q] & (EXPM * 0x10001u), ONE * 0x10001u);
-                const uint32_t eb = __vmaxu2(rb[q] & (EXPM * 0x10001u), ONE * 0x10001u);
-                // 1 per lane where both elements are nonzero, widened to a lane mask
-                const uint32_t live = __vminu2(__vminu2(ra[q] & 0x7FFF7FFFu, rb[q] & 0x7FFF7FFFu), 0x00010001u) * 0xFFFFu;
-                mx = __vmaxu2(mx, (ea + eb) & live);      // field sums stay below 2^16: no carry between the lanes
-                if (EK == EK_F16) {
-                    const float2 fa = __half22float2(*reinterpret_cast<const __half2*>(&ra[q]));
-                    const float2 fb = __half22float2(*reinterpret_cast<const __half2*>(&rb[q]));
-                    pf[2 * q < L ? 2 * q : 0] = __fmul_rn(fa.x, fb.x);
-                    pf[2 * q + 1 < L ? 2 * q + 1 : 0] = __fmul_rn(fa.y, fb.y);
-                } else {
-                    pd[2 * q < L ? 2 * q : 0] = __dmul_rn(double(__uint_as_float(ra[q] << 16)), double(__uint_as_float(rb[q] << 16)));
-                    pd[2 * q + 1 < L ? 2 * q + 1 : 0] = __dmul_rn(double(__uint_as_float(ra[q] & 0xFFFF0000u)), double(__uint_as_float(rb[q] & 0xFFFF0000u)));
-                }
-            }
-            const uint32_t m1 = max(mx & 0xFFFFu, mx >> 16);
-            e_prod = m1 ? int(m1 >> E::MBITS) - 2 * E::BIAS : NO_EXP;
-        } else {
-            uint32_t mx = 0u;
-#pragma unroll
-            for (int k = 0; k < L; ++k) {
-                const uint32_t xa = ra[k] & 0x7FFFE000u, xb = rb[k] & 0x7FFFE000u;
-                const uint32_t es = max(xa >> 23, 1u) + max(xb >> 23, 1u);
-                mx = max(mx, (xa && xb) ? es : 0u);
-                pd[EK == EK_F16 ? 0 : k] = __dmul_rn(double(__uint_as_float(ra[k] & 0xFFFFE000u)), double(__uint_as_float(rb[k] & 0xFFFFE000u)));
-            }
-            e_prod = mx ? int(mx) - 2 * E::BIAS : NO_EXP;
-        }
+        const int e_prod = products<EK, L>(rows, k0, pf, pd);
         const uint32_t cfield = ACC16 ? (cw >> 10) & 0x1Fu : (cw >> 23) & 0xFFu;
         const int e_c = (cw & (ACC16 ? 0x7FFFu : 0x7FFFFFFFu)) ? int(max(cfield, 1u)) - (ACC16 ? 15 : 127) : NO_EXP;
         const double cd = ACC16 ? double(__half2float(__ushort_as_half((unsigned short)cw))) : double(__uint_as_float(cw));
@@ -217,17 +234,119 @@ __device__ __forceinline__ uint32_t tfdpa_dot(const Rows& rows, int K, int F, ui
     return positive_zero(cw, ACC16 ? 0x7FFFu : 0x7FFFFFFFu);
 }
 
-template <int EK, int L, int RHO, bool STAGED>
-__global__ void __launch_bounds__(DOT_THREADS)
-dot_tfdpa_kernel(DevModel m, int64_t n, int64_t K, const void* A, const void* B, const void* C, void* D) {
+// TR-FDPA (Algorithm 10; F = 24, F2 = 31, RNE-FP32) the same way: the truncated sum T of the products at their own maximum, then T
+// and the accumulator rounded down to the grid of the larger exponent, each by one fused multiply-add, and one conversion.
+template <int EK, int L, class Rows>
+__device__ __forceinline__ uint32_t trfdpa_dot(const Rows& rows, int K, uint32_t cw) {
+    constexpr int F = 24, F2 = 31;
+    constexpr double M = 6755399441055744.0;              // 1.5 * 2^52: one ulp = 1
+    for (int k0 = 0; k0 < K; k0 += L) {
+        float pf[EK == EK_F16 ? L : 1];
+        double pd[EK == EK_F16 ? 1 : L];
+        const int e_prod = products<EK, L>(rows, k0, pf, pd);
+        const int e_max = max(e_prod, -400);
+        const double scale = __hiloint2double((1023 + F - e_max) << 20, 0);
+        double T0 = 0.0, T1 = 0.0;
+#pragma unroll
+        for (int k = 0; k < L; ++k) {
+            double p = EK == EK_F16 ? double(pf[EK == EK_F16 ? k : 0]) : pd[EK == EK_F16 ? 0 : k];
+            if (EK != EK_F16 && fabs(p) >= 3.402823669209385e38 && p == p)       // a product of 2^128 or more is an infinity (Section 4.2)
+                p = __hiloint2double((__double2hiint(p) & int(0x80000000u)) | 0x7FF00000, 0);
+            const double t = trunc_scaled(p, scale, __double2hiint(p));
+            if (k & 1) T1 += t; else T0 += t;
+        }
+        const double c = double(__uint_as_float(cw));
+        const uint32_t cfield = (cw >> 23) & 0xFFu;
+        const int E = max(e_max, (cw & 0x7FFFFFFFu) ? int(max(cfield, 1u)) - 127 : NO_EXP);
+        // T counts 2^(e_max - F); onto the grid 2^(E - F2), c onto 2^(E - F)
+        const double T2 = __fma_rd(T0 + T1, __hiloint2double((1023 + e_max - F + F2 - E) << 20, 0), M) - M;
+        const double c2 = __fma_rd(c, __hiloint2double((1023 + F - E) << 20, 0), M) - M;
+        const double v = __dmul_rn(__fma_rn(c2, double(1 << (F2 - F)), T2), __hiloint2double((1023 + E - F2) << 20, 0));
+        cw = (v != v) ? 0x7FC00000u : __float_as_uint(__double2float_rn(v));
+    }
+    return cw;
+}
+
+// T-FDPA for 8-bit inputs.  The exponents of four elements are two words of 16-bit lanes.  F = 13: products, scaled terms (below 2^15)
+// and sums (below 2^21) are exact in FP32, where the floor goes onto 2^23; F = 25: FP64, as above.
+template <bool E5M2>
+__device__ __forceinline__ float2 two_floats(uint32_t w, int half) {
+    uint32_t h;
+    const unsigned short p = (unsigned short)(w >> (16 * half));
+    if (E5M2) asm("cvt.rn.f16x2.e5m2x2 %0, %1;" : "=r"(h) : "h"(p));
+    else asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h) : "h"(p));
+    return __half22float2(*reinterpret_cast<const __half2*>(&h));
+}
+template <bool E5M2, bool F13, int L, int RHO, class Rows>
+__device__ __forceinline__ uint32_t tfdpa8_dot(const Rows& rows, int K, uint32_t cw) {
     constexpr bool ACC16 = RHO == RHO_RNE_FP16;
-    extern __shared__ __align__(16) unsigned char dot_smem[];
-    const int row_bytes = int(K) * Elem<EK>::BYTES;
-    const int F = m.F;
+    constexpr int F = F13 ? 13 : 25, NRAW = L / 4, MB = E5M2 ? 2 : 3, BIAS = E5M2 ? 15 : 7;
+    constexpr uint32_t EXPM = (0x7Fu >> MB << MB) * 0x10001u, ONE = (1u << MB) * 0x10001u;
+    for (int k0 = 0; k0 < K; k0 += L) {
+        uint32_t ra[NRAW], rb[NRAW], mx = 0u;
+        load_raw<1, L>(rows, false, k0, ra);
+        load_raw<1, L>(rows, true, k0, rb);
+        float p[L];
+#pragma unroll
+        for (int q = 0; q < NRAW; ++q) {
+#pragma unroll
+            for (int odd = 0; odd < 2; ++odd) {
+                const uint32_t xa = ra[q] >> (8 * odd), xb = rb[q] >> (8 * odd);
+                const uint32_t live = __vminu2(__vminu2(xa & 0x007F007Fu, xb & 0x007F007Fu), 0x00010001u) * 0xFFFFu;
+                mx = __vmaxu2(mx, (__vmaxu2(xa & EXPM, ONE) + __vmaxu2(xb & EXPM, ONE)) & live);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float2 fa = two_floats<E5M2>(ra[q], h), fb = two_floats<E5M2>(rb[q], h);
+                p[4 * q + 2 * h] = __fmul_rn(fa.x, fb.x);
+                p[4 * q + 2 * h + 1] = __fmul_rn(fa.y, fb.y);
+            }
+        }
+        const uint32_t m1 = max(mx & 0xFFFFu, mx >> 16);
+        const int e_prod = m1 ? int(m1 >> MB) - 2 * BIAS : NO_EXP;
+        const uint32_t cfield = ACC16 ? (cw >> 10) & 0x1Fu : (cw >> 23) & 0xFFu;
+        const int e_c = (cw & (ACC16 ? 0x7FFFu : 0x7FFFFFFFu)) ? int(max(cfield, 1u)) - (ACC16 ? 15 : 127) : NO_EXP;
+        const float cf = ACC16 ? __half2float(__ushort_as_half((unsigned short)cw)) : __uint_as_float(cw);
+        if (F13) {
+            // without a nonzero product the sum is c alone, and any scale that keeps its bits will do (a NaN product stays one)
+            const bool none = e_prod == NO_EXP;
+            const int emax = none ? 0 : max(e_prod, e_c);
+            const float scale = __uint_as_float(uint32_t(127 + F - emax) << 23);
+            float S0 = 0.f, S1 = 0.f;
+            auto term = [&](float x) {
+                const float n = __fadd_rn(__fmaf_rd(fabsf(x), scale, 8388608.f), -8388608.f);
+                return __uint_as_float(__float_as_uint(n) | (__float_as_uint(x) & 0x80000000u));
+            };
+#pragma unroll
+            for (int k = 0; k < L; k += 2) { S0 = __fadd_rn(S0, term(p[k])); S1 = __fadd_rn(S1, term(p[k + 1])); }
+            const float S = __fadd_rn(S0, S1);
+            const float v = none ? __fadd_rn(cf, S) : __fmul_rn(__fadd_rn(S, term(cf)), __uint_as_float(uint32_t(127 + emax - F) << 23));
+            if (ACC16) cw = (v != v) ? 0x7FFFu : uint32_t(__half_as_ushort(__float2half_rn(v)));
+            else cw = (v != v) ? 0x7FFFFFFFu : __float_as_uint(v) & (RHO == RHO_RZ_E8M13 ? 0xFFFFFC00u : 0xFFFFFFFFu);
+        } else {
+            const int emax = max(max(e_prod, e_c), -400);
+            const double scale = __hiloint2double((1023 + F - emax) << 20, 0), cd = double(cf);
+            double S0 = trunc_scaled(cd, scale, __double2hiint(cd)), S1 = 0.0;
+#pragma unroll
+            for (int k = 0; k < L; ++k) {
+                const double t = trunc_scaled(double(p[k]), scale, __float_as_int(p[k]));
+                if (k & 1) S1 += t; else S0 += t;
+            }
+            const double v = __dmul_rn(S0 + S1, __hiloint2double((1023 + emax - F) << 20, 0));
+            if (ACC16) cw = (v != v) ? 0x7FFFu : uint32_t(__half_as_ushort(__double2half(v)));
+            else if (fabs(v) >= 3.402823669209385e38) cw = (__double2hiint(v) < 0 ? 0xFF800000u : 0x7F800000u);
+            else cw = (v != v) ? 0x7FFFFFFFu : __float_as_uint(__double2float_rz(v));
+        }
+    }
+    return positive_zero(cw, ACC16 ? 0x7FFFu : 0x7FFFFFFFu);
+}
+
+// One dot product per thread through `body(rows, c)`.
+template <int BYTES, bool ACC16, bool STAGED, class Body>
+__device__ __forceinline__ void one_dot(unsigned char* smem, int64_t n, int64_t K, const void* A, const void* B, const void* C, void* D, Body body) {
+    const int row_bytes = int(K) * BYTES;
     if (STAGED) {
-        staged_tile<ACC16>(dot_smem, n, row_bytes, A, B, C, D, [&](const StagedRows& rows, int64_t, uint32_t c) {
-            return tfdpa_dot<EK, L, RHO>(rows, int(K), F, c);
-        });
+        staged_tile<ACC16>(smem, n, row_bytes, A, B, C, D, [&](const StagedRows& rows, int64_t, uint32_t c) { return body(rows, c); });
     } else {
         const int64_t t = int64_t(blockIdx.x) * DOT_THREADS + threadIdx.x;
         if (t >= n) return;
@@ -236,10 +355,30 @@ dot_tfdpa_kernel(DevModel m, int64_t n, int64_t K, const void* A, const void* B,
         GlobalRows rows;
         rows.a = static_cast<const unsigned char*>(A) + t * row_bytes;
         rows.b = static_cast<const unsigned char*>(B) + t * row_bytes;
-        cw = tfdpa_dot<EK, L, RHO>(rows, int(K), F, cw);
+        cw = body(rows, cw);
         if (ACC16) static_cast<uint16_t*>(D)[t] = uint16_t(cw);
         else static_cast<uint32_t*>(D)[t] = cw;
     }
+}
+
+template <int EK, int L, bool STAGED>
+__global__ void __launch_bounds__(DOT_THREADS)
+dot_trfdpa_kernel(int64_t n, int64_t K, const void* A, const void* B, const void* C, void* D) {
+    extern __shared__ __align__(16) unsigned char dot_smem[];
+    one_dot<Elem<EK>::BYTES, false, STAGED>(dot_smem, n, K, A, B, C, D, [&](const auto& rows, uint32_t c) { return trfdpa_dot<EK, L>(rows, int(K), c); });
+}
+template <bool E5M2, bool F13, int L, int RHO, bool STAGED>
+__global__ void __launch_bounds__(DOT_THREADS)
+dot_tfdpa8_kernel(int64_t n, int64_t K, const void* A, const void* B, const void* C, void* D) {
+    extern __shared__ __align__(16) unsigned char dot_smem[];
+    one_dot<1, RHO == RHO_RNE_FP16, STAGED>(dot_smem, n, K, A, B, C, D, [&](const auto& rows, uint32_t c) { return tfdpa8_dot<E5M2, F13, L, RHO>(rows, int(K), c); });
+}
+
+template <int EK, int L, int RHO, bool STAGED>
+__global__ void __launch_bounds__(DOT_THREADS)
+dot_tfdpa_kernel(DevModel m, int64_t n, int64_t K, const void* A, const void* B, const void* C, void* D) {
+    extern __shared__ __align__(16) unsigned char dot_smem[];
+    one_dot<Elem<EK>::BYTES, RHO == RHO_RNE_FP16, STAGED>(dot_smem, n, K, A, B, C, D, [&](const auto& rows, uint32_t c) { return tfdpa_dot<EK, L, RHO>(rows, int(K), m.F, c); });
 }
 
 // FTZ-Add / FTZ-Mul (Algorithm 1) as the hardware's flush-to-zero operations: operands are never subnormal here
@@ -298,25 +437,12 @@ template <int EK, int P, int STEP, bool STAGED>
 __global__ void __launch_bounds__(DOT_THREADS)
 dot_ftz_kernel(int64_t n, int64_t K, const void* A, const void* B, const void* C, void* D) {
     extern __shared__ __align__(16) unsigned char dot_smem[];
-    const int row_bytes = int(K) * 2;
-    if (STAGED) {
-        staged_tile<false>(dot_smem, n, row_bytes, A, B, C, D, [&](const StagedRows& rows, int64_t, uint32_t c) {
-            return ftz_word(ftz_dot<EK, P, STEP>(rows, int(K), flush_c(c)));
-        });
-    } else {
-        const int64_t t = int64_t(blockIdx.x) * DOT_THREADS + threadIdx.x;
-        if (t >= n) return;
-        GlobalRows rows;
-        rows.a = static_cast<const unsigned char*>(A) + t * row_bytes;
-        rows.b = static_cast<const unsigned char*>(B) + t * row_bytes;
-        const float d = ftz_dot<EK, P, STEP>(rows, int(K), flush_c(C ? static_cast<const uint32_t*>(C)[t] : 0u));
-        static_cast<uint32_t*>(D)[t] = ftz_word(d);
-    }
+    one_dot<2, false, STAGED>(dot_smem, n, K, A, B, C, D, [&](const auto& rows, uint32_t c) { return ftz_word(ftz_dot<EK, P, STEP>(rows, int(K), flush_c(c))); });
 }
 
-// Rows of 8 to 128 bytes (a power of two) are staged through shared memory: 2 * 128 rows per CTA.
+// Rows of 4 to 128 bytes (a power of two) are staged through shared memory: 2 * 128 rows per CTA.
 bool staged_rows(int64_t row_bytes) {
-    return row_bytes == 8 || row_bytes == 16 || row_bytes == 32 || row_bytes == 64 || row_bytes == 128;
+    return row_bytes == 4 || row_bytes == 8 || row_bytes == 16 || row_bytes == 32 || row_bytes == 64 || row_bytes == 128;
 }
 
 template <class Kernel, class... Args>
@@ -354,6 +480,34 @@ cudaError_t launch_t_l(const DevModel& m, const GemmArgs& g, int L, cudaStream_t
     }
 }
 
+template <int EK, int L>
+cudaError_t launch_tr(const GemmArgs& g, cudaStream_t st) {
+    const int64_t rb = g.K * Elem<EK>::BYTES;
+    if (staged_rows(rb)) return launch_dot(dot_trfdpa_kernel<EK, L, true>, true, g.M, rb, st, g.M, g.K, g.A, g.B, g.C, g.D);
+    return launch_dot(dot_trfdpa_kernel<EK, L, false>, false, g.M, rb, st, g.M, g.K, g.A, g.B, g.C, g.D);
+}
+
+template <bool E5M2, bool F13, int L, int RHO>
+cudaError_t launch_8l(const GemmArgs& g, cudaStream_t st) {
+    if (staged_rows(g.K)) return launch_dot(dot_tfdpa8_kernel<E5M2, F13, L, RHO, true>, true, g.M, g.K, st, g.M, g.K, g.A, g.B, g.C, g.D);
+    return launch_dot(dot_tfdpa8_kernel<E5M2, F13, L, RHO, false>, false, g.M, g.K, st, g.M, g.K, g.A, g.B, g.C, g.D);
+}
+template <bool E5M2, bool F13, int RHO>
+cudaError_t launch_8r(const GemmArgs& g, int L, cudaStream_t st) {
+    switch (L) {
+        case 4: return launch_8l<E5M2, F13, 4, RHO>(g, st);
+        case 8: return launch_8l<E5M2, F13, 8, RHO>(g, st);
+        case 16: return launch_8l<E5M2, F13, 16, RHO>(g, st);
+        case 32: return launch_8l<E5M2, F13, 32, RHO>(g, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+template <bool E5M2>
+cudaError_t launch_8(const DevModel& m, const GemmArgs& g, int L, cudaStream_t st) {
+    if (m.F == 13) return m.rho == RHO_RNE_FP16 ? launch_8r<E5M2, true, RHO_RNE_FP16>(g, L, st) : launch_8r<E5M2, true, RHO_RZ_E8M13>(g, L, st);
+    return m.rho == RHO_RNE_FP16 ? launch_8r<E5M2, false, RHO_RNE_FP16>(g, L, st) : launch_8r<E5M2, false, RHO_RZ_FP32>(g, L, st);
+}
+
 template <int EK, int P>
 cudaError_t launch_ftz(const GemmArgs& g, cudaStream_t st) {
     const int64_t rb = g.K * 2;
@@ -371,6 +525,20 @@ cudaError_t launch_ftz(const GemmArgs& g, cudaStream_t st) {
 bool dot_stream_supported(const DevModel& m, const GemmArgs& g) {
     if (!g.dot_mode || m.fmt_a != m.fmt_b) return false;
     const int bytes = fmt_desc(m.fmt_a).storage_bits / 8;
+    if (m.family == FAM_T && (m.fmt_a == EF_E4M3 || m.fmt_a == EF_E5M2)) {
+        const int L = int(g.K < m.L ? g.K : m.L);
+        if (L != 4 && L != 8 && L != 16 && L != 32) return false;
+        if ((m.rho == RHO_RNE_FP16) != (m.acc == ACC_F16)) return false;
+        if (m.rho != RHO_RNE_FP16 && !(m.F == 13 && m.rho == RHO_RZ_E8M13) && !(m.F == 25 && m.rho == RHO_RZ_FP32)) return false;
+        if (m.F != 13 && m.F != 25) return false;
+        return g.K % (L < 16 ? L : 16) == 0;                        // every row starts on a vector-load boundary
+    }
+    if (m.family == FAM_TR) {
+        if (m.fmt_a != EF_F16 && m.fmt_a != EF_BF16 && m.fmt_a != EF_TF32) return false;
+        const int L = int(g.K < m.L ? g.K : m.L);
+        if ((L != 4 && L != 8) || m.F != 24 || m.F2 != 31 || m.rho != RHO_RNE_FP32 || m.inner_round || m.acc != ACC_F32) return false;
+        return (g.K * bytes) % (L * bytes >= 16 ? 16 : 8) == 0;
+    }
     if (m.family == FAM_T) {
         if (m.fmt_a != EF_F16 && m.fmt_a != EF_BF16 && m.fmt_a != EF_TF32) return false;
         const int L = int(g.K < m.L ? g.K : m.L);
@@ -386,10 +554,17 @@ bool dot_stream_supported(const DevModel& m, const GemmArgs& g) {
 
 int launch_dot_stream(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
     cudaError_t err = cudaErrorInvalidValue;
-    if (m.family == FAM_T) {
-        const int L = int(g.K < m.L ? g.K : m.L);
+    const int L = int(g.K < m.L ? g.K : m.L);
+    if (m.family == FAM_TR) {
+        set_kernel_name("dot_trfdpa");
+        if (m.fmt_a == EF_F16) err = L == 4 ? launch_tr<EK_F16, 4>(g, stream) : launch_tr<EK_F16, 8>(g, stream);
+        else if (m.fmt_a == EF_BF16) err = L == 4 ? launch_tr<EK_BF16, 4>(g, stream) : launch_tr<EK_BF16, 8>(g, stream);
+        else err = L == 4 ? launch_tr<EK_TF32, 4>(g, stream) : launch_tr<EK_TF32, 8>(g, stream);
+    } else if (m.family == FAM_T) {
         set_kernel_name("dot_tfdpa");
-        if (m.fmt_a == EF_F16) err = launch_t_l<EK_F16>(m, g, L, stream);
+        if (m.fmt_a == EF_E4M3) err = launch_8<false>(m, g, L, stream);
+        else if (m.fmt_a == EF_E5M2) err = launch_8<true>(m, g, L, stream);
+        else if (m.fmt_a == EF_F16) err = launch_t_l<EK_F16>(m, g, L, stream);
         else if (m.fmt_a == EF_BF16) err = launch_t_l<EK_BF16>(m, g, L, stream);
         else err = launch_t_l<EK_TF32>(m, g, L, stream);
     } else {
