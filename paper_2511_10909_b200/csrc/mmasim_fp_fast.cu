@@ -11,20 +11,24 @@
 // hardware's flush coincide here: products of two BF16 / FP16 values have at most 22 significant bits, and sums of
 // two normal-or-zero FP32 values below 2^-125 are multiples of 2^-149, so no result is rounded across the 2^-126
 // boundary.  Inputs are never subnormal (Algorithm 2 flushes A, B and C to +0 first; every intermediate is flushed).
+//
+// Any K and any row stride: the last chunk is filled up with -0 in A and +0 in B, whose products are -0, which every accumulator
+// (a -0 too) takes without a change.  Tiles in two sizes; see use_small.
 #include <cuda_fp16.h>
+#include <algorithm>
 #include "mmasim_internal.h"
 
 namespace mmasim {
 namespace {
 
-constexpr int NT = 256, KC = 16;
+constexpr int NT = 256;
 
 enum FpMode : int { FP_FMA32 = 0, FP_FTZ_F16 = 2, FP_FTZ_BF16 = 3 };
 
 template <int MODE> struct ModeTraits;
-template <> struct ModeTraits<FP_FMA32> { using acc_t = float; using in_t = float; static constexpr int TM = 8, TN = 8, IN_BYTES = 4; };
-template <> struct ModeTraits<FP_FTZ_F16> { using acc_t = float; using in_t = float; static constexpr int TM = 8, TN = 4, IN_BYTES = 2; };
-template <> struct ModeTraits<FP_FTZ_BF16> { using acc_t = float; using in_t = float; static constexpr int TM = 8, TN = 4, IN_BYTES = 2; };
+template <> struct ModeTraits<FP_FMA32> { static constexpr int TM = 8, TN = 8, IN_BYTES = 4; };
+template <> struct ModeTraits<FP_FTZ_F16> { static constexpr int TM = 8, TN = 4, IN_BYTES = 2; };
+template <> struct ModeTraits<FP_FTZ_BF16> { static constexpr int TM = 8, TN = 4, IN_BYTES = 2; };
 
 __device__ __forceinline__ float add_ftz(float x, float y) {
     float z;
@@ -43,12 +47,14 @@ __device__ __forceinline__ float load_flushed(uint32_t w, bool bf16) {
     return ((w & 0x7C00u) == 0u && (w & 0x03FFu)) ? 0.0f : __half2float(__ushort_as_half((unsigned short)w));
 }
 
-template <int MODE, int P>
-__global__ void __launch_bounds__(NT, 2) fp_kernel(GemmArgs g) {
+// TM x TN: outputs per thread; KC: elements of K per chunk; rows at any address (ROWS_ANY), on 16 bytes (ROWS_16), or on 16 bytes with K a
+// multiple of a chunk (ROWS_WHOLE: without the tests for the end of K, 2 - 5 % faster).
+enum Rows : int { ROWS_ANY = 0, ROWS_16, ROWS_WHOLE };
+template <int MODE, int P, int TM, int TN, int KC, int ROWS>
+__global__ void __launch_bounds__(NT, TM >= 8 ? 2 : 3) fp_kernel(GemmArgs g) {
     using T = ModeTraits<MODE>;
-    using in_t = typename T::in_t;
-    using acc_t = typename T::acc_t;
-    constexpr int TM = T::TM, TN = T::TN;
+    using in_t = float;
+    using acc_t = float;
     constexpr int BM = 16 * TM, BN = 16 * TN;
     constexpr bool FTZ = MODE == FP_FTZ_F16 || MODE == FP_FTZ_BF16;
     constexpr int EPT = 16 / T::IN_BYTES;                   // elements per 16-byte load
@@ -95,10 +101,25 @@ __global__ void __launch_bounds__(NT, 2) fp_kernel(GemmArgs g) {
             const int rows = is_a ? BM : BN;
             const int r = u % rows, h = u / rows;
             const int64_t grow = (is_a ? row0 : col0) + r;
-            raw[it] = make_uint4(0u, 0u, 0u, 0u);
-            if (task < TASKS && grow < (is_a ? g.M : g.N))
-                raw[it] = *reinterpret_cast<const uint4*>(static_cast<const unsigned char*>(is_a ? g.A : g.B) +
-                                                          (grow * (is_a ? g.lda : g.ldb) + k0 + h * EPT) * T::IN_BYTES);
+            const uint32_t pad = is_a ? (T::IN_BYTES == 4 ? 0x80000000u : 0x80008000u) : 0u;
+            raw[it] = make_uint4(pad, pad, pad, pad);
+            const int64_t k = k0 + h * EPT;
+            if (task >= TASKS || grow >= (is_a ? g.M : g.N) || (ROWS != ROWS_WHOLE && k >= g.K)) continue;
+            const unsigned char* p = static_cast<const unsigned char*>(is_a ? g.A : g.B) + (grow * (is_a ? g.lda : g.ldb) + k) * T::IN_BYTES;
+            if (ROWS == ROWS_WHOLE || (ROWS == ROWS_16 && k + EPT <= g.K)) raw[it] = *reinterpret_cast<const uint4*>(p);
+            else {
+                uint32_t w[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    w[q] = pad;
+                    if (T::IN_BYTES == 4) { if (k + q < g.K) w[q] = reinterpret_cast<const uint32_t*>(p)[q]; }
+                    else {
+                        if (k + 2 * q < g.K) w[q] = (w[q] & 0xFFFF0000u) | reinterpret_cast<const uint16_t*>(p)[2 * q];
+                        if (k + 2 * q + 1 < g.K) w[q] = (w[q] & 0x0000FFFFu) | uint32_t(reinterpret_cast<const uint16_t*>(p)[2 * q + 1]) << 16;
+                    }
+                }
+                raw[it] = make_uint4(w[0], w[1], w[2], w[3]);
+            }
         }
     };
     fetch(0);
@@ -127,7 +148,7 @@ __global__ void __launch_bounds__(NT, 2) fp_kernel(GemmArgs g) {
 
         if (!FTZ) {
             // fully unrolled: with a partial unroll the compiler rotates the accumulators through register moves
-#pragma unroll
+#pragma unroll 16
             for (int kk = 0; kk < KC; ++kk) {
                 in_t a[TM], b[TN];
 #pragma unroll
@@ -193,49 +214,56 @@ __global__ void __launch_bounds__(NT, 2) fp_kernel(GemmArgs g) {
 // raw doubles of A and B reach shared memory by 16-byte asynchronous copies, three chunks of 16 k in flight, rows with
 // a pitch of 20 doubles so that the fragment loads (lane (g, t) reads element (row 8 i + g, k 4 s + t)) are conflict-free.
 namespace dm {
-constexpr int BM = 128, BN = 64, DKC = 16, KP = DKC + 4, DNT = 256, STAGES = 3;
+constexpr int DKC = 16, KP = DKC + 4, STAGES = 3;
+template <int BM, int BN>
 struct Stage {
     double a[BM][KP];
     double b[BN][KP];
 };
 }  // namespace dm
 
-__global__ void __launch_bounds__(dm::DNT, 2) fma64_mma_kernel(GemmArgs g) {
+// WR x WC warps of TI x TJ accumulator tiles; UNIT: bytes per asynchronous copy (16, or 8 where a row stride or K is odd); TAIL: K is no
+// multiple of a chunk (the test for it in every chunk cost 2048 x 2048 x 2048 684 instead of 620 us).
+template <int WR, int WC, int TI, int TJ, int UNIT, bool TAIL>
+__global__ void __launch_bounds__(32 * WR * WC, 2) fma64_mma_kernel(GemmArgs g) {
     using namespace dm;
+    constexpr int BM = 8 * WR * TI, BN = 8 * WC * TJ, DNT = 32 * WR * WC, SEGS = DKC * 8 / UNIT, PER = UNIT / 8;
+    using ST = Stage<BM, BN>;
     extern __shared__ __align__(16) unsigned char dm_smem[];
-    Stage* stages = reinterpret_cast<Stage*>(dm_smem);
+    ST* stages = reinterpret_cast<ST*>(dm_smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int wr = warp >> 1, wc = warp & 1, gq = lane >> 2, tq = lane & 3;
+    const int wr = warp / WC, wc = warp % WC, gq = lane >> 2, tq = lane & 3;
     const int64_t row0 = int64_t(blockIdx.y) * BM, col0 = int64_t(blockIdx.x) * BN;
-    const int NCH = int(g.K / DKC);
+    const int NCH = TAIL ? int((g.K + DKC - 1) / DKC) : int(g.K / DKC), tail = int(g.K % DKC);
 
-    double acc[4][4][2];
+    double acc[TI][TJ][2];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < TI; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int j = 0; j < TJ; ++j)
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                const int64_t r = row0 + wr * 32 + 8 * i + gq, c = col0 + wc * 32 + 8 * j + 2 * tq + e;
+                const int64_t r = row0 + 8 * (wr * TI + i) + gq, c = col0 + 8 * (wc * TJ + j) + 2 * tq + e;
                 acc[i][j][e] = (g.C && r < g.M && c < g.N) ? static_cast<const double*>(g.C)[r * g.ldc + c] : 0.0;
             }
 
-    // one chunk: 192 rows x 8 segments of 16 bytes, consecutive threads on consecutive segments of a row; rows beyond the
-    // matrix are filled with zeros (a copy of size 0)
+    // one chunk: consecutive threads on consecutive segments of a row; rows and K beyond the matrix are filled with zeros (a
+    // shorter copy, or none)
     auto issue = [&](int n) {
-        Stage& s = stages[n % STAGES];
+        ST& s = stages[n % STAGES];
 #pragma unroll
-        for (int it = 0; it < (BM + BN) * 8 / DNT; ++it) {
+        for (int it = 0; it < (BM + BN) * SEGS / DNT; ++it) {
             const int task = it * DNT + tid;
-            const bool is_a = task < BM * 8;
-            const int u = is_a ? task : task - BM * 8;
-            const int r = u >> 3, seg = u & 7;
-            const int64_t grow = (is_a ? row0 : col0) + r;
-            const bool valid = grow < (is_a ? g.M : g.N);
+            const bool is_a = task < BM * SEGS;
+            const int u = is_a ? task : task - BM * SEGS;
+            const int r = u / SEGS, seg = u % SEGS;
+            const int64_t grow = (is_a ? row0 : col0) + r, k = int64_t(n) * DKC + PER * seg;
+            const bool inside = grow < (is_a ? g.M : g.N) && (!TAIL || k < g.K);      // (all of a copy is inside, or nothing)
             const double* base = static_cast<const double*>(is_a ? g.A : g.B);
-            const double* src = valid ? base + grow * (is_a ? g.lda : g.ldb) + int64_t(n) * DKC + 2 * seg : base;
-            const uint32_t dst = uint32_t(__cvta_generic_to_shared(is_a ? &s.a[r][2 * seg] : &s.b[r][2 * seg]));
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
+            const double* src = inside ? base + grow * (is_a ? g.lda : g.ldb) + k : base;
+            const uint32_t dst = uint32_t(__cvta_generic_to_shared(is_a ? &s.a[r][PER * seg] : &s.b[r][PER * seg]));
+            if (UNIT == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(inside ? 16 : 0) : "memory");
+            else asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(inside ? 8 : 0) : "memory");
         }
     };
     issue(0);
@@ -248,18 +276,22 @@ __global__ void __launch_bounds__(dm::DNT, 2) fma64_mma_kernel(GemmArgs g) {
         __syncthreads();                                        // ... for every thread, and everybody has left chunk n - 1
         if (n + 2 < NCH) issue(n + 2);                          // into the buffer of chunk n - 1
         asm volatile("cp.async.commit_group;" ::: "memory");
-        const Stage& s = stages[n % STAGES];
+        const ST& s = stages[n % STAGES];
+        const bool last = TAIL && n == NCH - 1;
 #pragma unroll
         for (int ks = 0; ks < DKC / 4; ++ks) {
-            double af[4], bf[4];
+            double af[TI], bf[TJ];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) af[i] = s.a[wr * 32 + 8 * i + gq][4 * ks + tq];
+            for (int i = 0; i < TI; ++i) {
+                af[i] = s.a[8 * (wr * TI + i) + gq][4 * ks + tq];
+                if (last && 4 * ks + tq >= tail) af[i] = -0.0;
+            }
 #pragma unroll
-            for (int j = 0; j < 4; ++j) bf[j] = s.b[wc * 32 + 8 * j + gq][4 * ks + tq];
+            for (int j = 0; j < TJ; ++j) bf[j] = s.b[8 * (wc * TJ + j) + gq][4 * ks + tq];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < TI; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
+                for (int j = 0; j < TJ; ++j)
                     asm volatile("mma.sync.aligned.m8n8k4.row.col.rn.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
                                  : "+d"(acc[i][j][0]), "+d"(acc[i][j][1]) : "d"(af[i]), "d"(bf[j]));
         }
@@ -267,12 +299,12 @@ __global__ void __launch_bounds__(dm::DNT, 2) fma64_mma_kernel(GemmArgs g) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < TI; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int j = 0; j < TJ; ++j)
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                const int64_t r = row0 + wr * 32 + 8 * i + gq, c = col0 + wc * 32 + 8 * j + 2 * tq + e;
+                const int64_t r = row0 + 8 * (wr * TI + i) + gq, c = col0 + 8 * (wc * TJ + j) + 2 * tq + e;
                 if (r >= g.M || c >= g.N) continue;
                 const double v = acc[i][j][e];
                 unsigned long long w = (unsigned long long)__double_as_longlong(v);
@@ -281,23 +313,46 @@ __global__ void __launch_bounds__(dm::DNT, 2) fma64_mma_kernel(GemmArgs g) {
             }
 }
 
-cudaError_t launch_fma64_mma(const GemmArgs& g, cudaStream_t stream) {
-    using namespace dm;
-    constexpr size_t sh = sizeof(Stage) * STAGES;
-    cudaError_t err = cudaFuncSetAttribute(fma64_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sh));
-    if (err != cudaSuccess) return err;
-    dim3 grid((unsigned)((g.N + BN - 1) / BN), (unsigned)((g.M + BM - 1) / BM), 1);
-    fma64_mma_kernel<<<grid, DNT, sh, stream>>>(g);
-    return cudaGetLastError();
+int64_t up_div(int64_t x, int64_t y) { return (x + y - 1) / y; }
+
+// Small tiles where the large ones leave SMs idle: the work on the fullest SM, in large tiles; a small tile is its share of the outputs
+// times `overhead` (more operand traffic per output), and a few of them take 0.35 of a large tile however small (latency).  Large / small
+// in us: FP32 512^3 77 / 27, 1024^3 149 / 156; FP64 512^3 54 / 17, 1024 x 1024 x 256 34 / 31; CDNA2 FP16 560 x 192 x 128 20 / 11.
+bool use_small(const GemmArgs& g, int bm, int bn, int sm, int sn, double overhead) {
+    const double large = double(up_div(up_div(g.M, bm) * up_div(g.N, bn), 148));
+    const double share = double(sm * sn) / double(bm * bn), n = double(up_div(up_div(g.M, sm) * up_div(g.N, sn), 148));
+    return std::max(n * share * overhead, 0.35) < large;
 }
 
+template <int WR, int WC, int TI, int TJ>
+cudaError_t launch_fma64_tile(const GemmArgs& g, cudaStream_t stream) {
+    constexpr int BM = 8 * WR * TI, BN = 8 * WC * TJ;
+    constexpr size_t sh = sizeof(dm::Stage<BM, BN>) * dm::STAGES;
+    auto kernel = (g.lda | g.ldb | g.K) & 1 ? fma64_mma_kernel<WR, WC, TI, TJ, 8, true>
+                                            : (g.K % dm::DKC ? fma64_mma_kernel<WR, WC, TI, TJ, 16, true> : fma64_mma_kernel<WR, WC, TI, TJ, 16, false>);
+    const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sh));
+    if (err != cudaSuccess) return err;
+    kernel<<<dim3(unsigned(up_div(g.N, BN)), unsigned(up_div(g.M, BM))), 32 * WR * WC, sh, stream>>>(g);
+    return cudaGetLastError();
+}
+cudaError_t launch_fma64_mma(const GemmArgs& g, cudaStream_t stream) {
+    return use_small(g, 128, 64, 32, 32, 1.15) ? launch_fma64_tile<2, 2, 2, 2>(g, stream) : launch_fma64_tile<4, 2, 4, 4>(g, stream);
+}
+
+template <int MODE, int P, int TM, int TN, int KC>
+cudaError_t launch_fp_tile(const GemmArgs& g, cudaStream_t stream) {
+    constexpr int B = ModeTraits<MODE>::IN_BYTES;
+    const dim3 grid(unsigned(up_div(g.N, 16 * TN)), unsigned(up_div(g.M, 16 * TM)), 1);
+    if ((g.lda * B) % 16 || (g.ldb * B) % 16) fp_kernel<MODE, P, TM, TN, KC, ROWS_ANY><<<grid, NT, 0, stream>>>(g);
+    else if (g.K % KC) fp_kernel<MODE, P, TM, TN, KC, ROWS_16><<<grid, NT, 0, stream>>>(g);
+    else fp_kernel<MODE, P, TM, TN, KC, ROWS_WHOLE><<<grid, NT, 0, stream>>>(g);
+    return cudaGetLastError();
+}
 template <int MODE, int P>
 cudaError_t launch_fp(const GemmArgs& g, cudaStream_t stream) {
     using T = ModeTraits<MODE>;
-    constexpr int BM = 16 * T::TM, BN = 16 * T::TN;
-    dim3 grid((unsigned)((g.N + BN - 1) / BN), (unsigned)((g.M + BM - 1) / BM), 1);
-    fp_kernel<MODE, P><<<grid, NT, 0, stream>>>(g);
-    return cudaGetLastError();
+    if (use_small(g, 16 * T::TM, 16 * T::TN, 32, 64, MODE == FP_FMA32 ? 2.1 : 1.6)) return launch_fp_tile<MODE, P, 2, 4, 32>(g, stream);
+    return launch_fp_tile<MODE, P, T::TM, T::TN, 16>(g, stream);
 }
 
 }  // namespace
@@ -305,11 +360,8 @@ cudaError_t launch_fp(const GemmArgs& g, cudaStream_t stream) {
 bool fast_fp_supported(const DevModel& m, const GemmArgs& g) {
     if (g.dot_mode || g.k_chunk || g.row_scale) return false;
     if (m.family != FAM_FMA && m.family != FAM_FTZ) return false;
-    const int bytes = fmt_desc(m.fmt_a).storage_bits / 8;
-    if (g.K % KC) return false;
-    if (((g.lda * bytes) % 16) || ((g.ldb * bytes) % 16)) return false;
-    if (g.M > 65535ll * 32) return false;
-    return true;
+    if (g.K > 0x7FFF0000ll) return false;
+    return g.M <= 65535ll * 32;
 }
 
 int launch_fast_fp(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
@@ -323,6 +375,8 @@ int launch_fast_fp(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
         else if (m.P == 4) err = launch_fp<FP_FTZ_BF16, 4>(g, stream);
         else err = launch_fp<FP_FTZ_BF16, 2>(g, stream);
     }
+    const int bytes = fmt_desc(m.fmt_a).storage_bits / 8;
+    if ((g.lda * bytes) % 16 || (g.ldb * bytes) % 16) set_kernel_name("generic");       // the any-shape route: rows at any address
     if (err != cudaSuccess) {
         set_error("floating-point kernel launch failed: %s", cudaGetErrorString(err));
         return MMASIM_ERR_CUDA;
