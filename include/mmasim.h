@@ -238,6 +238,11 @@ int mmasim_hw_umma(int kind, int64_t M, int64_t K, const void* A, const void* B,
  * All pointers are device pointers. */
 int mmasim_error_stats(int acc_fmt, int64_t n, const void* D, const double* ref, double* stats, void* stream);
 
+/* That reference for one model's operands: ref (M x N doubles) = A x B^T + C in FP64, the values widened exactly, the FP64
+ * multiply-add chain in ascending k.  Packed operands of unscaled models whose A and B have one type, FP32, TF32, BF16, FP16 or FP8. */
+int mmasim_reference_fp64(const mmasim_model* model, int64_t M, int64_t N, int64_t K, const void* A, const void* B, const void* C,
+                          double* ref, void* stream);
+
 /* Issue-rate micro-benchmarks, the roofline denominators (no counterpart in the paper).  Launches `blocks` CTAs of
  * 256 threads; every thread runs `iters` (rounded up to a multiple of 8) times 8 rounds of independent operations of
  * the given kind.  `sink` (device, >= 4 bytes) receives a value that keeps the work alive.  The caller times the

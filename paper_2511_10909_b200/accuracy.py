@@ -41,7 +41,12 @@ def deviation_stats(model: mmasim.Model, A, B, C=None, ref=None) -> dict:
     """Run the model and reduce delta = D - D_real: count, mean, mean |delta|, rms, share of negative / positive
     deviations, max |delta|, mean relative error."""
     if ref is None:
-        ref = reference_fp64(model.in_fmt, model.acc, A, B, C)
+        packed = all(t is None or (t.is_cuda and t.dim() == 2 and t.is_contiguous()) for t in (A, B, C))
+        if packed and model.b_fmt == model.in_fmt and model.in_fmt in ("fp16", "bf16", "bf16_1k", "tf32", "fp32", "e4m3", "e5m2") \
+                and model.acc != "fp64" and A.shape[1] == B.shape[1]:
+            ref = mmasim.reference_fp64(model, A, B, C)       # the operands widened in one launch
+        else:
+            ref = reference_fp64(model.in_fmt, model.acc, A, B, C)
     D = mmasim.gemm(model, A, B, C)
     s = mmasim.error_stats(model.acc, D, ref).cpu().tolist()
     n = max(s[0], 1.0)

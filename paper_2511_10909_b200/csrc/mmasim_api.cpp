@@ -471,6 +471,24 @@ int mmasim_error_stats(int acc_fmt, int64_t n, const void* D, const double* ref,
                               static_cast<cudaStream_t>(stream));
 }
 
+int mmasim_reference_fp64(const mmasim_model* model, int64_t M, int64_t N, int64_t K, const void* A, const void* B, const void* C,
+                          double* ref, void* stream) {
+    GemmArgs g;
+    int st = build_args(model, M, N, K, A, B, C, ref, nullptr, &g);
+    if (st != MMASIM_OK) return st;
+    const DevModel& m = model->dev;
+    const int f = m.fmt_a;
+    if (f != m.fmt_b || (f != EF_F16 && f != EF_BF16 && f != EF_TF32 && f != EF_F32 && f != EF_E4M3 && f != EF_E5M2) || m.k_block || m.acc == ACC_F64) {
+        set_error("mmasim_reference_fp64: unscaled models of FP32, TF32, BF16, FP16 and FP8 inputs of one type");
+        return MMASIM_ERR_UNSUPPORTED;
+    }
+    if ((st = check_device_ptr(A, "A")) != MMASIM_OK) return st;
+    if ((st = check_device_ptr(B, "B")) != MMASIM_OK) return st;
+    if ((st = check_device_ptr(ref, "ref")) != MMASIM_OK) return st;
+    if (C && (st = check_device_ptr(C, "C")) != MMASIM_OK) return st;
+    return launch_reference_fp64(f, m.acc, M, N, K, A, B, C, ref, static_cast<cudaStream_t>(stream));
+}
+
 int mmasim_host_release(void) {
     std::lock_guard<std::mutex> lock(g_pool_mutex);
     cudaError_t err = cudaSuccess;

@@ -116,6 +116,7 @@ int launch_hw_umma(int kind, int64_t M, int64_t K, const void* A, const void* B,
                    const void* sfb, int32_t* status, cudaStream_t stream);
 // mmasim_stats.cu
 int launch_error_stats(int acc, int64_t n, const void* D, const double* ref, double* stats, cudaStream_t stream);
+int launch_reference_fp64(int fmt, int acc, int64_t M, int64_t N, int64_t K, const void* A, const void* B, const void* C, double* ref, cudaStream_t stream);
 // mmasim_peak.cu
 int launch_int_peak(int kind, int64_t blocks, int64_t iters, void* sink, int32_t* ops_per_round, cudaStream_t stream);
 // mmasim_api.cpp

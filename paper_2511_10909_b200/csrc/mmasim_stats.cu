@@ -1,7 +1,10 @@
 // Error statistics of model outputs against an FP64 reference: the reduction behind the accuracy analysis of
-// Section 6 (the deviations delta = D - D_real of Figure 3, their sign balance and size).  A grid-stride pass over
-// the outputs, per-thread partial sums in FP64, warp shuffles, one atomic per warp and statistic.
+// Section 6 (the deviations delta = D - D_real of Figure 3, their sign balance and size), and the widening of that
+// reference's operands.  A grid-stride pass over the outputs, four in flight per thread, per-thread partial sums in FP64, reduced
+// over the CTA, one atomic per CTA and statistic (one per warp, 9472 on each of eight addresses, took 85 of the 89 us
+// of a 1024 x 1024 reduction).
 #include <cuda_fp16.h>
+#include <cstring>
 #include "mmasim_internal.h"
 
 namespace mmasim {
@@ -23,6 +26,7 @@ __device__ __forceinline__ double warp_max(double v) {
 template <bool ACC16>
 __global__ void __launch_bounds__(256) stats_kernel(int64_t n, const void* D, const double* ref, double* stats) {
     double cnt = 0.0, sum = 0.0, sabs = 0.0, ssq = 0.0, nneg = 0.0, npos = 0.0, mx = 0.0, srel = 0.0;
+#pragma unroll 4
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
         const double d = ACC16 ? double(__half2float(__ushort_as_half(static_cast<const unsigned short*>(D)[i])))
                                : double(__uint_as_float(static_cast<const uint32_t*>(D)[i]));
@@ -40,13 +44,50 @@ __global__ void __launch_bounds__(256) stats_kernel(int64_t n, const void* D, co
     }
     const double v[NSTAT] = {warp_sum(cnt), warp_sum(sum), warp_sum(sabs), warp_sum(ssq), warp_sum(nneg), warp_sum(npos),
                              warp_max(mx), warp_sum(srel)};
+    __shared__ double part[NSTAT][8];
     if ((threadIdx.x & 31) == 0) {
 #pragma unroll
-        for (int s = 0; s < NSTAT; ++s) {
-            if (s == 6) atomicMax(reinterpret_cast<unsigned long long*>(stats + s), (unsigned long long)__double_as_longlong(v[s]));   // non-negative doubles order like their bit patterns
-            else atomicAdd(stats + s, v[s]);
+        for (int s = 0; s < NSTAT; ++s) part[s][threadIdx.x >> 5] = v[s];
+    }
+    __syncthreads();
+    if (threadIdx.x < NSTAT) {
+        const int s = threadIdx.x;
+        double t = part[s][0];
+#pragma unroll
+        for (int w = 1; w < 8; ++w) t = s == 6 ? fmax(t, part[s][w]) : t + part[s][w];
+        if (s == 6) atomicMax(reinterpret_cast<unsigned long long*>(stats + s), (unsigned long long)__double_as_longlong(t));   // non-negative doubles order like their bit patterns
+        else atomicAdd(stats + s, t);
+    }
+}
+
+// Up to three operands widened exactly to FP64, four elements per thread.
+struct Widen {
+    const void* src[3];
+    double* dst[3];
+    int64_t n[3];
+    int fmt[3];
+};
+__device__ __forceinline__ double widen_one(int fmt, const void* p, int64_t i) {
+    switch (fmt) {
+        case EF_F16: return double(__half2float(__ushort_as_half(static_cast<const unsigned short*>(p)[i])));
+        case EF_BF16: return double(__uint_as_float(uint32_t(static_cast<const uint16_t*>(p)[i]) << 16));
+        case EF_TF32: return double(__uint_as_float(static_cast<const uint32_t*>(p)[i] & ~0x1FFFu));
+        case EF_F32: return double(__uint_as_float(static_cast<const uint32_t*>(p)[i]));
+        default: {
+            const unsigned short x = static_cast<const uint8_t*>(p)[i];
+            uint32_t h;
+            if (fmt == EF_E5M2) asm("cvt.rn.f16x2.e5m2x2 %0, %1;" : "=r"(h) : "h"(x));
+            else asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h) : "h"(x));
+            return double(__half2float(__ushort_as_half((unsigned short)h)));
         }
     }
+}
+__global__ void __launch_bounds__(256) widen_kernel(Widen w) {
+    const int o = blockIdx.y;
+    const int64_t first = (int64_t(blockIdx.x) * 256 + threadIdx.x) * 4;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (first + q < w.n[o]) w.dst[o][first + q] = widen_one(w.fmt[o], w.src[o], first + q);
 }
 
 }  // namespace
@@ -54,12 +95,45 @@ __global__ void __launch_bounds__(256) stats_kernel(int64_t n, const void* D, co
 int launch_error_stats(int acc, int64_t n, const void* D, const double* ref, double* stats, cudaStream_t stream) {
     if (acc != ACC_F32 && acc != ACC_F16) { set_error("mmasim_error_stats: the accumulator format must be FP32 or FP16"); return MMASIM_ERR_INVALID_ARG; }
     const int64_t want = (n + 255) / 256;
-    const unsigned blocks = unsigned(want < 148 * 8 ? want : 148 * 8);
+    const unsigned blocks = unsigned(want < 148 * 4 ? want : 148 * 4);
     if (acc == ACC_F16) stats_kernel<true><<<blocks, 256, 0, stream>>>(n, D, ref, stats);
     else stats_kernel<false><<<blocks, 256, 0, stream>>>(n, D, ref, stats);
     const cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) { set_error("mmasim_error_stats launch failed: %s", cudaGetErrorString(err)); return MMASIM_ERR_CUDA; }
     return MMASIM_OK;
+}
+
+// D_real = A x B^T + C in FP64 (Phi_FMA): the operands widened to scratch memory in one launch, then the FP64 kernel.
+int launch_reference_fp64(int fmt, int acc, int64_t M, int64_t N, int64_t K, const void* A, const void* B, const void* C, double* ref, cudaStream_t stream) {
+    cudaMemPool_t pool;
+    double* scratch = nullptr;
+    cudaError_t err = scratch_pool(&pool);
+    const int64_t na = M * K, nb = N * K, nc = C ? M * N : 0, a_at = 0, b_at = (na + 1) / 2 * 2, c_at = b_at + (nb + 1) / 2 * 2;
+    if (err == cudaSuccess) err = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&scratch), size_t(c_at + nc) * 8, pool, stream);
+    int st = MMASIM_OK;
+    if (err == cudaSuccess) {
+        const Widen w = {{A, B, C}, {scratch + a_at, scratch + b_at, scratch + c_at}, {na, nb, nc}, {fmt, fmt, acc == ACC_F16 ? EF_F16 : EF_F32}};
+        const int64_t most = na > nb ? (na > nc ? na : nc) : (nb > nc ? nb : nc);
+        widen_kernel<<<dim3(unsigned((most + 1023) / 1024), C ? 3 : 2), 256, 0, stream>>>(w);
+        err = cudaGetLastError();
+    }
+    if (err == cudaSuccess) {
+        DevModel m;
+        std::memset(&m, 0, sizeof(m));
+        m.family = FAM_FMA;
+        m.fmt_a = m.fmt_b = EF_F64;
+        m.acc = ACC_F64;
+        GemmArgs g;
+        std::memset(&g, 0, sizeof(g));
+        g.M = M; g.N = N; g.K = K;
+        g.A = scratch + a_at; g.B = scratch + b_at; g.C = C ? scratch + c_at : nullptr; g.D = ref;
+        g.lda = g.ldb = K;
+        g.ldc = g.ldd = N;
+        st = launch_fast_fp(m, g, stream);
+    }
+    if (scratch) cudaFreeAsync(scratch, stream);
+    if (err != cudaSuccess) { set_error("mmasim_reference_fp64: %s", cudaGetErrorString(err)); return MMASIM_ERR_CUDA; }
+    return st;
 }
 
 }  // namespace mmasim

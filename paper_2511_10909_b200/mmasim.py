@@ -79,6 +79,8 @@ def _load():
     lib.mmasim_hw_umma.argtypes = [c_int, c_int64, c_int64, c_void_p, c_void_p, c_void_p, c_void_p, c_void_p, c_void_p, c_void_p, c_void_p]
     lib.mmasim_error_stats.restype = c_int
     lib.mmasim_error_stats.argtypes = [c_int, c_int64, c_void_p, c_void_p, c_void_p, c_void_p]
+    lib.mmasim_reference_fp64.restype = c_int
+    lib.mmasim_reference_fp64.argtypes = [c_void_p, c_int64, c_int64, c_int64, c_void_p, c_void_p, c_void_p, c_void_p, c_void_p]
     lib.mmasim_host_release.restype = c_int
     lib.mmasim_host_release.argtypes = []
     lib.mmasim_last_kernel.restype = c_char_p
@@ -361,6 +363,18 @@ def copy_timeouts() -> int:
 def host_release():
     """Destroys the device memory pools that gemm_host keeps between calls."""
     _check(_lib.mmasim_host_release())
+
+
+def reference_fp64(model: Model, A, B, C=None, *, stream=None):
+    """A x B^T + C in FP64 for packed operands of ``model``'s types (mmasim_reference_fp64): an M x N FP64 CUDA tensor."""
+    import torch
+    dev, M, N, K = A.device, A.shape[0], B.shape[0], A.shape[1]
+    for t, name, rows, cols, bits in ((A, "A", M, K, model.a_bits), (B, "B", N, K, model.b_bits), (C, "C", M, N, 8 * model.acc_bytes)):
+        if t is not None and _matrix(t, name, rows, cols, bits, dev) != cols:
+            raise MmasimError(3, f"{name} must be a packed {rows} x {cols} matrix")
+    ref = torch.empty((M, N), dtype=torch.float64, device=dev)
+    _check(_lib.mmasim_reference_fp64(model._h, M, N, K, _ptr(A), _ptr(B), _ptr(C), _ptr(ref), _stream(stream)))
+    return ref
 
 
 STAT_NAMES = ["count", "sum", "sum_abs", "sum_sq", "negative", "positive", "max_abs", "sum_rel"]
