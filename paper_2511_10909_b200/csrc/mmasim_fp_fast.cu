@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(32 * WR * WC, 2) fma64_mma_kernel(GemmArgs g) 
         if (n + 2 < NCH) issue(n + 2);                          // into the buffer of chunk n - 1
         asm volatile("cp.async.commit_group;" ::: "memory");
         const ST& s = stages[n % STAGES];
-        const bool last = TAIL && n == NCH - 1;
+        const bool last = TAIL && tail && n == NCH - 1;
 #pragma unroll
         for (int ks = 0; ks < DKC / 4; ++ks) {
             double af[TI], bf[TJ];

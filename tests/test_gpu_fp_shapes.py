@@ -16,7 +16,7 @@ def test_any_k_and_stride(key):
     from paper_2511_10909_b200 import mmasim
     model = mmasim.Model(*key)
     unit = model.P or 1
-    for n, (M, N, K) in enumerate([(1, 1, 1), (33, 65, 5), (31, 64, 17), (130, 129, 35), (700, 1300, 36), (1290, 1300, 52)]):
+    for n, (M, N, K) in enumerate([(1, 1, 1), (33, 65, 5), (31, 64, 17), (34, 70, 64), (130, 129, 35), (700, 1300, 36), (1290, 1300, 52)]):
         K = -(-K // unit) * unit
         g = wl.rng(60 + n)
         inp = wl.normal_inputs(key[1], key[2], M, N, K, seed=n)
