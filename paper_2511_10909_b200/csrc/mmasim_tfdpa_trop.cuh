@@ -8,8 +8,9 @@
 // u - the shift by e_max - e_k, the truncation and the addition of Algorithm 7 in one instruction, the alignment
 // distance carried by the register's exponent.  Operands are the element values (A) and the element values with an
 // offset 2^-(pre + guard) below the last significand bit (B), so that a negative product is never on the grid and
-// floors to the one's complement of its truncated magnitude; a population count over sign / nonzero masks adds the
-// number of negative nonzero terms back.  The accumulator enters by one addition rounded toward minus infinity (its
+// floors to the one's complement of its truncated magnitude; a population count over sign masks adds the number of
+// negative terms back (a zero is staged as a tiny number of its sign, TINY: far below any unit, its negative products too
+// fall one short, so that no mask of nonzero elements is needed: 4.21 -> 4.1 ms).  The accumulator enters by one addition rounded toward minus infinity (its
 // lowest mantissa bit set, so that a negative c floors likewise; the +1 is added to the register's starting value),
 // and the block's value S * u leaves by one exact subtraction of 1.5 * 2^23 * u; rho is a mask (RZ-E8M13) or a
 // conversion (RNE-FP16).  The accumulator between blocks is the output word itself.
@@ -82,7 +83,7 @@ struct Geo {
 struct LutEntryT {      // 8 bytes: one shared load per staged element
     uint32_t op;        // staged FP32 operand
     uint32_t y;         // bits 0..14: BF16 word of pe(x); bit 15: infinity / NaN (a pe of -0: harmless in P);
-                        // bit 16: sign; bit 24: finite and nonzero
+                        // bit 16: sign; bit 24: zero
 };
 
 // One operand's share of a chunk of KC = 32 elements of K, decoded: R rows of A (or columns of B).  A decode kernel
@@ -91,9 +92,10 @@ template <int R>
 struct BlkT {
     uint32_t op[KC][R];                 // [k][permuted row]: FP32 operands
     uint16_t pe[R][PE_STRIDE];          // [row][k]: BF16 exponent powers for the tensor cores
-    uint32_t sgn[R], nz[R];             // [permuted row]: bit k = sign / nonzero of element k of the chunk
+    uint32_t sgn[R];                    // [permuted row]: bit k = sign of element k of the chunk
     uint32_t special;                   // nonzero: the block holds an infinity or a NaN
-    uint32_t pad[3];
+    uint32_t sparse;                    // nonzero: a row (of the matrix) has a block of L with half or more of its elements zero
+    uint32_t pad[2];
 };
 static_assert(sizeof(BlkT<128>) % 16 == 0 && sizeof(BlkT<64>) % 16 == 0, "bulk copies move multiples of 16 bytes");
 
@@ -113,38 +115,42 @@ __device__ __forceinline__ int perm_row(int r) {
 }
 __device__ __forceinline__ int perm_col(int c) { return (c & ~31) | (((c >> 1) & 3) << 3) | (((c >> 3) & 3) << 1) | (c & 1); }
 
+constexpr float TINY = 7.888609052210118e-31f;          // 2^-100: times an element below 2^-83, the smallest unit is 2^-43
+
 template <int BASE>
 __device__ __forceinline__ void init_lut_t(LutEntryT* lut_a, LutEntryT* lut_b, const FmtDesc& fa, const FmtDesc& fb, int pre, int guard, int tid) {
     const uint32_t da = decode_elem(fa, uint32_t(tid)), db = decode_elem(fb, uint32_t(tid));
     const bool fin_a = dec_cls(da) == CLS_FINITE, fin_b = dec_cls(db) == CLS_FINITE;
     const bool nz_a = fin_a && dec_sig(da) != 0u, nz_b = fin_b && dec_sig(db) != 0u;
     LutEntryT ea, eb;
-    ea.op = __float_as_uint(ldexpf(float(fin_a ? dec_ssig(da) : 0), fin_a ? dec_exp(da) : 0));
+    auto tiny = [](uint32_t d) { return __float_as_uint(dec_sign(d) ? -TINY : TINY); };
+    ea.op = nz_a ? __float_as_uint(ldexpf(float(dec_ssig(da)), dec_exp(da))) : tiny(da);
     ea.y = (nz_a ? uint32_t((127 + BASE * (dec_exp(da) - PE_CENTER)) << 7) : 0u) | (fin_a ? 0u : 0x8000u) |
-           (fin_a ? (dec_sign(da) << 16) | (uint32_t(nz_a) << 24) : 0u);
+           (dec_sign(da) << 16) | (uint32_t(!nz_a) << 24);
     const int sb = fin_b ? dec_ssig(db) : 0;
     const int ub = dec_sign(db) ? -1 : 1;
     // a_op * b_op = a * b * (1 + 2^-(pre + guard) / |sig_b|): the true product with the offset that makes a negative one inexact
-    eb.op = nz_b ? __float_as_uint(ldexpf(float(sb * (1 << (pre + guard)) + ub), dec_exp(db) - (fa.mbits + fb.mbits + pre + guard))) : 0u;
+    eb.op = nz_b ? __float_as_uint(ldexpf(float(sb * (1 << (pre + guard)) + ub), dec_exp(db) - (fa.mbits + fb.mbits + pre + guard))) : tiny(db);
     eb.y = (nz_b ? uint32_t((127 + pe_shift(BASE) + BASE * (dec_exp(db) - PE_CENTER)) << 7) : 0u) | (fin_b ? 0u : 0x8000u) |
-           (fin_b ? (dec_sign(db) << 16) | (uint32_t(nz_b) << 24) : 0u);
+           (dec_sign(db) << 16) | (uint32_t(!nz_b) << 24);
     lut_a[tid] = ea;
     lut_b[tid] = eb;
 }
 
-// N = 16 or 8 elements of one row: operands k-major, pe words row-major, sign / nonzero bits into the masks.
+// N = 16 or 8 elements of one row: operands k-major, pe words row-major, sign bits into the masks.  Returns the table's flags
+// (bit 15: infinity / NaN) and in bits 16.. the number of zeros.
 template <int N, int R>
 __device__ __forceinline__ uint32_t stage_row(const LutEntryT* lut, BlkT<R>& s, const uint32_t (&w)[N / 4], int r, int pr, int part) {
     uint32_t* op = &s.op[part * N][pr];
-    uint32_t acc = 0u, spec = 0u, pw[N / 2];
+    uint32_t acc = 0u, spec = 0u, zeros = 0u, pw[N / 2];
 #pragma unroll
     for (int q = 0; q < N; q += 2) {
         const uint2 e0 = *reinterpret_cast<const uint2*>(&lut[(w[q / 4] >> (8 * (q % 4))) & 0xFFu]);
         const uint2 e1 = *reinterpret_cast<const uint2*>(&lut[(w[q / 4] >> (8 * (q % 4) + 8)) & 0xFFu]);
         op[q * R] = e0.x;
         op[(q + 1) * R] = e1.x;
-        // sign byte -> bits 0.., nonzero byte -> bits 16..
-        acc += (__byte_perm(e0.y, 0u, 0x4342) << q) + (__byte_perm(e1.y, 0u, 0x4342) << (q + 1));
+        acc += ((e0.y >> 16 & 1u) << q) + ((e1.y >> 16 & 1u) << (q + 1));
+        zeros += (e0.y >> 24) + (e1.y >> 24);
         spec |= e0.y | e1.y;
         pw[q / 2] = __byte_perm(e0.y, e1.y, 0x5410);
     }
@@ -154,12 +160,10 @@ __device__ __forceinline__ uint32_t stage_row(const LutEntryT* lut, BlkT<R>& s, 
         reinterpret_cast<uint4*>(pe)[q] = make_uint4(pw[4 * q], pw[4 * q + 1], pw[4 * q + 2], pw[4 * q + 3]);
     if (N == 16) {
         reinterpret_cast<uint16_t*>(&s.sgn[pr])[part] = uint16_t(acc);
-        reinterpret_cast<uint16_t*>(&s.nz[pr])[part] = uint16_t(acc >> 16);
     } else {
         reinterpret_cast<uint8_t*>(&s.sgn[pr])[part] = uint8_t(acc);
-        reinterpret_cast<uint8_t*>(&s.nz[pr])[part] = uint8_t(acc >> 16);
     }
-    return spec;
+    return (spec & 0x8000u) | zeros << 16;
 }
 
 // Decode pass: one CTA decodes one block (R rows of A or columns of B x 32 elements of K) through a 256-entry table of
@@ -175,7 +179,7 @@ __global__ void __launch_bounds__(NT) trop_decode_kernel(DevModel m, const unsig
     const int tid = threadIdx.x;
     const FmtDesc fa = fmt_desc(m.fmt_a), fb = fmt_desc(m.fmt_b);
     init_lut_t<BASE>(lut_a, lut_b, fa, fb, F - (fa.mbits + fb.mbits), fa.mbits + 1, tid);
-    if (tid == 0) { blk.special = 0u; blk.pad[0] = blk.pad[1] = blk.pad[2] = 0u; }
+    if (tid == 0) { blk.special = blk.sparse = 0u; blk.pad[0] = blk.pad[1] = 0u; }
     constexpr int N = R * KC / NT;                      // elements per thread: 16 or 8
     const int r = tid % R, part = tid / R;
     const int64_t i = int64_t(blockIdx.y) * R + r, k0 = int64_t(blockIdx.x) * KC;
@@ -192,6 +196,9 @@ __global__ void __launch_bounds__(NT) trop_decode_kernel(DevModel m, const unsig
     __syncthreads();
     const uint32_t spec = stage_row<N, R>(IS_A ? lut_a : lut_b, blk, w, r, IS_A ? perm_row<TH>(r) : perm_col(r), part);
     if (spec & 0x8000u) atomicOr(&blk.special, 1u);
+    // (two rows with less than half of their elements zero meet in a nonzero product; a thread sees a part of a block of L, and
+    // parts with less than half of theirs add up to one)
+    if (i < rows && (spec >> 16) * 2 >= uint32_t(N)) atomicOr(&blk.sparse, 1u);
     __syncthreads();
     uint4* out = reinterpret_cast<uint4*>(dst + (int64_t(blockIdx.y) * gridDim.x + blockIdx.x));
     const uint4* in = reinterpret_cast<const uint4*>(&blk);
@@ -265,6 +272,7 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
     uint32_t cw[TH][TW];
     mask_t sp_nan = 0, sp_pinf = 0, sp_ninf = 0;        // per output (bit h * TW + x)
     float promoted[PROMOTE ? TH : 1][PROMOTE ? TW : 1];
+    int big = 0;
 #define MMASIM_SP_GET(h, x) (uint32_t((sp_nan >> ((h) * TW + (x))) & 1u) | (uint32_t((sp_pinf >> ((h) * TW + (x))) & 1u) << 1) | (uint32_t((sp_ninf >> ((h) * TW + (x))) & 1u) << 2))
 #define MMASIM_SP_WORD(h, x, w) (MMASIM_SP_GET(h, x) ? special_word(((MMASIM_SP_GET(h, x) & 1u) || (MMASIM_SP_GET(h, x) & 6u) == 6u) ? 1 : ((MMASIM_SP_GET(h, x) & 2u) ? 2 : 3), ACC16, true) : (w))
 #pragma unroll
@@ -283,10 +291,13 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
                 if (d.cls == CLS_NAN) sp_nan |= bit; else if (d.sign) sp_ninf |= bit; else sp_pinf |= bit;
                 w = 0u;
             }
+            big = big || fabsf(__uint_as_float(w)) > 1.2676506e30f;         // 2^100
             cw[h][x] = w;
         }
 
-    __syncthreads();                                       // the barriers are initialised
+    // (the barriers are initialised.)  An output can only leave the range of the sum register where it has no nonzero product, or
+    // from a huge C: K products of at most 2^32 each move an accumulator by less than 2^64.
+    big = __syncthreads_or(!ACC16 && !PROMOTE && big);
     for (int chunk = 0; chunk < NCH; ++chunk) {
         const int k0 = chunk * KC;
         // a wait that runs out is recorded and the chunk computed on whatever is there; every thread sees the flag after
@@ -294,7 +305,7 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
         if (!mbar_wait(&sm.full[chunk & 1], uint32_t(chunk >> 1) & 1u)) *reinterpret_cast<volatile int*>(&sm.error) = 1;
         const BlkT<BM>& sa_blk = sm.a[chunk & 1];
         const BlkT<BN>& sb_blk = sm.b[chunk & 1];
-        const bool chunk_special = (sa_blk.special | sb_blk.special) != 0u;
+        const bool chunk_special = (sa_blk.special | sb_blk.special) != 0u, chunk_range = big || (sa_blk.sparse | sb_blk.sparse) != 0u;
 
 #pragma unroll 1
         for (int blk = 0; blk < NBLK; ++blk) {
@@ -390,11 +401,16 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
                             // |c| and t1 are positive FP32 patterns: their order as numbers is their order as words, and
                             // the absolute value rides on the instruction
                             e = __float_as_uint(fmaxf(__uint_as_float(t1), fabsf(__uint_as_float(cw[h][x]))));
-                            out_of_range = __viaddmax_u32(e, 0u - E_LOW, out_of_range);
                         }
                         p = e;
                     }
-                if (!ACC16 && out_of_range > E_HIGH - E_LOW) {     // rare: turn the outputs out of range into markers (see above)
+                if (!ACC16 && chunk_range) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) out_of_range = __viaddmax_u32(P[j][i], 0u - E_LOW, out_of_range);
+                }
+                if (!ACC16 && chunk_range && out_of_range > E_HIGH - E_LOW) {     // rare: turn the outputs out of range into markers (see above)
                     rare = true;
 #pragma unroll
                     for (int hh = 0; hh < 2; ++hh)
@@ -467,23 +483,20 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
             // ---- sign corrections and rho ----
             const uint32_t kmask = (L == 32) ? 0xFFFFFFFFu : (((1u << L) - 1u) << kb);
             uint32_t wmax = 0u;
-            uint32_t sbv[TW], nzb[TW];
+            uint32_t sbv[TW];
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 const uint4 u = *reinterpret_cast<const uint4*>(&sb_blk.sgn[wc * 32 + 8 * tq + 4 * q]);
-                const uint4 v = *reinterpret_cast<const uint4*>(&sb_blk.nz[wc * 32 + 8 * tq + 4 * q]);
                 sbv[4 * q] = u.x; sbv[4 * q + 1] = u.y; sbv[4 * q + 2] = u.z; sbv[4 * q + 3] = u.w;
-                nzb[4 * q] = v.x; nzb[4 * q + 1] = v.y; nzb[4 * q + 2] = v.z; nzb[4 * q + 3] = v.w;
             }
             auto finish = [&](auto with_markers) {
 #pragma unroll
                 for (int h = 0; h < TH; ++h) {
                     const uint32_t sa = sa_blk.sgn[wr * G::WROWS + TH * gq + h];
-                    const uint32_t nza = sa_blk.nz[wr * G::WROWS + TH * gq + h] & kmask;
                     uint32_t bitsv[TW], vv[TW];
 #pragma unroll
-                    for (int x = 0; x < TW; ++x)                   // every negative nonzero term fell one unit short:
-                        bitsv[x] = cw[h][x] + uint32_t(__popc((sa ^ sbv[x]) & nza & nzb[x]));   // (1.5 * 2^23 + S) * unit
+                    for (int x = 0; x < TW; ++x)                   // every negative term fell one unit short:
+                        bitsv[x] = cw[h][x] + uint32_t(__popc((sa ^ sbv[x]) & kmask));   // (1.5 * 2^23 + S) * unit
 #pragma unroll
                     for (int xp = 0; xp < TW / 2; ++xp)            // S * unit, exact; two columns per packed subtraction
                         asm("{\n\t.reg .b64 a, b, r;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tsub.rn.f32x2 r, a, b;\n\tmov.b64 {%0, %1}, r;\n\t}"
