@@ -127,7 +127,7 @@ __host__ __device__ constexpr int min_ctas(int tiles, int L, int warps) {
 // unit_a / unit_b: bytes per asynchronous copy that the row starts allow (the natural 16, or 8 for 8-bit elements; 4), or 0:
 // rows at odd addresses, read element by element in the decode step.
 template <int FAM, int EK, int L, int RHO, bool PROMOTE, int TM, int CN, int WR, int WC, int PW, int TASK>
-__global__ void __launch_bounds__(32 * (WR * WC + PW), min_ctas(TM * CN, L, WR * WC + PW)) direct_kernel(DevModel m, GemmArgs g, int unit_a, int unit_b) {
+__device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g, int unit_a, int unit_b, int64_t row0, int64_t col0) {
     static_assert(FAM == FAM_T || FAM == FAM_ST || FAM == FAM_TR || FAM == FAM_GTR || FAM == FAM_E, "FDPA families");
     constexpr bool T = FAM == FAM_T || FAM == FAM_ST, GTR = FAM == FAM_GTR, E = FAM == FAM_E;
     constexpr bool ACC16 = RHO == RHO_RNE_FP16, E8M13 = RHO == RHO_RZ_E8M13;
@@ -145,8 +145,6 @@ __global__ void __launch_bounds__(32 * (WR * WC + PW), min_ctas(TM * CN, L, WR *
     const bool stager = warp >= NC;                     // the first WR * WC warps compute, the others decode
     const int tid = int(threadIdx.x) - 32 * NC;         // (of a staging thread)
     const int wr = warp / WC, wc = warp % WC, gq = lane >> 2, tq = lane & 3;
-    const int64_t row0 = int64_t(blockIdx.y) * BM, col0 = int64_t(blockIdx.x) * BN;
-    if (T && !tile_wanted(g, row0, BM, col0, BN)) return;
     auto row_at = [&](int r) { return wr * 8 * TM + 8 * r + gq; };                       // inside the CTA tile
     auto col_at = [&](int c) { return wc * 8 * CN + 8 * (c >> 1) + 2 * tq + (c & 1); };
     const FmtDesc fa = fmt_desc(m.fmt_a), fb = fmt_desc(m.fmt_b);
@@ -713,6 +711,38 @@ __global__ void __launch_bounds__(32 * (WR * WC + PW), min_ctas(TM * CN, L, WR *
         }
 }
 
+template <int FAM, int EK, int L, int RHO, bool PROMOTE, int TM, int CN, int WR, int WC, int PW, int TASK>
+__global__ void __launch_bounds__(32 * (WR * WC + PW), min_ctas(TM * CN, L, WR * WC + PW)) direct_kernel(DevModel m, GemmArgs g, int unit_a, int unit_b) {
+    direct_tile<FAM, EK, L, RHO, PROMOTE, TM, CN, WR, WC, PW, TASK>(m, g, unit_a, unit_b, int64_t(blockIdx.y) * (8 * TM * WR), int64_t(blockIdx.x) * (8 * CN * WC));
+}
+
+// The tiles that the matrix instruction has to leave to the emulation (GemmArgs::least_a), on a fixed grid: almost always there are
+// none, and every CTA reads the smallest exponents and leaves (1024 x 4096: 3 us; a CTA per tile that looks at its own rows: 18 us).
+template <int FAM, int EK, int L, int RHO, int TM, int CN, int WR, int WC, int PW, int TASK>
+__global__ void __launch_bounds__(32 * (WR * WC + PW), min_ctas(TM * CN, L, WR * WC + PW)) direct_rest_kernel(DevModel m, GemmArgs g, int unit_a, int unit_b) {
+    constexpr int BM = 8 * TM * WR, BN = 8 * CN * WC;
+    __shared__ int least[2];
+    if (threadIdx.x < 2) least[threadIdx.x] = 1 << 20;
+    __syncthreads();
+    int a = 1 << 20, b = 1 << 20;
+#pragma unroll 8
+    for (int64_t i = threadIdx.x; i < g.M; i += blockDim.x) a = min(a, g.least_a[i]);
+#pragma unroll 8
+    for (int64_t j = threadIdx.x; j < g.N; j += blockDim.x) b = min(b, g.least_b[j]);
+    a = __reduce_min_sync(0xFFFFFFFFu, a);
+    b = __reduce_min_sync(0xFFFFFFFFu, b);
+    if (threadIdx.x % 32 == 0) { atomicMin(&least[0], a); atomicMin(&least[1], b); }
+    __syncthreads();
+    if (least[0] + least[1] >= -126) return;
+    const int64_t tn = (g.N + BN - 1) / BN, tiles = (g.M + BM - 1) / BM * tn;
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int64_t row0 = t / tn * BM, col0 = t % tn * BN;
+        if (!tile_wanted(g, row0, BM, col0, BN)) continue;
+        direct_tile<FAM, EK, L, RHO, false, TM, CN, WR, WC, PW, TASK>(m, g, unit_a, unit_b, row0, col0);
+        __syncthreads();
+    }
+}
+
 // Bytes per asynchronous copy that rows `ld` elements apart allow (bases are 16-byte aligned).
 template <int EK, int TASK>
 int copy_unit(int64_t ld) {
@@ -732,6 +762,18 @@ cudaError_t launch_tile(const DevModel& m, const GemmArgs& g, cudaStream_t st) {
     }
     const dim3 grid((unsigned)((g.N + BN - 1) / BN), (unsigned)((g.M + BM - 1) / BM), 1);
     kernel<<<grid, NTH, sh, st>>>(m, g, copy_unit<EK, TASK>(g.lda), copy_unit<EK, TASK>(g.ldb));
+    return cudaGetLastError();
+}
+
+template <int FAM, int EK, int L, int RHO>
+cudaError_t launch_rest(const DevModel& m, const GemmArgs& g, cudaStream_t st) {
+    constexpr int PW = 4, TASK = 8, NTH = 32 * (4 + PW);
+    constexpr size_t sh = sizeof(Smem<EK, 32, 32, 32 * PW, TASK>);
+    auto kernel = direct_rest_kernel<FAM, EK, L, RHO, 2, 2, 2, 2, PW, TASK>;
+    const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sh));
+    if (err != cudaSuccess) return err;
+    const int64_t tiles = (g.M + 31) / 32 * ((g.N + 31) / 32);
+    kernel<<<unsigned(tiles < 296 ? tiles : 296), NTH, sh, st>>>(m, g, copy_unit<EK, TASK>(g.lda), copy_unit<EK, TASK>(g.ldb));
     return cudaGetLastError();
 }
 

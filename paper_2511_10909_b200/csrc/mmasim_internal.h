@@ -93,8 +93,7 @@ bool fast_tfdpa_supported(const DevModel& m, const GemmArgs& g);
 int launch_fast_tfdpa(const DevModel& m, const GemmArgs& g, cudaStream_t stream);
 // the small-tile kernels (mmasim_direct.cuh): any K, any row stride; DIRECT_NONE: the large kernel is the better one
 enum DirectSize : int { DIRECT_NONE = 0, DIRECT_8x16, DIRECT_16x16, DIRECT_32x32 };
-// (`or_large` false: the best of the small tiles; `us`: about what the emulation takes)
-DirectSize direct_size(const DevModel& m, const GemmArgs& g, bool or_large = true, double* us = nullptr);
+DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us = nullptr);       // `us`: about what the emulation takes
 int launch_direct(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStream_t stream);
 int launch_gemm_noalloc(const DevModel& m, const GemmArgs& g, cudaStream_t stream);   // status code; sets the error message
 // mmasim_umma.cu: the rows that the B200's own matrix instruction computes

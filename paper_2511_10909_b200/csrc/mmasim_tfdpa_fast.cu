@@ -92,7 +92,7 @@ bool rows16(const DevModel& m, const GemmArgs& g) {                          // 
 // (its decode pass and two more launches: about 6 us, fifteen units of one chunk).  Examples, small against large in us, on both
 // sides of the line: Hopper FP16 128 x 2048 x 2048 128 / 337, 2352 x 192 x 3328 320 / 771, 1000 x 1111 x 992 245 / 254,
 // 1024^3 225 / 175, 2048 x 2048 x 512 449 / 340.
-DirectSize direct_size(const DevModel& m, const GemmArgs& g, bool or_large, double* us) {
+DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us) {
     const int kind = kind_of(m);
     if (!kind || g.dot_mode || m.literal_emax) return DIRECT_NONE;
     if ((kind == KIND_TR || kind == KIND_E) && g.k_chunk) return DIRECT_NONE;
@@ -104,7 +104,7 @@ DirectSize direct_size(const DevModel& m, const GemmArgs& g, bool or_large, doub
     const double large = f13 ? 13.5 : (bits8 ? 9.5 : (kind == KIND_E ? 22.0 : (kind == KIND_TR ? 18.0 : (m.L >= 16 ? 14.0 : 20.0))));
     const double c8 = 0.5 + 0.6 * fullest(8, 16), c16 = 0.6 + fullest(16, 16), c32 = 0.6 + mid * fullest(32, 32);
     const double chunks = double((g.K + fast::KC - 1) / fast::KC);
-    const double big = or_large && fast_tfdpa_supported(m, g) ? large * fullest(fast::BM, f13 && m.acc != ACC_F16 && !g.k_chunk ? 128 : fast::BN) + 15.0 / chunks : 1e30;
+    const double big = fast_tfdpa_supported(m, g) ? large * fullest(fast::BM, f13 && m.acc != ACC_F16 && !g.k_chunk ? 128 : fast::BN) + 15.0 / chunks : 1e30;
     if (us) *us = 3.0 + 0.45 * chunks * std::min(std::min(c8, c16), std::min(c32, big));
     if (big <= c8 && big <= c16 && big <= c32) return DIRECT_NONE;
     return c8 <= c16 && c8 <= c32 ? DIRECT_8x16 : (c16 <= c32 ? DIRECT_16x16 : DIRECT_32x32);

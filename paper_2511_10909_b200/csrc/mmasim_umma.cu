@@ -558,7 +558,7 @@ bool umma_supported(const DevModel& m, const GemmArgs& g) {
     if (overlap(g)) return false;
     if (mk == MK_MXF4) return fast_gst_supported(m, g);
     double us = 0.0;
-    direct_size(m, g, true, &us);
+    direct_size(m, g, &us);
     return us > 14.0;
 }
 
@@ -647,7 +647,7 @@ int launch_umma(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
         GemmArgs e = g;
         e.least_a = least_a;
         e.least_b = least_b;
-        st = mk == MK_MXF4 ? launch_fast_gst(m, e, stream) : launch_direct(m, e, direct_size(m, e, false), stream);
+        st = mk == MK_MXF4 ? launch_fast_gst(m, e, stream) : launch_direct(m, e, DIRECT_32x32, stream);
     }
     if (scratch) cudaFreeAsync(scratch, stream);
     // the names of the kernels that emulate the same rows: they say whose arithmetic it is
