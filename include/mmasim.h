@@ -166,7 +166,7 @@ int mmasim_dot_batch(const mmasim_model* model, int64_t n, int64_t K,
  * library creates per device on first use and that keeps up to 1 GiB between calls, so repeated calls do not pay
  * for allocation; mmasim_host_release() destroys the pools and returns the memory.  The device's default memory
  * pool and its attributes are not touched.  Pinned host buffers make the copies asynchronous.
- * Problems of 1024 rows and 32 MiB or more are cut into up to eight row panels of D (outputs are independent,
+ * Problems of 512 rows and 6 MiB or more are cut into up to six row panels of D (outputs are independent,
  * Section 3.1 Step 1): B is copied once, then each panel's rows of A and C go in, its kernel runs and its rows of D
  * come back on separate streams, so that with pinned buffers the copies run beside the arithmetic.
  * With opts->ldd > N only the N words of every row of D are written; the words between rows stay the caller's.
@@ -174,7 +174,7 @@ int mmasim_dot_batch(const mmasim_model* model, int64_t n, int64_t K,
 int mmasim_gemm_host(const mmasim_model* model, int64_t M, int64_t N, int64_t K,
                      const void* A, const void* B, const void* C, void* D, const mmasim_gemm_opts* opts);
 
-/* Destroys the memory pools mmasim_gemm_host created (every device); no mmasim_gemm_host call may be in flight.
+/* Destroys the memory pools, streams and events that mmasim_gemm_host keeps between calls (every device); no mmasim_gemm_host call may be in flight.
  * The next mmasim_gemm_host call creates a new pool.  No counterpart in the paper. */
 int mmasim_host_release(void);
 

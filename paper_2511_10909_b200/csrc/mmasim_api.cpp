@@ -1,10 +1,12 @@
 // C ABI of libmmasim: argument validation, model objects, dispatch to the kernels.
+#include <atomic>
 #include <cstdarg>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <vector>
 #include "mmasim_internal.h"
 
 namespace mmasim {
@@ -57,11 +59,12 @@ int check_k(const DevModel& m, int64_t K) {
     return MMASIM_OK;
 }
 
-int run_gemm(const mmasim_model* model, const GemmArgs& g, int flags, cudaStream_t stream) {
+// `whole`: the product that g is a row panel of, if it is one: its size decides on the tiles (panels run beside each other).
+int run_gemm(const mmasim_model* model, const GemmArgs& g, int flags, cudaStream_t stream, const GemmArgs* whole = nullptr) {
     const DevModel& m = model->dev;
     if (!(flags & MMASIM_GEMM_FORCE_GENERIC) && !m.literal_emax) {
         if (!(flags & MMASIM_GEMM_LARGE_TILES) && umma_supported(m, g)) return launch_umma(m, g, stream);
-        const DirectSize size = (flags & MMASIM_GEMM_LARGE_TILES) && fast_tfdpa_supported(m, g) ? DIRECT_NONE : direct_size(m, g);
+        const DirectSize size = (flags & MMASIM_GEMM_LARGE_TILES) && fast_tfdpa_supported(m, g) ? DIRECT_NONE : direct_size(m, whole ? *whole : g);
         if (size != DIRECT_NONE) return launch_direct(m, g, size, stream);
         if (fast_tfdpa_supported(m, g)) return launch_fast_tfdpa(m, g, stream);
         if (fast_fp_supported(m, g)) return launch_fast_fp(m, g, stream);
@@ -144,6 +147,9 @@ cudaError_t scratch_pool(cudaMemPool_t* out) {
         if (err != cudaSuccess) return err;
         unsigned long long keep = 1ull << 30;
         err = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        // a buffer that another stream will free must not make this stream wait for it: row panels run beside each other
+        int no = 0;
+        if (err == cudaSuccess) err = cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &no);
         if (err != cudaSuccess) { cudaMemPoolDestroy(pool); return err; }
         g_pools[dev] = pool;
     }
@@ -151,6 +157,67 @@ cudaError_t scratch_pool(cudaMemPool_t* out) {
     return cudaSuccess;
 }
 
+namespace {
+// The streams and events of one mmasim_gemm_host call, and a word of mapped host memory that its kernels count given-up waits in (a copy
+// of the device's counter before and after each call cost 15 us).  Creating them took about 100 us of every call, so up to
+// LANES_KEPT sets per device wait for the next one; a call has its set to itself, and mmasim_host_release destroys those that wait.
+struct HostLane {
+    static constexpr int PANELS = 6;        // (with the streams of the copies eight: more would share the hardware's eight queues)
+    int device = -1;
+    cudaStream_t in = nullptr, out = nullptr, k[PANELS] = {};
+    cudaEvent_t ev_in[PANELS] = {}, ev_k[PANELS] = {};
+    unsigned int* gave_up = nullptr;        // host address
+    unsigned int* gave_up_dev = nullptr;    // device address
+};
+constexpr int LANES_KEPT = 4;
+std::atomic<unsigned int> g_host_timeouts[MAX_DEVICES];     // what the words of finished calls held
+std::mutex g_lane_mutex;
+std::vector<HostLane> g_lanes[MAX_DEVICES];
+
+void destroy_lane(HostLane& l) {
+    for (int p = 0; p < HostLane::PANELS; ++p) {
+        if (l.ev_in[p]) cudaEventDestroy(l.ev_in[p]);
+        if (l.ev_k[p]) cudaEventDestroy(l.ev_k[p]);
+        if (l.k[p]) cudaStreamDestroy(l.k[p]);
+    }
+    if (l.in) cudaStreamDestroy(l.in);
+    if (l.out) cudaStreamDestroy(l.out);
+    if (l.gave_up) cudaFreeHost(l.gave_up);
+    l = HostLane();
+}
+cudaError_t take_lane(HostLane* out) {
+    int dev = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess) return err;
+    if (dev < 0 || dev >= MAX_DEVICES) return cudaErrorInvalidDevice;
+    {
+        std::lock_guard<std::mutex> lock(g_lane_mutex);
+        if (!g_lanes[dev].empty()) { *out = g_lanes[dev].back(); g_lanes[dev].pop_back(); return cudaSuccess; }
+    }
+    HostLane l;
+    l.device = dev;
+    err = cudaHostAlloc(reinterpret_cast<void**>(&l.gave_up), sizeof(unsigned int), cudaHostAllocMapped);
+    if (err == cudaSuccess) err = cudaHostGetDevicePointer(reinterpret_cast<void**>(&l.gave_up_dev), l.gave_up, 0);
+    if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&l.in, cudaStreamNonBlocking);
+    if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&l.out, cudaStreamNonBlocking);
+    for (int p = 0; p < HostLane::PANELS && err == cudaSuccess; ++p) {
+        err = cudaStreamCreateWithFlags(&l.k[p], cudaStreamNonBlocking);
+        if (err == cudaSuccess) err = cudaEventCreateWithFlags(&l.ev_in[p], cudaEventDisableTiming);
+        if (err == cudaSuccess) err = cudaEventCreateWithFlags(&l.ev_k[p], cudaEventDisableTiming);
+    }
+    if (err != cudaSuccess) destroy_lane(l);
+    *out = l;
+    return err;
+}
+void give_lane(HostLane& l, bool sound) {
+    if (l.device < 0) return;
+    if (sound) {
+        std::lock_guard<std::mutex> lock(g_lane_mutex);
+        if (g_lanes[l.device].size() < LANES_KEPT) { g_lanes[l.device].push_back(l); return; }
+    }
+    destroy_lane(l);
+}
+}  // namespace
 
 }  // namespace mmasim
 
@@ -294,64 +361,41 @@ int mmasim_gemm_host(const mmasim_model* model, int64_t M, int64_t N, int64_t K,
     const mmasim_info& info = model->info;
     const size_t a_bytes = size_t((M - 1) * g.lda + K) * info.a_bits / 8;
     const size_t b_bytes = size_t((N - 1) * g.ldb + K) * info.b_bits / 8;
-    const size_t c_bytes = size_t((M - 1) * g.ldc + N) * info.acc_bytes;
+    const size_t c_bytes = g.C ? size_t((M - 1) * g.ldc + N) * info.acc_bytes : 0;
     const size_t d_bytes = size_t((M - 1) * g.ldd + N) * info.acc_bytes;
     const size_t sfa_bytes = g.sfa ? size_t(M * g.ld_sfa) : 0, sfb_bytes = g.sfb ? size_t(N * g.ld_sfb) : 0;
-    void *dA = nullptr, *dB = nullptr, *dC = nullptr, *dD = nullptr, *dSA = nullptr, *dSB = nullptr, *dRS = nullptr, *dCS = nullptr;
-    cudaError_t err = cudaSuccess;
-    // Stream-ordered allocations on a stream of this call's own: after the first call the buffers come out of the
-    // library's own memory pool (which keeps up to 1 GiB between calls) and the call synchronises once, at the end.
-    // Large problems are cut into a few row panels of D (outputs are independent, Section 3.1 Step 1): B once, then per
-    // panel its rows of A and C in, the kernel, its rows of D out, on three streams chained by events, so that the
-    // copies of one panel run beside the arithmetic of another (two compute streams, so that a panel's last CTAs
-    // share the SMs with the next panel's first).
-    // the counter of bulk-copy timeouts before the call: a kernel of this call that gives up makes it grow
-    unsigned int timeouts_before = 0u;
-    if (g.copy_timeouts) cudaMemcpy(&timeouts_before, g.copy_timeouts, sizeof(unsigned int), cudaMemcpyDeviceToHost);
-    constexpr int MAX_PANELS = 16;
-    int panels = 1;
-    int64_t panel_rows = M;
-    if (M >= 1024 && a_bytes + b_bytes + c_bytes + d_bytes >= (size_t(32) << 20)) {
-        // whole CTA tiles, at most about eight panels, and at least 256 tiles of 128 x 128 per panel: with fewer a
-        // panel's kernel leaves most of the 296 CTA slots of the GPU empty
-        panel_rows = ((M + 7) / 8 + 127) / 128 * 128;
-        const int64_t fill_rows = 128 * ((256 + (N + 127) / 128 - 1) / ((N + 127) / 128));
-        if (panel_rows < fill_rows) panel_rows = fill_rows;
-        if (panel_rows < 512) panel_rows = 512;
-        panels = int((M + panel_rows - 1) / panel_rows);
-        if (panels > MAX_PANELS) { panels = 1; panel_rows = M; }
-    }
-    cudaStream_t s_in = nullptr, s_k[2] = {nullptr, nullptr}, s_out = nullptr;
-    cudaEvent_t ev_in[MAX_PANELS] = {}, ev_k[MAX_PANELS] = {};
-    err = cudaStreamCreateWithFlags(&s_in, cudaStreamNonBlocking);
-    if (err == cudaSuccess && panels > 1) {
-        err = cudaStreamCreateWithFlags(&s_k[0], cudaStreamNonBlocking);
-        if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&s_k[1], cudaStreamNonBlocking);
-        if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&s_out, cudaStreamNonBlocking);
-        for (int p = 0; p < panels && err == cudaSuccess; ++p) {
-            err = cudaEventCreateWithFlags(&ev_in[p], cudaEventDisableTiming);
-            if (err == cudaSuccess) err = cudaEventCreateWithFlags(&ev_k[p], cudaEventDisableTiming);
-        }
-    }
+    // Row panels of D (outputs are independent, Section 3.1 Step 1): B once, then per panel its rows of A and C in, the kernel, its rows
+    // of D out, so that copies in, arithmetic and copies out run beside each other.  A panel is whole CTA tiles and, with its copies,
+    // about 3 MB (55 us of the bus, against some 10 us that its calls cost), at most six; every panel has a stream of its own, because
+    // one alone does not fill the SMs.  Large tiles want 512 rows: every one walks all of K, and the last panel's come last.
+    // In us, one panel / several: Ampere BF16 1475 x 1214 x 1072 890 / 675, 1477 x 1229 x 144 283 / 256, 1216 x 1306 x 624 604 / 430,
+    // Hopper E4M3 2048 x 2048 x 2048 1460 / 1130 (384 rows: 1215).
+    const bool large_tiles = fast_tfdpa_supported(model->dev, g) && !umma_supported(model->dev, g) && direct_size(model->dev, g) == DIRECT_NONE;
+    int panels = int((a_bytes + c_bytes + d_bytes) / (size_t(3) << 20));
+    panels = panels < 1 || M < 512 ? 1 : (panels > HostLane::PANELS ? HostLane::PANELS : panels);
+    int64_t panel_rows = panels > 1 ? ((M + panels - 1) / panels + 127) / 128 * 128 : M;
+    if (large_tiles && panels > 1 && panel_rows < 512) panel_rows = 512;
+    panels = int((M + panel_rows - 1) / panel_rows);
+    HostLane lane;
+    cudaError_t err = take_lane(&lane);
     cudaMemPool_t pool = nullptr;
     if (err == cudaSuccess) err = scratch_pool(&pool);
-    auto alloc = [&](void** dst, const void* src, size_t bytes) {
+    // one allocation, stream-ordered out of the library's own pool (which keeps up to 1 GiB between calls)
+    auto up256 = [](size_t x) { return (x + 255) / 256 * 256; };
+    const size_t sizes[8] = {a_bytes, b_bytes, c_bytes, d_bytes, sfa_bytes, sfb_bytes, g.row_scale ? size_t(M) * 4 : 0, g.col_scale ? size_t(N) * 4 : 0};
+    size_t total = 0;
+    for (size_t x : sizes) total += up256(x);
+    unsigned char* base = nullptr;
+    if (err == cudaSuccess) err = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&base), total, pool, lane.in);
+    unsigned char* at[8];
+    size_t off = 0;
+    for (int i = 0; i < 8; ++i) { at[i] = sizes[i] ? base + off : nullptr; off += up256(sizes[i]); }
+    unsigned char *dA = at[0], *dB = at[1], *dC = at[2], *dD = at[3], *dSA = at[4], *dSB = at[5], *dRS = at[6], *dCS = at[7];
+    auto h2d = [&](void* dst, const void* src, size_t at_byte, size_t bytes) {
         if (err != cudaSuccess || !src || !bytes) return;
-        err = cudaMallocFromPoolAsync(dst, bytes, pool, s_in);
+        err = cudaMemcpyAsync(static_cast<unsigned char*>(dst) + at_byte, static_cast<const unsigned char*>(src) + at_byte, bytes, cudaMemcpyHostToDevice, lane.in);
     };
-    auto h2d = [&](void* dst, const void* src, size_t off, size_t bytes) {
-        if (err != cudaSuccess || !src || !bytes) return;
-        err = cudaMemcpyAsync(static_cast<unsigned char*>(dst) + off, static_cast<const unsigned char*>(src) + off, bytes,
-                              cudaMemcpyHostToDevice, s_in);
-    };
-    alloc(&dA, A, a_bytes);
-    alloc(&dB, B, b_bytes);
-    alloc(&dC, C, c_bytes);
-    alloc(&dSA, g.sfa, sfa_bytes);
-    alloc(&dSB, g.sfb, sfb_bytes);
-    alloc(&dRS, g.row_scale, size_t(M) * 4);
-    alloc(&dCS, g.col_scale, size_t(N) * 4);
-    alloc(&dD, D, d_bytes);
+    if (err == cudaSuccess) { *lane.gave_up = 0u; g.copy_timeouts = lane.gave_up_dev; }
     h2d(dB, B, 0, b_bytes);
     h2d(dSB, g.sfb, 0, sfb_bytes);
     h2d(dRS, g.row_scale, 0, size_t(M) * 4);
@@ -367,64 +411,56 @@ int mmasim_gemm_host(const mmasim_model* model, int64_t M, int64_t N, int64_t K,
         h2d(dC, C, c_off, c_len);
         h2d(dSA, host.sfa, size_t(r0 * host.ld_sfa), host.sfa ? size_t(rows * host.ld_sfa) : 0);
         if (err != cudaSuccess) break;
-        cudaStream_t sk = panels > 1 ? s_k[p & 1] : s_in;
+        const cudaStream_t sk = panels > 1 ? lane.k[p] : lane.in, so = panels > 1 ? lane.out : lane.in;
         if (panels > 1) {
-            err = cudaEventRecord(ev_in[p], s_in);
-            if (err == cudaSuccess) err = cudaStreamWaitEvent(sk, ev_in[p], 0);
+            err = cudaEventRecord(lane.ev_in[p], lane.in);
+            if (err == cudaSuccess) err = cudaStreamWaitEvent(sk, lane.ev_in[p], 0);
             if (err != cudaSuccess) break;
         }
         GemmArgs q = host;
         q.M = rows;
-        q.A = static_cast<const unsigned char*>(dA) + a_off;
+        q.A = dA + a_off;
         q.B = dB;
-        q.C = dC ? static_cast<const unsigned char*>(dC) + c_off : nullptr;
-        q.D = static_cast<unsigned char*>(dD) + d_off;
-        q.sfa = dSA ? static_cast<const uint8_t*>(dSA) + r0 * host.ld_sfa : nullptr;
-        q.sfb = static_cast<const uint8_t*>(dSB);
-        q.row_scale = dRS ? static_cast<const float*>(dRS) + r0 : nullptr;
-        q.col_scale = static_cast<const float*>(dCS);
-        st = run_gemm(model, q, opts ? opts->flags : 0, sk);
+        q.C = dC ? dC + c_off : nullptr;
+        q.D = dD + d_off;
+        q.sfa = dSA ? dSA + r0 * host.ld_sfa : nullptr;
+        q.sfb = dSB;
+        q.row_scale = dRS ? reinterpret_cast<const float*>(dRS) + r0 : nullptr;
+        q.col_scale = reinterpret_cast<const float*>(dCS);
+        st = run_gemm(model, q, opts ? opts->flags : 0, sk, &host);
         if (st != MMASIM_OK) break;
-        cudaStream_t so = panels > 1 ? s_out : s_in;
         if (panels > 1) {
-            err = cudaEventRecord(ev_k[p], sk);
-            if (err == cudaSuccess) err = cudaStreamWaitEvent(so, ev_k[p], 0);
+            err = cudaEventRecord(lane.ev_k[p], sk);
+            if (err == cudaSuccess) err = cudaStreamWaitEvent(so, lane.ev_k[p], 0);
             if (err != cudaSuccess) break;
         }
         // only the N words of every row go back: with ldd > N the words between the rows of the caller's D are not the library's
         if (host.ldd == N)
-            err = cudaMemcpyAsync(static_cast<unsigned char*>(D) + d_off, static_cast<unsigned char*>(dD) + d_off, d_len,
-                                  cudaMemcpyDeviceToHost, so);
+            err = cudaMemcpyAsync(static_cast<unsigned char*>(D) + d_off, dD + d_off, d_len, cudaMemcpyDeviceToHost, so);
         else
-            err = cudaMemcpy2DAsync(static_cast<unsigned char*>(D) + d_off, size_t(host.ldd) * info.acc_bytes,
-                                    static_cast<unsigned char*>(dD) + d_off, size_t(host.ldd) * info.acc_bytes,
+            err = cudaMemcpy2DAsync(static_cast<unsigned char*>(D) + d_off, size_t(host.ldd) * info.acc_bytes, dD + d_off, size_t(host.ldd) * info.acc_bytes,
                                     size_t(N) * info.acc_bytes, size_t(rows), cudaMemcpyDeviceToHost, so);
     }
     // everything drains, then the buffers go back to the pool in the order of the stream they came from
-    cudaStream_t all[] = {s_k[0], s_k[1], s_out};
-    for (cudaStream_t s : all)
-        if (s) { const cudaError_t e2 = cudaStreamSynchronize(s); if (err == cudaSuccess) err = e2; }
-    if (s_in) {
-        void* bufs[] = {dA, dB, dC, dD, dSA, dSB, dRS, dCS};
-        for (void* b : bufs) if (b) cudaFreeAsync(b, s_in);
-        const cudaError_t e2 = cudaStreamSynchronize(s_in);
-        if (err == cudaSuccess) err = e2;
+    bool sound = err == cudaSuccess;
+    if (lane.in) {
+        for (int p = 0; p < panels && panels > 1; ++p) { const cudaError_t e = cudaStreamSynchronize(lane.k[p]); if (err == cudaSuccess) err = e; }
+        if (panels > 1) { const cudaError_t e = cudaStreamSynchronize(lane.out); if (err == cudaSuccess) err = e; }
+        if (base) cudaFreeAsync(base, lane.in);
+        const cudaError_t e = cudaStreamSynchronize(lane.in);
+        if (err == cudaSuccess) err = e;
     }
-    for (int p = 0; p < MAX_PANELS; ++p) { if (ev_in[p]) cudaEventDestroy(ev_in[p]); if (ev_k[p]) cudaEventDestroy(ev_k[p]); }
-    cudaStream_t streams[] = {s_in, s_k[0], s_k[1], s_out};
-    for (cudaStream_t s : streams) if (s) cudaStreamDestroy(s);
+    const unsigned int count = err == cudaSuccess ? *static_cast<volatile unsigned int*>(lane.gave_up) : 0u;
+    if (count) g_host_timeouts[lane.device] += count;
+    give_lane(lane, sound && err == cudaSuccess);
     if (err != cudaSuccess) {
         cudaGetLastError();
         set_error("mmasim_gemm_host: %s", cudaGetErrorString(err));
         return MMASIM_ERR_CUDA;
     }
-    if (st == MMASIM_OK && g.copy_timeouts) {
-        unsigned int timeouts_after = timeouts_before;
-        cudaMemcpy(&timeouts_after, g.copy_timeouts, sizeof(unsigned int), cudaMemcpyDeviceToHost);
-        if (timeouts_after != timeouts_before) {
-            set_error("mmasim_gemm_host: %u CTAs gave up waiting for a bulk copy and stored nothing", timeouts_after - timeouts_before);
-            return MMASIM_ERR_TIMEOUT;
-        }
+    if (st == MMASIM_OK && count) {
+        set_error("mmasim_gemm_host: %u CTAs gave up waiting for a bulk copy and stored nothing", count);
+        return MMASIM_ERR_TIMEOUT;
     }
     return st;
 }
@@ -490,6 +526,17 @@ int mmasim_reference_fp64(const mmasim_model* model, int64_t M, int64_t N, int64
 }
 
 int mmasim_host_release(void) {
+    {
+        std::lock_guard<std::mutex> lanes(g_lane_mutex);
+        int current = 0;
+        const bool known = cudaGetDevice(&current) == cudaSuccess;
+        for (int d = 0; d < MAX_DEVICES; ++d) {
+            if (!g_lanes[d].empty()) cudaSetDevice(d);
+            for (HostLane& l : g_lanes[d]) destroy_lane(l);
+            g_lanes[d].clear();
+        }
+        if (known) cudaSetDevice(current);
+    }
     std::lock_guard<std::mutex> lock(g_pool_mutex);
     cudaError_t err = cudaSuccess;
     for (int d = 0; d < MAX_DEVICES; ++d)
@@ -512,9 +559,11 @@ int mmasim_copy_timeouts(uint64_t* count) {
     if (!count) { set_error("count is NULL"); return MMASIM_ERR_INVALID_ARG; }
     unsigned int* p = copy_timeout_counter();
     unsigned int v = 0u;
+    int dev = 0;
     cudaError_t err = p ? cudaMemcpy(&v, p, sizeof(v), cudaMemcpyDeviceToHost) : cudaErrorUnknown;
+    if (err == cudaSuccess) err = cudaGetDevice(&dev);
     if (err != cudaSuccess) { set_error("mmasim_copy_timeouts: %s", cudaGetErrorString(err)); return MMASIM_ERR_CUDA; }
-    *count = v;
+    *count = v + (dev < MAX_DEVICES ? g_host_timeouts[dev].load() : 0u);
     return MMASIM_OK;
 }
 const char* mmasim_last_error(void) { return g_error; }

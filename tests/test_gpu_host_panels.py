@@ -1,0 +1,37 @@
+"""mmasim_gemm_host in one panel, in several, and with a last panel shorter than the others, from several threads at once and after the
+kept streams were given back, against the same product on device memory."""
+import threading
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2511_10909_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+gu = pytest.importorskip("gpu_util") if torch.cuda.is_available() else None
+
+
+@pytest.mark.parametrize("key,shape", [(("hopper", "e4m3", "fp32"), (2100, 1100, 256)), (("ampere", "bf16", "fp32"), (1500, 1300, 40)),
+                                       (("hopper", "fp16", "fp32"), (513, 6000, 64)), (("blackwell", "nvf4", "fp32"), (1700, 1600, 128)),
+                                       (("volta", "fp16", "fp16"), (40, 30, 20))], ids=str)
+def test_panels_and_threads(key, shape):
+    from paper_2511_10909_b200 import mmasim
+    M, N, K = shape
+    inp = wl.normal_inputs(key[1], key[2], M, N, K, seed=5)
+    want = gu.run_gemm(key, inp)
+    model = mmasim.Model(*key)
+    got = [None] * 3
+
+    def call(i):
+        got[i] = mmasim.gemm_host(model, inp["A"], inp["B"], inp["C"], K=K, sfa=inp.get("sfa"), sfb=inp.get("sfb"))
+    threads = [threading.Thread(target=call, args=(i,)) for i in range(3)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for x in got:
+        assert np.array_equal(x.view(want.dtype), want)
+    mmasim.host_release()
+    call(0)
+    assert np.array_equal(got[0].view(want.dtype), want)
