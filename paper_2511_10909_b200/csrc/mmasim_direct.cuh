@@ -108,6 +108,7 @@ struct Smem {
     __align__(16) uint32_t e[BUF][ROWS][EP];            // exponents of elements 2 p (low half) and 2 p + 1 (high half)
     uint32_t sgn[BUF][ROWS], nz[BUF][ROWS];             // bit k: sign / finite and nonzero
     int special[BUF];                                   // n + 1: chunk n holds an infinity or a NaN (ST: or a NaN scale factor)
+    int wild[BUF];                                      // n + 1: chunk n holds a nonzero element outside [2^-48, 2^40)
     uint32_t max_exp[BUF][2];                           // (n + 1) << 11 | largest Exp + EB of chunk n's A and B (TR-FDPA, wide formats)
 };
 
@@ -134,6 +135,9 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
     constexpr int TN = 2 * CN, BM = 8 * TM * WR, BN = 8 * CN * WC, NTH = 32 * PW;     // NTH: the staging threads
     constexpr int BYTES = Elem<EK>::BYTES;
     constexpr bool TOP = FAM == FAM_TR && (EK == fast::EK_BF16 || EK == fast::EK_TF32);     // products that may reach 2^128
+    // results are tested for the range of normal FP32 numbers only where they can leave it (see mmasim_tfdpa_f64.cuh); the small tiles
+    // wait for the chain of a block, not for the integer pipe: a second body of code gained and lost 2 - 6 % from size to size
+    constexpr bool TAMEABLE = FAM == FAM_T && !ACC16 && TM * CN >= 4;
     static_assert(TM * TN <= 16 && KC % L == 0, "sticky flags are 16-bit masks; blocks tile the chunk");
     constexpr int NC = WR * WC, NBLK = KC / L;
     using SM = Smem<EK, BM, BN, NTH, TASK>;
@@ -196,7 +200,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
     };
     auto stage = [&](int n) {                           // decode the thread's own raw words of chunk n into buffer n mod 3
         const int buf = n % BUF;
-        uint32_t spec = 0u, top_a = 0u, top_b = 0u;
+        uint32_t spec = 0u, wild = 0u, top_a = 0u, top_b = 0u;
 #pragma unroll
         for (int it = 0; it < SM::PER; ++it) {
             const int task = it * NTH + tid;
@@ -247,6 +251,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
                 nbits = __funnelshift_l(mag + 0x7FFFFFFFu, nbits, 1);
                 if (q & 1) ep[q / 2] = expb << 16; else ep[q / 2] |= expb;
             }
+            if (WIDE && TAMEABLE) wild |= uint32_t(top >= uint32_t(127 + 40) << 23) | uint32_t(low < (uint32_t(127 - 48) << 23) - 1u);
             if (top >= 0x7F800000u || (WIDE && low < 0x007FFFFFu) || sc_nan) {
                 // rare: infinities and NaNs are staged as zeros without exponent, like the rows of a NaN scale factor; an FP32
                 // subnormal is a small integer times 2^-149
@@ -301,6 +306,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
             }
         }
         if (spec) sm.special[buf] = n + 1;
+        if (wild) sm.wild[buf] = n + 1;
         if (TOP) {
             if (top_a) atomicMax(&sm.max_exp[buf][0], uint32_t(n + 1) << 11 | top_a);
             if (top_b) atomicMax(&sm.max_exp[buf][1], uint32_t(n + 1) << 11 | top_b);
@@ -334,7 +340,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
     };
     // (exponent sum + CB) << 20 becomes the exponent field e_max + 1023 (T), or that of the constant 1.5 * 2^52 * 2^(e_max - F) (TR)
     const int key_add = T ? -(1 << 20) : (1023 + 52 - m.F - CB) << 20;
-    if (threadIdx.x < BUF) { sm.special[threadIdx.x] = 0; sm.max_exp[threadIdx.x][0] = sm.max_exp[threadIdx.x][1] = 0u; }
+    if (threadIdx.x < BUF) { sm.special[threadIdx.x] = sm.wild[threadIdx.x] = 0; sm.max_exp[threadIdx.x][0] = sm.max_exp[threadIdx.x][1] = 0u; }
     __syncthreads();
     if (stager) {
         // during chunk n, which looks ahead at the exponents of chunk n + 1, chunk n + 2 is decoded
@@ -435,8 +441,9 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
         fetch_fragments(nb, nkb, ks);
         fetch_exponents(nb, nkb, ks);
     };
-    auto block = [&](int kb, int nb, int nkb, auto careful) {
-        constexpr bool CAREFUL = decltype(careful)::value;
+    enum { PLAIN = 0, CAREFULLY, IN_RANGE };
+    auto block = [&](int kb, int nb, int nkb, auto mode) {
+        constexpr bool CAREFUL = decltype(mode)::value == CAREFULLY, TAME = decltype(mode)::value == IN_RANGE;
         const uint32_t kmask = (L == 32) ? 0xFFFFFFFFu : (((1u << (L % 32)) - 1u) << kb);
         if constexpr (T) {
             // blocks of at most 8 terms, and F = 13: the sum register's low word, started at 2^31, never carries
@@ -480,9 +487,11 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
                         v = __dsub_rn(__longlong_as_double(__double_as_longlong(acc[r][c]) + (long long)nneg), __hiloint2double(mhi[r][c], 0));
                     if constexpr (SPLIT) v = __dadd_rn(v, __dsub_rn(acc2[r][c], __hiloint2double(mhi[r][c], 0)));
                     if (ACC16) asm("cvt.f64.f16 %0, %1;" : "=d"(v) : "h"(__half_as_ushort(__double2half(v))));
-                    const uint32_t twice = uint32_t(imad(__double2hiint(v), c_mul64[6], 0));          // (the sign leaves at the top)
-                    seen_max = max(seen_max, twice);
-                    seen_min = __viaddmin_u32(twice, 0xFFFFFFFFu, seen_min);                          // (zero wraps: it needs nothing)
+                    if (!TAME) {
+                        const uint32_t twice = uint32_t(imad(__double2hiint(v), c_mul64[6], 0));      // (the sign leaves at the top)
+                        seen_max = max(seen_max, twice);
+                        seen_min = __viaddmin_u32(twice, 0xFFFFFFFFu, seen_min);                      // (zero wraps: it needs nothing)
+                    }
                     if (ACC16) cs[r][c] = __hiloint2double(__double2hiint(v), __double2loint(v) | 1);
                     else if (E8M13) cs[r][c] = __hiloint2double(__double2hiint(v) & int(0xFFFFFF80u), 1);
                     else cs[r][c] = __hiloint2double(__double2hiint(v), (__double2loint(v) & int(0xE0000000u)) | 1);
@@ -597,6 +606,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
         sp_nan = sp_pinf = sp_ninf = 0u;
         subnormal = false;
     };
+    bool c_tame = false;
     subnormal = __any_sync(0xFFFFFFFFu, subnormal);     // (matrix instructions need the whole warp: what they depend on is voted)
     for (int chunk = 0; chunk < NCH; ++chunk) {
         const int buf = chunk % BUF, next_buf = (chunk + 1) % BUF, k0 = chunk * KC, kc = min(KC, K - k0), nblk = (kc + L - 1) / L;
@@ -619,7 +629,29 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
         // ---- a whole chunk without special values, promotion or odd accumulators runs through plain blocks; if one of them
         // notes a result outside the normal range, the chunk is done again from the accumulators it began with ----
         bool again = true;
-        if (!rare && !subnormal && nblk == NBLK && !(PROMOTE && until < KC)) {
+        const bool whole = !rare && !subnormal && nblk == NBLK && !(PROMOTE && until < KC);
+        bool tame = TAMEABLE && whole && !(WIDE && sm.wild[buf] == chunk + 1);
+        if (tame && !c_tame) {
+            bool ok = true;
+#pragma unroll
+            for (int r = 0; r < TM; ++r)
+#pragma unroll
+                for (int c = 0; c < TN; ++c) {
+                    const uint32_t h = uint32_t(__double2hiint(cs[E ? 0 : r][E ? 0 : c])) & 0x7FFFFFFFu;
+                    ok = ok && (h == 0u || h - (uint32_t(1023 - 100) << 20) < (200u << 20));
+                }
+            c_tame = __all_sync(0xFFFFFFFFu, ok);
+        }
+        tame = tame && c_tame;
+        c_tame = tame;
+        constexpr int UNROLL = NBLK * TM * TN <= 32 ? NBLK : (32 / (TM * TN) > 1 ? 32 / (TM * TN) : 1);
+        if (TAMEABLE && tame) {
+#pragma unroll UNROLL
+            for (int blk = 0; blk < NBLK; ++blk)
+                block(blk * L, blk + 1 < NBLK ? buf : next_buf, blk + 1 < NBLK ? blk * L + L : 0, std::integral_constant<int, TAMEABLE ? IN_RANGE : PLAIN>{});
+            again = false;
+            if (PROMOTE && (until -= KC) == 0) promote();
+        } else if (whole) {
             double cs0[E ? 1 : TM][E ? 1 : TN];
             uint32_t cw0[E ? TM : 1][E ? TN : 1];
 #pragma unroll
@@ -630,9 +662,8 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
             seen_min = 0xFFFFFFFFu;
             seen_top = 0.f;
             slow = 0u;
-            constexpr int UNROLL = NBLK * TM * TN <= 32 ? NBLK : (32 / (TM * TN) > 1 ? 32 / (TM * TN) : 1);
 #pragma unroll UNROLL
-            for (int blk = 0; blk < NBLK; ++blk) block(blk * L, blk + 1 < NBLK ? buf : next_buf, blk + 1 < NBLK ? blk * L + L : 0, std::false_type{});
+            for (int blk = 0; blk < NBLK; ++blk) block(blk * L, blk + 1 < NBLK ? buf : next_buf, blk + 1 < NBLK ? blk * L + L : 0, std::integral_constant<int, PLAIN>{});
             const bool done = T ? seen_max < 2u * TOPHI && seen_min >= 2u * LOWHI - 1u : (E ? slow == 0u : seen_top <= 3.4028234663852886e38f);
             again = __any_sync(0xFFFFFFFFu, !done);
             if (again) {
@@ -673,7 +704,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
                         }
                 }
                 slow = 0u;
-                block(kb, blk + 1 < nblk ? buf : next_buf, blk + 1 < nblk ? kb + L : 0, std::true_type{});
+                block(kb, blk + 1 < nblk ? buf : next_buf, blk + 1 < nblk ? kb + L : 0, std::integral_constant<int, CAREFULLY>{});
                 if (E && slow) {                        // by the book on the raw words
 #pragma unroll
                     for (int r = 0; r < TM; ++r)

@@ -254,7 +254,8 @@ struct Blk64 {
     uint8_t sf[R];                  // [permuted row]: the E8M0 scale factor of the row for this block of 32 (ST-FDPA), else 127
     uint32_t special;               // the block holds an infinity or a NaN
     uint32_t max_exp;               // the largest Exp(x) + EB of the block's elements (0: all zero)
-    uint32_t pad[2];
+    uint32_t wild;                  // some nonzero element lies outside [2^-48, 2^40)
+    uint32_t pad;
 };
 static_assert(sizeof(Blk64<BM>) % 16 == 0 && sizeof(Blk64<BN>) % 16 == 0, "bulk copies move multiples of 16 bytes");
 
@@ -276,7 +277,10 @@ __host__ __device__ constexpr int pe64_sub(int base) { return base == 8 ? 32 : (
 // place dst[tile][chunk].  Rows beyond the matrix decode as zeros.
 // EOSPLIT (GTR-FDPA, blocks of 16): inside each block of 16 the operand plane holds the even elements first, then the odd
 // ones, so that a matrix instruction sums four elements of one group; exponent pairs and masks keep the order of K.
-template <int EK, int R, bool IS_A, int BASE, bool EOSPLIT = false>
+// TINY_ZEROS (the T-FDPA kernels without a tensor-core maximum): a zero is staged as 2^-900 of its sign.  Its products are far below any
+// unit of a sum register, so that a positive one adds nothing and a negative one falls one unit short like every other
+// negative product: the sign masks alone count them, without the masks of nonzero elements.
+template <int EK, int R, bool IS_A, int BASE, bool EOSPLIT = false, bool TINY_ZEROS = false>
 __global__ void __launch_bounds__(256) decode64_kernel(DevModel m, const unsigned char* src, int64_t rows, int64_t ld, Blk64<R>* dst,
                                                        const uint8_t* sf = nullptr, int64_t ld_sf = 0) {
     using E = Elem<EK>;
@@ -297,10 +301,10 @@ __global__ void __launch_bounds__(256) decode64_kernel(DevModel m, const unsigne
         e.bits = (fin ? dec_sign(dd) : 0u) | (fin ? 0u : 2u) | (sg ? 4u : 0u);
         lut[tid] = e;
     }
-    if (tid == 0) { blk.special = 0u; blk.max_exp = 0u; blk.pad[0] = blk.pad[1] = 0u; }
+    if (tid == 0) { blk.special = 0u; blk.max_exp = 0u; blk.wild = blk.pad = 0u; }
     __syncthreads();
     const int64_t k0 = int64_t(blockIdx.x) * KC;
-    uint32_t spec = 0u, top_exp = 0u;
+    uint32_t spec = 0u, top_exp = 0u, wild = 0u;
     for (int task = tid; task < TASKS; task += 256) {
         const int r = task % R, h = task / R;
         const int pr = IS_A ? perm_row64(r) : perm_col64(r);
@@ -360,7 +364,9 @@ __global__ void __launch_bounds__(256) decode64_kernel(DevModel m, const unsigne
                 } else {
                     nzbit = 0u;
                     spec |= uint32_t(field == TOP);
+                    if (TINY_ZEROS) hi = uint32_t(1023 - 900) << 20;
                 }
+                if (E::EBITS == 8) wild |= uint32_t(expb - uint32_t(EB - 48) >= 88u && expb != 0u);
                 op = __hiloint2double(int(hi | (sign << 31)), int(lo));
                 bits += (sign | (nzbit << 16)) << q;
             }
@@ -384,6 +390,7 @@ __global__ void __launch_bounds__(256) decode64_kernel(DevModel m, const unsigne
         }
     }
     if (spec) atomicOr(&blk.special, 1u);
+    if (wild) atomicOr(&blk.wild, 1u);
     if (tid < R) {                                      // the scale factors travel with the block (rows beyond the matrix: 2^0)
         const int64_t grow = int64_t(blockIdx.y) * R + tid;
         blk.sf[IS_A ? perm_row64(tid) : perm_col64(tid)] = (sf && grow < rows) ? sf[grow * ld_sf + blockIdx.x] : uint8_t(127);
@@ -537,6 +544,12 @@ __global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, 
     };
     // the range of normal numbers of the accumulator's format, as exponent fields of doubles
     constexpr int EXP_LOW = ACC16 ? -14 : -126, EXP_TOP = ACC16 ? 16 : 128;
+    // Where results cannot leave the range of normal FP32 numbers they are not tested for it (an eighth of the integer work of a block of
+    // eight): accumulators that are zero or within 2^-100 .. 2^100, and a chunk whose nonzero elements are within 2^-48 .. 2^40.  A
+    // nonzero sum is then a multiple of 2^-123 (of 2^(-96 - F), or an accumulator unchanged), and K products of at most 2^83 each
+    // stay below 2^116.  FP16 elements always are within.
+    constexpr bool TAMEABLE = BASE == 0 && !ACC16 && !ST;
+    bool c_tame = false;
     double cs[DS ? TM : 1][DS ? TN : 1];
     uint32_t sub_mask = 0u;                             // outputs whose accumulator is a nonzero FP32 subnormal: Exp(c) = -126
     uint32_t cw[TM][TN];                                // the words of C as read (finite ones; the rest become flags)
@@ -607,6 +620,22 @@ __global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, 
             sp_nan |= scale_nan;                        // a NaN scale factor makes the block result NaN
         }
 
+        bool tame = TAMEABLE && !(E::EBITS == 8 && (sa_blk.wild | sb_blk.wild) != 0u);
+        if (tame && !c_tame) {
+            bool ok = true;
+#pragma unroll
+            for (int r = 0; r < TM; ++r)
+#pragma unroll
+                for (int c = 0; c < TN; ++c) {
+                    const uint32_t h = uint32_t(__double2hiint(cs[DS ? r : 0][DS ? c : 0])) & 0x7FFFFFFFu;
+                    ok = ok && (h == 0u || h - (uint32_t(1023 - 100) << 20) < (200u << 20));
+                }
+            c_tame = __all_sync(0xFFFFFFFFu, ok);       // (matrix instructions need the whole warp)
+        }
+        tame = tame && c_tame;
+        c_tame = tame;
+        auto run_blocks = [&](auto in_range) {
+        constexpr bool TAME = decltype(in_range)::value;
 #pragma unroll UNROLL_BLK
         for (int blk = 0; blk < NBLK; ++blk) {
             const int kb = blk * L;
@@ -733,7 +762,7 @@ __global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, 
                 }
             };
             auto restart_subnormals = [&](int r0) {     // rare: redo the outputs whose accumulator is an FP32 subnormal
-                if (DS && sub_mask) {
+                if (DS && !TAME && sub_mask) {
 #pragma unroll
                     for (int r = r0; r < r0 + 2; ++r)
 #pragma unroll
@@ -766,9 +795,12 @@ __global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, 
             constexpr uint32_t LOWHI = uint32_t(1023 + EXP_LOW) << 20, SPANHI = uint32_t(EXP_TOP - EXP_LOW) << 20;
             uint32_t urange = 0u;
             auto block_value = [&](int r, int c) -> double {
-                const uint32_t sa = sa_blk.sgn[prow + r], nza = sa_blk.nz[prow + r] & kmask;
-                const uint32_t live = nza & sb_blk.nz[pcol + c];
-                if (BASE) no_product = no_product || live == 0u;
+                const uint32_t sa = sa_blk.sgn[prow + r];
+                uint32_t live = kmask;                  // (BASE = 0: zeros are staged as tiny numbers of their sign)
+                if (BASE) {
+                    live &= sa_blk.nz[prow + r] & sb_blk.nz[pcol + c];
+                    no_product = no_product || live == 0u;
+                }
                 const int nneg = __popc((sa ^ sb_blk.sgn[pcol + c]) & live);
                 double v;
                 if (NARROW) {
@@ -798,7 +830,7 @@ __global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, 
                     if (BASE) nv[BASE ? r : 0][BASE ? c : 0] = st; else cs[DS ? r : 0][DS ? c : 0] = st;
                 } else if (DS) {
                     // (twice the high word: the sign leaves at the top, and a multiply-add is not on the integer pipe)
-                    urange = max(uint32_t(imad(__double2hiint(v), c_mul64[6], int(0u - 2u * LOWHI))), urange);
+                    if (!TAME) urange = max(uint32_t(imad(__double2hiint(v), c_mul64[6], int(0u - 2u * LOWHI))), urange);
                     // RZ-FP32 of a number in the normal range: the low 29 bits of the double's significand go
                     const double st = __hiloint2double(__double2hiint(v), (__double2loint(v) & int(0xE0000000u)) | 1);
                     if (BASE) nv[BASE ? r : 0][BASE ? c : 0] = st; else cs[DS ? r : 0][DS ? c : 0] = st;
@@ -846,7 +878,7 @@ __global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, 
 #pragma unroll
             for (int o = 8; o < 16; ++o) finish(o / TN, o % TN);
 
-            if (DS) {
+            if (DS && !TAME) {
                 bool odd = urange >= 2u * SPANHI;       // some result is not a normal FP32 number
                 if (BASE && no_product) {               // rare: no nonzero product: the block returns its accumulator
                     odd = true;
@@ -881,6 +913,9 @@ __global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, 
                 }
             }
         }
+        };
+        if (TAMEABLE && tame) run_blocks(std::integral_constant<bool, TAMEABLE>{});
+        else run_blocks(std::false_type{});
         __syncthreads();                                // everybody has finished with this buffer
         if (*reinterpret_cast<volatile int*>(&sm.error)) break;
         if (tid == 0 && chunk + 2 < NCH) issue(chunk + 2);
@@ -942,8 +977,8 @@ cudaError_t launch_one64b(const DevModel& m, const GemmArgs& g, cudaStream_t str
     cudaError_t err = cudaFuncSetAttribute(tfdpa64_kernel<EK, L, RHO, PROMOTE, ST, BASE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sh));
     if (err != cudaSuccess) return err;
     const size_t dsh_a = 256 * sizeof(LutEntry64) + sizeof(Blk64<BM>), dsh_b = 256 * sizeof(LutEntry64) + sizeof(Blk64<BN>);
-    if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BM, true, BASE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_a))) != cudaSuccess) return err;
-    if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BN, false, BASE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_b))) != cudaSuccess) return err;
+    if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BM, true, BASE, false, BASE == 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_a))) != cudaSuccess) return err;
+    if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BN, false, BASE, false, BASE == 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_b))) != cudaSuccess) return err;
     const int64_t tiles_m = (g.M + BM - 1) / BM, tiles_n = (g.N + BN - 1) / BN, nch = g.K / KC;
     // scratch: the decoded blocks of A and B, stream-ordered out of the library's pool and returned to it behind the kernel
     const size_t bytes_a = size_t(tiles_m * nch) * sizeof(Blk64<BM>), bytes_b = size_t(tiles_n * nch) * sizeof(Blk64<BN>);
@@ -953,9 +988,9 @@ cudaError_t launch_one64b(const DevModel& m, const GemmArgs& g, cudaStream_t str
     if ((err = cudaMallocFromPoolAsync(&ws, bytes_a + bytes_b, pool, stream)) != cudaSuccess) return err;
     Blk64<BM>* wa = static_cast<Blk64<BM>*>(ws);
     Blk64<BN>* wb = reinterpret_cast<Blk64<BN>*>(static_cast<unsigned char*>(ws) + bytes_a);
-    decode64_kernel<EK, BM, true, BASE><<<dim3((unsigned)nch, (unsigned)tiles_m), 256, dsh_a, stream>>>(
+    decode64_kernel<EK, BM, true, BASE, false, BASE == 0><<<dim3((unsigned)nch, (unsigned)tiles_m), 256, dsh_a, stream>>>(
         m, static_cast<const unsigned char*>(g.A), g.M, g.lda, wa, ST ? g.sfa : nullptr, g.ld_sfa);
-    decode64_kernel<EK, BN, false, BASE><<<dim3((unsigned)nch, (unsigned)tiles_n), 256, dsh_b, stream>>>(
+    decode64_kernel<EK, BN, false, BASE, false, BASE == 0><<<dim3((unsigned)nch, (unsigned)tiles_n), 256, dsh_b, stream>>>(
         m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, wb, ST ? g.sfb : nullptr, g.ld_sfb);
     dim3 grid((unsigned)tiles_n, (unsigned)tiles_m, 1);
     tfdpa64_kernel<EK, L, RHO, PROMOTE, ST, BASE><<<grid, NT, sh, stream>>>(m, g, wa, wb);
