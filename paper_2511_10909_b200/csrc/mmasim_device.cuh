@@ -8,13 +8,13 @@
 
 namespace mmasim {
 
-// Whether the CTA's tile is the emulation's to compute (GemmArgs::least_a): called by whole warps, the same answer in all.
+// Whether a tile is the emulation's to compute (GemmArgs::redo).
 __device__ __forceinline__ bool tile_wanted(const GemmArgs& g, int64_t row0, int rows, int64_t col0, int cols) {
-    if (!g.least_a) return true;
-    int a = 1 << 20, b = 1 << 20;
-    for (int64_t i = row0 + threadIdx.x % 32; i < min(row0 + rows, g.M); i += 32) a = min(a, g.least_a[i]);
-    for (int64_t j = col0 + threadIdx.x % 32; j < min(col0 + cols, g.N); j += 32) b = min(b, g.least_b[j]);
-    return __reduce_min_sync(0xFFFFFFFFu, a) + __reduce_min_sync(0xFFFFFFFFu, b) < -126;
+    if (!g.redo) return true;
+    for (int64_t j = col0 / 128; j <= (min(col0 + cols, g.N) - 1) / 128; ++j)
+        for (int64_t i = row0 / g.redo_rows; i <= (min(row0 + rows, g.M) - 1) / g.redo_rows; ++i)
+            if (g.redo[j * g.redo_across + i]) return true;
+    return false;
 }
 
 // ---------------------------------------------------------------------------------------------------------

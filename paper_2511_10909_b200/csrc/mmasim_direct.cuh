@@ -747,24 +747,15 @@ __global__ void __launch_bounds__(32 * (WR * WC + PW), min_ctas(TM * CN, L, WR *
     direct_tile<FAM, EK, L, RHO, PROMOTE, TM, CN, WR, WC, PW, TASK>(m, g, unit_a, unit_b, int64_t(blockIdx.y) * (8 * TM * WR), int64_t(blockIdx.x) * (8 * CN * WC));
 }
 
-// The tiles that the matrix instruction has to leave to the emulation (GemmArgs::least_a), on a fixed grid: almost always there are
-// none, and every CTA reads the smallest exponents and leaves (1024 x 4096: 3 us; a CTA per tile that looks at its own rows: 18 us).
+// The tiles that the matrix instruction has to leave to the emulation (GemmArgs::redo), on a fixed grid: almost always there are
+// none, and every CTA reads the flags and leaves (1024 x 4096: a CTA per tile that looked for itself took 18 us).
 template <int FAM, int EK, int L, int RHO, int TM, int CN, int WR, int WC, int PW, int TASK>
 __global__ void __launch_bounds__(32 * (WR * WC + PW), min_ctas(TM * CN, L, WR * WC + PW)) direct_rest_kernel(DevModel m, GemmArgs g, int unit_a, int unit_b) {
     constexpr int BM = 8 * TM * WR, BN = 8 * CN * WC;
-    __shared__ int least[2];
-    if (threadIdx.x < 2) least[threadIdx.x] = 1 << 20;
-    __syncthreads();
-    int a = 1 << 20, b = 1 << 20;
-#pragma unroll 8
-    for (int64_t i = threadIdx.x; i < g.M; i += blockDim.x) a = min(a, g.least_a[i]);
-#pragma unroll 8
-    for (int64_t j = threadIdx.x; j < g.N; j += blockDim.x) b = min(b, g.least_b[j]);
-    a = __reduce_min_sync(0xFFFFFFFFu, a);
-    b = __reduce_min_sync(0xFFFFFFFFu, b);
-    if (threadIdx.x % 32 == 0) { atomicMin(&least[0], a); atomicMin(&least[1], b); }
-    __syncthreads();
-    if (least[0] + least[1] >= -126) return;
+    const int64_t flags = (g.N + 127) / 128 * g.redo_across;
+    int any = 0;
+    for (int64_t i = threadIdx.x; i < flags; i += blockDim.x) any |= g.redo[i];
+    if (!__syncthreads_or(any)) return;
     const int64_t tn = (g.N + BN - 1) / BN, tiles = (g.M + BM - 1) / BM * tn;
     for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
         const int64_t row0 = t / tn * BM, col0 = t % tn * BN;

@@ -2,7 +2,7 @@
 #include "mmasim_direct.cuh"
 namespace mmasim { namespace direct {
 cudaError_t launch_lut8(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStream_t st) {
-    if (g.least_a) return launch_rest<FAM_ST, fast::EK_LUT8, 32, RHO_RZ_FP32>(m, g, st);
+    if (g.redo) return launch_rest<FAM_ST, fast::EK_LUT8, 32, RHO_RZ_FP32>(m, g, st);
     if (m.family == FAM_ST) return launch<FAM_ST, fast::EK_LUT8, 32, RHO_RZ_FP32>(m, g, size, st);
     if (m.L == 16) {
         if (m.rho == RHO_RZ_E8M13) return launch<FAM_T, fast::EK_LUT8, 16, RHO_RZ_E8M13>(m, g, size, st);

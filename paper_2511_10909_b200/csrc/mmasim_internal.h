@@ -68,10 +68,10 @@ struct GemmArgs {
     const float* row_scale;
     const float* col_scale;
     int dot_mode;                 // 1: n independent dots (row t of A with row t of B), N is ignored
-    // smallest exponent of every row of A and B, or NULL: the emulating kernels then leave a tile alone unless one of its rows of A
-    // and one of its rows of B have a smaller sum than -126 (the matrix instruction has done the tile; see mmasim_umma.cu)
-    const int* least_a;
-    const int* least_b;
+    // one byte per redo_rows rows of A x 128 rows of B, redo_across of them per 128 rows of B, or NULL: the emulating kernels then leave
+    // a tile alone unless it touches a set one (the matrix instruction has done the rest; see mmasim_umma.cu)
+    const unsigned char* redo;
+    int redo_rows, redo_across;
     unsigned int* copy_timeouts;  // device counter of CTAs whose bounded wait on a bulk copy ran out (may be NULL)
 };
 

@@ -60,12 +60,12 @@ __global__ void __launch_bounds__(256) stats_kernel(int64_t n, const void* D, co
     }
 }
 
-// Up to three operands widened exactly to FP64, four elements per thread.
+// An operand widened exactly to FP64, two elements per thread and step: 16-byte stores, consecutive threads side by side.
 struct Widen {
-    const void* src[3];
-    double* dst[3];
-    int64_t n[3];
-    int fmt[3];
+    const void* src;
+    double* dst;
+    int64_t n;
+    int fmt;
 };
 __device__ __forceinline__ double widen_one(int fmt, const void* p, int64_t i) {
     switch (fmt) {
@@ -82,12 +82,14 @@ __device__ __forceinline__ double widen_one(int fmt, const void* p, int64_t i) {
         }
     }
 }
-__global__ void __launch_bounds__(256) widen_kernel(Widen w) {
-    const int o = blockIdx.y;
-    const int64_t first = (int64_t(blockIdx.x) * 256 + threadIdx.x) * 4;
+__global__ void __launch_bounds__(256) widen_kernel(Widen a, Widen b, Widen c) {
+    const Widen w = blockIdx.y == 0 ? a : (blockIdx.y == 1 ? b : c);
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-        if (first + q < w.n[o]) w.dst[o][first + q] = widen_one(w.fmt[o], w.src[o], first + q);
+    for (int q = 0; q < 4; ++q) {
+        const int64_t i = ((int64_t(blockIdx.x) * 4 + q) * 256 + threadIdx.x) * 2;
+        if (i + 1 < w.n) *reinterpret_cast<double2*>(w.dst + i) = make_double2(widen_one(w.fmt, w.src, i), widen_one(w.fmt, w.src, i + 1));
+        else if (i < w.n) w.dst[i] = widen_one(w.fmt, w.src, i);
+    }
 }
 
 }  // namespace
@@ -112,9 +114,9 @@ int launch_reference_fp64(int fmt, int acc, int64_t M, int64_t N, int64_t K, con
     if (err == cudaSuccess) err = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&scratch), size_t(c_at + nc) * 8, pool, stream);
     int st = MMASIM_OK;
     if (err == cudaSuccess) {
-        const Widen w = {{A, B, C}, {scratch + a_at, scratch + b_at, scratch + c_at}, {na, nb, nc}, {fmt, fmt, acc == ACC_F16 ? EF_F16 : EF_F32}};
+        const Widen wa = {A, scratch + a_at, na, fmt}, wb = {B, scratch + b_at, nb, fmt}, wc = {C, scratch + c_at, nc, acc == ACC_F16 ? EF_F16 : EF_F32};
         const int64_t most = na > nb ? (na > nc ? na : nc) : (nb > nc ? nb : nc);
-        widen_kernel<<<dim3(unsigned((most + 1023) / 1024), C ? 3 : 2), 256, 0, stream>>>(w);
+        widen_kernel<<<dim3(unsigned((most + 2047) / 2048), C ? 3 : 2), 256, 0, stream>>>(wa, wb, wc);
         err = cudaGetLastError();
     }
     if (err == cudaSuccess) {
