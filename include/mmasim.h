@@ -243,6 +243,11 @@ int mmasim_error_stats(int acc_fmt, int64_t n, const void* D, const double* ref,
 int mmasim_reference_fp64(const mmasim_model* model, int64_t M, int64_t N, int64_t K, const void* A, const void* B, const void* C,
                           double* ref, void* stream);
 
+/* The whole of it: the model's product, that reference and the statistics of their deviations (from zero) in `stats`, eight doubles in
+ * HOST memory.  Works in library memory on `stream` and waits for it. */
+int mmasim_deviation_stats(const mmasim_model* model, int64_t M, int64_t N, int64_t K, const void* A, const void* B, const void* C,
+                           double* stats, void* stream);
+
 /* Issue-rate micro-benchmarks, the roofline denominators (no counterpart in the paper).  Launches `blocks` CTAs of
  * 256 threads; every thread runs `iters` (rounded up to a multiple of 8) times 8 rounds of independent operations of
  * the given kind.  `sink` (device, >= 4 bytes) receives a value that keeps the work alive.  The caller times the

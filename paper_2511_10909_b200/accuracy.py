@@ -40,15 +40,14 @@ def reference_fp64(in_fmt: str, acc: str, A, B, C=None):
 def deviation_stats(model: mmasim.Model, A, B, C=None, ref=None) -> dict:
     """Run the model and reduce delta = D - D_real: count, mean, mean |delta|, rms, share of negative / positive
     deviations, max |delta|, mean relative error."""
-    if ref is None:
-        packed = all(t is None or (t.is_cuda and t.dim() == 2 and t.is_contiguous()) for t in (A, B, C))
-        if packed and model.b_fmt == model.in_fmt and model.in_fmt in ("fp16", "bf16", "bf16_1k", "tf32", "fp32", "e4m3", "e5m2") \
-                and model.acc != "fp64" and A.shape[1] == B.shape[1]:
-            ref = mmasim.reference_fp64(model, A, B, C)       # the operands widened in one launch
-        else:
+    packed = all(t is None or (t.is_cuda and t.dim() == 2 and t.is_contiguous()) for t in (A, B, C))
+    if ref is None and packed and model.b_fmt == model.in_fmt and model.in_fmt in ("fp16", "bf16", "bf16_1k", "tf32", "fp32", "e4m3", "e5m2") \
+            and model.acc != "fp64" and A.shape[1] == B.shape[1]:
+        s = mmasim.deviation_stats(model, A, B, C)           # one call of the library
+    else:
+        if ref is None:
             ref = reference_fp64(model.in_fmt, model.acc, A, B, C)
-    D = mmasim.gemm(model, A, B, C)
-    s = mmasim.error_stats(model.acc, D, ref).cpu().tolist()
+        s = mmasim.error_stats(model.acc, mmasim.gemm(model, A, B, C), ref).cpu().tolist()
     n = max(s[0], 1.0)
     return {"count": int(s[0]), "mean": s[1] / n, "mean_abs": s[2] / n, "rms": (s[3] / n) ** 0.5, "negative": s[4] / n,
             "positive": s[5] / n, "max_abs": s[6], "mean_rel": s[7] / n}

@@ -158,7 +158,7 @@ cudaError_t scratch_pool(cudaMemPool_t* out) {
 }
 
 namespace {
-// The streams and events of one mmasim_gemm_host call, and a word of mapped host memory that its kernels count given-up waits in (a copy
+// The streams and events of one mmasim_gemm_host call (mmasim_deviation_stats uses only the memory), and a word of mapped host memory that its kernels count given-up waits in (a copy
 // of the device's counter before and after each call cost 15 us).  Creating them took about 100 us of every call, so up to
 // LANES_KEPT sets per device wait for the next one; a call has its set to itself, and mmasim_host_release destroys those that wait.
 struct HostLane {
@@ -168,6 +168,7 @@ struct HostLane {
     cudaEvent_t ev_in[PANELS] = {}, ev_k[PANELS] = {};
     unsigned int* gave_up = nullptr;        // host address
     unsigned int* gave_up_dev = nullptr;    // device address
+    double* stats = nullptr;                // eight doubles behind it (mmasim_deviation_stats)
 };
 constexpr int LANES_KEPT = 4;
 std::atomic<unsigned int> g_host_timeouts[MAX_DEVICES];     // what the words of finished calls held
@@ -196,8 +197,9 @@ cudaError_t take_lane(HostLane* out) {
     }
     HostLane l;
     l.device = dev;
-    err = cudaHostAlloc(reinterpret_cast<void**>(&l.gave_up), sizeof(unsigned int), cudaHostAllocMapped);
+    err = cudaHostAlloc(reinterpret_cast<void**>(&l.gave_up), 128, cudaHostAllocMapped);
     if (err == cudaSuccess) err = cudaHostGetDevicePointer(reinterpret_cast<void**>(&l.gave_up_dev), l.gave_up, 0);
+    if (err == cudaSuccess) l.stats = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(l.gave_up) + 64);
     if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&l.in, cudaStreamNonBlocking);
     if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&l.out, cudaStreamNonBlocking);
     for (int p = 0; p < HostLane::PANELS && err == cudaSuccess; ++p) {
@@ -507,14 +509,67 @@ int mmasim_error_stats(int acc_fmt, int64_t n, const void* D, const double* ref,
                               static_cast<cudaStream_t>(stream));
 }
 
+namespace {
+bool has_reference(const DevModel& m) {
+    const int f = m.fmt_a;
+    return f == m.fmt_b && (f == EF_F16 || f == EF_BF16 || f == EF_TF32 || f == EF_F32 || f == EF_E4M3 || f == EF_E5M2) && !m.k_block && m.acc != ACC_F64;
+}
+}  // namespace
+
+// One call for the pipeline that was five (reference, product, zeroed statistics, statistics, copy): one allocation of kept memory, the
+// eight doubles into pinned memory, and the next launch is queued long before the last kernel ends.  CDNA3 FP16, 1024 x 1024 x 256:
+// 169 us as five calls from Python, 149 us as one; about 125 us of it are the kernels.
+int mmasim_deviation_stats(const mmasim_model* model, int64_t M, int64_t N, int64_t K, const void* A, const void* B, const void* C,
+                           double* stats, void* stream) {
+    GemmArgs g;
+    int st = build_args(model, M, N, K, A, B, C, stats, nullptr, &g);
+    if (st != MMASIM_OK) return st;
+    const DevModel& m = model->dev;
+    if (!has_reference(m)) {
+        set_error("mmasim_deviation_stats: unscaled models of FP32, TF32, BF16, FP16 and FP8 inputs of one type");
+        return MMASIM_ERR_UNSUPPORTED;
+    }
+    if (!aligned16(A) || !aligned16(B) || (C && !aligned16(C))) { set_error("A, B and C must be 16-byte aligned"); return MMASIM_ERR_ALIGN; }
+    if ((st = check_device_ptr(A, "A")) != MMASIM_OK) return st;
+    if ((st = check_device_ptr(B, "B")) != MMASIM_OK) return st;
+    if (C && (st = check_device_ptr(C, "C")) != MMASIM_OK) return st;
+    const cudaStream_t s = static_cast<cudaStream_t>(stream);
+    HostLane lane;
+    cudaError_t err = take_lane(&lane);
+    cudaMemPool_t pool = nullptr;
+    if (err == cudaSuccess) err = scratch_pool(&pool);
+    const size_t words = size_t(M) * size_t(N), d_at = 64, ref_at = d_at + (words * model->info.acc_bytes + 255) / 256 * 256;
+    unsigned char* base = nullptr;
+    if (err == cudaSuccess) err = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&base), ref_at + words * 8, pool, s);
+    double *dev_stats = reinterpret_cast<double*>(base), *ref = reinterpret_cast<double*>(base + ref_at);
+    if (err == cudaSuccess) err = cudaMemsetAsync(dev_stats, 0, 64, s);
+    if (err == cudaSuccess) {
+        st = launch_reference_fp64(m.fmt_a, m.acc, M, N, K, A, B, C, ref, s);
+        g.D = base + d_at;
+        if (st == MMASIM_OK) st = run_gemm(model, g, 0, s);
+        if (st == MMASIM_OK) st = launch_error_stats(m.acc, int64_t(words), g.D, ref, dev_stats, s);
+        if (st == MMASIM_OK) err = cudaMemcpyAsync(lane.stats, dev_stats, 64, cudaMemcpyDeviceToHost, s);
+    }
+    if (base) cudaFreeAsync(base, s);
+    const cudaError_t e = cudaStreamSynchronize(s);
+    if (err == cudaSuccess) err = e;
+    if (err == cudaSuccess && st == MMASIM_OK) std::memcpy(stats, lane.stats, 64);
+    give_lane(lane, err == cudaSuccess);
+    if (err != cudaSuccess) {
+        cudaGetLastError();
+        set_error("mmasim_deviation_stats: %s", cudaGetErrorString(err));
+        return MMASIM_ERR_CUDA;
+    }
+    return st;
+}
+
 int mmasim_reference_fp64(const mmasim_model* model, int64_t M, int64_t N, int64_t K, const void* A, const void* B, const void* C,
                           double* ref, void* stream) {
     GemmArgs g;
     int st = build_args(model, M, N, K, A, B, C, ref, nullptr, &g);
     if (st != MMASIM_OK) return st;
     const DevModel& m = model->dev;
-    const int f = m.fmt_a;
-    if (f != m.fmt_b || (f != EF_F16 && f != EF_BF16 && f != EF_TF32 && f != EF_F32 && f != EF_E4M3 && f != EF_E5M2) || m.k_block || m.acc == ACC_F64) {
+    if (!has_reference(m)) {
         set_error("mmasim_reference_fp64: unscaled models of FP32, TF32, BF16, FP16 and FP8 inputs of one type");
         return MMASIM_ERR_UNSUPPORTED;
     }
@@ -522,7 +577,7 @@ int mmasim_reference_fp64(const mmasim_model* model, int64_t M, int64_t N, int64
     if ((st = check_device_ptr(B, "B")) != MMASIM_OK) return st;
     if ((st = check_device_ptr(ref, "ref")) != MMASIM_OK) return st;
     if (C && (st = check_device_ptr(C, "C")) != MMASIM_OK) return st;
-    return launch_reference_fp64(f, m.acc, M, N, K, A, B, C, ref, static_cast<cudaStream_t>(stream));
+    return launch_reference_fp64(m.fmt_a, m.acc, M, N, K, A, B, C, ref, static_cast<cudaStream_t>(stream));
 }
 
 int mmasim_host_release(void) {

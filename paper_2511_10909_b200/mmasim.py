@@ -81,6 +81,8 @@ def _load():
     lib.mmasim_error_stats.argtypes = [c_int, c_int64, c_void_p, c_void_p, c_void_p, c_void_p]
     lib.mmasim_reference_fp64.restype = c_int
     lib.mmasim_reference_fp64.argtypes = [c_void_p, c_int64, c_int64, c_int64, c_void_p, c_void_p, c_void_p, c_void_p, c_void_p]
+    lib.mmasim_deviation_stats.restype = c_int
+    lib.mmasim_deviation_stats.argtypes = [c_void_p, c_int64, c_int64, c_int64, c_void_p, c_void_p, c_void_p, c_void_p, c_void_p]
     lib.mmasim_host_release.restype = c_int
     lib.mmasim_host_release.argtypes = []
     lib.mmasim_last_kernel.restype = c_char_p
@@ -365,13 +367,27 @@ def host_release():
     _check(_lib.mmasim_host_release())
 
 
-def reference_fp64(model: Model, A, B, C=None, *, stream=None):
-    """A x B^T + C in FP64 for packed operands of ``model``'s types (mmasim_reference_fp64): an M x N FP64 CUDA tensor."""
-    import torch
+def _packed(model, A, B, C):
     dev, M, N, K = A.device, A.shape[0], B.shape[0], A.shape[1]
     for t, name, rows, cols, bits in ((A, "A", M, K, model.a_bits), (B, "B", N, K, model.b_bits), (C, "C", M, N, 8 * model.acc_bytes)):
         if t is not None and _matrix(t, name, rows, cols, bits, dev) != cols:
             raise MmasimError(3, f"{name} must be a packed {rows} x {cols} matrix")
+    return dev, M, N, K
+
+
+def deviation_stats(model: Model, A, B, C=None, *, stream=None):
+    """The eight statistics (STAT_NAMES) of the deviations of ``model``'s product of packed operands from the FP64 result
+    (mmasim_deviation_stats): a list of floats, once the GPU is done."""
+    _, M, N, K = _packed(model, A, B, C)
+    stats = (ctypes.c_double * 8)()
+    _check(_lib.mmasim_deviation_stats(model._h, M, N, K, _ptr(A), _ptr(B), _ptr(C), ctypes.addressof(stats), _stream(stream)))
+    return list(stats)
+
+
+def reference_fp64(model: Model, A, B, C=None, *, stream=None):
+    """A x B^T + C in FP64 for packed operands of ``model``'s types (mmasim_reference_fp64): an M x N FP64 CUDA tensor."""
+    import torch
+    dev, M, N, K = _packed(model, A, B, C)
     ref = torch.empty((M, N), dtype=torch.float64, device=dev)
     _check(_lib.mmasim_reference_fp64(model._h, M, N, K, _ptr(A), _ptr(B), _ptr(C), _ptr(ref), _stream(stream)))
     return ref

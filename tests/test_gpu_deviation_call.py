@@ -1,0 +1,25 @@
+"""mmasim_deviation_stats against the same pipeline in three calls: FP32 and FP16 accumulators, ragged sizes, with and without C."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2511_10909_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+gu = pytest.importorskip("gpu_util") if torch.cuda.is_available() else None
+
+
+@pytest.mark.parametrize("key", [("cdna3", "fp16", "fp32"), ("hopper", "fp16", "fp16"), ("hopper", "e4m3", "fp32"), ("cdna2", "bf16", "fp32")],
+                         ids=lambda k: "-".join(k))
+def test_one_call_against_three(key):
+    from paper_2511_10909_b200 import accuracy, mmasim
+    model = mmasim.Model(*key)
+    for M, N, K in ((1, 1, 32), (130, 301, 96)):
+        A, B, C = (gu.dev(wl.normal_inputs(key[1], key[2], M, N, K, seed=8)[k]) for k in ("A", "B", "C"))
+        for c in (C, None):
+            got = mmasim.deviation_stats(model, A, B, c)
+            ref = accuracy.reference_fp64(key[1], key[2], A, B, c)
+            want = mmasim.error_stats(key[2], mmasim.gemm(model, A, B, c), ref).cpu().numpy()
+            # FP64 sums of M N terms in another order: at most M N ulps of the sum of magnitudes
+            scale = np.maximum(np.abs(want), [1, want[2], 0, 0, 1, 1, 0, 0])
+            assert np.all(np.abs(np.array(got) - want) <= M * N * 2.0 ** -52 * scale), (key, (M, N, K), got, want)
