@@ -104,11 +104,16 @@ PIPES = {
     "fp64_fma": ("FP64 fused multiply-add issue", FP64_KINDS, 64.0),
     "int_dp4a": ("4-way byte dot-product issue", ("dp4a",), 64.0),
     "int_alu": ("3-input integer add issue", ("iadd3",), 64.0),
+    "tcgen05": ("tcgen05.mma", (), 4096.0),
 }
+# dense rates of tcgen05.mma by storage of an element, as multiples of the 16-bit kinds'
+TCGEN05_RATE = {"tf32": 0.5, "fp16": 1.0, "bf16": 1.0, "mxf4": 4.0, "nvf4": 4.0}
 
 
 def pipe_of(kernel: str, model):
     """(pipe key, pipe instructions per emulated MAC) of the kernel a model dispatches to."""
+    if model.family in ("ST", "GST") or (model.family == "T" and model.F == 25):
+        return "tcgen05", 1.0               # the model is the GPU's own matrix instruction
     if kernel == "tfdpa_lut8" and model.F <= 13:
         return "fp32_fma", 1.0
     if kernel in ("tfdpa_lut8", "tfdpa_f16", "tfdpa_bf16", "tfdpa_tf32", "trfdpa", "gtrfdpa", "efdpa", "fma_f64"):
@@ -403,7 +408,7 @@ def run_ours(args):
     # occupancies per pipe, the best counts): the pipe the timed kernel is bound by, and the 3-input integer add that is
     # the unit of the paper-level operation count
     pipe_key, pipe_ops_per_mac = pipe_of(kernel_name, model)
-    peaks = measure_pipe_peaks(mmasim, torch, dev, sorted({pipe_key, "int_alu"})) if not is_dot else {}
+    peaks = measure_pipe_peaks(mmasim, torch, dev, sorted({pipe_key, "int_alu"} - {"tcgen05"})) if not is_dot else {}
 
     # ---- timed region: K steps, device timers, L2 flushed between steps ----
     sampler = ClockSampler(local_rank)
@@ -460,15 +465,21 @@ def run_ours(args):
 
     per_gpu_macs_s = value / world
     sm_mhz = clocks.get("sm_mhz") or 1965.0
-    hbm_peak, hbm_src = 6650.0, "fallback 6.65 TB/s (MEASURED_PEAKS.json absent)"
+    hbm_peak, hbm_src, bf16_peak = 6650.0, "fallback 6.65 TB/s (MEASURED_PEAKS.json absent)", 1590.0
     try:
-        hbm_peak = float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["hbm_gbs"])
+        measured_peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
+        hbm_peak, bf16_peak = float(measured_peaks["hbm_gbs"]), float(measured_peaks["bf16_tflops"])
         hbm_src = "MEASURED_PEAKS.json hbm_gbs (STREAM-style copy)"
     except (OSError, KeyError, ValueError):
         pass
 
-    def pipe_view(pipe, ops_per_mac, macs_s):
-        """Fractions of one pipe: against the best live witness and against the nominal rate at the sampled clock."""
+    def pipe_view(pipe, ops_per_mac, macs_s, in_fmt=""):
+        """Fractions of one pipe: against the best live witness and against the nominal rate at the sampled clock (the matrix
+        instruction: against the measured library BF16 GEMM times the kind's multiple of its rate)."""
+        if pipe == "tcgen05":
+            rate = TCGEN05_RATE.get(in_fmt, 2.0)
+            peak, nominal = bf16_peak * 1e12 / 2 * rate, SMS * PIPES[pipe][2] * rate * sm_mhz * 1e6
+            return {"pipe": PIPES[pipe][0], "pipe_ops_per_mac": 1.0, "frac": macs_s / peak, "frac_nominal": macs_s / nominal}
         label, _, per_clk = PIPES[pipe]
         nominal = SMS * per_clk * sm_mhz * 1e6
         measured = peaks[pipe]["peak"]
@@ -492,7 +503,7 @@ def run_ours(args):
         int_view["note"] = ("the count of 6 integer operations per term + 25 per block is not a floor for this formulation: the "
                             "kernel replaces multiply / distance / shift / add by one fused multiply-add and the maximum by a "
                             "tensor-core product of powers, so this fraction may exceed 1 and bounds nothing")
-        roofline = {"bound": "alu", **pipe_view(pipe_key, pipe_ops_per_mac, per_gpu_macs_s), "kernel": kernel_name,
+        roofline = {"bound": "alu", **pipe_view(pipe_key, pipe_ops_per_mac, per_gpu_macs_s, key[1]), "kernel": kernel_name,
                     "traffic": NCU_DRAM_BYTES.get(name),
                     "traffic_source": "stored constant from a one-pass ncu capture of this workload at full size, main kernel + both decode launches (not measured in this run)" if name in NCU_DRAM_BYTES else None,
                     "algorithmic_bytes": NCU_ALGORITHMIC_BYTES.get(name),
@@ -535,10 +546,10 @@ def run_ours(args):
                          "macs_per_s": float(size) ** 3 / (tot / 3 * 1e-3), "_pipe": pp, "_opm": opm})
             del out
         cache.clear()
-        peaks.update(measure_pipe_peaks(mmasim, torch, dev, sorted(pm_peaks_needed - set(peaks))))
+        peaks.update(measure_pipe_peaks(mmasim, torch, dev, sorted(pm_peaks_needed - set(peaks) - {"tcgen05"})))
         per_model = []
         for r in rows:
-            v = pipe_view(r.pop("_pipe"), r.pop("_opm"), r["macs_per_s"])
+            v = pipe_view(r.pop("_pipe"), r.pop("_opm"), r["macs_per_s"], r["model"].split("-")[1])
             r.update(pipe=v["pipe"], pipe_ops_per_mac=v["pipe_ops_per_mac"], frac=v["frac"], frac_nominal=v["frac_nominal"])
             per_model.append(r)
         # the HBM-bound probe-style batch (config 4): 2^20 dots of length 32, FP16, both kernel kinds
@@ -590,7 +601,7 @@ def run_ours(args):
         "dtype": compute_dtype(kernel_name, model), "data": "synthetic",
         "config": {"workload": f"{name}: {desc}", "model": "-".join(key), "M": M, "N": N, "K": K,
                    "l2": "flushed between timed steps (256 MiB write)", "parallelism": f"replicas x{world} (independent batches, no exchange)"},
-        "clocks": clocks, "e2e": e2e, "gpu_launches": args.steps * KERNELS_PER_CALL.get(kernel_name, 1),
+        "clocks": clocks, "e2e": e2e, "gpu_launches": args.steps * (1 if pipe_key == "tcgen05" else KERNELS_PER_CALL.get(kernel_name, 1)),
         "roofline": roofline,
         "cpu_baseline": {"value": cpu_value, "unit": UNIT, "kind": "oracle", **cpu_info},
         "per_model": per_model, "per_model_size": args.per_model_size if per_model else None, "dot_batch": dot_line,

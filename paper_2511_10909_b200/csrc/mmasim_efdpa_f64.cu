@@ -37,29 +37,30 @@ __device__ __noinline__ uint32_t efdpa_by_the_book(DevModel m, const void* A, co
 }
 
 template <int EK, int L>
-__global__ void __launch_bounds__(NT, 1) efdpa64_kernel(DevModel m, GemmArgs g, const Blk64<BM>* __restrict__ wa,
-                                                        const Blk64<BN>* __restrict__ wb) {
+__global__ void __launch_bounds__(NT, 2) efdpa64_kernel(DevModel m, GemmArgs g, const Blk64<BM, EXP_NONE>* __restrict__ wa,
+                                                        const Blk64<BN, EXP_NONE>* __restrict__ wb) {
     constexpr int NBLK = KC / L;
     constexpr bool SCALAR = L == 2;                     // (with blocks of 4 the matrix instruction wins: 12.3 against 15.4 ms at 4096^3)
     static_assert(L == 2 || L == 4, "one matrix instruction (four terms) per block");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    SmemMM& sm = *reinterpret_cast<SmemMM*>(smem_raw);
+    SmemMM<EXP_NONE>& sm = *reinterpret_cast<SmemMM<EXP_NONE>*>(smem_raw);
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
-    const int wr = warp >> 2, wc = warp & 3, gq = lane >> 2, tq = lane & 3;      // warp grid 4 x 4, warp tile 32 x 16
+    const int wr = warp >> 2, wc = warp & 3, gq = lane >> 2, tq = lane & 3;      // warp grid 2 x 4, warp tile 32 x 16
     auto row_at = [&](int r) { return wr * 32 + gq + 8 * r; };                   // inside the CTA tile
     auto col_at = [&](int c) { return wc * 16 + 8 * (c >> 1) + 2 * tq + (c & 1); };
-    const int64_t row0 = int64_t(blockIdx.y) * BM, col0 = int64_t(blockIdx.x) * BN;
+    const unsigned tiles_n = unsigned((g.N + BN - 1) / BN), tile_m = blockIdx.x / tiles_n, tile_n = blockIdx.x % tiles_n;
+    const int64_t row0 = int64_t(tile_m) * BM, col0 = int64_t(tile_n) * BN;
 
     const int NCH = int(g.K / KC);
-    const Blk64<BM>* src_a = wa + int64_t(blockIdx.y) * NCH;
-    const Blk64<BN>* src_b = wb + int64_t(blockIdx.x) * NCH;
+    const Blk64<BM, EXP_NONE>* src_a = wa + int64_t(tile_m) * NCH;
+    const Blk64<BN, EXP_NONE>* src_b = wb + int64_t(tile_n) * NCH;
     auto issue = [&](int n) {                              // one thread: both copies of chunk n into buffer n & 1
         unsigned long long* bar = &sm.full[n & 1];
-        fast::mbar_expect_tx(bar, uint32_t(sizeof(Blk64<BM>) + sizeof(Blk64<BN>)));
-        fast::bulk_load(&sm.a[n & 1], src_a + n, uint32_t(sizeof(Blk64<BM>)), bar);
-        fast::bulk_load(&sm.b[n & 1], src_b + n, uint32_t(sizeof(Blk64<BN>)), bar);
+        fast::mbar_expect_tx(bar, uint32_t(sizeof(Blk64<BM, EXP_NONE>) + sizeof(Blk64<BN, EXP_NONE>)));
+        fast::bulk_load(&sm.a[n & 1], src_a + n, uint32_t(sizeof(Blk64<BM, EXP_NONE>)), bar);
+        fast::bulk_load(&sm.b[n & 1], src_b + n, uint32_t(sizeof(Blk64<BN, EXP_NONE>)), bar);
     };
     if (tid == 0) {
         sm.error = 0;
@@ -83,8 +84,8 @@ __global__ void __launch_bounds__(NT, 1) efdpa64_kernel(DevModel m, GemmArgs g, 
     for (int chunk = 0; chunk < NCH; ++chunk) {
         const int64_t k0 = int64_t(chunk) * KC;
         if (!fast::mbar_wait(&sm.full[chunk & 1], uint32_t(chunk >> 1) & 1u)) *reinterpret_cast<volatile int*>(&sm.error) = 1;
-        const Blk64<BM>& sa_blk = sm.a[chunk & 1];
-        const Blk64<BN>& sb_blk = sm.b[chunk & 1];
+        const Blk64<BM, EXP_NONE>& sa_blk = sm.a[chunk & 1];
+        const Blk64<BN, EXP_NONE>& sb_blk = sm.b[chunk & 1];
         const bool chunk_special = (sa_blk.special | sb_blk.special) != 0u;
 
 #pragma unroll 1
@@ -202,27 +203,26 @@ __global__ void __launch_bounds__(NT, 1) efdpa64_kernel(DevModel m, GemmArgs g, 
 
 template <int EK, int L>
 cudaError_t launch_e_one(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
-    const size_t sh = sizeof(SmemMM);
+    const size_t sh = sizeof(SmemMM<EXP_NONE>);
     cudaError_t err = cudaFuncSetAttribute(efdpa64_kernel<EK, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sh));
     if (err != cudaSuccess) return err;
-    const size_t dsh_a = 256 * sizeof(LutEntry64) + sizeof(Blk64<BM>), dsh_b = 256 * sizeof(LutEntry64) + sizeof(Blk64<BN>);
-    if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BM, true, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_a))) != cudaSuccess) return err;
-    if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BN, false, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_b))) != cudaSuccess) return err;
+    const size_t dsh_a = 256 * sizeof(LutEntry64) + sizeof(Blk64<BM, EXP_NONE>), dsh_b = 256 * sizeof(LutEntry64) + sizeof(Blk64<BN, EXP_NONE>);
+    if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BM, true, 0, false, false, EXP_NONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_a))) != cudaSuccess) return err;
+    if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BN, false, 0, false, false, EXP_NONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_b))) != cudaSuccess) return err;
     const int64_t tiles_m = (g.M + BM - 1) / BM, tiles_n = (g.N + BN - 1) / BN, nch = g.K / KC;
     // scratch: the decoded blocks of A and B, stream-ordered out of the library's pool and returned to it behind the kernel
-    const size_t bytes_a = size_t(tiles_m * nch) * sizeof(Blk64<BM>), bytes_b = size_t(tiles_n * nch) * sizeof(Blk64<BN>);
+    const size_t bytes_a = size_t(tiles_m * nch) * sizeof(Blk64<BM, EXP_NONE>), bytes_b = size_t(tiles_n * nch) * sizeof(Blk64<BN, EXP_NONE>);
     cudaMemPool_t pool = nullptr;
     if ((err = scratch_pool(&pool)) != cudaSuccess) return err;
     void* ws = nullptr;
     if ((err = cudaMallocFromPoolAsync(&ws, bytes_a + bytes_b, pool, stream)) != cudaSuccess) return err;
-    Blk64<BM>* wa = static_cast<Blk64<BM>*>(ws);
-    Blk64<BN>* wb = reinterpret_cast<Blk64<BN>*>(static_cast<unsigned char*>(ws) + bytes_a);
-    decode64_kernel<EK, BM, true, 0><<<dim3((unsigned)nch, (unsigned)tiles_m), 256, dsh_a, stream>>>(
-        m, static_cast<const unsigned char*>(g.A), g.M, g.lda, wa);
-    decode64_kernel<EK, BN, false, 0><<<dim3((unsigned)nch, (unsigned)tiles_n), 256, dsh_b, stream>>>(
-        m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, wb);
-    dim3 grid((unsigned)tiles_n, (unsigned)tiles_m, 1);
-    efdpa64_kernel<EK, L><<<grid, NT, sh, stream>>>(m, g, wa, wb);
+    Blk64<BM, EXP_NONE>* wa = static_cast<Blk64<BM, EXP_NONE>*>(ws);
+    Blk64<BN, EXP_NONE>* wb = reinterpret_cast<Blk64<BN, EXP_NONE>*>(static_cast<unsigned char*>(ws) + bytes_a);
+    decode64_kernel<EK, BM, true, 0, false, false, EXP_NONE><<<unsigned(nch * tiles_m), 256, dsh_a, stream>>>(
+        m, static_cast<const unsigned char*>(g.A), g.M, g.lda, unsigned(nch), wa);
+    decode64_kernel<EK, BN, false, 0, false, false, EXP_NONE><<<unsigned(nch * tiles_n), 256, dsh_b, stream>>>(
+        m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, unsigned(nch), wb);
+    efdpa64_kernel<EK, L><<<unsigned(tiles_n * tiles_m), NT, sh, stream>>>(m, g, wa, wb);
     err = cudaGetLastError();
     const cudaError_t err2 = cudaFreeAsync(ws, stream);
     return err != cudaSuccess ? err : err2;

@@ -35,52 +35,20 @@
 namespace mmasim {
 namespace fast64 {
 
-using fast::BM;
-using fast::BN;
 using fast::KC;
 using fast::EB;
 using fast::CB;
 using fast::Elem;
 using fast::raw_elem;
 
-// 512 threads own the 128 x 64 tile of D, 4 x 4 outputs each (a warp: 32 x 16, the accumulator tiles of eight FP64 matrix
-// instructions): sixteen warps per SM keep the FP64 pipe fed while the per-thread state (accumulators, product exponents
-// of the next block, operand fragments) stays within 128 registers.
-constexpr int TM = 4, TN = 4, NT = 512;
-
-// The raw words of one chunk, E::TASK consecutive elements of one row of A or B per task (as in the integer kernels).
-template <int EK>
-struct RawChunk {
-    static constexpr int TPR = KC / Elem<EK>::TASK;
-    static constexpr int TASKS = (BM + BN) * TPR;
-    static constexpr int PER_THREAD = (TASKS + NT - 1) / NT;
-    static constexpr int WORDS = Elem<EK>::TASK * Elem<EK>::BYTES / 4;
-    uint32_t w[PER_THREAD][WORDS];
-};
-
-template <int EK>
-__device__ __forceinline__ void load_chunk(RawChunk<EK>& raw, const GemmArgs& g, int64_t row0, int64_t col0, int64_t k0, int tid) {
-    using E = Elem<EK>;
-    using R = RawChunk<EK>;
-#pragma unroll
-    for (int it = 0; it < R::PER_THREAD; ++it) {
-        const int task = it * NT + tid;
-        const bool is_a = task < BM * R::TPR;
-        const int u = is_a ? task : task - BM * R::TPR;
-        const int rows = is_a ? BM : BN;
-        const int r = u % rows, h = u / rows;              // consecutive threads take consecutive rows
-        const int64_t grow = (is_a ? row0 : col0) + r;
-        const bool valid = task < R::TASKS && grow < (is_a ? g.M : g.N);
-        const unsigned char* base = static_cast<const unsigned char*>(is_a ? g.A : g.B) +
-                                    (grow * (is_a ? g.lda : g.ldb) + k0 + h * E::TASK) * E::BYTES;
-#pragma unroll
-        for (int q = 0; q < R::WORDS / 4; ++q) {
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (valid) v = reinterpret_cast<const uint4*>(base)[q];
-            raw.w[it][4 * q] = v.x; raw.w[it][4 * q + 1] = v.y; raw.w[it][4 * q + 2] = v.z; raw.w[it][4 * q + 3] = v.w;
-        }
-    }
-}
+// 256 threads own a 64 x 64 tile of D, 4 x 4 outputs each (a warp: 32 x 16, the accumulator tiles of eight FP64 matrix
+// instructions), and two CTAs share an SM.  Sixteen warps per SM within 128 registers a thread either way, but next to one
+// CTA of 128 x 64: the integer phases of one CTA run beside the FP64 phases of the other (no barrier joins them), and an SM
+// that has one tile less than another idles for half as long.  2048 x 2048 x 2048: Ampere BF16 1598 -> 1422 us, TF32
+// 2358 -> 2025; x 1024: Volta FP16 1181 -> 1040, CDNA3 FP16 1016 -> 902, CDNA3 E4M3 1003 -> 855, CDNA1 FP16 912 -> 790;
+// 4096 x 4096 x 1024 (even numbers of tiles for both) 2796 -> 2777.  One CTA alone on an SM reaches 86 % of the rate of two.
+constexpr int BM = 64, BN = 64;
+constexpr int TM = 4, TN = 4, NT = 256;
 
 constexpr int G_OFF = 30;          // the B offset sits 30 bits below the element's last significand bit (bit 22 - mbits of a double's low word)
 
@@ -92,47 +60,14 @@ struct LutEntry64 {
 
 // Operand planes are row-major (k contiguous) with a pitch of KP doubles = 288 bytes: the fragment loads of the FP64
 // matrix instruction (lane (g, t) reads element (row 8 i + g, k 4 s + t)) then hit sixteen different bank pairs per
-// half-warp.  Exponent planes and masks are indexed by the permuted row / column (see perm_row64 / perm_col64), so that
+// half-warp.  Exponent pairs and masks are indexed by the permuted row / column (see perm_row64 / perm_col64), so that
 // the four rows and the four columns of a thread are adjacent.
 constexpr int KP = KC + 4;
-template <int EK, bool ROWMAJOR = false>
-struct Planes64;
-template <int EK>
-struct Planes64<EK, true> {
-    static constexpr bool ROW_MAJOR = true;
-    double a_d[BM][KP];
-    double b_d[BN][KP];
-    uint32_t a_exp2[KC / 2][BM];    // [pair p][permuted row]: exponents of elements 2p (low half) and 2p + 1 (high half)
-    uint32_t b_exp2[KC / 2][BN];
-    uint32_t a_sgn[BM], b_sgn[BN];  // [permuted row]: bit k = sign of element k of the chunk
-    uint32_t a_nz[BM], b_nz[BN];    // [permuted row]: bit k = element k is finite and nonzero
-};
-// The k-major layout of the kernels that still issue one scalar FP64 multiply-add per term (TR-, GTR- and E-FDPA): a
-// thread owns rows 4 ty .. 4 ty + 3 and the columns col_of(tx, c); nothing is permuted.
-template <int EK>
-struct Planes64<EK, false> {
-    static constexpr bool ROW_MAJOR = false;
-    double a_d[KC][BM];
-    double b_d[KC][BN];
-    uint32_t a_exp2[KC / 2][BM];
-    uint32_t b_exp2[KC / 2][BN];
-    uint32_t a_sgn[BM], b_sgn[BN];
-    uint32_t a_nz[BM], b_nz[BN];
-};
-
 // A warp owns 32 rows x 16 columns of the CTA tile, as four by two accumulator tiles of the 8 x 8 x 4 FP64 matrix
 // instruction; a thread's outputs are its share of those tiles: rows g + 8 r (g = lane / 4, r = 0..3) and columns
 // 8 (c / 2) + 2 t + c % 2 (t = lane % 4, c = 0..3).  Permuted positions put a thread's rows / columns side by side.
 __device__ __forceinline__ int perm_row64(int r) { return (r & ~31) | ((r & 7) << 2) | ((r >> 3) & 3); }
 __device__ __forceinline__ int perm_col64(int c) { return (c & ~15) | (((c >> 1) & 3) << 2) | (((c >> 3) & 1) << 1) | (c & 1); }
-
-template <int EK, bool ROWMAJOR = false>
-struct Smem64 {
-    Planes64<EK, ROWMAJOR> pl[2];   // the chunk being computed and the one being decoded
-    LutEntry64 lut_a[Elem<EK>::SIGNMAG ? 1 : 256];
-    LutEntry64 lut_b[Elem<EK>::SIGNMAG ? 1 : 256];
-    int special[3];                 // chunk (by index mod 3) holds an infinity or a NaN
-};
 
 __device__ __forceinline__ double pow2d(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
@@ -146,110 +81,27 @@ __device__ __forceinline__ double operand_b(uint32_t sign, uint32_t sig, int exp
     return sign ? -mag : mag;
 }
 
-template <int EK, class SM>
-__device__ __forceinline__ void init_lut64(SM& s, const FmtDesc& fa, const FmtDesc& fb, int tid) {
-    if (!Elem<EK>::SIGNMAG && tid < 256) {
-        const uint32_t da = decode_elem(fa, uint32_t(tid)), db = decode_elem(fb, uint32_t(tid));
-        const bool fin_a = dec_cls(da) == CLS_FINITE, fin_b = dec_cls(db) == CLS_FINITE;
-        LutEntry64 ea, eb;
-        const uint32_t sga = fin_a ? dec_sig(da) : 0u, sgb = fin_b ? dec_sig(db) : 0u;
-        ea.op = operand_a(fin_a ? dec_sign(da) : 0u, sga, fin_a ? dec_exp(da) : 0, fa.mbits);
-        ea.exp = sga ? uint32_t(dec_exp(da) + EB) : 0u;
-        ea.bits = (fin_a ? dec_sign(da) : 0u) | (fin_a ? 0u : 2u) | (sga ? 4u : 0u);
-        eb.op = operand_b(fin_b ? dec_sign(db) : 0u, sgb, fin_b ? dec_exp(db) : 0, fb.mbits);
-        eb.exp = sgb ? uint32_t(dec_exp(db) + EB) : 0u;
-        eb.bits = (fin_b ? dec_sign(db) : 0u) | (fin_b ? 0u : 2u) | (sgb ? 4u : 0u);
-        s.lut_a[tid] = ea;
-        s.lut_b[tid] = eb;
-    }
-}
-
-// Decode the raw words of a chunk into double operands, packed exponent pairs and sign bit masks.
-template <int EK, class SM, class PL>
-__device__ __forceinline__ void store_chunk64(SM& sm, PL& s, const RawChunk<EK>& raw, int flag, int tid) {
-    using E = Elem<EK>;
-    using R = RawChunk<EK>;
-    uint32_t spec = 0u;
-#pragma unroll
-    for (int it = 0; it < R::PER_THREAD; ++it) {
-        const int task = it * NT + tid;
-        if (task >= R::TASKS) break;
-        const bool is_a = task < BM * R::TPR;
-        const int u = is_a ? task : task - BM * R::TPR;
-        const int rows = is_a ? BM : BN;
-        const int r = u % rows, h = u / rows;
-        const int pr = !PL::ROW_MAJOR ? r : (is_a ? perm_row64(r) : perm_col64(r));
-        uint32_t bits = 0u, prev_exp = 0u;
-#pragma unroll
-        for (int q = 0; q < E::TASK; ++q) {
-            const int kk = h * E::TASK + q;
-            double op;
-            uint32_t expb;
-            if (!E::SIGNMAG) {
-                const uint32_t byte = (raw.w[it][q / 4] >> (8 * (q % 4))) & 0xFFu;
-                const LutEntry64 e = is_a ? sm.lut_a[byte] : sm.lut_b[byte];
-                op = e.op;
-                expb = e.exp;
-                bits += ((e.bits & 1u) | ((e.bits & 4u) << 14)) << q;      // sign in the low half, nonzero in the high half
-                spec |= e.bits & 2u;
-            } else {
-                const uint32_t w = E::BYTES == 2 ? ((raw.w[it][q / 2] >> (16 * (q % 2))) & 0xFFFFu) : raw.w[it][q];
-                // A normal number becomes a double by moving its exponent and mantissa fields into place and rebiasing
-                // (no arithmetic); the offset of a B operand is then bit 22 - mbits of the low word.  Subnormals take
-                // the arithmetic route; zeros, infinities and NaNs are staged as zero without exponent.
-                constexpr uint32_t TOP = (1u << E::EBITS) - 1u;
-                const uint32_t xx = w >> E::LOW;
-                const uint32_t mag = xx & ((1u << (E::EBITS + E::MBITS)) - 1u);
-                const uint32_t field = mag >> E::MBITS;
-                const uint32_t sign = (xx >> (E::EBITS + E::MBITS)) & 1u;
-                uint32_t hi = 0u, lo = 0u, nzbit = 1u;
-                expb = 0u;
-                if (field - 1u < TOP - 1u) {
-                    hi = (mag << (20 - E::MBITS)) + (uint32_t(1023 - E::BIAS) << 20);
-                    lo = is_a ? 0u : (1u << (22 - E::MBITS));
-                    expb = field + uint32_t(EB - E::BIAS);
-                } else if (field == 0u && mag != 0u) {
-                    const double v = is_a ? operand_a(0u, mag, 1 - E::BIAS, E::MBITS) : operand_b(0u, mag, 1 - E::BIAS, E::MBITS);
-                    hi = uint32_t(__double2hiint(v));
-                    lo = uint32_t(__double2loint(v));
-                    expb = uint32_t(1 - E::BIAS + EB);
-                } else {
-                    nzbit = 0u;
-                    spec |= uint32_t(field == TOP);
-                }
-                op = __hiloint2double(int(hi | (sign << 31)), int(lo));
-                bits += (sign | (nzbit << 16)) << q;
-            }
-            if (PL::ROW_MAJOR) { if (is_a) s.a_d[r][kk] = op; else s.b_d[r][kk] = op; }
-            else { if (is_a) s.a_d[kk][r] = op; else s.b_d[kk][r] = op; }
-            if (q & 1) {
-                const uint32_t pair = prev_exp | (expb << 16);
-                if (is_a) s.a_exp2[kk / 2][pr] = pair; else s.b_exp2[kk / 2][pr] = pair;
-            }
-            prev_exp = expb;
-        }
-        // sign and nonzero bits of the task's elements go to bits [h * TASK, h * TASK + TASK) of the row's masks
-        if (E::TASK == 16) {
-            if (is_a) { reinterpret_cast<uint16_t*>(&s.a_sgn[pr])[h] = uint16_t(bits); reinterpret_cast<uint16_t*>(&s.a_nz[pr])[h] = uint16_t(bits >> 16); }
-            else { reinterpret_cast<uint16_t*>(&s.b_sgn[pr])[h] = uint16_t(bits); reinterpret_cast<uint16_t*>(&s.b_nz[pr])[h] = uint16_t(bits >> 16); }
-        } else {
-            if (is_a) { reinterpret_cast<uint8_t*>(&s.a_sgn[pr])[h] = uint8_t(bits); reinterpret_cast<uint8_t*>(&s.a_nz[pr])[h] = uint8_t(bits >> 16); }
-            else { reinterpret_cast<uint8_t*>(&s.b_sgn[pr])[h] = uint8_t(bits); reinterpret_cast<uint8_t*>(&s.b_nz[pr])[h] = uint8_t(bits >> 16); }
-        }
-    }
-    if (spec) atomicOr(&sm.special[flag], 1);
-}
-
 // One operand's share of a chunk of KC = 32 elements of K, decoded for the matrix-instruction kernel: R rows of A (or
 // columns of B).  A decode kernel writes these blocks to scratch memory once per GEMM; the main kernel brings them in with
-// one bulk copy each.  Layouts as in Planes64<EK, true>; `pe` holds BF16 powers 2^(BASE (Exp - 1)) for the tensor-core
-// exponent maximum of the element kinds whose exponent sums fit (FP16 and the 8-bit kinds).
+// one bulk copy each.  Exponents come in the form that the kernel takes the block maximum from: pairs for the add-max
+// instructions, or BF16 powers 2^(BASE (Exp - 1)) for the tensor cores (element kinds whose exponent sums fit: FP16 and the
+// 8-bit kinds), or not at all (E-FDPA).
 constexpr int PE_STRIDE64 = KC + 8;     // 80 bytes per row: fragment loads hit 32 different banks
+enum { EXP_NONE, EXP_PAIRS, EXP_POWERS };
+__host__ __device__ constexpr int exp_form(int base) { return base ? EXP_POWERS : EXP_PAIRS; }
+template <int R, int FORM>
+struct Exp64 {};
 template <int R>
-struct Blk64 {
-    double d[R][KP];
-    uint32_t exp2[KC / 2][R];
+struct Exp64<R, EXP_PAIRS> {
+    uint32_t exp2[KC / 2][R];           // [pair p][permuted row]: exponents of elements 2p (low half) and 2p + 1 (high half)
+};
+template <int R>
+struct Exp64<R, EXP_POWERS> {
     uint16_t pe[R][PE_STRIDE64];
+};
+template <int R, int FORM>
+struct Blk64 : Exp64<R, FORM> {
+    double d[R][KP];
     uint32_t sgn[R], nz[R];
     uint8_t sf[R];                  // [permuted row]: the E8M0 scale factor of the row for this block of 32 (ST-FDPA), else 127
     uint32_t special;               // the block holds an infinity or a NaN
@@ -257,11 +109,13 @@ struct Blk64 {
     uint32_t wild;                  // some nonzero element lies outside [2^-48, 2^40)
     uint32_t pad;
 };
-static_assert(sizeof(Blk64<BM>) % 16 == 0 && sizeof(Blk64<BN>) % 16 == 0, "bulk copies move multiples of 16 bytes");
+static_assert(sizeof(Blk64<BM, EXP_NONE>) % 16 == 0 && sizeof(Blk64<BM, EXP_PAIRS>) % 16 == 0 && sizeof(Blk64<BM, EXP_POWERS>) % 16 == 0,
+              "bulk copies move multiples of 16 bytes");
 
+template <int FORM>
 struct SmemMM {
-    Blk64<BM> a[2];
-    Blk64<BN> b[2];
+    Blk64<BM, FORM> a[2];
+    Blk64<BN, FORM> b[2];
     unsigned long long full[2];         // mbarriers: the bulk copies of a buffer have landed
     int error;                          // a bounded wait ran out
 };
@@ -271,6 +125,7 @@ struct SmemMM {
 //   FP16 x FP16 (sums -28..30): BASE 4, sub-blocks of 8 terms; 8-bit kinds: 8 (E4M3 / FP6 / FP4 only: one accumulation of
 //   32), 5 (one E5M2 operand: sub-blocks of 16), 4 (two: sub-blocks of 8); BF16 and TF32 do not fit: BASE 0, add-max pass.
 __host__ __device__ constexpr int pe64_shift(int base) { return base == 5 ? 3 : 1; }       // (127 + shift) % base == 0
+__host__ __device__ constexpr bool tiny_zeros(int ek, int base) { return base == 0 || ek == fast::EK_F16; }
 __host__ __device__ constexpr int pe64_sub(int base) { return base == 8 ? 32 : (base == 5 ? 16 : 8); }
 
 // Decode pass: one CTA of 256 threads decodes one block (R rows x 32 elements) into shared memory and copies it to its
@@ -280,14 +135,14 @@ __host__ __device__ constexpr int pe64_sub(int base) { return base == 8 ? 32 : (
 // TINY_ZEROS (the T-FDPA kernels without a tensor-core maximum): a zero is staged as 2^-900 of its sign.  Its products are far below any
 // unit of a sum register, so that a positive one adds nothing and a negative one falls one unit short like every other
 // negative product: the sign masks alone count them, without the masks of nonzero elements.
-template <int EK, int R, bool IS_A, int BASE, bool EOSPLIT = false, bool TINY_ZEROS = false>
-__global__ void __launch_bounds__(256) decode64_kernel(DevModel m, const unsigned char* src, int64_t rows, int64_t ld, Blk64<R>* dst,
+template <int EK, int R, bool IS_A, int BASE, bool EOSPLIT = false, bool TINY_ZEROS = false, int FORM = exp_form(BASE)>
+__global__ void __launch_bounds__(256) decode64_kernel(DevModel m, const unsigned char* src, int64_t rows, int64_t ld, unsigned nch, Blk64<R, FORM>* dst,
                                                        const uint8_t* sf = nullptr, int64_t ld_sf = 0) {
     using E = Elem<EK>;
     constexpr int TPR = KC / E::TASK, TASKS = R * TPR, WORDS = E::TASK * E::BYTES / 4;
     extern __shared__ __align__(16) unsigned char dec_smem[];
     LutEntry64* lut = reinterpret_cast<LutEntry64*>(dec_smem);
-    Blk64<R>& blk = *reinterpret_cast<Blk64<R>*>(dec_smem + 256 * sizeof(LutEntry64));
+    Blk64<R, FORM>& blk = *reinterpret_cast<Blk64<R, FORM>*>(dec_smem + 256 * sizeof(LutEntry64));
     const int tid = threadIdx.x;
     if (!E::SIGNMAG) {
         const FmtDesc f = fmt_desc(IS_A ? m.fmt_a : m.fmt_b);
@@ -303,12 +158,12 @@ __global__ void __launch_bounds__(256) decode64_kernel(DevModel m, const unsigne
     }
     if (tid == 0) { blk.special = 0u; blk.max_exp = 0u; blk.wild = blk.pad = 0u; }
     __syncthreads();
-    const int64_t k0 = int64_t(blockIdx.x) * KC;
+    const int64_t tile = blockIdx.x / nch, chunk = blockIdx.x % nch, k0 = chunk * KC;
     uint32_t spec = 0u, top_exp = 0u, wild = 0u;
     for (int task = tid; task < TASKS; task += 256) {
         const int r = task % R, h = task / R;
         const int pr = IS_A ? perm_row64(r) : perm_col64(r);
-        const int64_t grow = int64_t(blockIdx.y) * R + r;
+        const int64_t grow = tile * R + r;
         uint32_t w[WORDS];
 #pragma unroll
         for (int q = 0; q < WORDS / 4; ++q) {
@@ -322,7 +177,7 @@ __global__ void __launch_bounds__(256) decode64_kernel(DevModel m, const unsigne
         int sc20 = 0;
         bool sc_nan = false;
         if (sf) {
-            const uint32_t sbyte = grow < rows ? uint32_t(sf[grow * ld_sf + blockIdx.x]) : 127u;
+            const uint32_t sbyte = grow < rows ? uint32_t(sf[grow * ld_sf + chunk]) : 127u;
             sc20 = (int(sbyte) - 127) << 20;
             sc_nan = sbyte == 0xFFu;
         }
@@ -374,15 +229,17 @@ __global__ void __launch_bounds__(256) decode64_kernel(DevModel m, const unsigne
             // BF16 word of 2^(BASE (Exp - 1)) (the B plane times 2^shift); 0 for an element without exponent
             const uint32_t pe = (BASE && expb) ? uint32_t((127 + (IS_A ? 0 : pe64_shift(BASE)) + BASE * (int(expb) - EB - 1)) << 7) : 0u;
             if (q & 1) {
-                blk.exp2[kk / 2][pr] = prev_exp | (expb << 16);
+                if constexpr (FORM == EXP_PAIRS) blk.exp2[kk / 2][pr] = prev_exp | (expb << 16);
                 pw[q / 2] |= pe << 16;
             } else pw[q / 2] = pe;
             prev_exp = expb;
             top_exp = max(top_exp, expb);
         }
+        if constexpr (FORM == EXP_POWERS) {
 #pragma unroll
-        for (int q = 0; q < E::TASK / 8; ++q)
-            reinterpret_cast<uint4*>(&blk.pe[r][h * E::TASK])[q] = make_uint4(pw[4 * q], pw[4 * q + 1], pw[4 * q + 2], pw[4 * q + 3]);
+            for (int q = 0; q < E::TASK / 8; ++q)
+                reinterpret_cast<uint4*>(&blk.pe[r][h * E::TASK])[q] = make_uint4(pw[4 * q], pw[4 * q + 1], pw[4 * q + 2], pw[4 * q + 3]);
+        }
         if (E::TASK == 16) {
             reinterpret_cast<uint16_t*>(&blk.sgn[pr])[h] = uint16_t(bits); reinterpret_cast<uint16_t*>(&blk.nz[pr])[h] = uint16_t(bits >> 16);
         } else {
@@ -392,41 +249,15 @@ __global__ void __launch_bounds__(256) decode64_kernel(DevModel m, const unsigne
     if (spec) atomicOr(&blk.special, 1u);
     if (wild) atomicOr(&blk.wild, 1u);
     if (tid < R) {                                      // the scale factors travel with the block (rows beyond the matrix: 2^0)
-        const int64_t grow = int64_t(blockIdx.y) * R + tid;
-        blk.sf[IS_A ? perm_row64(tid) : perm_col64(tid)] = (sf && grow < rows) ? sf[grow * ld_sf + blockIdx.x] : uint8_t(127);
+        const int64_t grow = tile * R + tid;
+        blk.sf[IS_A ? perm_row64(tid) : perm_col64(tid)] = (sf && grow < rows) ? sf[grow * ld_sf + chunk] : uint8_t(127);
     }
     top_exp = __reduce_max_sync(0xFFFFFFFFu, top_exp);
     if ((tid & 31) == 0 && top_exp) atomicMax(&blk.max_exp, top_exp);
     __syncthreads();
-    uint4* out = reinterpret_cast<uint4*>(dst + (int64_t(blockIdx.y) * gridDim.x + blockIdx.x));
+    uint4* out = reinterpret_cast<uint4*>(dst + blockIdx.x);
     const uint4* in = reinterpret_cast<const uint4*>(&blk);
-    for (int q = tid; q < int(sizeof(Blk64<R>) / 16); q += 256) out[q] = in[q];
-}
-
-// Columns of a thread's micro-tile in the k-major layout: two adjacent pairs, 32 columns apart, so that the sixteen
-// threads of a row of the thread grid read 256 contiguous bytes of B operands per 16-byte load.
-__device__ __forceinline__ int col_of(int tx, int c) { return (c >> 1) * (BN / 2) + tx * 2 + (c & 1); }
-
-// Largest exponent sum of the products of one block (pass 1 of Algorithm 7 without the accumulator), two elements
-// per instruction: lane 0 holds the even elements' maximum, lane 1 the odd ones'.  k-major layout.
-template <int L>
-__device__ __forceinline__ void product_exponents(const uint32_t* ea_p, const uint32_t* eb_p, uint32_t (&emp)[TM][TN]) {
-#pragma unroll
-    for (int r = 0; r < TM; ++r)
-#pragma unroll
-        for (int c = 0; c < TN; ++c) emp[r][c] = 0u;
-#pragma unroll
-    for (int kp = 0; kp < L / 2; ++kp) {
-        const uint4 ea0 = *reinterpret_cast<const uint4*>(ea_p + kp * BM);
-        const uint2 eb0 = *reinterpret_cast<const uint2*>(eb_p + kp * BN);
-        const uint2 eb1 = *reinterpret_cast<const uint2*>(eb_p + kp * BN + BN / 2);
-        const uint32_t ea[TM] = {ea0.x, ea0.y, ea0.z, ea0.w};
-        const uint32_t ebv[TN] = {eb0.x, eb0.y, eb1.x, eb1.y};
-#pragma unroll
-        for (int r = 0; r < TM; ++r)
-#pragma unroll
-            for (int c = 0; c < TN; ++c) emp[r][c] = __viaddmax_s16x2(ea[r], ebv[c], emp[r][c]);
-    }
+    for (int q = tid; q < int(sizeof(Blk64<R, FORM>) / 16); q += 256) out[q] = in[q];
 }
 
 // Multipliers read from the constant bank, so that the compiler keeps integer multiply-adds (which issue beside the
@@ -452,7 +283,8 @@ __device__ __forceinline__ uint32_t imad_hi(uint32_t a, int b, uint32_t c) {
     return d;
 }
 
-// The same for the permuted layout: ea_p / eb_p point at the thread's four adjacent (permuted) rows / columns of the
+// Largest exponent sum of the products of one block (pass 1 of Algorithm 7 without the accumulator), two elements per
+// instruction: lane 0 holds the even elements' maximum, lane 1 the odd ones'.  ea_p / eb_p point at the thread's four adjacent (permuted) rows / columns of the
 // first pair of the block.
 template <int L>
 __device__ __forceinline__ void product_exponents_adj(const uint32_t* ea_p, const uint32_t* eb_p, uint32_t (&emp)[TM][TN]) {
@@ -469,14 +301,14 @@ __device__ __forceinline__ void product_exponents_adj(const uint32_t* ea_p, cons
     }
 }
 
-// One CTA per SM, 512 threads, a 4 x 4 micro-tile per thread.  The FP64 pipe is the bound (one fma.rm.f64 per term),
+// The FP64 pipe is the floor (one fma.rm.f64 per term), the integer pipe is nearer (73 % busy in blocks of eight),
 // so everything else is arranged to run beside it: the staged planes are double-buffered (the next chunk is decoded
 // between two barriers while its raw words were fetched a chunk earlier), and the product-exponent pass of block
 // n + 1 is fused, instruction by instruction, into the multiply-add pass of block n - the integer pipe works in
 // the issue slots that the FP64 pipe leaves free.
 template <int EK, int L, int RHO, bool PROMOTE, bool ST, int BASE>
-__global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, const Blk64<BM>* __restrict__ wa,
-                                                        const Blk64<BN>* __restrict__ wb) {
+__global__ void __launch_bounds__(NT, 2) tfdpa64_kernel(DevModel m, GemmArgs g, const Blk64<BM, exp_form(BASE)>* __restrict__ wa,
+                                                        const Blk64<BN, exp_form(BASE)>* __restrict__ wb) {
     // BASE > 0: the block maximum of the product exponents comes from the tensor cores (a product of powers BASE^Exp on
     // BF16 planes, as in the F = 13 kernel); BASE = 0: from fused add-max instructions on packed exponent pairs.
     static_assert(BASE == 0 || ((BASE == 4 || BASE == 8) && L >= 8), "see pe64_shift / pe64_sub");
@@ -489,26 +321,27 @@ __global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, 
     static_assert(KC % L == 0 && L % 4 == 0, "blocks tile the chunk; pass 1 handles pairs of elements");
     static_assert(!ST || L == KC, "ST-FDPA: one scale factor pair per block of 32 (Algorithm 8)");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    SmemMM& sm = *reinterpret_cast<SmemMM*>(smem_raw);
+    SmemMM<exp_form(BASE)>& sm = *reinterpret_cast<SmemMM<exp_form(BASE)>*>(smem_raw);
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
-    const int wr = warp >> 2, wc = warp & 3, gq = lane >> 2, tq = lane & 3;      // warp grid 4 x 4, warp tile 32 x 16
+    const int wr = warp >> 2, wc = warp & 3, gq = lane >> 2, tq = lane & 3;      // warp grid 2 x 4, warp tile 32 x 16
     const int prow = wr * 32 + gq * 4, pcol = wc * 16 + tq * 4;                  // the thread's first permuted row / column
     auto row_at = [&](int r) { return wr * 32 + gq + 8 * r; };                   // inside the CTA tile
     auto col_at = [&](int c) { return wc * 16 + 8 * (c >> 1) + 2 * tq + (c & 1); };
-    const int64_t row0 = int64_t(blockIdx.y) * BM, col0 = int64_t(blockIdx.x) * BN;
+    const unsigned tiles_n = unsigned((g.N + BN - 1) / BN), tile_m = blockIdx.x / tiles_n, tile_n = blockIdx.x % tiles_n;
+    const int64_t row0 = int64_t(tile_m) * BM, col0 = int64_t(tile_n) * BN;
     const FmtDesc fa = fmt_desc(m.fmt_a), fb = fmt_desc(m.fmt_b);
 
     // the decoded blocks of this tile row of A and tile column of B, chunk after chunk, land in two buffers by bulk copies
     const int NCH = int(g.K / KC);
-    const Blk64<BM>* src_a = wa + int64_t(blockIdx.y) * NCH;
-    const Blk64<BN>* src_b = wb + int64_t(blockIdx.x) * NCH;
+    const Blk64<BM, exp_form(BASE)>* src_a = wa + int64_t(tile_m) * NCH;
+    const Blk64<BN, exp_form(BASE)>* src_b = wb + int64_t(tile_n) * NCH;
     auto issue = [&](int n) {                              // one thread: both copies of chunk n into buffer n & 1
         unsigned long long* bar = &sm.full[n & 1];
-        fast::mbar_expect_tx(bar, uint32_t(sizeof(Blk64<BM>) + sizeof(Blk64<BN>)));
-        fast::bulk_load(&sm.a[n & 1], src_a + n, uint32_t(sizeof(Blk64<BM>)), bar);
-        fast::bulk_load(&sm.b[n & 1], src_b + n, uint32_t(sizeof(Blk64<BN>)), bar);
+        fast::mbar_expect_tx(bar, uint32_t(sizeof(Blk64<BM, exp_form(BASE)>) + sizeof(Blk64<BN, exp_form(BASE)>)));
+        fast::bulk_load(&sm.a[n & 1], src_a + n, uint32_t(sizeof(Blk64<BM, exp_form(BASE)>)), bar);
+        fast::bulk_load(&sm.b[n & 1], src_b + n, uint32_t(sizeof(Blk64<BN, exp_form(BASE)>)), bar);
     };
     if (tid == 0) {
         sm.error = 0;
@@ -548,7 +381,11 @@ __global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, 
     // eight): accumulators that are zero or within 2^-100 .. 2^100, and a chunk whose nonzero elements are within 2^-48 .. 2^40.  A
     // nonzero sum is then a multiple of 2^-123 (of 2^(-96 - F), or an accumulator unchanged), and K products of at most 2^83 each
     // stay below 2^116.  FP16 elements always are within.
-    constexpr bool TAMEABLE = BASE == 0 && !ACC16 && !ST;
+    // With the tensor-core maximum (FP16) a block without a nonzero product reads as e_max = -30, two below the smallest
+    // exponent sum of FP16.  That returns c unchanged all the same, where c is a multiple of 2^(-30 - F): one of 2^-30 and above
+    // as an initial accumulator, and every sum since (a block's unit is 2^(-30 - F) or more).
+    constexpr bool TAMEABLE = (BASE == 0 || EK == fast::EK_F16) && !ACC16 && !ST;
+    constexpr int C_LOW = BASE ? -30 : -100;            // (FP16: see below)
     bool c_tame = false;
     double cs[DS ? TM : 1][DS ? TN : 1];
     uint32_t sub_mask = 0u;                             // outputs whose accumulator is a nonzero FP32 subnormal: Exp(c) = -126
@@ -588,11 +425,11 @@ __global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, 
         // a wait that runs out is recorded and the chunk computed on whatever is there; every thread sees the flag after
         // the barrier at the end of the chunk, and the CTA leaves together without storing anything
         if (!fast::mbar_wait(&sm.full[chunk & 1], uint32_t(chunk >> 1) & 1u)) *reinterpret_cast<volatile int*>(&sm.error) = 1;
-        const Blk64<BM>& sa_blk = sm.a[chunk & 1];
-        const Blk64<BN>& sb_blk = sm.b[chunk & 1];
+        const Blk64<BM, exp_form(BASE)>& sa_blk = sm.a[chunk & 1];
+        const Blk64<BN, exp_form(BASE)>& sb_blk = sm.b[chunk & 1];
         const bool chunk_special = (sa_blk.special | sb_blk.special) != 0u;
         // the first block's product exponents (the other blocks' are taken beside the multiply-adds of their predecessor)
-        if (BASE == 0) product_exponents_adj<L>(&sa_blk.exp2[0][prow], &sb_blk.exp2[0][pcol], emp);
+        if constexpr (BASE == 0) product_exponents_adj<L>(&sa_blk.exp2[0][prow], &sb_blk.exp2[0][pcol], emp);
 
         // ST-FDPA (Algorithm 8): Exp(alpha) of this thread's rows and Exp(beta) of its columns for this block of 32, as
         // exponent-field increments.  The staged operands already carry the scale factors (decode pass), so the products,
@@ -628,7 +465,7 @@ __global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, 
 #pragma unroll
                 for (int c = 0; c < TN; ++c) {
                     const uint32_t h = uint32_t(__double2hiint(cs[DS ? r : 0][DS ? c : 0])) & 0x7FFFFFFFu;
-                    ok = ok && (h == 0u || h - (uint32_t(1023 - 100) << 20) < (200u << 20));
+                    ok = ok && (h == 0u || h - (uint32_t(1023 + C_LOW) << 20) < (uint32_t(100 - C_LOW) << 20));
                 }
             c_tame = __all_sync(0xFFFFFFFFu, ok);       // (matrix instructions need the whole warp)
         }
@@ -661,7 +498,7 @@ __global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, 
                     }
             }
 
-            if (BASE) {
+            if constexpr (BASE != 0) {
                 // ---- pass 1 on the tensor cores: P = sum_k pe(a_k) pe(b_k) per sub-block of KSUB terms, the block's P the
                 // integer maximum of their words; emp receives the raw words (0: no nonzero product) ----
                 constexpr int KSUB = pe64_sub(BASE) < L ? pe64_sub(BASE) : L, NSUB = L / KSUB;
@@ -796,10 +633,11 @@ __global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, 
             uint32_t urange = 0u;
             auto block_value = [&](int r, int c) -> double {
                 const uint32_t sa = sa_blk.sgn[prow + r];
-                uint32_t live = kmask;                  // (BASE = 0: zeros are staged as tiny numbers of their sign)
-                if (BASE) {
-                    live &= sa_blk.nz[prow + r] & sb_blk.nz[pcol + c];
-                    no_product = no_product || live == 0u;
+                uint32_t live = kmask;                  // (TINY: zeros are staged as tiny numbers of their sign)
+                if (BASE && !TAME) {
+                    const uint32_t nz = sa_blk.nz[prow + r] & sb_blk.nz[pcol + c] & kmask;
+                    no_product = no_product || nz == 0u;
+                    if (!tiny_zeros(EK, BASE)) live = nz;
                 }
                 const int nneg = __popc((sa ^ sb_blk.sgn[pcol + c]) & live);
                 double v;
@@ -827,13 +665,13 @@ __global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, 
                     asm("cvt.f64.f16 %0, %1;" : "=d"(x) : "h"(__half_as_ushort(__double2half(v))));
                     urange = max(uint32_t(imad(__double2hiint(x), c_mul64[6], int(0u - 2u * LOWHI))), urange);
                     const double st = __hiloint2double(__double2hiint(x), __double2loint(x) | 1);
-                    if (BASE) nv[BASE ? r : 0][BASE ? c : 0] = st; else cs[DS ? r : 0][DS ? c : 0] = st;
+                    if (BASE && !TAME) nv[BASE ? r : 0][BASE ? c : 0] = st; else cs[DS ? r : 0][DS ? c : 0] = st;
                 } else if (DS) {
                     // (twice the high word: the sign leaves at the top, and a multiply-add is not on the integer pipe)
                     if (!TAME) urange = max(uint32_t(imad(__double2hiint(v), c_mul64[6], int(0u - 2u * LOWHI))), urange);
                     // RZ-FP32 of a number in the normal range: the low 29 bits of the double's significand go
                     const double st = __hiloint2double(__double2hiint(v), (__double2loint(v) & int(0xE0000000u)) | 1);
-                    if (BASE) nv[BASE ? r : 0][BASE ? c : 0] = st; else cs[DS ? r : 0][DS ? c : 0] = st;
+                    if (BASE && !TAME) nv[BASE ? r : 0][BASE ? c : 0] = st; else cs[DS ? r : 0][DS ? c : 0] = st;
                 }
             };
 
@@ -859,7 +697,7 @@ __global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, 
 #pragma unroll
                 for (int q = 0; q < PER; ++q)
                     if (ksi * PER + q < 8) finish((ksi * PER + q) / TN, (ksi * PER + q) % TN);
-                if (fuse) {                             // the product exponents of the next block (add-max kinds)
+                if constexpr (BASE == 0) if (fuse) {    // the product exponents of the next block (add-max kinds)
                     const uint32_t* ea_p = &sa_blk.exp2[(kb + L) / 2 < KC / 2 ? (kb + L) / 2 : 0][prow];
                     const uint32_t* eb_p = &sb_blk.exp2[(kb + L) / 2 < KC / 2 ? (kb + L) / 2 : 0][pcol];
 #pragma unroll
@@ -973,38 +811,38 @@ __global__ void __launch_bounds__(NT, 1) tfdpa64_kernel(DevModel m, GemmArgs g, 
 
 template <int EK, int L, int RHO, bool PROMOTE, bool ST, int BASE>
 cudaError_t launch_one64b(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
-    const size_t sh = sizeof(SmemMM);
+    const size_t sh = sizeof(SmemMM<exp_form(BASE)>);
     cudaError_t err = cudaFuncSetAttribute(tfdpa64_kernel<EK, L, RHO, PROMOTE, ST, BASE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sh));
     if (err != cudaSuccess) return err;
-    const size_t dsh_a = 256 * sizeof(LutEntry64) + sizeof(Blk64<BM>), dsh_b = 256 * sizeof(LutEntry64) + sizeof(Blk64<BN>);
-    if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BM, true, BASE, false, BASE == 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_a))) != cudaSuccess) return err;
-    if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BN, false, BASE, false, BASE == 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_b))) != cudaSuccess) return err;
+    const size_t dsh_a = 256 * sizeof(LutEntry64) + sizeof(Blk64<BM, exp_form(BASE)>), dsh_b = 256 * sizeof(LutEntry64) + sizeof(Blk64<BN, exp_form(BASE)>);
+    if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BM, true, BASE, false, tiny_zeros(EK, BASE)>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_a))) != cudaSuccess) return err;
+    if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BN, false, BASE, false, tiny_zeros(EK, BASE)>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_b))) != cudaSuccess) return err;
     const int64_t tiles_m = (g.M + BM - 1) / BM, tiles_n = (g.N + BN - 1) / BN, nch = g.K / KC;
     // scratch: the decoded blocks of A and B, stream-ordered out of the library's pool and returned to it behind the kernel
-    const size_t bytes_a = size_t(tiles_m * nch) * sizeof(Blk64<BM>), bytes_b = size_t(tiles_n * nch) * sizeof(Blk64<BN>);
+    const size_t bytes_a = size_t(tiles_m * nch) * sizeof(Blk64<BM, exp_form(BASE)>), bytes_b = size_t(tiles_n * nch) * sizeof(Blk64<BN, exp_form(BASE)>);
     cudaMemPool_t pool = nullptr;
     if ((err = scratch_pool(&pool)) != cudaSuccess) return err;
     void* ws = nullptr;
     if ((err = cudaMallocFromPoolAsync(&ws, bytes_a + bytes_b, pool, stream)) != cudaSuccess) return err;
-    Blk64<BM>* wa = static_cast<Blk64<BM>*>(ws);
-    Blk64<BN>* wb = reinterpret_cast<Blk64<BN>*>(static_cast<unsigned char*>(ws) + bytes_a);
-    decode64_kernel<EK, BM, true, BASE, false, BASE == 0><<<dim3((unsigned)nch, (unsigned)tiles_m), 256, dsh_a, stream>>>(
-        m, static_cast<const unsigned char*>(g.A), g.M, g.lda, wa, ST ? g.sfa : nullptr, g.ld_sfa);
-    decode64_kernel<EK, BN, false, BASE, false, BASE == 0><<<dim3((unsigned)nch, (unsigned)tiles_n), 256, dsh_b, stream>>>(
-        m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, wb, ST ? g.sfb : nullptr, g.ld_sfb);
-    dim3 grid((unsigned)tiles_n, (unsigned)tiles_m, 1);
-    tfdpa64_kernel<EK, L, RHO, PROMOTE, ST, BASE><<<grid, NT, sh, stream>>>(m, g, wa, wb);
+    Blk64<BM, exp_form(BASE)>* wa = static_cast<Blk64<BM, exp_form(BASE)>*>(ws);
+    Blk64<BN, exp_form(BASE)>* wb = reinterpret_cast<Blk64<BN, exp_form(BASE)>*>(static_cast<unsigned char*>(ws) + bytes_a);
+    decode64_kernel<EK, BM, true, BASE, false, tiny_zeros(EK, BASE)><<<unsigned(nch * tiles_m), 256, dsh_a, stream>>>(
+        m, static_cast<const unsigned char*>(g.A), g.M, g.lda, unsigned(nch), wa, ST ? g.sfa : nullptr, g.ld_sfa);
+    decode64_kernel<EK, BN, false, BASE, false, tiny_zeros(EK, BASE)><<<unsigned(nch * tiles_n), 256, dsh_b, stream>>>(
+        m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, unsigned(nch), wb, ST ? g.sfb : nullptr, g.ld_sfb);
+    tfdpa64_kernel<EK, L, RHO, PROMOTE, ST, BASE><<<unsigned(tiles_n * tiles_m), NT, sh, stream>>>(m, g, wa, wb);
     err = cudaGetLastError();
     const cudaError_t err2 = cudaFreeAsync(ws, stream);
     return err != cudaSuccess ? err : err2;
 }
 
-// The base of the tensor-core exponent maximum by element kinds: FP16 (blocks of 16) 4; 8-bit kinds 4 with an E5M2
-// operand, else 8; BF16, TF32 and blocks of 4 and 8: the add-max pass (for blocks of 8 it is as fast, and two of them
-// are unrolled per loop trip).
+// The base of the tensor-core exponent maximum by element kinds: FP16 4; 8-bit kinds 4 with an E5M2 operand, else 8; BF16 and
+// TF32 (their exponent sums do not fit) and blocks of 4: the add-max pass.  FP16 in blocks of 8 with FP32 accumulators,
+// 2048 x 2048 x 1024: 647 us against 700 with add-max; with FP16 accumulators, which keep the masks of nonzero elements beside
+// the tensor-core maximum, 876 against 802: add-max.
 template <int EK, int L, int RHO, bool PROMOTE, bool ST = false>
 cudaError_t launch_one64(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
-    if constexpr (EK == fast::EK_F16 && L >= 16) return launch_one64b<EK, L, RHO, PROMOTE, ST, 4>(m, g, stream);
+    if constexpr (EK == fast::EK_F16 && (L >= 16 || (L == 8 && RHO != RHO_RNE_FP16))) return launch_one64b<EK, L, RHO, PROMOTE, ST, 4>(m, g, stream);
     else if constexpr (EK == fast::EK_LUT8 && L >= 8) {
         if (m.fmt_a == EF_E5M2 || m.fmt_b == EF_E5M2) return launch_one64b<EK, L, RHO, PROMOTE, ST, 4>(m, g, stream);
         return launch_one64b<EK, L, RHO, PROMOTE, ST, 8>(m, g, stream);

@@ -74,7 +74,7 @@ bool fast_tfdpa_supported(const DevModel& m, const GemmArgs& g) {
     if (g.k_chunk % fast::KC) return false;
     if ((kind == KIND_TR || kind == KIND_E) && g.k_chunk) return false;
     if (((g.lda * bytes) % 16) || ((g.ldb * bytes) % 16)) return false;      // 16-byte row starts for the vector loads
-    if (g.M > 65535ll * fast::BM) return false;                             // grid.y
+    if (m.F == 13 && g.M > 65535ll * fast::BM) return false;                // grid.y
     if (g.N > 0x7FFFFFFFll - 128 || g.K > 0x7FFFFFFFll - 64) return false;   // 32-bit tile origins and k offsets in the kernels
     return true;
 }
@@ -87,11 +87,11 @@ bool rows16(const DevModel& m, const GemmArgs& g) {                          // 
 }  // namespace
 
 // Small tiles, or the large kernel?  What an SM does per chunk of 32 elements of K decides: CTAs on the fullest SM times the time
-// of one, plus the latency of a chunk when there are few.  In units of a 16 x 16 tile's chunk (0.33 - 0.55 us by family), measured
-// on full grids (4096 x 4096 x 256) and on single waves: 8 x 16 tiles 0.6, 32 x 32 tiles `mid`, tiles of the large kernel `large`
-// (its decode pass and two more launches: about 6 us, fifteen units of one chunk).  Examples, small against large in us, on both
-// sides of the line: Hopper FP16 128 x 2048 x 2048 128 / 337, 2352 x 192 x 3328 320 / 771, 1000 x 1111 x 992 245 / 254,
-// 1024^3 225 / 175, 2048 x 2048 x 512 449 / 340.
+// of one, plus the latency of a chunk when there are few.  In units of a 16 x 16 tile's chunk (about 0.45 us), measured on one to
+// eighteen CTAs per SM at K = 1024 and 256: 8 x 16 tiles 0.6, 32 x 32 tiles `mid`, tiles of the large kernel `large` (two to an SM;
+// one that is alone takes 16 % longer) and 17 us for its decode pass and two more launches (F = 13: 7).  Small against large in us,
+// on both sides of the line, K = 1024: Ampere FP16 512 x 512 75 / 124, 768 x 768 142 / 126, 1024 x 1536 370 / 297; CDNA3 FP16
+// 768 x 768 150 / 166, 1024 x 1536 394 / 404, 2048 x 2048 - / 889; CDNA3 E4M3 768 x 768 188 / 161.
 DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us) {
     const int kind = kind_of(m);
     if (!kind || g.dot_mode || m.literal_emax) return DIRECT_NONE;
@@ -100,11 +100,16 @@ DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us) {
     constexpr int64_t SMS = 148;
     auto fullest = [&](int bm, int bn) { return double((((g.M + bm - 1) / bm) * ((g.N + bn - 1) / bn) + SMS - 1) / SMS); };
     const bool f13 = kind == 1 + fast::EK_LUT8 && m.F == 13, bits8 = kind == 1 + fast::EK_LUT8;
-    const double mid = bits8 ? 2.1 : (kind == KIND_E ? 3.4 : (kind == KIND_TR ? 2.7 : (m.L >= 16 ? 2.7 : 3.2)));
-    const double large = f13 ? 13.5 : (bits8 ? 9.5 : (kind == KIND_E ? 22.0 : (kind == KIND_TR ? 18.0 : (m.L >= 16 ? 14.0 : 20.0))));
+    const double mid = bits8 ? 2.1 : (kind == KIND_E ? 2.3 : (kind == KIND_TR ? (m.family == FAM_GTR ? 3.05 : 2.4) : (m.L <= 4 ? 3.2 : 2.3)));
+    const double large = f13 ? 13.5 : (bits8 ? 5.0 : (kind == KIND_E ? 7.6 : (kind == KIND_TR ? (m.family == FAM_GTR ? 8.3 : 8.7) :
+                         (m.L <= 4 ? 10.1 : (kind == 1 + fast::EK_F16 ? (m.acc == ACC_F16 ? 7.8 : 6.3) : 7.3)))));
     const double c8 = 0.5 + 0.6 * fullest(8, 16), c16 = 0.6 + fullest(16, 16), c32 = 0.6 + mid * fullest(32, 32);
     const double chunks = double((g.K + fast::KC - 1) / fast::KC);
-    const double big = fast_tfdpa_supported(m, g) ? large * fullest(fast::BM, f13 && m.acc != ACC_F16 && !g.k_chunk ? 128 : fast::BN) + 15.0 / chunks : 1e30;
+    double big = 1e30;
+    if (fast_tfdpa_supported(m, g)) {
+        const double n = f13 ? fullest(fast::BM, m.acc != ACC_F16 && !g.k_chunk ? 128 : fast::BN) : fullest(64, 64);
+        big = large * (f13 || int64_t(n) % 2 == 0 ? n : n + 0.16 / n) + (f13 ? 15.0 : 38.0) / chunks;
+    }
     if (us) *us = 3.0 + 0.45 * chunks * std::min(std::min(c8, c16), std::min(c32, big));
     if (big <= c8 && big <= c16 && big <= c32) return DIRECT_NONE;
     return c8 <= c16 && c8 <= c32 ? DIRECT_8x16 : (c16 <= c32 ? DIRECT_16x16 : DIRECT_32x32);

@@ -28,20 +28,21 @@ using fast::EK_BF16;
 using fast::EK_TF32;
 
 template <int EK, int L, bool GTR>
-__global__ void __launch_bounds__(NT, 1) trfdpa64_kernel(DevModel m, GemmArgs g, const Blk64<BM>* __restrict__ wa,
-                                                         const Blk64<BN>* __restrict__ wb) {
+__global__ void __launch_bounds__(NT, 2) trfdpa64_kernel(DevModel m, GemmArgs g, const Blk64<BM, EXP_PAIRS>* __restrict__ wa,
+                                                         const Blk64<BN, EXP_PAIRS>* __restrict__ wb) {
     constexpr int NBLK = KC / L;
     static_assert(KC % L == 0 && L % 4 == 0 && (!GTR || L == 16), "blocks tile the chunk; a matrix instruction takes four terms");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    SmemMM& sm = *reinterpret_cast<SmemMM*>(smem_raw);
+    SmemMM<EXP_PAIRS>& sm = *reinterpret_cast<SmemMM<EXP_PAIRS>*>(smem_raw);
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
-    const int wr = warp >> 2, wc = warp & 3, gq = lane >> 2, tq = lane & 3;      // warp grid 4 x 4, warp tile 32 x 16
+    const int wr = warp >> 2, wc = warp & 3, gq = lane >> 2, tq = lane & 3;      // warp grid 2 x 4, warp tile 32 x 16
     const int prow = wr * 32 + gq * 4, pcol = wc * 16 + tq * 4;                  // the thread's first permuted row / column
     auto row_at = [&](int r) { return wr * 32 + gq + 8 * r; };                   // inside the CTA tile
     auto col_at = [&](int c) { return wc * 16 + 8 * (c >> 1) + 2 * tq + (c & 1); };
-    const int64_t row0 = int64_t(blockIdx.y) * BM, col0 = int64_t(blockIdx.x) * BN;
+    const unsigned tiles_n = unsigned((g.N + BN - 1) / BN), tile_m = blockIdx.x / tiles_n, tile_n = blockIdx.x % tiles_n;
+    const int64_t row0 = int64_t(tile_m) * BM, col0 = int64_t(tile_n) * BN;
     const FmtDesc fa = fmt_desc(m.fmt_a), fb = fmt_desc(m.fmt_b);
     const int F = m.F, F2 = m.F2;
     const int frac = fa.mbits + fb.mbits;
@@ -50,13 +51,13 @@ __global__ void __launch_bounds__(NT, 1) trfdpa64_kernel(DevModel m, GemmArgs g,
 
     // the decoded blocks of this tile row of A and tile column of B, chunk after chunk, land in two buffers by bulk copies
     const int NCH = int(g.K / KC);
-    const Blk64<BM>* src_a = wa + int64_t(blockIdx.y) * NCH;
-    const Blk64<BN>* src_b = wb + int64_t(blockIdx.x) * NCH;
+    const Blk64<BM, EXP_PAIRS>* src_a = wa + int64_t(tile_m) * NCH;
+    const Blk64<BN, EXP_PAIRS>* src_b = wb + int64_t(tile_n) * NCH;
     auto issue = [&](int n) {                              // one thread: both copies of chunk n into buffer n & 1
         unsigned long long* bar = &sm.full[n & 1];
-        fast::mbar_expect_tx(bar, uint32_t(sizeof(Blk64<BM>) + sizeof(Blk64<BN>)));
-        fast::bulk_load(&sm.a[n & 1], src_a + n, uint32_t(sizeof(Blk64<BM>)), bar);
-        fast::bulk_load(&sm.b[n & 1], src_b + n, uint32_t(sizeof(Blk64<BN>)), bar);
+        fast::mbar_expect_tx(bar, uint32_t(sizeof(Blk64<BM, EXP_PAIRS>) + sizeof(Blk64<BN, EXP_PAIRS>)));
+        fast::bulk_load(&sm.a[n & 1], src_a + n, uint32_t(sizeof(Blk64<BM, EXP_PAIRS>)), bar);
+        fast::bulk_load(&sm.b[n & 1], src_b + n, uint32_t(sizeof(Blk64<BN, EXP_PAIRS>)), bar);
     };
     if (tid == 0) {
         sm.error = 0;
@@ -95,8 +96,8 @@ __global__ void __launch_bounds__(NT, 1) trfdpa64_kernel(DevModel m, GemmArgs g,
         // a wait that runs out is recorded and the chunk computed on whatever is there; every thread sees the flag after
         // the barrier at the end of the chunk, and the CTA leaves together without storing anything
         if (!fast::mbar_wait(&sm.full[chunk & 1], uint32_t(chunk >> 1) & 1u)) *reinterpret_cast<volatile int*>(&sm.error) = 1;
-        const Blk64<BM>& sa_blk = sm.a[chunk & 1];
-        const Blk64<BN>& sb_blk = sm.b[chunk & 1];
+        const Blk64<BM, EXP_PAIRS>& sa_blk = sm.a[chunk & 1];
+        const Blk64<BN, EXP_PAIRS>& sb_blk = sm.b[chunk & 1];
         const bool chunk_special = (sa_blk.special | sb_blk.special) != 0u;
         // no product of the chunk reaches 2^126 when the largest exponents of its A and B elements do not add up to it (a
         // bound from the decode pass: crossing it only sends the chunk's blocks through the exact scan below)
@@ -309,27 +310,26 @@ __global__ void __launch_bounds__(NT, 1) trfdpa64_kernel(DevModel m, GemmArgs g,
 
 template <int EK, int L, bool GTR>
 cudaError_t launch_tr_one(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
-    const size_t sh = sizeof(SmemMM);
+    const size_t sh = sizeof(SmemMM<EXP_PAIRS>);
     cudaError_t err = cudaFuncSetAttribute(trfdpa64_kernel<EK, L, GTR>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sh));
     if (err != cudaSuccess) return err;
-    const size_t dsh_a = 256 * sizeof(LutEntry64) + sizeof(Blk64<BM>), dsh_b = 256 * sizeof(LutEntry64) + sizeof(Blk64<BN>);
+    const size_t dsh_a = 256 * sizeof(LutEntry64) + sizeof(Blk64<BM, EXP_PAIRS>), dsh_b = 256 * sizeof(LutEntry64) + sizeof(Blk64<BN, EXP_PAIRS>);
     if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BM, true, 0, GTR>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_a))) != cudaSuccess) return err;
     if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BN, false, 0, GTR>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_b))) != cudaSuccess) return err;
     const int64_t tiles_m = (g.M + BM - 1) / BM, tiles_n = (g.N + BN - 1) / BN, nch = g.K / KC;
     // scratch: the decoded blocks of A and B, stream-ordered out of the library's pool and returned to it behind the kernel
-    const size_t bytes_a = size_t(tiles_m * nch) * sizeof(Blk64<BM>), bytes_b = size_t(tiles_n * nch) * sizeof(Blk64<BN>);
+    const size_t bytes_a = size_t(tiles_m * nch) * sizeof(Blk64<BM, EXP_PAIRS>), bytes_b = size_t(tiles_n * nch) * sizeof(Blk64<BN, EXP_PAIRS>);
     cudaMemPool_t pool = nullptr;
     if ((err = scratch_pool(&pool)) != cudaSuccess) return err;
     void* ws = nullptr;
     if ((err = cudaMallocFromPoolAsync(&ws, bytes_a + bytes_b, pool, stream)) != cudaSuccess) return err;
-    Blk64<BM>* wa = static_cast<Blk64<BM>*>(ws);
-    Blk64<BN>* wb = reinterpret_cast<Blk64<BN>*>(static_cast<unsigned char*>(ws) + bytes_a);
-    decode64_kernel<EK, BM, true, 0, GTR><<<dim3((unsigned)nch, (unsigned)tiles_m), 256, dsh_a, stream>>>(
-        m, static_cast<const unsigned char*>(g.A), g.M, g.lda, wa);
-    decode64_kernel<EK, BN, false, 0, GTR><<<dim3((unsigned)nch, (unsigned)tiles_n), 256, dsh_b, stream>>>(
-        m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, wb);
-    dim3 grid((unsigned)tiles_n, (unsigned)tiles_m, 1);
-    trfdpa64_kernel<EK, L, GTR><<<grid, NT, sh, stream>>>(m, g, wa, wb);
+    Blk64<BM, EXP_PAIRS>* wa = static_cast<Blk64<BM, EXP_PAIRS>*>(ws);
+    Blk64<BN, EXP_PAIRS>* wb = reinterpret_cast<Blk64<BN, EXP_PAIRS>*>(static_cast<unsigned char*>(ws) + bytes_a);
+    decode64_kernel<EK, BM, true, 0, GTR><<<unsigned(nch * tiles_m), 256, dsh_a, stream>>>(
+        m, static_cast<const unsigned char*>(g.A), g.M, g.lda, unsigned(nch), wa);
+    decode64_kernel<EK, BN, false, 0, GTR><<<unsigned(nch * tiles_n), 256, dsh_b, stream>>>(
+        m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, unsigned(nch), wb);
+    trfdpa64_kernel<EK, L, GTR><<<unsigned(tiles_n * tiles_m), NT, sh, stream>>>(m, g, wa, wb);
     err = cudaGetLastError();
     const cudaError_t err2 = cudaFreeAsync(ws, stream);
     return err != cudaSuccess ? err : err2;
