@@ -10,8 +10,9 @@
 // offset 2^-(pre + guard) below the last significand bit (B), so that a negative product is never on the grid and
 // floors to the one's complement of its truncated magnitude; a population count over sign masks adds the number of
 // negative terms back (a zero is staged as a tiny number of its sign, TINY: far below any unit, its negative products too
-// fall one short, so that no mask of nonzero elements is needed: 4.21 -> 4.1 ms).  The accumulator enters by one addition rounded toward minus infinity (its
-// lowest mantissa bit set, so that a negative c floors likewise; the +1 is added to the register's starting value),
+// fall one short, so that no mask of nonzero elements is needed).  The accumulator enters by one fused multiply-add rounded toward minus infinity (times
+// 1 + 2^-23: with its last mantissa bit clear, a c off the grid moves by less than its distance to the next grid point and one on the
+// grid leaves it, so that a negative c floors likewise; the +1 is added to the register's starting value),
 // and the block's value S * u leaves by one exact subtraction of 1.5 * 2^23 * u; rho is a mask (RZ-E8M13) or a
 // conversion (RNE-FP16).  The accumulator between blocks is the output word itself.
 //
@@ -24,7 +25,7 @@
 // is 2^5 or 2^4 and P is taken over sub-blocks of 16 or 8 terms (see pe_shift below).  P for the 32 x 32 outputs
 // of a warp and one block of 32 is sixteen mma.sync.m16n8k16 on BF16 planes of pe values (a power of two is exact in
 // BF16), instead of sixteen fused add-max instructions per output; P = 0 (every product zero: no exponent) converts
-// to an exponent below every real one.  The division by the base is one high multiply on the bits of P, which leaves
+// to an exponent below every real one.  The fragments come by ldmatrix.  The division by the base is one high multiply on the bits of P, which leaves
 // the result as an FP32 exponent field in place, comparable with the bits of |c| and a mask away from the sum
 // register's starting value.
 //
@@ -34,6 +35,11 @@
 // planes are stored with rows and columns permuted accordingly (the four rows of a thread adjacent, its eight
 // columns contiguous): three 16-byte shared loads feed the 32 fused multiply-adds of one k, which are issued as
 // sixteen packed ones (fma.rm.f32x2: two adjacent columns per instruction).
+//
+// What bounds it: the packed multiply-adds with their loads and moves (2.5 of the 3.97 ms at 4096^3 that the kernel took with every phase
+// on; 1.9 at the nominal rate), then the integer work per output and block (0.95 ms) and the tensor-core pass (0.5 ms); the phases
+// add up, integer and FP32 instructions of one SM partition do not run beside each other at full rate.  4096^3, Hopper E4M3 -> FP32:
+// 4.21 ms -> 3.97 (zeros as tiny numbers, range test left out) -> 3.84 (accumulator by multiply-add, ldmatrix).
 #pragma once
 #include <type_traits>
 #include "mmasim_tfdpa_fast.cuh"
@@ -114,6 +120,11 @@ __device__ __forceinline__ int perm_row(int r) {
     return TH == 4 ? ((r & ~31) | ((r & 7) << 2) | ((r >> 3) & 3)) : ((r & ~63) | ((r & 7) << 3) | ((r >> 3) & 7));
 }
 __device__ __forceinline__ int perm_col(int c) { return (c & ~31) | (((c >> 1) & 3) << 3) | (((c >> 3) & 3) << 1) | (c & 1); }
+
+// four 8 x 8 tiles of 16-bit elements, lane l gives row l % 8 of tile l / 8 (stride 80 bytes: eight rows in eight bank groups)
+__device__ __forceinline__ void ldmatrix4(uint32_t* r, const void* row) {
+    asm("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr(row)) : "memory");
+}
 
 constexpr float TINY = 7.888609052210118e-31f;          // 2^-100: times an element below 2^-83, the smallest unit is 2^-43
 
@@ -291,6 +302,9 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
                 if (d.cls == CLS_NAN) sp_nan |= bit; else if (d.sign) sp_ninf |= bit; else sp_pinf |= bit;
                 w = 0u;
             }
+            // an FP32 accumulator enters with the bits that its own exponent keeps (units of 2^(Exp(c) - F): the first block's are as
+            // coarse or coarser), so that its last mantissa bit is clear; zeros are +0
+            if (!ACC16) w = (w & 0x7FFFFFFFu & RHO_MASK) ? w & RHO_MASK : 0u;
             big = big || fabsf(__uint_as_float(w)) > 1.2676506e30f;         // 2^100
             cw[h][x] = w;
         }
@@ -333,47 +347,38 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
             // ---- pass 1 on the tensor cores: P = sum_k pe(a_k) pe(b_k), one accumulation per sub-block of KSUB terms,
             // the block's P the integer maximum of their words; one accumulator fragment row (16 x 32 outputs of the
             // warp, two rows of the micro-tile) at a time, followed at once by its sum registers ----
-            constexpr int NK = KSUB >= 16 ? KSUB / 16 : 1;                 // matrix instructions per accumulation
-            constexpr int AR = KSUB >= 16 ? 4 : 2, BR = KSUB >= 16 ? 2 : 1;
+            // (fragments by ldmatrix, the columns' kept for all rows: 12 instead of 96 loads per block of 32)
+            constexpr int NK = KSUB >= 16 ? KSUB / 16 : 1, K8 = L / 8;     // matrix instructions per accumulation; tiles of 8 along K
             bool rare = false;
+            uint32_t bf[4 * K8];                                           // [column tile j][k8]
+#pragma unroll
+            for (int q = 0; q < K8; ++q) {
+                const int t = 4 * q + (lane >> 3);
+                ldmatrix4(&bf[4 * q], &sb_blk.pe[wc * 32 + 8 * (t / K8) + (lane & 7)][kb + 8 * (t % K8)]);
+            }
 #pragma unroll
             for (int mt = 0; mt < TH / 2; ++mt) {
-                uint32_t P[4][4];
+                uint32_t P[4][4], af[2 * K8];                              // af: [k8][upper / lower 8 rows]
+#pragma unroll
+                for (int q = 0; q < K8 / 2; ++q)
+                    ldmatrix4(&af[4 * q], &sa_blk.pe[wr * G::WROWS + 16 * mt + (lane & 15)][kb + 8 * (2 * q + (lane >> 4))]);
 #pragma unroll
                 for (int sub = 0; sub < NSUB; ++sub) {
-                    uint32_t af[NK][AR];
-                    const int ar = wr * G::WROWS + 16 * mt + gq;
-#pragma unroll
-                    for (int ks = 0; ks < NK; ++ks) {
-                        const int kq = kb + sub * KSUB + 16 * ks + 2 * tq;
-                        af[ks][0] = *reinterpret_cast<const uint32_t*>(&sa_blk.pe[ar][kq]);
-                        af[ks][1] = *reinterpret_cast<const uint32_t*>(&sa_blk.pe[ar + 8][kq]);
-                        if (AR == 4) {
-                            af[ks][AR - 2] = *reinterpret_cast<const uint32_t*>(&sa_blk.pe[ar][kq + 8]);
-                            af[ks][AR - 1] = *reinterpret_cast<const uint32_t*>(&sa_blk.pe[ar + 8][kq + 8]);
-                        }
-                    }
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        uint32_t bf[NK][BR];
-#pragma unroll
-                        for (int ks = 0; ks < NK; ++ks) {
-                            const int kq = kb + sub * KSUB + 16 * ks + 2 * tq;
-                            bf[ks][0] = *reinterpret_cast<const uint32_t*>(&sb_blk.pe[wc * 32 + 8 * j + gq][kq]);
-                            if (BR == 2) bf[ks][BR - 1] = *reinterpret_cast<const uint32_t*>(&sb_blk.pe[wc * 32 + 8 * j + gq][kq + 8]);
-                        }
                         float d[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                         for (int ks = 0; ks < NK; ++ks) {
-                            if (KSUB >= 16)
+                            const int k8 = (sub * KSUB + 16 * ks) / 8;
+                            if constexpr (KSUB >= 16)
                                 asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                                              : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                                             : "r"(af[ks][0]), "r"(af[ks][1]), "r"(af[ks][AR - 2]), "r"(af[ks][AR - 1]),
-                                               "r"(bf[ks][0]), "r"(bf[ks][BR - 1]));
+                                             : "r"(af[2 * k8]), "r"(af[2 * k8 + 1]), "r"(af[2 * k8 + 2]), "r"(af[2 * k8 + 3]),
+                                               "r"(bf[j * K8 + k8]), "r"(bf[j * K8 + k8 + 1]));
                             else
                                 asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
                                              : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                                             : "r"(af[ks][0]), "r"(af[ks][1]), "r"(bf[ks][0]));
+                                             : "r"(af[2 * k8]), "r"(af[2 * k8 + 1]), "r"(bf[j * K8 + k8]));
                         }
 #pragma unroll
                         for (int i = 0; i < 4; ++i)
@@ -439,8 +444,12 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
                             const uint32_t c = cw[h][2 * xp + q];
                             magic[q] = (e & FIELD) + MAGIC_ADD + (c >> (ACC16 ? 15 : 31));
                             const float cf = ACC16 ? __half2float(__ushort_as_half((unsigned short)c)) : __uint_as_float(c);
-                            cb[q] = __float_as_uint(cf) | 1u;
+                            cb[q] = ACC16 ? __float_as_uint(cf) | 1u : c;
                         }
+                        if (!ACC16)
+                            asm("{\n\t.reg .b64 a, b, r;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tfma.rm.f32x2 r, a, %6, b;\n\tmov.b64 {%0, %1}, r;\n\t}"
+                                : "=r"(cw[h][2 * xp]), "=r"(cw[h][2 * xp + 1]) : "r"(cb[0]), "r"(cb[1]), "r"(magic[0]), "r"(magic[1]), "l"(0x3F8000013F800001ull));
+                        else
                         asm("{\n\t.reg .b64 a, b, r;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tadd.rm.f32x2 r, a, b;\n\tmov.b64 {%0, %1}, r;\n\t}"
                             : "=r"(cw[h][2 * xp]), "=r"(cw[h][2 * xp + 1]) : "r"(cb[0]), "r"(cb[1]), "r"(magic[0]), "r"(magic[1]));
                     }
