@@ -112,7 +112,7 @@ TCGEN05_RATE = {"tf32": 0.5, "fp16": 1.0, "bf16": 1.0, "mxf4": 4.0, "nvf4": 4.0}
 
 def pipe_of(kernel: str, model):
     """(pipe key, pipe instructions per emulated MAC) of the kernel a model dispatches to."""
-    if model.family in ("ST", "GST") or (model.family == "T" and model.F == 25):
+    if model.family in ("st", "gst") or (model.family == "t" and model.F == 25):
         return "tcgen05", 1.0               # the model is the GPU's own matrix instruction
     if kernel == "tfdpa_lut8" and model.F <= 13:
         return "fp32_fma", 1.0
