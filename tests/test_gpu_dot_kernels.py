@@ -10,7 +10,8 @@ pytestmark = pytest.mark.gpu
 gu = pytest.importorskip("gpu_util") if torch.cuda.is_available() else None
 
 KEYS = [("hopper", "e4m3", "fp32"), ("hopper", "e5m2", "fp16"), ("ada", "e4m3", "fp32"), ("ada", "e5m2", "fp16"), ("blackwell", "e4m3", "fp32"),
-        ("blackwell", "e5m2", "fp16"), ("cdna3", "fp16", "fp32"), ("cdna3", "bf16", "fp32"), ("cdna3", "tf32", "fp32")]
+        ("blackwell", "e5m2", "fp16"), ("cdna3", "fp16", "fp32"), ("cdna3", "bf16", "fp32"), ("cdna3", "tf32", "fp32"),
+        ("volta", "fp16", "fp32"), ("hopper", "fp16", "fp32"), ("hopper", "fp16", "fp16"), ("ampere", "bf16", "fp32"), ("hopper", "tf32", "fp32")]
 
 
 @pytest.mark.parametrize("key", KEYS, ids=lambda k: "-".join(k))
