@@ -534,6 +534,7 @@ cudaError_t launch_ftz(const GemmArgs& g, cudaStream_t st) {
 bool dot_stream_supported(const DevModel& m, const GemmArgs& g) {
     if (!g.dot_mode || m.fmt_a != m.fmt_b) return false;
     const int bytes = fmt_desc(m.fmt_a).storage_bits / 8;
+    if (g.K > 0x7FFFFFFFll / bytes) return false;                   // offsets inside a row are 32-bit
     if (m.family == FAM_T && (m.fmt_a == EF_E4M3 || m.fmt_a == EF_E5M2)) {
         const int L = int(g.K < m.L ? g.K : m.L);
         if (L != 4 && L != 8 && L != 16 && L != 32) return false;

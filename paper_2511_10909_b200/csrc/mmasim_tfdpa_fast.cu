@@ -96,7 +96,12 @@ DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us) {
     const int kind = kind_of(m);
     if (!kind || g.dot_mode || m.literal_emax) return DIRECT_NONE;
     if ((kind == KIND_TR || kind == KIND_E) && g.k_chunk) return DIRECT_NONE;
-    if (g.M > 65535ll * 8 || g.N > 0x7FFFFFFFll - 128 || g.K > 0x7FFFFFFFll - 256) return DIRECT_NONE;     // grid.y, 32-bit k
+    if (g.M > 65535ll * 8 || g.N > 0x7FFFFFFFll - 128) return DIRECT_NONE;                                 // grid.y, 32-bit columns
+    // The kernels count the bytes left in a row, and the chunks, in 32 bits; TR-FDPA of the wide formats tags exponents with the chunk's
+    // number in 21 bits.
+    const int64_t row = g.K * (fmt_desc(m.fmt_a).storage_bits / 8);
+    const bool tagged = m.family == FAM_TR && (m.fmt_a == EF_BF16 || m.fmt_a == EF_TF32);
+    if (row > 0x7FFFFFFFll - 1024 || (tagged && g.K > (int64_t(1) << 21) * fast::KC - 256)) return DIRECT_NONE;
     constexpr int64_t SMS = 148;
     auto fullest = [&](int bm, int bn) { return double((((g.M + bm - 1) / bm) * ((g.N + bn - 1) / bn) + SMS - 1) / SMS); };
     const bool f13 = kind == 1 + fast::EK_LUT8 && m.F == 13, bits8 = kind == 1 + fast::EK_LUT8;
