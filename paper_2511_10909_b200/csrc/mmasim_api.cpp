@@ -26,6 +26,11 @@ namespace {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+bool ranges_meet(const void* p, size_t p_bytes, const void* q, size_t q_bytes) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p), b = reinterpret_cast<uintptr_t>(q);
+    return p_bytes && q_bytes && a < b + q_bytes && b < a + p_bytes;
+}
+
 // MMASIM_OK if p is device-accessible memory; ERR_INVALID_ARG for plain host memory; ERR_CUDA otherwise.
 int check_device_ptr(const void* p, const char* name) {
     cudaPointerAttributes attr;
@@ -375,6 +380,10 @@ int mmasim_gemm_host(const mmasim_model* model, int64_t M, int64_t N, int64_t K,
     const bool large_tiles = fast_tfdpa_supported(model->dev, g) && !umma_supported(model->dev, g) && direct_size(model->dev, g) == DIRECT_NONE;
     int panels = int((a_bytes + c_bytes + d_bytes) / (size_t(3) << 20));
     panels = panels < 1 || M < 512 ? 1 : (panels > HostLane::PANELS ? HostLane::PANELS : panels);
+    // D over an operand that later panels still read: everything goes in before anything comes out.  (C in place is fine: a panel's rows of
+    // D replace its own rows of C.)
+    const bool in_place = g.C == g.D && g.ldc == g.ldd;
+    if (ranges_meet(D, d_bytes, A, a_bytes) || ranges_meet(D, d_bytes, g.sfa, sfa_bytes) || (!in_place && ranges_meet(D, d_bytes, C, c_bytes))) panels = 1;
     int64_t panel_rows = panels > 1 ? ((M + panels - 1) / panels + 127) / 128 * 128 : M;
     if (large_tiles && panels > 1 && panel_rows < 512) panel_rows = 512;
     panels = int((M + panel_rows - 1) / panel_rows);

@@ -1,5 +1,5 @@
 """mmasim_gemm_host in one panel, in several, and with a last panel shorter than the others, from several threads at once and after the
-kept streams were given back, against the same product on device memory."""
+kept streams were given back, and with D over the memory of an operand, against the same product on device memory."""
 import threading
 
 import numpy as np
@@ -35,3 +35,23 @@ def test_panels_and_threads(key, shape):
     mmasim.host_release()
     call(0)
     assert np.array_equal(got[0].view(want.dtype), want)
+
+
+def test_output_over_an_operand():
+    """D in the place of C, one row further, and over the second half of A's rows: the words of the product of what was there before."""
+    from paper_2511_10909_b200 import mmasim
+    key, (M, N, K) = ("hopper", "e4m3", "fp32"), (1024, 1024, 2048)
+    inp = wl.normal_inputs(key[1], key[2], M, N, K, seed=6)
+    want = gu.run_gemm(key, inp)
+    model = mmasim.Model(*key)
+    for shift in (0, 1):
+        buf = np.zeros((M + 1, N), dtype=np.uint32)
+        buf[:M] = inp["C"]
+        got = mmasim.gemm_host(model, inp["A"], inp["B"], buf[:M], out=buf[shift:M + shift])
+        assert np.array_equal(got, want), shift
+    half = M * K // 2
+    flat = np.zeros(half + 4 * M * N, dtype=np.uint8)
+    A = flat[:M * K].reshape(M, K)
+    A[:] = inp["A"]
+    got = mmasim.gemm_host(model, A, inp["B"], inp["C"], out=flat[half:].view(np.uint32).reshape(M, N))
+    assert np.array_equal(got, want)
