@@ -369,6 +369,7 @@ __global__ void __launch_bounds__(Layout<MK, BN>::NTHREADS, 1) umma_kernel(const
                     if (c * LY::SPC + i >= nst) break;
                     ok = ok && warp_wait(bar_full + 8 * s, phase, &gave_up, budget);       // (the stage's columns are free)
                     if (ok) {
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");    // behind the instructions that read them
                         const uint32_t sfl = tmem + quarter + LY::ACCS * BN + s * LY::SF_COLS, sfq = sfl + 4 * SF;
                         uint32_t wl[SF ? 4 * SF : 4], wq[SF ? 4 * SF * LY::NRB : 4];
 #pragma unroll

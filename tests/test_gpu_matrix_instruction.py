@@ -68,6 +68,23 @@ def test_matrix_instruction_against_generic(key):
     assert mmasim.copy_timeouts() == 0
 
 
+@pytest.mark.parametrize("key", [("blackwell", "mxe4m3", "fp32"), ("blackwell", "mxf4", "fp32"), ("blackwell", "nvf4", "fp32")],
+                         ids=lambda k: "-".join(k))
+def test_scale_factors_round_the_ring(key):
+    """Every stage's columns of scale factors are written over many times, by values that differ from block to block: long K, more tiles
+    than SMs."""
+    from paper_2511_10909_b200 import mmasim
+    model = mmasim.Model(*key)
+    for n, (M, N, K) in enumerate([(20, 2400, 8192), (300, 150, 16384), (1500, 2000, 2048)]):
+        v = wl.normal_inputs(key[1], key[2], M, N, K, seed=320 + n)
+        g = wl.rng(321 + n)
+        lo, hi = (40, 72) if key[1] == "nvf4" else (112, 132)
+        for k in ("sfa", "sfb"):
+            v[k] = g.integers(lo, hi, v[k].shape, dtype=np.uint8)
+        _compare(model, v, K, v["C"], (key, (M, N, K)))
+    assert mmasim.copy_timeouts() == 0
+
+
 @pytest.mark.parametrize("key,K", [(("hopper", "fp16", "fp32"), 8), (("blackwell", "e4m3", "fp32"), 16), (("blackwell", "mxe4m3", "fp32"), 16),
                                    (("blackwell", "mxf4", "fp32"), 32), (("blackwell", "nvf4", "fp32"), 32)], ids=str)
 def test_block_shorter_than_the_instruction_and_dequantisation(key, K):
