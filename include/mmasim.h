@@ -38,7 +38,7 @@ typedef enum {
     MMASIM_ERR_SHAPE = 3,       /* M, N, K < 1, K not a multiple of the model's block, bad k_chunk or ld */
     MMASIM_ERR_ALIGN = 4,       /* pointer or leading dimension not aligned as documented */
     MMASIM_ERR_CUDA = 5,        /* a CUDA runtime call failed (message holds the CUDA error string) */
-    MMASIM_ERR_TIMEOUT = 6      /* a bounded device-side wait gave up (mmasim_hw_umma's status word, mmasim_gemm_host, mmasim_copy_timeouts) */
+    MMASIM_ERR_TIMEOUT = 6      /* a bounded device-side wait gave up (mmasim_hw_umma's status word, mmasim_gemm_host, mmasim_deviation_stats, mmasim_copy_timeouts) */
 } mmasim_status;
 
 /* The ten architectures of Section 3.2. */
@@ -244,7 +244,8 @@ int mmasim_reference_fp64(const mmasim_model* model, int64_t M, int64_t N, int64
                           double* ref, void* stream);
 
 /* The whole of it: the model's product, that reference and the statistics of their deviations (from zero) in `stats`, eight doubles in
- * HOST memory.  Works in library memory on `stream` and waits for it. */
+ * HOST memory.  Works in library memory on `stream` and waits for it.  MMASIM_ERR_TIMEOUT, and nothing in `stats`, if a kernel's
+ * bounded wait ran out (the tiles it did not store would count as deviations). */
 int mmasim_deviation_stats(const mmasim_model* model, int64_t M, int64_t N, int64_t K, const void* A, const void* B, const void* C,
                            double* stats, void* stream);
 

@@ -163,8 +163,8 @@ cudaError_t scratch_pool(cudaMemPool_t* out) {
 }
 
 namespace {
-// The streams and events of one mmasim_gemm_host call (mmasim_deviation_stats uses only the memory), and a word of mapped host memory that its kernels count given-up waits in (a copy
-// of the device's counter before and after each call cost 15 us).  Creating them took about 100 us of every call, so up to
+// The streams and events of one mmasim_gemm_host call (mmasim_deviation_stats uses only the memory), and a word of mapped host memory
+// that its kernels count given-up waits in (a copy of the device's counter before and after each call cost 15 us).  Creating them took about 100 us of every call, so up to
 // LANES_KEPT sets per device wait for the next one; a call has its set to itself, and mmasim_host_release destroys those that wait.
 struct HostLane {
     static constexpr int PANELS = 6;        // (with the streams of the copies eight: more would share the hardware's eight queues)
@@ -225,6 +225,13 @@ void give_lane(HostLane& l, bool sound) {
     destroy_lane(l);
 }
 }  // namespace
+
+int given_up_waits(int st, unsigned int count, int device, const char* call) {
+    if (count && device >= 0 && device < MAX_DEVICES) g_host_timeouts[device] += count;
+    if (!count || st != MMASIM_OK) return st;
+    set_error("%s: %u CTAs gave up waiting for a bulk copy and stored nothing", call, count);
+    return MMASIM_ERR_TIMEOUT;
+}
 
 }  // namespace mmasim
 
@@ -475,19 +482,15 @@ int mmasim_gemm_host(const mmasim_model* model, int64_t M, int64_t N, int64_t K,
         const cudaError_t e = cudaStreamSynchronize(lane.in);
         if (err == cudaSuccess) err = e;
     }
+    const int device = lane.device;
     const unsigned int count = err == cudaSuccess ? *static_cast<volatile unsigned int*>(lane.gave_up) : 0u;
-    if (count) g_host_timeouts[lane.device] += count;
     give_lane(lane, sound && err == cudaSuccess);
     if (err != cudaSuccess) {
         cudaGetLastError();
         set_error("mmasim_gemm_host: %s", cudaGetErrorString(err));
         return MMASIM_ERR_CUDA;
     }
-    if (st == MMASIM_OK && count) {
-        set_error("mmasim_gemm_host: %u CTAs gave up waiting for a bulk copy and stored nothing", count);
-        return MMASIM_ERR_TIMEOUT;
-    }
-    return st;
+    return given_up_waits(st, count, device, "mmasim_gemm_host");
 }
 
 int mmasim_int_peak(int kind, int64_t blocks, int64_t iters, void* sink, int32_t* ops_per_round, void* stream) {
@@ -567,6 +570,8 @@ int mmasim_deviation_stats(const mmasim_model* model, int64_t M, int64_t N, int6
     double *dev_stats = reinterpret_cast<double*>(base), *ref = reinterpret_cast<double*>(base + ref_at);
     if (err == cudaSuccess) err = cudaMemsetAsync(dev_stats, 0, 64, s);
     if (err == cudaSuccess) {
+        *lane.gave_up = 0u;
+        g.copy_timeouts = lane.gave_up_dev;
         st = launch_reference_fp64(m.fmt_a, m.acc, M, N, K, A, B, C, ref, s);
         g.D = base + d_at;
         if (st == MMASIM_OK) st = run_gemm(model, g, 0, s);
@@ -576,14 +581,16 @@ int mmasim_deviation_stats(const mmasim_model* model, int64_t M, int64_t N, int6
     if (base) cudaFreeAsync(base, s);
     const cudaError_t e = cudaStreamSynchronize(s);
     if (err == cudaSuccess) err = e;
-    if (err == cudaSuccess && st == MMASIM_OK) std::memcpy(stats, lane.stats, 64);
+    const int device = lane.device;
+    const unsigned int count = err == cudaSuccess ? *static_cast<volatile unsigned int*>(lane.gave_up) : 0u;
+    if (err == cudaSuccess && st == MMASIM_OK && !count) std::memcpy(stats, lane.stats, 64);
     give_lane(lane, err == cudaSuccess);
     if (err != cudaSuccess) {
         cudaGetLastError();
         set_error("mmasim_deviation_stats: %s", cudaGetErrorString(err));
         return MMASIM_ERR_CUDA;
     }
-    return st;
+    return given_up_waits(st, count, device, "mmasim_deviation_stats");
 }
 
 int mmasim_reference_fp64(const mmasim_model* model, int64_t M, int64_t N, int64_t K, const void* A, const void* B, const void* C,

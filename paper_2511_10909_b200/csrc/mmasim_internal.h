@@ -121,6 +121,8 @@ int launch_int_peak(int kind, int64_t blocks, int64_t iters, void* sink, int32_t
 // mmasim_api.cpp
 unsigned int* copy_timeout_counter();          // the current device's counter (a device variable of the library; NULL on failure)
 cudaError_t scratch_pool(cudaMemPool_t* out);   // the library's own memory pool of the current device (created on first use)
+// The status of a call that came to `st` and whose kernels counted `count` given-up waits, which join the device's total.
+int given_up_waits(int st, unsigned int count, int device, const char* call);
 void set_error(const char* fmt, ...);
 void set_kernel_name(const char* name);
 }  // namespace mmasim

@@ -78,3 +78,18 @@ def read_table(name):
             if line:
                 rows.append(line.split())
     return rows
+
+
+def host_program(folder, source):
+    """Compiles C++ source that uses the library's internal header against libmmasim.so; returns a function that runs it with
+    arguments and gives the lines it prints."""
+    import os
+    import subprocess
+    from paper_2511_10909_b200.build import CSRC, build
+    lib = build()
+    src, exe = os.path.join(str(folder), "program.cpp"), os.path.join(str(folder), "program")
+    with open(src, "w") as f:
+        f.write(source)
+    subprocess.run(["g++", "-std=c++17", f"-I{CSRC}", "-I/usr/local/cuda/include", src, "-o", exe, lib,
+                    f"-Wl,-rpath,{os.path.dirname(lib)}"], check=True)
+    return lambda *args: subprocess.run([exe, *map(str, args)], check=True, capture_output=True, text=True).stdout.splitlines()

@@ -1,11 +1,8 @@
 """Where the kernels whose offsets inside a row are 32-bit end: the dispatcher's own predicates, called on the host, at the row lengths
 on both sides of the limit (2 GiB rows; 2^21 chunks for the kernels that tag a chunk's number in 21 bits)."""
-import os
-import subprocess
-
 import pytest
 
-ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+from helpers import host_program
 
 PROGRAM = r"""
 #include <cstdio>
@@ -35,21 +32,10 @@ int main(int argc, char** argv) {       // arch, input type, accumulator type, t
 
 @pytest.fixture(scope="module")
 def ask(tmp_path_factory):
-    from paper_2511_10909_b200.build import build
-    lib = build()
+    run = host_program(tmp_path_factory.mktemp("limits"), PROGRAM)
     from paper_2511_10909_b200 import mmasim
-    d = tmp_path_factory.mktemp("limits")
-    (d / "limits.cpp").write_text(PROGRAM)
-    exe = str(d / "limits")
-    csrc = os.path.join(ROOT, "paper_2511_10909_b200", "csrc")
-    subprocess.run(["g++", "-std=c++17", f"-I{csrc}", "-I/usr/local/cuda/include", str(d / "limits.cpp"), "-o", exe, lib,
-                    f"-Wl,-rpath,{os.path.dirname(lib)}"], check=True)
-
-    def run(key, *K):
-        args = [mmasim.ARCH[key[0]], mmasim.FMT[key[1]], mmasim.ACC[key[2]], *K]
-        text = subprocess.run([exe, *map(str, args)], check=True, capture_output=True, text=True).stdout
-        return [tuple(x == "1" for x in line.split()) for line in text.splitlines()]
-    return run
+    return lambda key, *K: [tuple(x == "1" for x in line.split())
+                            for line in run(mmasim.ARCH[key[0]], mmasim.FMT[key[1]], mmasim.ACC[key[2]], *K)]
 
 
 # bytes per element; the largest K of the small-tile kernels, if it is not that of 2 GiB rows
