@@ -370,7 +370,7 @@ def host_release():
 def _packed(model, A, B, C):
     dev, M, N, K = A.device, A.shape[0], B.shape[0], A.shape[1]
     for t, name, rows, cols, bits in ((A, "A", M, K, model.a_bits), (B, "B", N, K, model.b_bits), (C, "C", M, N, 8 * model.acc_bytes)):
-        if t is not None and _matrix(t, name, rows, cols, bits, dev) != cols:
+        if t is not None and _matrix(t, name, rows, cols, bits, dev) != cols and rows > 1:
             raise MmasimError(3, f"{name} must be a packed {rows} x {cols} matrix")
     return dev, M, N, K
 

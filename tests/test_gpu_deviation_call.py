@@ -23,3 +23,16 @@ def test_one_call_against_three(key):
             # FP64 sums of M N terms in another order: at most M N ulps of the sum of magnitudes
             scale = np.maximum(np.abs(want), [1, want[2], 0, 0, 1, 1, 0, 0])
             assert np.all(np.abs(np.array(got) - want) <= M * N * 2.0 ** -52 * scale), (key, (M, N, K), got, want)
+
+
+def test_operands_that_are_parts_of_larger_ones():
+    """Single rows of wider matrices (contiguous whatever their row stride), and a C of more rows and columns than the product has."""
+    from paper_2511_10909_b200 import accuracy, mmasim
+    key = ("cdna3", "fp16", "fp32")
+    model = mmasim.Model(*key)
+    inp = wl.normal_inputs(key[1], key[2], 40, 48, 64, seed=9)
+    A, B, C = (gu.dev(inp[k]) for k in ("A", "B", "C"))
+    wide = torch.nn.functional.pad(A, (0, 32))
+    assert accuracy.deviation_stats(model, wide[:1, :64], B, C[:1]) == pytest.approx(accuracy.deviation_stats(model, A[:1].clone(), B, C[:1].clone()), rel=1e-9)
+    large = torch.nn.functional.pad(C, (0, 16, 0, 3))
+    assert accuracy.deviation_stats(model, A, B, large) == pytest.approx(accuracy.deviation_stats(model, A, B, C), rel=1e-9)
