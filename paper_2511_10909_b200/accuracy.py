@@ -41,10 +41,15 @@ def deviation_stats(model: mmasim.Model, A, B, C=None, ref=None) -> dict:
     """Run the model and reduce delta = D - D_real: count, mean, mean |delta|, rms, share of negative / positive
     deviations, max |delta|, mean relative error."""
     packed = all(t is None or (t.is_cuda and t.dim() == 2 and t.is_contiguous()) for t in (A, B, C))
+    s = None
     if ref is None and packed and model.b_fmt == model.in_fmt and model.in_fmt in ("fp16", "bf16", "bf16_1k", "tf32", "fp32", "e4m3", "e5m2") \
             and model.acc != "fp64" and A.shape[1] == B.shape[1] and (C is None or C.shape == (A.shape[0], B.shape[0])):
-        s = mmasim.deviation_stats(model, A, B, C)           # one call of the library
-    else:
+        try:
+            s = mmasim.deviation_stats(model, A, B, C)       # one call of the library
+        except mmasim.MmasimError as e:
+            if "out of memory" not in str(e):                # (what torch's allocator keeps is out of the library's reach)
+                raise
+    if s is None:
         if ref is None:
             ref = reference_fp64(model.in_fmt, model.acc, A, B, C)
         s = mmasim.error_stats(model.acc, mmasim.gemm(model, A, B, C), ref).cpu().tolist()

@@ -65,7 +65,7 @@ int check_k(const DevModel& m, int64_t K) {
 }
 
 // `whole`: the product that g is a row panel of, if it is one: its size decides on the tiles (panels run beside each other).
-int run_gemm(const mmasim_model* model, const GemmArgs& g, int flags, cudaStream_t stream, const GemmArgs* whole = nullptr) {
+int dispatch(const mmasim_model* model, const GemmArgs& g, int flags, cudaStream_t stream, const GemmArgs* whole) {
     const DevModel& m = model->dev;
     if (!(flags & MMASIM_GEMM_FORCE_GENERIC) && !m.literal_emax) {
         if (!(flags & MMASIM_GEMM_LARGE_TILES) && umma_supported(m, g)) return launch_umma(m, g, stream);
@@ -77,6 +77,11 @@ int run_gemm(const mmasim_model* model, const GemmArgs& g, int flags, cudaStream
     }
     set_kernel_name("generic");
     return launch_generic(m, g, stream);
+}
+int run_gemm(const mmasim_model* model, const GemmArgs& g, int flags, cudaStream_t stream, const GemmArgs* whole = nullptr) {
+    const int st = dispatch(model, g, flags, stream, whole);
+    if (st == MMASIM_ERR_CUDA) cudaGetLastError();      // (an allocation that failed is this call's error, not the next launch's)
+    return st;
 }
 
 int build_args(const mmasim_model* model, int64_t M, int64_t N, int64_t K, const void* A, const void* B,
@@ -578,6 +583,7 @@ int mmasim_deviation_stats(const mmasim_model* model, int64_t M, int64_t N, int6
         if (st == MMASIM_OK) st = launch_error_stats(m.acc, int64_t(words), g.D, ref, dev_stats, s);
         if (st == MMASIM_OK) err = cudaMemcpyAsync(lane.stats, dev_stats, 64, cudaMemcpyDeviceToHost, s);
     }
+    if (st == MMASIM_ERR_CUDA) cudaGetLastError();
     if (base) cudaFreeAsync(base, s);
     const cudaError_t e = cudaStreamSynchronize(s);
     if (err == cudaSuccess) err = e;
@@ -607,7 +613,9 @@ int mmasim_reference_fp64(const mmasim_model* model, int64_t M, int64_t N, int64
     if ((st = check_device_ptr(B, "B")) != MMASIM_OK) return st;
     if ((st = check_device_ptr(ref, "ref")) != MMASIM_OK) return st;
     if (C && (st = check_device_ptr(C, "C")) != MMASIM_OK) return st;
-    return launch_reference_fp64(m.fmt_a, m.acc, M, N, K, A, B, C, ref, static_cast<cudaStream_t>(stream));
+    st = launch_reference_fp64(m.fmt_a, m.acc, M, N, K, A, B, C, ref, static_cast<cudaStream_t>(stream));
+    if (st == MMASIM_ERR_CUDA) cudaGetLastError();
+    return st;
 }
 
 int mmasim_host_release(void) {

@@ -36,3 +36,23 @@ def test_operands_that_are_parts_of_larger_ones():
     assert accuracy.deviation_stats(model, wide[:1, :64], B, C[:1]) == pytest.approx(accuracy.deviation_stats(model, A[:1].clone(), B, C[:1].clone()), rel=1e-9)
     large = torch.nn.functional.pad(C, (0, 16, 0, 3))
     assert accuracy.deviation_stats(model, A, B, large) == pytest.approx(accuracy.deviation_stats(model, A, B, C), rel=1e-9)
+
+
+def test_separate_calls_where_the_library_gets_no_memory(monkeypatch):
+    """What torch's allocator keeps for itself serves the separate calls; other errors come through."""
+    from paper_2511_10909_b200 import accuracy, mmasim
+    key = ("hopper", "e4m3", "fp32")
+    model = mmasim.Model(*key)
+    inp = wl.normal_inputs(key[1], key[2], 40, 48, 64, seed=10)
+    A, B, C = (gu.dev(inp[k]) for k in ("A", "B", "C"))
+    want = accuracy.deviation_stats(model, A, B, C)
+
+    def fail(message):
+        def call(*args, **kw):
+            raise mmasim.MmasimError(5, message)
+        monkeypatch.setattr(mmasim, "deviation_stats", call)
+    fail("mmasim_deviation_stats: out of memory")
+    assert accuracy.deviation_stats(model, A, B, C) == pytest.approx(want, rel=1e-9)
+    fail("mmasim_deviation_stats: invalid argument")
+    with pytest.raises(mmasim.MmasimError):
+        accuracy.deviation_stats(model, A, B, C)
