@@ -89,7 +89,13 @@ PyObject* gemm(PyObject*, PyObject* const* a, Py_ssize_t n) {
         if (a[4] == Py_None) fresh = at::empty({M, N}, at::TensorOptions().dtype(word(info.acc_bytes)).device(dev));
         else out = tensor(a[4]);
         if ((o.ldd = matrix(out, M, N, info.acc_bytes, dev)) < 0) Py_RETURN_NONE;
-        if (p_gemm_ex(model, M, N, K, A->data_ptr(), B->data_ptr(), C ? C->data_ptr() : nullptr, out->data_ptr(), &o, stream())) Py_RETURN_NONE;
+        const void *a_ptr = A->data_ptr(), *b_ptr = B->data_ptr(), *c_ptr = C ? C->data_ptr() : nullptr;
+        void *d_ptr = out->data_ptr(), *s = stream();
+        int st;
+        Py_BEGIN_ALLOW_THREADS                              // (a launch waits where the stream's queue is full, an allocation too)
+        st = p_gemm_ex(model, M, N, K, a_ptr, b_ptr, c_ptr, d_ptr, &o, s);
+        Py_END_ALLOW_THREADS
+        if (st) Py_RETURN_NONE;
         if (a[4] == Py_None) return THPVariable_Wrap(fresh);
         Py_INCREF(a[4]);
         return a[4];
@@ -115,7 +121,13 @@ PyObject* dot_batch(PyObject*, PyObject* const* a, Py_ssize_t n) {
         if (a[4] == Py_None) fresh = at::empty({dots}, at::TensorOptions().dtype(word(info.acc_bytes)).device(dev));
         else out = tensor(a[4]);
         if (!vector(out, dots, info.acc_bytes, dev)) Py_RETURN_NONE;
-        if (p_dot_batch(model, dots, K, A->data_ptr(), B->data_ptr(), C ? C->data_ptr() : nullptr, out->data_ptr(), stream())) Py_RETURN_NONE;
+        const void *a_ptr = A->data_ptr(), *b_ptr = B->data_ptr(), *c_ptr = C ? C->data_ptr() : nullptr;
+        void *d_ptr = out->data_ptr(), *s = stream();
+        int st;
+        Py_BEGIN_ALLOW_THREADS
+        st = p_dot_batch(model, dots, K, a_ptr, b_ptr, c_ptr, d_ptr, s);
+        Py_END_ALLOW_THREADS
+        if (st) Py_RETURN_NONE;
         if (a[4] == Py_None) return THPVariable_Wrap(fresh);
         Py_INCREF(a[4]);
         return a[4];
