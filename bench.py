@@ -88,8 +88,18 @@ NCU_DRAM_BYTES = {"cfg3": (980664832 + 65643264) + (16788480 + 52632832) + (1678
                   "cfg3_2k": (74762496 + 1387776) + 4204288 + 4204800}
 NCU_ALGORITHMIC_BYTES = {"cfg3": 2 * 4096 * 4096 + 2 * 4 * 4096 * 4096, "cfg3_2k": 2 * 2048 * 2048 + 2 * 4 * 2048 * 2048}
 
-# kernels one library call launches: the tuned fused-summation kernels decode A and B into scratch blocks first
-KERNELS_PER_CALL = {"tfdpa_lut8": 3, "tfdpa_f16": 3, "tfdpa_bf16": 3, "tfdpa_tf32": 3, "trfdpa": 3, "gtrfdpa": 3, "efdpa": 3}
+DECODING = ("tfdpa_lut8", "tfdpa_f16", "tfdpa_bf16", "tfdpa_tf32", "trfdpa", "gtrfdpa", "efdpa")
+
+
+def kernels_per_call(kernel: str, variant: str, model) -> int:
+    """Kernels one library call launches: the large-tile fused-summation kernels decode A and B into scratch blocks first; in front
+    of the matrix instruction FP6 and FP4 codes are packed and the exponents of BF16 and TF32 rows looked at, and behind it the
+    emulation looks for tiles that it has to do (not for FP16, unscaled 8-bit and NVFP4 operands)."""
+    if variant == "matrix_instruction":
+        fmt = model.in_fmt
+        return 1 + (fmt.removeprefix("mx") in ("e2m3", "e3m2", "e2m1")) + 2 * (fmt in ("bf16", "tf32")) + fmt.startswith("mx")
+    return 3 if variant == "large_tiles" and kernel in DECODING else 1
+
 
 SMS = 148
 # The pipe that bounds each kernel: (name, instruction kinds of the issue-rate micro-benchmark that witness its rate,
@@ -110,9 +120,9 @@ PIPES = {
 TCGEN05_RATE = {"tf32": 0.5, "fp16": 1.0, "bf16": 1.0, "mxf4": 4.0, "nvf4": 4.0}
 
 
-def pipe_of(kernel: str, model):
-    """(pipe key, pipe instructions per emulated MAC) of the kernel a model dispatches to."""
-    if model.family in ("st", "gst") or (model.family == "t" and model.F == 25):
+def pipe_of(kernel: str, variant: str, model):
+    """(pipe key, pipe instructions per emulated MAC) of the kernel that ran."""
+    if variant == "matrix_instruction":
         return "tcgen05", 1.0               # the model is the GPU's own matrix instruction
     if kernel == "tfdpa_lut8" and model.F <= 13:
         return "fp32_fma", 1.0
@@ -402,12 +412,12 @@ def run_ours(args):
     for _ in range(max(args.warmup, 3)):
         step()
     torch.cuda.synchronize()
-    kernel_name = mmasim.last_kernel()
+    kernel_name, variant = mmasim.last_kernel(), mmasim.last_variant()
 
     # issue-rate peaks, measured live (independent chains of one instruction kind on every SM, several witnesses and
     # occupancies per pipe, the best counts): the pipe the timed kernel is bound by, and the 3-input integer add that is
     # the unit of the paper-level operation count
-    pipe_key, pipe_ops_per_mac = pipe_of(kernel_name, model)
+    pipe_key, pipe_ops_per_mac = pipe_of(kernel_name, variant, model)
     peaks = measure_pipe_peaks(mmasim, torch, dev, sorted({pipe_key, "int_alu"} - {"tcgen05"})) if not is_dot else {}
 
     # ---- timed region: K steps, device timers, L2 flushed between steps ----
@@ -528,7 +538,7 @@ def run_ours(args):
             for _ in range(2):          # the host generated this model's inputs for seconds: let the clocks come back up
                 mmasim.gemm(mdl, t["A"], t["B"], t["C"], out=out, K=size, **pkw)
             torch.cuda.synchronize()
-            kern = mmasim.last_kernel()
+            kern, var = mmasim.last_kernel(), mmasim.last_variant()
             best, tot = None, 0.0
             for _ in range(3):
                 flush.zero_()
@@ -540,7 +550,7 @@ def run_ours(args):
                 ms = e0.elapsed_time(e1)
                 tot += ms
                 best = ms if best is None else min(best, ms)
-            pp, opm = pipe_of(kern, mdl)
+            pp, opm = pipe_of(kern, var, mdl)
             pm_peaks_needed.add(pp)
             rows.append({"model": "-".join(pk), "kernel": kern, "ms": tot / 3, "ms_best": best,
                          "macs_per_s": float(size) ** 3 / (tot / 3 * 1e-3), "_pipe": pp, "_opm": opm})
@@ -601,7 +611,7 @@ def run_ours(args):
         "dtype": compute_dtype(kernel_name, model), "data": "synthetic",
         "config": {"workload": f"{name}: {desc}", "model": "-".join(key), "M": M, "N": N, "K": K,
                    "l2": "flushed between timed steps (256 MiB write)", "parallelism": f"replicas x{world} (independent batches, no exchange)"},
-        "clocks": clocks, "e2e": e2e, "gpu_launches": args.steps * (1 if pipe_key == "tcgen05" else KERNELS_PER_CALL.get(kernel_name, 1)),
+        "clocks": clocks, "e2e": e2e, "gpu_launches": args.steps * kernels_per_call(kernel_name, variant, model),
         "roofline": roofline,
         "cpu_baseline": {"value": cpu_value, "unit": UNIT, "kind": "oracle", **cpu_info},
         "per_model": per_model, "per_model_size": args.per_model_size if per_model else None, "dot_batch": dot_line,

@@ -275,9 +275,11 @@ int mmasim_deviation_stats(const mmasim_model* model, int64_t M, int64_t N, int6
  *                     multiply-add lanes are counted): whether the FP32 and the integer pipe issue side by side. */
 int mmasim_int_peak(int kind, int64_t blocks, int64_t iters, void* sink, int32_t* ops_per_round, void* stream);
 
-/* Whose arithmetic the last mmasim_gemm* call on this thread ran: the kernel family ("tfdpa_f16", "gstfdpa", ...; the same name for
- * its large-tile, small-tile and matrix-instruction kernels), or "generic". */
+/* Whose arithmetic the last mmasim_gemm* call on this thread ran: the kernel family ("tfdpa_f16", "gstfdpa", ...), or "generic"; and
+ * which of its kernels: "matrix_instruction" (tcgen05.mma, with the emulation behind it where the two can part), "large_tiles",
+ * "small_tiles", "streaming" (mmasim_dot_batch) or "generic". */
 const char* mmasim_last_kernel(void);
+const char* mmasim_last_variant(void);
 
 /* The tuned fused-summation kernels bring decoded operand blocks into shared memory with bulk copies and wait for each
  * with a bounded number of polls.  A CTA whose wait runs out (never in a healthy run) stores none of its outputs and

@@ -12,7 +12,7 @@
 namespace mmasim {
 
 static thread_local char g_error[512] = "";
-static thread_local char g_kernel[64] = "";
+static thread_local const char *g_kernel = "", *g_variant = "";     // (string literals)
 
 void set_error(const char* fmt, ...) {
     va_list ap;
@@ -20,7 +20,7 @@ void set_error(const char* fmt, ...) {
     vsnprintf(g_error, sizeof(g_error), fmt, ap);
     va_end(ap);
 }
-void set_kernel_name(const char* name) { snprintf(g_kernel, sizeof(g_kernel), "%s", name); }
+void set_kernel_name(const char* name, const char* variant) { g_kernel = name; g_variant = variant; }
 
 namespace {
 
@@ -75,7 +75,7 @@ int dispatch(const mmasim_model* model, const GemmArgs& g, int flags, cudaStream
         if (fast_fp_supported(m, g)) return launch_fast_fp(m, g, stream);
         if (fast_gst_supported(m, g)) return launch_fast_gst(m, g, stream);
     }
-    set_kernel_name("generic");
+    set_kernel_name("generic", "generic");
     return launch_generic(m, g, stream);
 }
 int run_gemm(const mmasim_model* model, const GemmArgs& g, int flags, cudaStream_t stream, const GemmArgs* whole = nullptr) {
@@ -368,7 +368,7 @@ int mmasim_dot_batch(const mmasim_model* model, int64_t n, int64_t K, const void
     g.ldc = g.ldd = 1;
     g.dot_mode = 1;
     if (!m.literal_emax && dot_stream_supported(m, g)) return launch_dot_stream(m, g, static_cast<cudaStream_t>(stream));
-    set_kernel_name("generic_dot");
+    set_kernel_name("generic_dot", "generic");
     return launch_generic(m, g, static_cast<cudaStream_t>(stream));
 }
 
@@ -647,6 +647,7 @@ int mmasim_host_release(void) {
 }
 
 const char* mmasim_last_kernel(void) { return g_kernel; }
+const char* mmasim_last_variant(void) { return g_variant; }
 
 int mmasim_copy_timeouts(uint64_t* count) {
     if (!count) { set_error("count is NULL"); return MMASIM_ERR_INVALID_ARG; }

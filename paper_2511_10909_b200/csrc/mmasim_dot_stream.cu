@@ -566,19 +566,19 @@ int launch_dot_stream(const DevModel& m, const GemmArgs& g, cudaStream_t stream)
     cudaError_t err = cudaErrorInvalidValue;
     const int L = int(g.K < m.L ? g.K : m.L);
     if (m.family == FAM_TR) {
-        set_kernel_name("dot_trfdpa");
+        set_kernel_name("dot_trfdpa", "streaming");
         if (m.fmt_a == EF_F16) err = L == 4 ? launch_tr<EK_F16, 4>(g, stream) : launch_tr<EK_F16, 8>(g, stream);
         else if (m.fmt_a == EF_BF16) err = L == 4 ? launch_tr<EK_BF16, 4>(g, stream) : launch_tr<EK_BF16, 8>(g, stream);
         else err = L == 4 ? launch_tr<EK_TF32, 4>(g, stream) : launch_tr<EK_TF32, 8>(g, stream);
     } else if (m.family == FAM_T) {
-        set_kernel_name("dot_tfdpa");
+        set_kernel_name("dot_tfdpa", "streaming");
         if (m.fmt_a == EF_E4M3) err = launch_8<false>(m, g, L, stream);
         else if (m.fmt_a == EF_E5M2) err = launch_8<true>(m, g, L, stream);
         else if (m.fmt_a == EF_F16) err = launch_t_l<EK_F16>(m, g, L, stream);
         else if (m.fmt_a == EF_BF16) err = launch_t_l<EK_BF16>(m, g, L, stream);
         else err = launch_t_l<EK_TF32>(m, g, L, stream);
     } else {
-        set_kernel_name("dot_ftz");
+        set_kernel_name("dot_ftz", "streaming");
         if (m.fmt_a == EF_F16) err = launch_ftz<EK_F16, 4>(g, stream);
         else if (m.P == 4) err = launch_ftz<EK_BF16, 4>(g, stream);
         else err = launch_ftz<EK_BF16, 2>(g, stream);

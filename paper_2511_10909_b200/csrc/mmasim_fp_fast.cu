@@ -336,7 +336,9 @@ cudaError_t launch_fma64_tile(const GemmArgs& g, cudaStream_t stream) {
     return cudaGetLastError();
 }
 cudaError_t launch_fma64_mma(const GemmArgs& g, cudaStream_t stream) {
-    return use_small(g, 128, 64, 32, 32, 1.15) ? launch_fma64_tile<2, 2, 2, 2>(g, stream) : launch_fma64_tile<4, 2, 4, 4>(g, stream);
+    const bool small = use_small(g, 128, 64, 32, 32, 1.15);
+    set_kernel_name("fma_f64", small ? "small_tiles" : "large_tiles");
+    return small ? launch_fma64_tile<2, 2, 2, 2>(g, stream) : launch_fma64_tile<4, 2, 4, 4>(g, stream);
 }
 
 template <int MODE, int P, int TM, int TN, int KC>
@@ -351,7 +353,9 @@ cudaError_t launch_fp_tile(const GemmArgs& g, cudaStream_t stream) {
 template <int MODE, int P>
 cudaError_t launch_fp(const GemmArgs& g, cudaStream_t stream) {
     using T = ModeTraits<MODE>;
-    if (use_small(g, 16 * T::TM, 16 * T::TN, 32, 64, MODE == FP_FMA32 ? 2.1 : 1.6)) return launch_fp_tile<MODE, P, 2, 4, 32>(g, stream);
+    const bool small = use_small(g, 16 * T::TM, 16 * T::TN, 32, 64, MODE == FP_FMA32 ? 2.1 : 1.6);
+    set_kernel_name(MODE == FP_FMA32 ? "fma_f32" : "ftz_addmul", small ? "small_tiles" : "large_tiles");
+    if (small) return launch_fp_tile<MODE, P, 2, 4, 32>(g, stream);
     return launch_fp_tile<MODE, P, T::TM, T::TN, 16>(g, stream);
 }
 
@@ -367,16 +371,12 @@ bool fast_fp_supported(const DevModel& m, const GemmArgs& g) {
 int launch_fast_fp(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
     cudaError_t err;
     if (m.family == FAM_FMA) {
-        set_kernel_name(m.acc == ACC_F64 ? "fma_f64" : "fma_f32");
         err = m.acc == ACC_F64 ? launch_fma64_mma(g, stream) : launch_fp<FP_FMA32, 2>(g, stream);
     } else {
-        set_kernel_name("ftz_addmul");
         if (m.fmt_a == EF_F16) err = launch_fp<FP_FTZ_F16, 4>(g, stream);
         else if (m.P == 4) err = launch_fp<FP_FTZ_BF16, 4>(g, stream);
         else err = launch_fp<FP_FTZ_BF16, 2>(g, stream);
     }
-    const int bytes = fmt_desc(m.fmt_a).storage_bits / 8;
-    if ((g.lda * bytes) % 16 || (g.ldb * bytes) % 16) set_kernel_name("generic");       // the any-shape route: rows at any address
     if (err != cudaSuccess) {
         set_error("floating-point kernel launch failed: %s", cudaGetErrorString(err));
         return MMASIM_ERR_CUDA;

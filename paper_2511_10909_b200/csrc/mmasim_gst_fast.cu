@@ -292,7 +292,7 @@ bool fast_gst_supported(const DevModel& m, const GemmArgs& g) {
 }
 
 int launch_fast_gst(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
-    set_kernel_name("gstfdpa");
+    set_kernel_name("gstfdpa", "large_tiles");
     const size_t sh = sizeof(Smem);
     dim3 grid((unsigned)((g.N + BN - 1) / BN), (unsigned)((g.M + BM - 1) / BM), 1);
     cudaError_t err;

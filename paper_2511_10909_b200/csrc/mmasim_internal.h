@@ -124,5 +124,5 @@ cudaError_t scratch_pool(cudaMemPool_t* out);   // the library's own memory pool
 // The status of a call that came to `st` and whose kernels counted `count` given-up waits, which join the device's total.
 int given_up_waits(int st, unsigned int count, int device, const char* call);
 void set_error(const char* fmt, ...);
-void set_kernel_name(const char* name);
+void set_kernel_name(const char* name, const char* variant);   // mmasim_last_kernel, mmasim_last_variant
 }  // namespace mmasim

@@ -79,13 +79,6 @@ bool fast_tfdpa_supported(const DevModel& m, const GemmArgs& g) {
     return true;
 }
 
-namespace {
-bool rows16(const DevModel& m, const GemmArgs& g) {                          // every row starts on a 16-byte boundary
-    const int bytes = fmt_desc(m.fmt_a).storage_bits / 8;
-    return (g.lda * bytes) % 16 == 0 && (g.ldb * bytes) % 16 == 0;
-}
-}  // namespace
-
 // Small tiles, or the large kernel?  What an SM does per chunk of 32 elements of K decides: CTAs on the fullest SM times the time
 // of one, plus the latency of a chunk when there are few.  In units of a 16 x 16 tile's chunk (about 0.45 us), measured on one to
 // eighteen CTAs per SM at K = 1024 and 256: 8 x 16 tiles 0.6, 32 x 32 tiles `mid`, tiles of the large kernel `large` (two to an SM;
@@ -124,19 +117,18 @@ int launch_direct(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStr
     cudaError_t err = cudaErrorInvalidValue;
     const int kind = kind_of(m);
     if (kind == KIND_TR) {
-        set_kernel_name(m.family == FAM_GTR ? "gtrfdpa" : "trfdpa");
+        set_kernel_name(m.family == FAM_GTR ? "gtrfdpa" : "trfdpa", "small_tiles");
         err = direct::launch_tr(m, g, size, stream);
     } else if (kind == KIND_E) {
-        set_kernel_name("efdpa");
+        set_kernel_name("efdpa", "small_tiles");
         err = direct::launch_e(m, g, size, stream);
     } else switch (kind - 1) {
-        case fast::EK_LUT8: set_kernel_name("tfdpa_lut8"); err = direct::launch_lut8(m, g, size, stream); break;
-        case fast::EK_F16: set_kernel_name("tfdpa_f16"); err = direct::launch_f16(m, g, size, stream); break;
-        case fast::EK_BF16: set_kernel_name("tfdpa_bf16"); err = direct::launch_bf16(m, g, size, stream); break;
-        case fast::EK_TF32: set_kernel_name("tfdpa_tf32"); err = direct::launch_tf32(m, g, size, stream); break;
+        case fast::EK_LUT8: set_kernel_name("tfdpa_lut8", "small_tiles"); err = direct::launch_lut8(m, g, size, stream); break;
+        case fast::EK_F16: set_kernel_name("tfdpa_f16", "small_tiles"); err = direct::launch_f16(m, g, size, stream); break;
+        case fast::EK_BF16: set_kernel_name("tfdpa_bf16", "small_tiles"); err = direct::launch_bf16(m, g, size, stream); break;
+        case fast::EK_TF32: set_kernel_name("tfdpa_tf32", "small_tiles"); err = direct::launch_tf32(m, g, size, stream); break;
         default: break;
     }
-    if (!rows16(m, g)) set_kernel_name("generic");      // the any-shape route: rows at any address
     if (err != cudaSuccess) {
         set_error("small-tile FDPA kernel launch failed: %s", cudaGetErrorString(err));
         return MMASIM_ERR_CUDA;
@@ -175,7 +167,7 @@ int launch_gemm_noalloc(const DevModel& m, const GemmArgs& g, cudaStream_t strea
                   "(about (ceil(M/128) + ceil(N/128)) * K/32 * 27 KiB); use mmasim_gemm_ex", need, cap);
         return MMASIM_ERR_SHAPE;
     }
-    set_kernel_name("tfdpa_lut8_noalloc");
+    set_kernel_name("tfdpa_lut8_noalloc", "large_tiles");
     const cudaError_t err = fast::launch_noalloc(m, g, stream);
     if (err != cudaSuccess) {
         set_error("mmasim_gemm_noalloc: %s", cudaGetErrorString(err));
@@ -187,16 +179,16 @@ int launch_gemm_noalloc(const DevModel& m, const GemmArgs& g, cudaStream_t strea
 int launch_fast_tfdpa(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
     cudaError_t err = cudaErrorInvalidValue;
     if (kind_of(m) == KIND_TR) {
-        set_kernel_name(m.family == FAM_GTR ? "gtrfdpa" : "trfdpa");
+        set_kernel_name(m.family == FAM_GTR ? "gtrfdpa" : "trfdpa", "large_tiles");
         err = fast::launch_tr(m, g, stream);
     } else if (kind_of(m) == KIND_E) {
-        set_kernel_name("efdpa");
+        set_kernel_name("efdpa", "large_tiles");
         err = fast::launch_e(m, g, stream);
     } else switch (kind_of(m) - 1) {
-        case fast::EK_LUT8: set_kernel_name("tfdpa_lut8"); err = fast::launch_lut8(m, g, stream); break;
-        case fast::EK_F16: set_kernel_name("tfdpa_f16"); err = fast::launch_f16(m, g, stream); break;
-        case fast::EK_BF16: set_kernel_name("tfdpa_bf16"); err = fast::launch_bf16(m, g, stream); break;
-        case fast::EK_TF32: set_kernel_name("tfdpa_tf32"); err = fast::launch_tf32(m, g, stream); break;
+        case fast::EK_LUT8: set_kernel_name("tfdpa_lut8", "large_tiles"); err = fast::launch_lut8(m, g, stream); break;
+        case fast::EK_F16: set_kernel_name("tfdpa_f16", "large_tiles"); err = fast::launch_f16(m, g, stream); break;
+        case fast::EK_BF16: set_kernel_name("tfdpa_bf16", "large_tiles"); err = fast::launch_bf16(m, g, stream); break;
+        case fast::EK_TF32: set_kernel_name("tfdpa_tf32", "large_tiles"); err = fast::launch_tf32(m, g, stream); break;
         default: break;
     }
     if (err != cudaSuccess) {

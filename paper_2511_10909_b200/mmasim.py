@@ -86,6 +86,7 @@ def _load():
     lib.mmasim_host_release.restype = c_int
     lib.mmasim_host_release.argtypes = []
     lib.mmasim_last_kernel.restype = c_char_p
+    lib.mmasim_last_variant.restype = c_char_p
     lib.mmasim_last_error.restype = c_char_p
     return lib
 
@@ -122,7 +123,13 @@ def _check(status: int):
 
 
 def last_kernel() -> str:
+    """The kernel family whose arithmetic the last call of this thread ran, or "generic"."""
     return _lib.mmasim_last_kernel().decode()
+
+
+def last_variant() -> str:
+    """Which of the family's kernels it was: "matrix_instruction", "large_tiles", "small_tiles", "streaming" or "generic"."""
+    return _lib.mmasim_last_variant().decode()
 
 
 class Model:

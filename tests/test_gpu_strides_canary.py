@@ -3,9 +3,9 @@
 Every matrix sits inside a larger buffer filled with sentinel words: A, B (packed FP4 included), the scale-factor
 matrices and C are surrounded by words that would poison the result if a kernel consumed them (NaN patterns where the
 format has one), and D by canary words that must be intact afterwards.  Shapes are ragged against every tile size
-(128 x 128, 128 x 64, 64 x 128, 16 x 16).  Row strides come in two kinds: a multiple of 16 bytes, which the tuned
-kernels accept, and an odd one, which only the generic kernels take; ldc differs from ldd.  Every output word is
-compared with the oracle.
+(128 x 128, 128 x 64, 64 x 128, 16 x 16).  Row strides come in two kinds: a multiple of 16 bytes, which every kernel
+accepts, and an odd one, which the small-tile, floating-point and generic kernels take; the generic kernels also run on
+their own.  ldc differs from ldd.  Every output word is compared with the oracle.
 """
 import numpy as np
 import pytest
@@ -46,10 +46,10 @@ def _poison(dtype):
     return np.array(-1).astype(np.int64).astype(dtype)                 # all ones: NaN in every format that has one
 
 
-@pytest.mark.parametrize("aligned", [True, False], ids=["ld16", "ldodd"])
+@pytest.mark.parametrize("aligned,generic", [(True, False), (False, False), (False, True)], ids=["ld16", "ldodd", "ldodd-generic"])
 @pytest.mark.parametrize("shape", SHAPES, ids=lambda s: f"{s[0]}x{s[1]}")
 @pytest.mark.parametrize("key", KEYS, ids=lambda k: "-".join(k))
-def test_padded_strides_and_canaries(key, shape, aligned):
+def test_padded_strides_and_canaries(key, shape, aligned, generic):
     from paper_2511_10909_b200 import mmasim
     M, N = shape
     K = 64
@@ -76,13 +76,16 @@ def test_padded_strides_and_canaries(key, shape, aligned):
         bufSA, vSA = _embed(inp["sfa"], inp["sfa"].shape[1], 64, np.uint8(0xFF))
         bufSB, vSB = _embed(inp["sfb"], inp["sfb"].shape[1], 64, np.uint8(0xFF))
         kw = dict(sfa=vSA, sfb=vSB)
-    D = mmasim.gemm(model, vA, vB, vC, out=vD, K=K, **kw)
+    D = mmasim.gemm(model, vA, vB, vC, out=vD, K=K, force_generic=generic, **kw)
     torch.cuda.synchronize()
     kernel = mmasim.last_kernel()
-    if aligned:
-        assert kernel != "generic", kernel                             # every model of KEYS has a tuned kernel
+    # every model of KEYS has a tuned kernel, and but for the group-scaled ones one that takes rows at any address
+    if generic or (packed and not aligned):
+        assert kernel == mmasim.last_variant() == "generic", kernel
     else:
-        assert kernel == "generic", kernel
+        assert kernel != "generic" and mmasim.last_variant() != "generic", kernel
+    if not aligned:
+        assert mmasim.last_variant() in ("small_tiles", "large_tiles", "generic")
     got = gu.host_words(D)
     want = gu.oracle_samples(key, inp, np.stack(np.meshgrid(np.arange(M), np.arange(N), indexing="ij"), -1).reshape(-1, 2))
     assert np.array_equal(got.astype(np.uint64).reshape(-1), want), (key, shape, kernel)
