@@ -6,7 +6,6 @@
 #include <cstring>
 #include <mutex>
 #include <new>
-#include <vector>
 #include "mmasim_internal.h"
 
 namespace mmasim {
@@ -183,7 +182,8 @@ struct HostLane {
 constexpr int LANES_KEPT = 4;
 std::atomic<unsigned int> g_host_timeouts[MAX_DEVICES];     // what the words of finished calls held
 std::mutex g_lane_mutex;
-std::vector<HostLane> g_lanes[MAX_DEVICES];
+HostLane g_lanes[MAX_DEVICES][LANES_KEPT];       // the first g_lane_count of a device (plain arrays: nothing here may throw)
+int g_lane_count[MAX_DEVICES] = {};
 
 void destroy_lane(HostLane& l) {
     for (int p = 0; p < HostLane::PANELS; ++p) {
@@ -203,7 +203,7 @@ cudaError_t take_lane(HostLane* out) {
     if (dev < 0 || dev >= MAX_DEVICES) return cudaErrorInvalidDevice;
     {
         std::lock_guard<std::mutex> lock(g_lane_mutex);
-        if (!g_lanes[dev].empty()) { *out = g_lanes[dev].back(); g_lanes[dev].pop_back(); return cudaSuccess; }
+        if (g_lane_count[dev]) { *out = g_lanes[dev][--g_lane_count[dev]]; return cudaSuccess; }
     }
     HostLane l;
     l.device = dev;
@@ -225,7 +225,7 @@ void give_lane(HostLane& l, bool sound) {
     if (l.device < 0) return;
     if (sound) {
         std::lock_guard<std::mutex> lock(g_lane_mutex);
-        if (g_lanes[l.device].size() < LANES_KEPT) { g_lanes[l.device].push_back(l); return; }
+        if (g_lane_count[l.device] < LANES_KEPT) { g_lanes[l.device][g_lane_count[l.device]++] = l; return; }
     }
     destroy_lane(l);
 }
@@ -624,9 +624,8 @@ int mmasim_host_release(void) {
         int current = 0;
         const bool known = cudaGetDevice(&current) == cudaSuccess;
         for (int d = 0; d < MAX_DEVICES; ++d) {
-            if (!g_lanes[d].empty()) cudaSetDevice(d);
-            for (HostLane& l : g_lanes[d]) destroy_lane(l);
-            g_lanes[d].clear();
+            if (g_lane_count[d]) cudaSetDevice(d);
+            while (g_lane_count[d]) destroy_lane(g_lanes[d][--g_lane_count[d]]);
         }
         if (known) cudaSetDevice(current);
     }

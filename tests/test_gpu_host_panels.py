@@ -12,6 +12,29 @@ pytestmark = pytest.mark.gpu
 gu = pytest.importorskip("gpu_util") if torch.cuda.is_available() else None
 
 
+def test_more_calls_at_once_than_sets_of_streams_are_kept():
+    """Ten calls at a time, twice, with the kept ones given back in between."""
+    from paper_2511_10909_b200 import mmasim
+    key, (M, N, K) = ("ampere", "fp16", "fp32"), (100, 90, 48)
+    inp = wl.normal_inputs(key[1], key[2], M, N, K, seed=7)
+    want = gu.run_gemm(key, inp)
+    model = mmasim.Model(*key)
+    for _ in range(2):
+        got = [None] * 10
+        gate = threading.Barrier(len(got))
+
+        def call(i):
+            gate.wait()
+            got[i] = mmasim.gemm_host(model, inp["A"], inp["B"], inp["C"])
+        threads = [threading.Thread(target=call, args=(i,)) for i in range(len(got))]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        assert all(np.array_equal(x, want) for x in got)
+        mmasim.host_release()
+
+
 @pytest.mark.parametrize("key,shape", [(("hopper", "e4m3", "fp32"), (2100, 1100, 256)), (("ampere", "bf16", "fp32"), (1500, 1300, 40)),
                                        (("hopper", "fp16", "fp32"), (513, 6000, 64)), (("blackwell", "nvf4", "fp32"), (1700, 1600, 128)),
                                        (("volta", "fp16", "fp16"), (40, 30, 20))], ids=str)
