@@ -24,9 +24,18 @@ def _nvcc() -> str:
     raise RuntimeError("nvcc not found")
 
 
+def built_against() -> str:
+    """What the extension module carries to say which torch it belongs to (its classes have no stable layout)."""
+    from importlib.metadata import version
+    return "torch " + version("torch")
+
+
 def _stale() -> bool:
     if not (os.path.exists(LIB) and os.path.exists(PY_EXT)):
         return True
+    with open(PY_EXT, "rb") as f:
+        if built_against().encode() + b"\0" not in f.read():
+            return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(PY_EXT))
     deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS + ["mmasim_py.cpp"]] + [__file__]
     return any(os.path.getmtime(d) > t for d in deps)
@@ -39,7 +48,7 @@ def _py_ext_cmd() -> list[str]:
     inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"), "/usr/local/cuda/include",
            sysconfig.get_paths()["include"]]
     return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
-            *(f"-I{d}" for d in inc), os.path.join(CSRC, "mmasim_py.cpp"), "-o", PY_EXT, "-L" + os.path.join(root, "lib"),
+            f'-DMMASIM_BUILT_AGAINST="{built_against()}"', *(f"-I{d}" for d in inc), os.path.join(CSRC, "mmasim_py.cpp"), "-o", PY_EXT, "-L" + os.path.join(root, "lib"),
             "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
 
 

@@ -143,4 +143,8 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_mmasim_py", nullptr, -1, methods,
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__mmasim_py() { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__mmasim_py() {
+    PyObject* m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_against", MMASIM_BUILT_AGAINST)) { Py_DECREF(m); return nullptr; }
+    return m;
+}

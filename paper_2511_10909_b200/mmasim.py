@@ -97,18 +97,34 @@ _lib = _load()
 _fast = None
 
 
-def _load_fast():
-    """The extension module, loaded with the first call on tensors (it needs torch's libraries in the process)."""
+class _NoFast:
+    """In the extension module's place: every call is left to the Python code below."""
+
+    @staticmethod
+    def gemm(*args):
+        return None
+
+    dot_batch = gemm
+
+
+def _load_fast(path=os.path.join(_HERE, "_mmasim_py.so")):
+    """The extension module, loaded with the first call on tensors (it needs torch's libraries in the process).  Without it, or with
+    one that belongs to another torch, gemm and dot_batch make the same library calls through ctypes, and a warning says so."""
     global _fast
     import importlib.util
-    import torch  # noqa: F401
-    path = os.path.join(_HERE, "_mmasim_py.so")
-    if not os.path.exists(path):
-        raise ImportError(f"{path} is missing: build it with `python -m paper_2511_10909_b200.build`")
-    spec = importlib.util.spec_from_file_location("_mmasim_py", path)
-    mod = importlib.util.module_from_spec(spec)
-    spec.loader.exec_module(mod)
-    mod.bind(*(ctypes.cast(f, c_void_p).value for f in (_lib.mmasim_gemm_ex, _lib.mmasim_dot_batch, _lib.mmasim_model_info)))
+    import torch
+    try:
+        spec = importlib.util.spec_from_file_location("_mmasim_py", path)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        if mod.built_against != "torch " + torch.__version__:
+            raise ImportError(f"it was built against {mod.built_against}, this is torch {torch.__version__}")
+        mod.bind(*(ctypes.cast(f, c_void_p).value for f in (_lib.mmasim_gemm_ex, _lib.mmasim_dot_batch, _lib.mmasim_model_info)))
+    except (ImportError, OSError, AttributeError) as e:
+        import warnings
+        warnings.warn(f"{path} cannot be used ({e}): every gemm and dot_batch call takes some 12 us longer; build it with "
+                      "`python -m paper_2511_10909_b200.build`", RuntimeWarning, stacklevel=3)
+        mod = _NoFast
     _fast = mod
     return mod
 

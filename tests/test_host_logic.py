@@ -91,6 +91,32 @@ def test_binding_refuses_cpu_tensors(mm):
         mm.gemm(model, torch.zeros((4, 16), dtype=torch.int16), torch.zeros((4, 16), dtype=torch.int16))
 
 
+@pytest.mark.parametrize("state", ["missing", "not a library", "other torch"])
+def test_call_path_without_a_usable_extension_module(mm, monkeypatch, tmp_path, state):
+    """gemm and dot_batch go on through ctypes, with a warning (here as far as CPU tensors go: the refusal of the Python code)."""
+    import torch
+    path = tmp_path / "_mmasim_py.so"
+    if state == "not a library":
+        path.write_bytes(b"nothing")
+    elif state == "other torch":
+        path = os.path.join(os.path.dirname(mm.__file__), "_mmasim_py.so")
+        monkeypatch.setattr(torch, "__version__", "0.0")
+    monkeypatch.setattr(mm, "_fast", None)
+    with pytest.warns(RuntimeWarning, match="build it with"):
+        mm._load_fast(str(path))
+    model = mm.Model("hopper", "fp16", "fp32")
+    for call in (mm.gemm, mm.dot_batch):
+        with pytest.raises(mm.MmasimError):
+            call(model, torch.zeros((4, 16), dtype=torch.int16), torch.zeros((4, 16), dtype=torch.int16))
+
+
+def test_extension_module_of_another_torch_is_stale(mm, monkeypatch):
+    from paper_2511_10909_b200 import build
+    assert not build._stale()
+    monkeypatch.setattr(build, "built_against", lambda: "torch 0.0")
+    assert build._stale()
+
+
 def test_product_never_imports_the_oracle():
     pkg = os.path.join(ROOT, "paper_2511_10909_b200")
     for dirpath, _, files in os.walk(pkg):
