@@ -107,6 +107,7 @@ struct Smem {
     __align__(16) double d[BUF][ROWS][KP];              // rows of A, then rows of B
     __align__(16) uint32_t e[BUF][ROWS][EP];            // exponents of elements 2 p (low half) and 2 p + 1 (high half)
     uint32_t sgn[BUF][ROWS], nz[BUF][ROWS];             // bit k: sign / finite and nonzero
+    uint32_t nan[BUF][ROWS], inf[BUF][ROWS];            // bit k: NaN (ST: all of them under a NaN scale factor) / infinity
     int special[BUF];                                   // n + 1: chunk n holds an infinity or a NaN (ST: or a NaN scale factor)
     int wild[BUF];                                      // n + 1: chunk n holds a nonzero element outside [2^-48, 2^40)
     uint32_t max_exp[BUF][2];                           // (n + 1) << 11 | largest Exp + EB of chunk n's A and B (TR-FDPA, wide formats)
@@ -138,7 +139,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
     // results are tested for the range of normal FP32 numbers only where they can leave it (see mmasim_tfdpa_f64.cuh); the small tiles
     // wait for the chain of a block, not for the integer pipe: a second body of code gained and lost 2 - 6 % from size to size
     constexpr bool TAMEABLE = FAM == FAM_T && !ACC16 && TM * CN >= 4;
-    static_assert(TM * TN <= 16 && KC % L == 0, "sticky flags are 16-bit masks; blocks tile the chunk");
+    static_assert(TM * TN <= 16 && KC % L == 0 && TASK == 8, "sticky flags are 16-bit masks; blocks tile the chunk; a task fills a byte of the masks");
     constexpr int NC = WR * WC, NBLK = KC / L;
     using SM = Smem<EK, BM, BN, NTH, TASK>;
     constexpr int TPR = SM::TPR;
@@ -200,6 +201,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
     };
     auto stage = [&](int n) {                           // decode the thread's own raw words of chunk n into buffer n mod 3
         const int buf = n % BUF;
+        const bool marked = sm.special[buf] != 0;
         uint32_t spec = 0u, wild = 0u, top_a = 0u, top_b = 0u;
 #pragma unroll
         for (int it = 0; it < SM::PER; ++it) {
@@ -231,7 +233,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
                 sc_exp += byte - 127u;
                 sc_nan = byte == 0xFFu;
             }
-            uint32_t x[TASK], sbits = 0u, nbits = 0u, ep[TASK / 2], top = 0u, low = 0xFFFFFFFFu;
+            uint32_t x[TASK], sbits = 0u, nbits = 0u, nans = 0u, infs = 0u, ep[TASK / 2], top = 0u, low = 0xFFFFFFFFu;
             to_fp32<EK, TASK>(w, is_a ? m.fmt_a : m.fmt_b, x);
             const uint32_t off = (E || is_a) ? 0u : OFFSET_BIT;
             const uint32_t min_field = is_a ? min_a : min_b;
@@ -263,6 +265,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
                         v[q] = 0.0;
                         nbits &= ~(1u << q);
                         ep[q / 2] &= (q & 1) ? 0x0000FFFFu : 0xFFFF0000u;
+                        if (mag == 0x7F800000u && !sc_nan) infs |= 1u << q; else nans |= 1u << q;
                         spec = 1u;
                     } else if (WIDE && mag - 1u < 0x007FFFFFu) {
                         const double d = __dmul_rn(__uint2double_rn(mag), __hiloint2double((1023 - 149) << 20, 0));
@@ -290,19 +293,13 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
                 for (int q = 0; q < TASK; q += 2) *reinterpret_cast<double2*>(dp + h * TASK + q) = make_double2(v[q], v[q + 1]);
             }
             if (!E) {
-                if constexpr (TASK == 8) {
-                    *reinterpret_cast<uint4*>(&sm.e[buf][r][h * 4]) = make_uint4(ep[0], ep[1], ep[2], ep[3]);
-                    reinterpret_cast<uint8_t*>(&sm.sgn[buf][r])[h] = uint8_t(sbits);
-                    reinterpret_cast<uint8_t*>(&sm.nz[buf][r])[h] = uint8_t(nbits);
-                } else {                                // two neighbouring threads share a byte of the masks
-                    *reinterpret_cast<uint2*>(&sm.e[buf][r][h * 2]) = make_uint2(ep[0], ep[1]);
-                    const uint32_t both = sbits | nbits << 8;
-                    const uint32_t byte = both | __shfl_down_sync(0xFFFFFFFFu, both, 1) << 4;
-                    if (!(h & 1)) {
-                        reinterpret_cast<uint8_t*>(&sm.sgn[buf][r])[h / 2] = uint8_t(byte);
-                        reinterpret_cast<uint8_t*>(&sm.nz[buf][r])[h / 2] = uint8_t(byte >> 8);
-                    }
-                }
+                *reinterpret_cast<uint4*>(&sm.e[buf][r][h * 4]) = make_uint4(ep[0], ep[1], ep[2], ep[3]);
+                reinterpret_cast<uint8_t*>(&sm.sgn[buf][r])[h] = uint8_t(sbits);
+                reinterpret_cast<uint8_t*>(&sm.nz[buf][r])[h] = uint8_t(nbits);
+            }
+            if (marked || (nans | infs)) {              // (zero until the buffer first holds a special value)
+                reinterpret_cast<uint8_t*>(&sm.nan[buf][r])[h] = uint8_t(nans);
+                reinterpret_cast<uint8_t*>(&sm.inf[buf][r])[h] = uint8_t(infs);
             }
         }
         if (spec) sm.special[buf] = n + 1;
@@ -340,6 +337,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
     };
     // (exponent sum + CB) << 20 becomes the exponent field e_max + 1023 (T), or that of the constant 1.5 * 2^52 * 2^(e_max - F) (TR)
     const int key_add = T ? -(1 << 20) : (1023 + 52 - m.F - CB) << 20;
+    for (int i = threadIdx.x; i < BUF * (BM + BN); i += 32 * (NC + PW)) (&sm.nan[0][0])[i] = (&sm.inf[0][0])[i] = 0u;
     if (threadIdx.x < BUF) { sm.special[threadIdx.x] = sm.wild[threadIdx.x] = 0; sm.max_exp[threadIdx.x][0] = sm.max_exp[threadIdx.x][1] = 0u; }
     __syncthreads();
     if (stager) {
@@ -429,7 +427,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
     uint32_t negm[E ? 1 : TM][E ? 1 : TN];              // bit k: product k of the chunk is negative and nonzero
     uint32_t seen_max = 0u, seen_min = 0xFFFFFFFFu;     // T: twice the high words of the results, and the same minus one
     float seen_top = 0.f;                               // TR, GTR: the largest magnitude
-    bool rare = false;                                  // the chunk holds special values, or products that may reach 2^128
+    bool rare = false;                                  // the chunk holds products that may reach 2^128 (E-FDPA: special values)
     uint32_t slow = 0u;                                 // E: outputs whose block sum needs the exact route
     auto mma = [&](double (&acc)[TM][TN], int ks, int nb, int nkb) {    // four terms per output, each rounded toward minus infinity
 #pragma unroll
@@ -584,7 +582,15 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
             for (int r = 0; r < TM; ++r)
 #pragma unroll
                 for (int c = 0; c < TN; ++c) {
-                    const bool fits = !(CAREFUL && rare) && lo[r][c] == hi[r][c] && __double2hiint(lo[r][c]) == __double2hiint(hi[r][c]);
+                    // the same double (bit for bit): the exact sum; block by block also bounds that round to one word, which leave no other for
+                    // the sum between them (a zero only if both are zero, and no NaN)
+                    bool fits = lo[r][c] == hi[r][c] && __double2hiint(lo[r][c]) == __double2hiint(hi[r][c]);
+                    if (CAREFUL) {
+                        const uint32_t w = __float_as_uint(__double2float_rn(lo[r][c]));
+                        fits = fits || (w == __float_as_uint(__double2float_rn(hi[r][c])) && (w & 0x7FFFFFFFu) - 1u < 0x7F800000u);
+                        if (lo[r][c] == 0.0 && hi[r][c] == 0.0) { lo[r][c] = 0.0; fits = true; }
+                        fits = fits && !((slow >> (r * TN + c)) & 1u);
+                    }
                     if (!fits) slow |= 1u << (r * TN + c);
                     if (!CAREFUL || fits) cw[r][c] = __float_as_uint(__double2float_rn(lo[r][c]));
                 }
@@ -610,10 +616,11 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
     subnormal = __any_sync(0xFFFFFFFFu, subnormal);     // (matrix instructions need the whole warp: what they depend on is voted)
     for (int chunk = 0; chunk < NCH; ++chunk) {
         const int buf = chunk % BUF, next_buf = (chunk + 1) % BUF, k0 = chunk * KC, kc = min(KC, K - k0), nblk = (kc + L - 1) / L;
-        rare = sm.special[buf] == chunk + 1;
+        const bool special = sm.special[buf] == chunk + 1;
+        bool top_reached = false;                       // some product may reach 2^128
         if (TOP) {
             auto top = [&](int x) { const uint32_t v = sm.max_exp[buf][x]; return v >> 11 == uint32_t(chunk + 1) ? int(v & 0x7FFu) : 0; };
-            rare = rare || top(0) + top(1) - CB >= 126;
+            top_reached = top(0) + top(1) - CB >= 126;
         }
         if (!E) {
             uint32_t sb[TN], nb[TN];
@@ -626,6 +633,34 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
                 for (int c = 0; c < TN; ++c) negm[E ? 0 : r][E ? 0 : c] = (sa ^ sb[c]) & na & nb[c];
             }
         }
+        // Special-value events (Section 4.2) of the elements in `bits`, from the masks; the flags are sticky, so that a chunk whose results
+        // stay finite runs like any other (the stand-ins are zeros) and notes them all behind it.  Loops, because they are rare and the
+        // registers are not.  Read and decoded element by element for every output, raw bit patterns took 1000 x 1111 x 1000 7.8 ms
+        // (Ampere FP16; the generic kernel 2.1, this way 0.34).
+        auto note_specials = [&](uint32_t bits) {
+#pragma unroll 1
+            for (int o = 0; o < TM * TN; ++o) {
+                const int a = row_at(o / TN), b = BM + col_at(o % TN);
+                const uint32_t an = sm.nan[buf][a], ai = sm.inf[buf][a], bn = sm.nan[buf][b], bi = sm.inf[buf][b];
+                const uint32_t az = ~(an | ai | sm.nz[buf][a]), bz = ~(bn | bi | sm.nz[buf][b]);
+                const uint32_t bad = an | bn | (ai & bz) | (bi & az), infs = (ai | bi) & ~bad & bits, sign = sm.sgn[buf][a] ^ sm.sgn[buf][b];
+                if (bad & bits) sp_nan |= 1u << o;
+                if (infs & ~sign) sp_pinf |= 1u << o;
+                if (infs & sign) sp_ninf |= 1u << o;
+            }
+        };
+        auto note_overflows = [&](int kb) {             // products of 2^128 and more are infinities (the offset of a B operand does not get one there)
+#pragma unroll 1
+            for (int o = 0; o < TM * TN; ++o) {
+                if (((sp_nan | (sp_pinf & sp_ninf)) >> o) & 1u) continue;       // a NaN already
+#pragma unroll 1
+                for (int k = kb; k < kb + L; ++k) {
+                    const double p = __dmul_rn(sm.d[buf][row_at(o / TN)][k], sm.d[buf][BM + col_at(o % TN)][k]);
+                    if (fabs(p) >= 3.402823669209385e38) { if (p < 0.0) sp_ninf |= 1u << o; else sp_pinf |= 1u << o; }
+                }
+            }
+        };
+        rare = E ? special : top_reached;
         // ---- a whole chunk without special values, promotion or odd accumulators runs through plain blocks; if one of them
         // notes a result outside the normal range, the chunk is done again from the accumulators it began with ----
         bool again = true;
@@ -650,6 +685,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
             for (int blk = 0; blk < NBLK; ++blk)
                 block(blk * L, blk + 1 < NBLK ? buf : next_buf, blk + 1 < NBLK ? blk * L + L : 0, std::integral_constant<int, TAMEABLE ? IN_RANGE : PLAIN>{});
             again = false;
+            if (special) note_specials(0xFFFFFFFFu);
             if (PROMOTE && (until -= KC) == 0) promote();
         } else if (whole) {
             double cs0[E ? 1 : TM][E ? 1 : TN];
@@ -673,37 +709,27 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
                     for (int c = 0; c < TN; ++c) { if (E) cw[E ? r : 0][E ? c : 0] = cw0[E ? r : 0][E ? c : 0]; else cs[E ? 0 : r][E ? 0 : c] = cs0[E ? 0 : r][E ? 0 : c]; }
 #pragma unroll
                 for (int ks = 0; ks < NKS; ++ks) { fetch_fragments(buf, 0, ks); fetch_exponents(buf, 0, ks); }
-            } else if (PROMOTE && (until -= KC) == 0) promote();
+            } else {
+                if (!E && special) note_specials(0xFFFFFFFFu);
+                if (PROMOTE && (until -= KC) == 0) promote();
+            }
         }
         if (again) {
 #pragma unroll 1
             for (int blk = 0; blk < nblk; ++blk) {
                 const int kb = blk * L;
-                if (rare && !E) {                       // special-value events of this block (Section 4.2); flags are sticky
-#pragma unroll 1
-                    for (int r = 0; r < TM; ++r)
-#pragma unroll 1
-                        for (int c = 0; c < TN; ++c) {
-                            const int64_t i = row0 + row_at(r), j = col0 + col_at(c);
-                            if (i >= g.M || j >= g.N) continue;
-                            Special ev;
-                            if (FAM == FAM_ST && (g.sfa[i * g.ld_sfa + chunk] == 0xFFu || g.sfb[j * g.ld_sfb + chunk] == 0xFFu)) ev.nan = true;
-                            for (int kk = k0 + kb; kk < min(k0 + kb + L, K); ++kk) {
-                                const uint32_t x = decode_elem(fa, raw_elem<EK>(g.A, i * g.lda + kk));
-                                const uint32_t y = decode_elem(fb, raw_elem<EK>(g.B, j * g.ldb + kk));
-                                ev.product(x, y);
-                                if (TOP && (dec_cls(x) | dec_cls(y)) == 0u) {
-                                    const int sk = dec_ssig(x) * dec_ssig(y);
-                                    if (product_overflows(sk, dec_exp(x) + dec_exp(y), fa.mbits + fb.mbits)) ev.add_inf(sk < 0);
-                                }
-                            }
-                            const uint32_t bit = 1u << (r * TN + c);
-                            if (ev.nan) sp_nan |= bit;
-                            if (ev.pinf) sp_pinf |= bit;
-                            if (ev.ninf) sp_ninf |= bit;
-                        }
-                }
+                // (before the block: a finite overflow counts if it comes first)
+                if (special && !E) note_specials(L == 32 ? 0xFFFFFFFFu : ((1u << (L % 32)) - 1u) << kb);
+                if (TOP && top_reached) note_overflows(kb);
                 slow = 0u;
+                if (E && rare) {                        // outputs whose block holds a special value
+#pragma unroll 1
+                    for (int o = 0; o < TM * TN; ++o) {
+                        const int a = row_at(o / TN), b = BM + col_at(o % TN);
+                        const uint32_t any = sm.nan[buf][a] | sm.inf[buf][a] | sm.nan[buf][b] | sm.inf[buf][b];
+                        if ((any >> kb) & ((1u << (L % 32)) - 1u)) slow |= 1u << o;
+                    }
+                }
                 block(kb, blk + 1 < nblk ? buf : next_buf, blk + 1 < nblk ? kb + L : 0, std::integral_constant<int, CAREFULLY>{});
                 if (E && slow) {                        // by the book on the raw words
 #pragma unroll
@@ -713,6 +739,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
                             if ((slow >> (r * TN + c)) & 1u) {
                                 const int64_t i = row0 + row_at(r), j = col0 + col_at(c);
                                 uint32_t& w = cw[E ? r : 0][E ? c : 0];
+                                if ((w & 0x7FFFFFFFu) > 0x7F800000u) { w = special_word(1, false, false); continue; }      // a NaN stays one
                                 w = (i < g.M && j < g.N) ? by_the_book<EK>(m, g.A, g.B, i * g.lda + k0 + kb, j * g.ldb + k0 + kb, min(L, kc - kb), w) : 0u;
                             }
                 }

@@ -83,3 +83,36 @@ def test_large_tiles_against_generic(key):
                 want = mmasim.gemm(model, d["A"], d["B"], d["C"], force_generic=True, **kw, **sf)
                 got = mmasim.gemm(model, d["A"], d["B"], d["C"], large_tiles=True, **kw, **sf)
                 assert torch.equal(got, want), (key, (M, N, K), kw, int((got != want).sum()))
+
+
+@pytest.mark.parametrize("key", KEYS, ids=lambda k: "-".join(k))
+def test_special_values_among_others(key):
+    """A few infinities, NaNs, zeros opposite them and huge values (overflow before and after a special value of the same chunk) in whole
+    and partial chunks, and E-FDPA sums that no double holds: from a few rows to all of them."""
+    from paper_2511_10909_b200 import mmasim
+    model = mmasim.Model(*key)
+    unit = 32 if key[1].startswith("mx") else model.l_max
+    for n, (M, N, K, share) in enumerate([(40, 70, 256, 0.001), (100, 130, 160 + unit % 32, 0.004), (500, 600, 96, 0.02)]):
+        g = wl.rng(400 + n)
+        v = wl.normal_inputs(key[1], key[2], M, N, -(-K // 32) * 32, seed=400 + n)
+        for k in ("A", "B"):
+            v[k] = v[k][:, :K].copy()
+            size = v[k].dtype.itemsize
+            width = {"e2m1": 4, "e2m3": 6, "e3m2": 6}.get(key[1].replace("mx", ""), 8) if size == 1 else 8 * size
+            top = ((1 << (width - 1)) - 1) if size < 4 else 0x7FFFE000
+            exps = {"fp16": 0x7C00, "bf16": 0x7F80, "tf32": 0x7F800000}.get(key[1], 0x7C if "e5m2" in key[1] else top)
+            for word in (exps, top, 0, exps - (1 << 13 if size == 4 else 1)):        # infinity (or the largest pattern), NaN, zero, the largest number
+                at = g.random(v[k].shape) < share
+                v[k][at] = (word | (g.integers(0, 2, int(at.sum())) << (width - 1))).astype(v[k].dtype)
+        if model.family == "e":
+            v["C"][::2] = (v["C"][::2] & np.uint32(0x807FFFFF)) | np.uint32(0x08000000)      # far below the products
+        d = {k: gu.dev(x) for k, x in v.items()}
+        sf = {k: d[k] for k in ("sfa", "sfb") if k in d}
+        want = mmasim.gemm(model, d["A"], d["B"], d["C"], force_generic=True, **sf)
+        got = mmasim.gemm(model, d["A"], d["B"], d["C"], **sf)
+        assert torch.equal(got, want), (key, (M, N, K), int((got != want).sum()))
+        if key[2] == "fp32" and model.family in ("t", "st"):
+            for kc in {unit, K} if K % unit == 0 else {K}:
+                want = mmasim.gemm(model, d["A"], d["B"], d["C"], force_generic=True, k_chunk=kc, **sf)
+                got = mmasim.gemm(model, d["A"], d["B"], d["C"], k_chunk=kc, **sf)
+                assert torch.equal(got, want), (key, (M, N, K), kc, int((got != want).sum()))
