@@ -125,3 +125,29 @@ def test_products_below_the_smallest_normal(key):
         near = (g.integers(0, 2, (M, N)) << 31) | (np.clip(centre + 127 + g.integers(-9, 9, (M, N)), 0, 254) << 23) | g.integers(0, 1 << 23, (M, N))
         for C in (None, near.astype(np.uint32), np.where(g.random((M, N)) < 0.5, 0, 0x80000001).astype(np.uint32)):
             _compare(model, v, K, C, (key, centre, C is None))
+
+
+@pytest.mark.parametrize("key", [("blackwell", "mxe4m3", "fp32"), ("blackwell", "mxe5m2", "fp32"), ("blackwell", "mxe3m2", "fp32"),
+                                 ("rtx_blackwell", "mxe2m1", "fp32"), ("blackwell", "mxf4", "fp32")], ids=lambda k: "-".join(k))
+def test_zero_blocks_under_small_scale_factors(key):
+    """Blocks of zeros (of either sign, and with the unused bits of a code set) under the smallest and under arbitrary small factors, beside
+    blocks that are zero but for one element: the first flag nothing, the last do."""
+    from paper_2511_10909_b200 import mmasim
+    model = mmasim.Model(*key)
+    packed = key[1] == "mxf4"
+    per = 16 if packed else 32
+    sign = 0x88 if packed else 1 << (_width(key) - 1)
+    junk = 0 if packed else 0xFF & ~((1 << _width(key)) - 1)
+    for n, (M, N, K) in enumerate([(300, 260, 64), (515, 520, 1024), (130, 2500, 4096)]):
+        g = wl.rng(380 + n)
+        v = wl.normal_inputs(key[1], key[2], M, N, K, seed=380 + n)
+        for k, s in (("A", "sfa"), ("B", "sfb")):
+            blocks = v[k].reshape(v[k].shape[0], -1, per)
+            zero = g.random(blocks.shape[:2]) < 0.1
+            blocks[zero] = g.choice(np.array([0, sign, junk, sign | junk], dtype=np.uint8), (int(zero.sum()), per))
+            v[s] = np.where(zero, np.where(g.random(zero.shape) < 0.5, 0, g.integers(0, 80, zero.shape)), g.integers(112, 132, zero.shape)).astype(np.uint8)
+            if n == 1:                                      # one element among the zeros: the product below 2^-126 counts
+                i, b = np.argwhere(zero)[3]
+                blocks[i, b, per - 1], v[s][i, b] = (0x10 if packed else 1), 0
+        for C in (v["C"], None):
+            _compare(model, v, K, C, (key, (M, N, K), C is None))
