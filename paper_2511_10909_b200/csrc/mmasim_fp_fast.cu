@@ -364,8 +364,17 @@ cudaError_t launch_fp(const GemmArgs& g, cudaStream_t stream) {
 bool fast_fp_supported(const DevModel& m, const GemmArgs& g) {
     if (g.dot_mode || g.k_chunk || g.row_scale) return false;
     if (m.family != FAM_FMA && m.family != FAM_FTZ) return false;
-    if (g.K > 0x7FFF0000ll) return false;
-    return g.M <= 65535ll * 32;
+    if (g.K > 0x7FFF0000ll || g.M > 65535ll * 32) return false;
+    // K off the chunks, or rows off 16 bytes, in FP32: while few CTAs (of 16 x 16 outputs) share an SM the generic kernels are the faster ones;
+    // they have one output per thread and wait for less at a time.  Here / there in us, K = 1000, at 1.1 and 2.4 CTAs per SM and odd
+    // strides: FP32 51 / 35 and 52 / 45, FP16 68 / 56 and 68 / 76, BF16 in pairs 70 / 64 and 70 / 89; on 16 bytes: FP32 43 / 35 and
+    // 43 / 45, FP16 0.4 per SM 47 / 41 and 1.1 48 / 56, BF16 in pairs 47 / 54.  (FP64 is faster here at any size: 25 / 35.)
+    const int bytes = fmt_desc(m.fmt_a).storage_bits / 8;
+    const bool on16 = (g.lda * bytes) % 16 == 0 && (g.ldb * bytes) % 16 == 0;
+    if (m.acc == ACC_F64 || (on16 && g.K % 16 == 0)) return true;
+    const int64_t per_sm = up_div(up_div(g.M, 16) * up_div(g.N, 16), 148);
+    const int generic_up_to = m.family == FAM_FMA ? (on16 ? 2 : 3) : (on16 ? (m.P == 4 ? 1 : 0) : 2);
+    return per_sm > generic_up_to;
 }
 
 int launch_fast_fp(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
