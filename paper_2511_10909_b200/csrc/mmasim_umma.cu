@@ -149,28 +149,36 @@ __device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t* x) {
 }
 
 // The smallest of sixteen E8M0 scale factors (four words, from block `k0` of a row on) by byte position, without those of blocks of zeros:
-// their products have no exponent, and quantisers give such a block the smallest factor there is.  Only the factors below `small` are
-// looked at; two of which neither is that small flag nothing.  (MXFP8 1024 x 4096 x 4096, one block in twenty zero under the
-// smallest factor: 3531 us with every tile flagged, now 140, most of it these looks; 2870 on the emulation alone.)
+// their products have no exponent, and quantisers give such a block the smallest factor there is.  Looked at are only the factors below
+// `small`, which becomes the smallest one that counts: of two that are not below the first `small` neither flags anything, and a row
+// needs its smallest alone.  Eight blocks at a time, their loads in flight together.  (MXFP8 1024 x 4096 x 4096, one block in twenty zero
+// under the smallest factor: 3531 us with every tile flagged, 2870 on the emulation alone.)
 template <int MK>
-__device__ __noinline__ uint32_t without_zero_blocks(const unsigned char* p, int row_bytes, uint32_t magnitude, int k0, uint4 w, uint32_t small) {
+__device__ __noinline__ uint32_t without_zero_blocks(const unsigned char* p, int row_bytes, uint32_t magnitude, int k0, uint4 w, uint32_t& small) {
     constexpr int BYTES = MK == MK_MXF4 ? 16 : 32;
     uint32_t least = 0xFFFFFFFFu;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        uint32_t e = q == 0 ? w.x : (q == 1 ? w.y : (q == 2 ? w.z : w.w));
 #pragma unroll 1
-        for (int b = 0; b < 4; ++b) {
-            if ((e >> (8 * b) & 0xFFu) >= (small & 0xFFu)) continue;
-            const int at = (k0 + 4 * q + b) * BYTES;
-            uint32_t any = 0u;
-            if (at + BYTES <= row_bytes)
-                for (int v = 0; v < BYTES; v += 16) { const uint4 x = *reinterpret_cast<const uint4*>(p + at + v); any |= x.x | x.y | x.z | x.w; }
-            else
-                for (int v = at; v < row_bytes; ++v) any |= p[v];
-            if (!(any & magnitude)) e |= 0xFFu << (8 * b);
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t e[2] = {h ? w.z : w.x, h ? w.w : w.y};
+        uint32_t any[8];
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            const int at = (k0 + 8 * h + b) * BYTES;
+            any[b] = magnitude;
+            if ((e[b / 4] >> (8 * (b % 4)) & 0xFFu) >= small) continue;
+            any[b] = 0u;
+            if (at + BYTES <= row_bytes) {
+#pragma unroll
+                for (int v = 0; v < BYTES; v += 16) { const uint4 x = *reinterpret_cast<const uint4*>(p + at + v); any[b] |= x.x | x.y | x.z | x.w; }
+            } else
+                for (int v = at; v < row_bytes; ++v) any[b] |= p[v];
         }
-        least = __vminu4(least, e);
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            const uint32_t factor = any[b] & magnitude ? e[b / 4] >> (8 * (b % 4)) & 0xFFu : 255u;
+            small = min(small, factor);
+            least = __vminu4(least, factor | 0xFFFFFF00u);
+        }
     }
     return least;
 }
@@ -312,7 +320,6 @@ __global__ void __launch_bounds__(Layout<MK, BN>::NTHREADS, 1) umma_kernel(const
         bool ok = true;
         // a thread's rows, one of the lane side and the others of the column side: 16 bytes of each at a time, tile after tile
         // without a gap (16 bytes are a stage of NVFP4, 0.5 us; two of MXFP4, four of MX8)
-        const uint32_t small = uint32_t(max(0, (-126 - g.least_sf + 1) / 2)) * 0x01010101u;
         auto row_at = [&](int64_t t, int i) -> int64_t { return i == 0 ? t / g.tiles_q * LANES + me : t % g.tiles_q * BN + me + 128 * i - LANES; };
         auto row_of = [&](int64_t t, int i) -> const uint8_t* {
             const int64_t row = row_at(t, i);
@@ -367,9 +374,10 @@ __global__ void __launch_bounds__(Layout<MK, BN>::NTHREADS, 1) umma_kernel(const
         // (a wait that ran out ends the waits and the stores, not the loops: the four warps meet at barriers)
         for (int64_t t = blockIdx.x; t < g.tiles; t += gridDim.x) {
             uint32_t least[PER];
+            uint32_t small[PER];                        // factors below this one are looked at
             bool inside[PER];
 #pragma unroll
-            for (int i = 0; i < PER; ++i) { least[i] = 0xFFFFFFFFu; inside[i] = MK != MK_NVF4 && row_of(t, i); }
+            for (int i = 0; i < PER; ++i) { least[i] = 0xFFFFFFFFu; small[i] = uint32_t(max(0, (-126 - g.least_sf + 1) / 2)); inside[i] = MK != MK_NVF4 && row_of(t, i); }
             for (int c = 0; c < nchunk; ++c) {
                 const uint32_t buf = ring + 16 * slot * LY::SF_ROWS;
                 asm volatile("cp.async.wait_group %0;" :: "n"(LY::SF_RING - 2) : "memory");
@@ -388,9 +396,9 @@ __global__ void __launch_bounds__(Layout<MK, BN>::NTHREADS, 1) umma_kernel(const
                                 w[q] |= over <= 0 ? 0u : (over >= 4 ? 0xFFFFFFFFu : ~(0xFFFFFFFFu >> (8 * over)));
                             }
                             uint32_t m4 = __vminu4(__vminu4(w[0], w[1]), __vminu4(w[2], w[3]));
-                            if (__vcmpltu4(m4, small))
+                            if (__vcmpltu4(m4, small[i] * 0x01010101u))
                                 m4 = without_zero_blocks<MK>(i == 0 ? g.codes_l + row_at(t, i) * g.pitch_l : g.codes_q + row_at(t, i) * g.pitch_q, g.row_bytes,
-                                                             i == 0 ? g.magnitude_l : g.magnitude_q, 16 * c, make_uint4(w[0], w[1], w[2], w[3]), small);
+                                                             i == 0 ? g.magnitude_l : g.magnitude_q, 16 * c, make_uint4(w[0], w[1], w[2], w[3]), small[i]);
                             least[i] = __vminu4(least[i], m4);
                         }
                 }
