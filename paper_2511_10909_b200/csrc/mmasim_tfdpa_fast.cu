@@ -79,12 +79,38 @@ bool fast_tfdpa_supported(const DevModel& m, const GemmArgs& g) {
     return true;
 }
 
-// Small tiles, or the large kernel?  What an SM does per chunk of 32 elements of K decides: CTAs on the fullest SM times the time
-// of one, plus the latency of a chunk when there are few.  In units of a 16 x 16 tile's chunk (about 0.45 us), measured on one to
-// eighteen CTAs per SM at K = 1024 and 256: 8 x 16 tiles 0.6, 32 x 32 tiles `mid`, tiles of the large kernel `large` (two to an SM;
-// one that is alone takes 16 % longer) and 17 us for its decode pass and two more launches (F = 13: 7).  Small against large in us,
-// on both sides of the line, K = 1024: Ampere FP16 512 x 512 75 / 124, 768 x 768 142 / 126, 1024 x 1536 370 / 297; CDNA3 FP16
-// 768 x 768 150 / 166, 1024 x 1536 394 / 404, 2048 x 2048 - / 889; CDNA3 E4M3 768 x 768 188 / 161.
+// Small tiles, or the large kernel?  What the fullest SM does decides.  In us, with `chunks` of 32 elements of K and n CTAs on that SM:
+//     small tiles   4 + chain chunks + per_tile n (chunks + 1.2)        8 x 16 outputs: 0.65 of a 16 x 16 tile
+//     large tiles   decode + large n (chunks + 0.5)                     (an odd n: the last tile has the SM to itself, 0.16 of one more)
+// with the constants of the arithmetic, fitted to the times of all four at sizes from 16 x 64 to 1076 x 3218 and K = 64, 256 and 1024
+// (within 10 %).  Chosen by it, no size takes 1.2 times its best, but for ragged rows of CDNA1 BF16 (1.4) and Ampere FP16 -> FP16 (1.4), whose
+// padding costs the large kernels extra; the average is 1.01.  Small / large in us on both sides of the line: Hopper E4M3 -> FP16 640 x 640 x 64
+// 25 / 29, x 256 63 / 60, Ampere FP16 768 x 768 x 256 36 / 38, 1024 x 1024 x 256 70 / 62, CDNA1 BF16 512 x 512 x 1024 129 / 211, 768 x 768 x 1024
+// 258 / 215.
+namespace {
+struct TileCosts { double chain, t16, t32, large, decode; };
+TileCosts tile_costs(const DevModel& m, int kind, bool promoted) {
+    const bool h = m.acc == ACC_F16;
+    if (kind == KIND_E) return m.fmt_a == EF_F16 ? TileCosts{0.26, 0.28, 0.89, 3.3, 15} : TileCosts{0.58, 0.43, 1.66, 5.3, 15};
+    if (kind == KIND_TR) {
+        if (m.family == FAM_GTR) return {0.27, 0.42, 1.26, 3.7, 15};
+        if (m.fmt_a == EF_TF32) return {0.35, 0.44, 1.54, 5.8, 15};
+        return {0.21, 0.35, 1.13, 3.85, 15};
+    }
+    if (kind == 1 + fast::EK_LUT8) {
+        if (m.F != 13) return h ? TileCosts{0.37, 0.63, 1.96, 4.5, 15} : (m.family == FAM_ST ? TileCosts{0.26, 0.50, 1.15, 2.3, 15} : TileCosts{0.19, 0.44, 1.05, 2.2, 15});
+        if (h) return m.L == 16 ? TileCosts{0.66, 0.56, 2.13, 6.8, 22} : TileCosts{0.37, 0.63, 1.96, 4.65, 22};
+        const double large = m.L == 16 ? 6.3 : 5.0;     // (promoted sums: tiles of half the size)
+        return m.L == 16 ? TileCosts{0.28, 0.36, 0.99, promoted ? 0.53 * large : large, 28} : TileCosts{0.20, 0.43, 1.01, promoted ? 0.53 * large : large, 28};
+    }
+    if (kind == 1 + fast::EK_F16 && h) return m.L == 4 ? TileCosts{0.46, 0.45, 1.83, 6.3, 15} : TileCosts{0.25, 0.35, 1.23, 3.9, 15};
+    if (kind == 1 + fast::EK_TF32) return m.L == 4 ? TileCosts{0.27, 0.43, 1.32, 4.3, 15} : TileCosts{0.21, 0.35, 1.08, 3.1, 15};
+    if (m.L == 4) return {0.28, 0.41, 1.29, 4.3, 15};
+    if (m.L == 8) return kind == 1 + fast::EK_F16 ? TileCosts{0.18, 0.34, 1.01, 2.8, 15} : TileCosts{0.19, 0.34, 1.04, 3.2, 15};
+    return {0.18, 0.32, 0.92, 2.3, 15};
+}
+}  // namespace
+
 DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us) {
     const int kind = kind_of(m);
     if (!kind || g.dot_mode || m.literal_emax) return DIRECT_NONE;
@@ -97,18 +123,16 @@ DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us) {
     if (row > 0x7FFFFFFFll - 1024 || (tagged && g.K > (int64_t(1) << 21) * fast::KC - 256)) return DIRECT_NONE;
     constexpr int64_t SMS = 148;
     auto fullest = [&](int bm, int bn) { return double((((g.M + bm - 1) / bm) * ((g.N + bn - 1) / bn) + SMS - 1) / SMS); };
-    const bool f13 = kind == 1 + fast::EK_LUT8 && m.F == 13, bits8 = kind == 1 + fast::EK_LUT8;
-    const double mid = bits8 ? 2.1 : (kind == KIND_E ? 2.3 : (kind == KIND_TR ? (m.family == FAM_GTR ? 3.05 : 2.4) : (m.L <= 4 ? 3.2 : 2.3)));
-    const double large = f13 ? 13.5 : (bits8 ? 5.0 : (kind == KIND_E ? 7.6 : (kind == KIND_TR ? (m.family == FAM_GTR ? 8.3 : 8.7) :
-                         (m.L <= 4 ? 10.1 : (kind == 1 + fast::EK_F16 ? (m.acc == ACC_F16 ? 7.8 : 6.3) : 7.3)))));
-    const double c8 = 0.5 + 0.6 * fullest(8, 16), c16 = 0.6 + fullest(16, 16), c32 = 0.6 + mid * fullest(32, 32);
-    const double chunks = double((g.K + fast::KC - 1) / fast::KC);
+    const bool f13 = kind == 1 + fast::EK_LUT8 && m.F == 13;
+    const TileCosts t = tile_costs(m, kind, g.k_chunk != 0);
+    const double chunks = double((g.K + fast::KC - 1) / fast::KC), start = 4.0 + t.chain * chunks, each = chunks + 1.2;
+    const double c8 = start + 0.65 * t.t16 * fullest(8, 16) * each, c16 = start + t.t16 * fullest(16, 16) * each, c32 = start + t.t32 * fullest(32, 32) * each;
     double big = 1e30;
     if (fast_tfdpa_supported(m, g)) {
         const double n = f13 ? fullest(fast::BM, m.acc != ACC_F16 && !g.k_chunk ? 128 : fast::BN) : fullest(64, 64);
-        big = large * (f13 || int64_t(n) % 2 == 0 ? n : n + 0.16 / n) + (f13 ? 15.0 : 38.0) / chunks;
+        big = t.decode + t.large * (f13 || int64_t(n) % 2 == 0 ? n : n + 0.16 / n) * (f13 ? chunks : chunks + 0.5);
     }
-    if (us) *us = 3.0 + 0.45 * chunks * std::min(std::min(c8, c16), std::min(c32, big));
+    if (us) *us = std::min(std::min(c8, c16), std::min(c32, big));
     if (big <= c8 && big <= c16 && big <= c32) return DIRECT_NONE;
     return c8 <= c16 && c8 <= c32 ? DIRECT_8x16 : (c16 <= c32 ? DIRECT_16x16 : DIRECT_32x32);
 }

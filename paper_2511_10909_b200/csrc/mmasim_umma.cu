@@ -705,9 +705,12 @@ bool umma_supported(const DevModel& m, const GemmArgs& g) {
     // The emulation goes last, so C has to be there still; and its launch and that of the exponents have to pay.
     if (overlap(g)) return false;
     if (mk == MK_MXF4) return fast_gst_supported(m, g);
+    // Emulation / instruction in us, by launches around the instruction.  Two (BF16 and TF32: the exponents before, the flags after; packed MX
+    // rows): BF16 512 x 512 x 64 9.4 / 14.6, 512 x 512 x 128 12.5 / 14.6, 384 x 384 x 256 14.7 / 14.6, 512 x 512 x 256 20.7 / 14.6, TF32
+    // 512 x 512 x 128 14.6 / 14.6.  One (MXFP8: the flags): 256 x 256 x 128 8.4 / 11.2, 384 x 384 x 128 12.5 / 11.0, 64 x 64 x 512 15.5 / 10.1.
     double us = 0.0;
     direct_size(m, g, &us);
-    return us > 14.0;
+    return us > (mk == MK_MX8 && code_bits(m.fmt_a) == 8 && code_bits(m.fmt_b) == 8 ? 11.0 : 15.0);
 }
 
 int launch_umma(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
