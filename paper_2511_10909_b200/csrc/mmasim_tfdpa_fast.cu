@@ -91,10 +91,10 @@ namespace {
 struct TileCosts { double chain, t16, t32, large, decode; };
 TileCosts tile_costs(const DevModel& m, int kind, bool promoted) {
     const bool h = m.acc == ACC_F16;
-    if (kind == KIND_E) return m.fmt_a == EF_F16 ? TileCosts{0.26, 0.28, 0.89, 3.3, 15} : TileCosts{0.58, 0.43, 1.66, 5.3, 15};
+    if (kind == KIND_E) return m.fmt_a == EF_F16 ? TileCosts{0.26, 0.28, 0.89, 3.3, 15} : TileCosts{0.58, 0.50, 1.55, 5.3, 15};
     if (kind == KIND_TR) {
         if (m.family == FAM_GTR) return {0.27, 0.42, 1.26, 3.7, 15};
-        if (m.fmt_a == EF_TF32) return {0.35, 0.44, 1.54, 5.8, 15};
+        if (m.fmt_a == EF_TF32) return {0.35, 0.46, 1.54, 5.8, 15};
         return {0.21, 0.35, 1.13, 3.85, 15};
     }
     if (kind == 1 + fast::EK_LUT8) {
@@ -103,7 +103,7 @@ TileCosts tile_costs(const DevModel& m, int kind, bool promoted) {
         const double large = m.L == 16 ? 6.3 : 5.0;     // (promoted sums: tiles of half the size)
         return m.L == 16 ? TileCosts{0.28, 0.36, 0.99, promoted ? 0.53 * large : large, 28} : TileCosts{0.20, 0.43, 1.01, promoted ? 0.53 * large : large, 28};
     }
-    if (kind == 1 + fast::EK_F16 && h) return m.L == 4 ? TileCosts{0.46, 0.45, 1.83, 6.3, 15} : TileCosts{0.25, 0.35, 1.23, 3.9, 15};
+    if (kind == 1 + fast::EK_F16 && h) return m.L == 4 ? TileCosts{0.46, 0.45, 1.83, 6.3, 15} : TileCosts{0.25, 0.36, 1.15, 3.75, 15};
     if (kind == 1 + fast::EK_TF32) return m.L == 4 ? TileCosts{0.27, 0.43, 1.32, 4.3, 15} : TileCosts{0.21, 0.35, 1.08, 3.1, 15};
     if (m.L == 4) return {0.28, 0.41, 1.29, 4.3, 15};
     if (m.L == 8) return kind == 1 + fast::EK_F16 ? TileCosts{0.18, 0.34, 1.01, 2.8, 15} : TileCosts{0.19, 0.34, 1.04, 3.2, 15};
