@@ -427,7 +427,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
     uint32_t negm[E ? 1 : TM][E ? 1 : TN];              // bit k: product k of the chunk is negative and nonzero
     uint32_t seen_max = 0u, seen_min = 0xFFFFFFFFu;     // T: twice the high words of the results, and the same minus one
     float seen_top = 0.f;                               // TR, GTR: the largest magnitude
-    bool rare = false;                                  // the chunk holds products that may reach 2^128 (E-FDPA: special values)
+    bool rare = false;                                  // the chunk holds special values, or products that may reach 2^128
     uint32_t slow = 0u;                                 // E: outputs whose block sum needs the exact route
     auto mma = [&](double (&acc)[TM][TN], int ks, int nb, int nkb) {    // four terms per output, each rounded toward minus infinity
 #pragma unroll
@@ -633,10 +633,10 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
                 for (int c = 0; c < TN; ++c) negm[E ? 0 : r][E ? 0 : c] = (sa ^ sb[c]) & na & nb[c];
             }
         }
-        // Special-value events (Section 4.2) of the elements in `bits`, from the masks; the flags are sticky, so that a chunk whose results
-        // stay finite runs like any other (the stand-ins are zeros) and notes them all behind it.  Loops, because they are rare and the
-        // registers are not.  Read and decoded element by element for every output, raw bit patterns took 1000 x 1111 x 1000 7.8 ms
-        // (Ampere FP16; the generic kernel 2.1, this way 0.34).
+        // Special-value events (Section 4.2) of the elements in `bits`, from the masks; the flags are sticky.  A loop, because they are rare
+        // and registers are not: a second call behind the plain blocks made special values cheaper (0.38 ms) and everything else 1 %
+        // dearer.  Read and decoded element by element for every output, raw bit patterns took 1000 x 1111 x 1000 7.8 ms (Ampere FP16;
+        // the generic kernel 2.1, this way 0.78).
         auto note_specials = [&](uint32_t bits) {
 #pragma unroll 1
             for (int o = 0; o < TM * TN; ++o) {
@@ -660,7 +660,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
                 }
             }
         };
-        rare = E ? special : top_reached;
+        rare = special || top_reached;
         // ---- a whole chunk without special values, promotion or odd accumulators runs through plain blocks; if one of them
         // notes a result outside the normal range, the chunk is done again from the accumulators it began with ----
         bool again = true;
@@ -685,7 +685,6 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
             for (int blk = 0; blk < NBLK; ++blk)
                 block(blk * L, blk + 1 < NBLK ? buf : next_buf, blk + 1 < NBLK ? blk * L + L : 0, std::integral_constant<int, TAMEABLE ? IN_RANGE : PLAIN>{});
             again = false;
-            if (special) note_specials(0xFFFFFFFFu);
             if (PROMOTE && (until -= KC) == 0) promote();
         } else if (whole) {
             double cs0[E ? 1 : TM][E ? 1 : TN];
@@ -710,7 +709,6 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
 #pragma unroll
                 for (int ks = 0; ks < NKS; ++ks) { fetch_fragments(buf, 0, ks); fetch_exponents(buf, 0, ks); }
             } else {
-                if (!E && special) note_specials(0xFFFFFFFFu);
                 if (PROMOTE && (until -= KC) == 0) promote();
             }
         }
@@ -722,7 +720,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
                 if (special && !E) note_specials(L == 32 ? 0xFFFFFFFFu : ((1u << (L % 32)) - 1u) << kb);
                 if (TOP && top_reached) note_overflows(kb);
                 slow = 0u;
-                if (E && rare) {                        // outputs whose block holds a special value
+                if (E && special) {                     // outputs whose block holds a special value
 #pragma unroll 1
                     for (int o = 0; o < TM * TN; ++o) {
                         const int a = row_at(o / TN), b = BM + col_at(o % TN);
