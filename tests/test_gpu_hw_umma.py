@@ -60,7 +60,8 @@ def test_blackwell_model_matches_tcgen05(kind, chain):
     hw = _run(kind, A, B, C)
     key = ("blackwell", fa, "fp32")
     model = mmasim.Model(*key, b_fmt=fb)
-    D = gu.host_words(mmasim.gemm(model, gu.dev(A), gu.dev(B), gu.dev(C)))
+    D = gu.host_words(mmasim.gemm(model, gu.dev(A), gu.dev(B), gu.dev(C), large_tiles=True))       # the emulation, not the same instruction
+    assert mmasim.last_variant() != "matrix_instruction"
     bad = np.argwhere(hw != D)
     assert bad.size == 0, (kind, K, len(bad), [(tuple(x), hex(int(hw[tuple(x)])), hex(int(D[tuple(x)]))) for x in bad[:6]])
     if fa == fb:
@@ -145,7 +146,8 @@ def test_block_scaled_models_match_tcgen05(kind, chain, wide):
     hw = gu.host_words(mmasim.hw_umma(kind, gu.dev(A), gu.dev(B), gu.dev(C), sfa=gu.dev(sfa), sfb=gu.dev(sfb), K=K))
     key = ("blackwell", kind, "fp32")
     inp = {"A": A, "B": B, "C": C, "sfa": sfa, "sfb": sfb}
-    D = gu.run_gemm(key, inp, K=K)
+    D = gu.run_gemm(key, inp, K=K, large_tiles=True)
+    assert mmasim.last_variant() != "matrix_instruction"
     bad = np.argwhere(hw != D)
     assert bad.size == 0, (kind, K, wide, len(bad), [(tuple(x), hex(int(hw[tuple(x)])), hex(int(D[tuple(x)]))) for x in bad[:6]])
     pairs = wl.sample_pairs(M, 16, 512, seed=96)
@@ -190,7 +192,8 @@ def test_blackwell_fp16_accumulator_rows_match_tcgen05(kind, chain):
     A, B, C = _tiles16(fa, K, M)
     hw = _run(kind, A, B, C)
     key = ("blackwell", fa, "fp16")
-    D = gu.host_words(mmasim.gemm(mmasim.Model(*key), gu.dev(A), gu.dev(B), gu.dev(C)))
+    D = gu.host_words(mmasim.gemm(mmasim.Model(*key), gu.dev(A), gu.dev(B), gu.dev(C), large_tiles=True))
+    assert mmasim.last_variant() != "matrix_instruction"
     bad = np.argwhere(hw != D)
     assert bad.size == 0, (kind, K, len(bad), [(tuple(x), hex(int(hw[tuple(x)])), hex(int(D[tuple(x)]))) for x in bad[:6]])
     pairs = wl.sample_pairs(M, 16, 768, seed=98)

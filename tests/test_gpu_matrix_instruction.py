@@ -46,13 +46,19 @@ def _variants(key, M, N, K, seed):
     return [inp, wild, small]
 
 
-def _compare(model, v, K, C, what, **kw):
+# kinds with products below 2^-126, which small calls leave to the emulation
+GUARDED = ("bf16", "tf32", "mxe4m3", "mxe5m2", "mxe2m3", "mxe3m2", "mxe2m1")
+
+
+def _compare(model, v, K, C, what, ran=True, **kw):
+    """`ran`: the matrix instruction has to be what computes it."""
     from paper_2511_10909_b200 import mmasim
     d = {k: gu.dev(x) for k, x in v.items()}
     sf = {k: d[k] for k in ("sfa", "sfb") if k in d}
     c = None if C is None else gu.dev(C)
     want = mmasim.gemm(model, d["A"], d["B"], c, K=K, force_generic=True, **kw, **sf)
     got = mmasim.gemm(model, d["A"], d["B"], c, K=K, **kw, **sf)
+    assert not ran or mmasim.last_variant() == "matrix_instruction", (what, mmasim.last_variant())
     assert torch.equal(got, want), (what, int((got != want).sum()))
 
 
@@ -64,8 +70,19 @@ def test_matrix_instruction_against_generic(key):
         K = model.l_max * blocks
         for v in _variants(key, M, N, K, 300 + n):
             for C in (v["C"], None):
-                _compare(model, v, K, C, (key, (M, N, K), C is None))
+                _compare(model, v, K, C, (key, (M, N, K), C is None), ran=key[1] not in GUARDED or M >= 1000)
     assert mmasim.copy_timeouts() == 0
+
+
+@pytest.mark.parametrize("key", [k for k in KEYS if k[1] in GUARDED], ids=lambda k: "-".join(k))
+def test_few_rows_of_kinds_with_small_products(key):
+    """Every width of tile (16 to 256 rows of A) with K long enough that the instruction runs; flags at the edges of such tiles."""
+    from paper_2511_10909_b200 import mmasim
+    model = mmasim.Model(*key)
+    for n, (M, N) in enumerate([(1, 300), (16, 129), (17, 257), (33, 140), (70, 300), (131, 390), (300, 700)]):
+        K = 4096 if M < 100 else 1024
+        for v in _variants(key, M, N, K, 310 + n):
+            _compare(model, v, K, v["C"], (key, (M, N, K)))
 
 
 @pytest.mark.parametrize("key", [("blackwell", "mxe4m3", "fp32"), ("blackwell", "mxf4", "fp32"), ("blackwell", "nvf4", "fp32")],
@@ -95,7 +112,7 @@ def test_block_shorter_than_the_instruction_and_dequantisation(key, K):
     rs, cs = (gu.dev(g.standard_normal(n).astype(np.float32)) for n in (M, N))
     for v in _variants(key, M, N, -(-K // 32) * 32, 330):
         for kw in ({}, dict(row_scale=rs, col_scale=cs)):
-            _compare(model, v, K, v["C"], (key, K, list(kw)), **kw)
+            _compare(model, v, K, v["C"], (key, K, list(kw)), ran=key[1] not in GUARDED + ("mxf4",), **kw)
 
 
 @pytest.mark.parametrize("key", [("hopper", "bf16", "fp32"), ("hopper", "tf32", "fp32"), ("blackwell", "mxe4m3", "fp32"),
@@ -105,7 +122,7 @@ def test_products_below_the_smallest_normal(key):
     """Exponent sums from far below -126 to just above, zero and nonzero accumulators; large enough that the matrix instruction runs."""
     from paper_2511_10909_b200 import mmasim
     model = mmasim.Model(*key)
-    M, N, K = 520, 500, 4 * model.l_max
+    M, N, K = 1100, 1000, 4 * model.l_max
     for n, centre in enumerate((-170, -156, -144, -132, -126, -120, -112, -104, -90)):
         g = wl.rng(350 + n)
         v = {k: x for k, x in wl.normal_inputs(key[1], key[2], M, N, K, seed=n).items()}
@@ -138,7 +155,7 @@ def test_zero_blocks_under_small_scale_factors(key):
     per = 16 if packed else 32
     sign = 0x88 if packed else 1 << (_width(key) - 1)
     junk = 0 if packed else 0xFF & ~((1 << _width(key)) - 1)
-    for n, (M, N, K) in enumerate([(300, 260, 64), (515, 520, 1024), (130, 2500, 4096)]):
+    for n, (M, N, K) in enumerate([(900, 800, 64), (515, 520, 1024), (130, 2500, 4096)]):
         g = wl.rng(380 + n)
         v = wl.normal_inputs(key[1], key[2], M, N, K, seed=380 + n)
         for k, s in (("A", "sfa"), ("B", "sfb")):

@@ -85,6 +85,22 @@ def test_large_tiles_against_generic(key):
                 assert torch.equal(got, want), (key, (M, N, K), kw, int((got != want).sum()))
 
 
+@pytest.mark.parametrize("key", [("blackwell", "mxf4", "fp32"), ("rtx_blackwell", "nvf4", "fp32")], ids=lambda k: "-".join(k))
+def test_group_scaled_rows_against_generic(key):
+    """The kernel that emulates the group-scaled rows, which otherwise only runs behind the matrix instruction (MXFP4) or not at all."""
+    from paper_2511_10909_b200 import mmasim
+    model = mmasim.Model(*key)
+    for n, (M, N, K) in enumerate([(1, 1, 64), (128, 64, 128), (129, 65, 192), (200, 300, 320)]):
+        for v in _inputs(key, M, N, K, 500 + n):
+            d = {k: gu.dev(x) for k, x in v.items()}
+            sf = {k: d[k] for k in ("sfa", "sfb")}
+            for c in (d["C"], None):
+                want = mmasim.gemm(model, d["A"], d["B"], c, K=K, force_generic=True, **sf)
+                got = mmasim.gemm(model, d["A"], d["B"], c, K=K, large_tiles=True, **sf)
+                assert mmasim.last_kernel() == "gstfdpa" and mmasim.last_variant() == "large_tiles"
+                assert torch.equal(got, want), (key, (M, N, K), c is None, int((got != want).sum()))
+
+
 @pytest.mark.parametrize("key", KEYS, ids=lambda k: "-".join(k))
 def test_special_values_among_others(key):
     """A few infinities, NaNs, zeros opposite them and huge values (overflow before and after a special value of the same chunk) in whole
