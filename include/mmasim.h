@@ -169,6 +169,7 @@ int mmasim_dot_batch(const mmasim_model* model, int64_t n, int64_t K,
  * Problems of 512 rows and 6 MiB or more are cut into up to six row panels of D (outputs are independent,
  * Section 3.1 Step 1): B is copied once, then each panel's rows of A and C go in, its kernel runs and its rows of D
  * come back on separate streams, so that with pinned buffers the copies run beside the arithmetic.
+ * D may lie over A, B or C: every operand counts as it was at the call (such a call runs as one panel, but for C in place).
  * With opts->ldd > N only the N words of every row of D are written; the words between rows stay the caller's.
  * Returns MMASIM_ERR_TIMEOUT if a kernel of the call gave up a bounded wait (see mmasim_copy_timeouts): D is then incomplete. */
 int mmasim_gemm_host(const mmasim_model* model, int64_t M, int64_t N, int64_t K,

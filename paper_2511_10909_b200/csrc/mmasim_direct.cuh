@@ -2,7 +2,7 @@
 // launch, no scratch memory, any K, any row stride.
 //
 // When they run.  The large kernels (mmasim_tfdpa_f64.cuh, mmasim_tfdpa_trop.cuh, mmasim_trfdpa_f64.cu, mmasim_efdpa_f64.cu)
-// own 128 x 64 or 128 x 128 outputs per CTA and read operands that a decode pass has laid out.  A matrix with few rows or few
+// own 64 x 64 (F = 13: 128 x 64 or 128 x 128) outputs per CTA and read operands that a decode pass has laid out.  A matrix with few rows or few
 // outputs gives them a handful of CTAs, each of which walks all of K at the full cost of its tile, most of it padding: every
 // output is a serial chain over K (the accumulator is rounded after each block), so nothing but more and smaller tiles makes
 // such a product faster.
@@ -17,7 +17,8 @@
 // What bounds it: the chain of a block - exponent maximum, one FP64 addition, L / 4 dependent matrix instructions (26 cycles
 // each), correction, rho - in one or two warps per scheduler, and the instructions around it.  So the next block's exponents and
 // operand fragments are fetched between this block's matrix instructions, and a chunk runs through blocks without a branch: what
-// needs one (subnormal or overflowing results, an inexact E-FDPA sum) is noted, and the chunk done again block by block.
+// needs one (subnormal or overflowing results, an inexact E-FDPA sum) is noted, and the chunk done again block by block;
+// chunks with infinities or NaNs, of which the staging warps keep masks, go block by block at once.
 // Against the large kernels (Hopper FP16): 16 x 4096 x 4096 1027 -> 112 us, 32 x 64 x 1536 353 -> 25, 128 x 2048 x 2048
 // 337 -> 128, 656 x 256 x 2688 647 -> 165; against the generic kernel: 1000 x 1111 x 1000 (Ampere BF16) 3590 -> 330 us.  Versions
 // on the way, 32 x 64 x 1536: staging by the computing warps 74 us, by warps of their own 45, branches out of the blocks 31;

@@ -16,7 +16,9 @@
 // -floor(|x|) - 1, every other term to floor(|x|), and the number of nonzero sign-differing terms of the block, a
 // population count over per-row / per-column sign and nonzero bit masks, is added back once per block, as an integer
 // added to the bit pattern of acc.  The accumulator operand c gets the same treatment: its double has bit 0 of the
-// mantissa set.  Zero elements (and the stand-ins of infinities and NaNs) are staged as 0: their products vanish.
+// mantissa set.  Zero elements (and the stand-ins of infinities and NaNs) are staged as 2^-900 of their sign, whose products lie far
+// below any q: a positive one adds nothing, a negative one falls short like any other and the sign masks alone count it.  (8-bit
+// elements with the tensor-core maximum: as 0, their products vanish, and masks of nonzero elements say which count.)
 //
 // A term whose value is zero has no exponent and takes no part in e_max: zero elements are staged with the exponent
 // word 0, far below every real exponent sum, and a zero c enters the maximum as 0 as well.
