@@ -82,10 +82,10 @@ def compute_dtype(kernel: str, model) -> str:
 # DRAM bytes per step (the main kernel and the two decode launches before it): dram__bytes_read.sum +
 # dram__bytes_write.sum of a one-pass ncu capture of the same workload at its full size, a STORED CONSTANT, not a figure
 # of this run.  Algorithmic bytes are 168 MB at 4096^3 (operands once, C and D); the rest is the decoded operand blocks
-# (226 MB, larger than the L2) written once and re-read by the tiles of later waves.  The kernels are bound by arithmetic:
-# 1.18 GB in 4.2 ms is 4 % of what the memory could move in that time.
-NCU_DRAM_BYTES = {"cfg3": (980664832 + 65643264) + (16788480 + 52632832) + (16789248 + 49752576),
-                  "cfg3_2k": (74762496 + 1387776) + 4204288 + 4204800}
+# (222 MB, larger than the L2) written once and re-read by the tiles of later waves.  The kernels are bound by arithmetic:
+# 1.16 GB in 3.84 ms is 5 % of what the memory could move in that time.
+NCU_DRAM_BYTES = {"cfg3": (958592768 + 64196608) + (16791552 + 54993920) + (16790528 + 49194752),
+                  "cfg3_2k": (73170688 + 6797824) + 4204288 + 4204800}
 NCU_ALGORITHMIC_BYTES = {"cfg3": 2 * 4096 * 4096 + 2 * 4 * 4096 * 4096, "cfg3_2k": 2 * 2048 * 2048 + 2 * 4 * 2048 * 2048}
 
 DECODING = ("tfdpa_lut8", "tfdpa_f16", "tfdpa_bf16", "tfdpa_tf32", "trfdpa", "gtrfdpa", "efdpa")

@@ -139,8 +139,8 @@ __device__ __forceinline__ void staged_tile(unsigned char* smem, int64_t n, int 
 // adds floor(x / q) for a positive x (the offset is below q and below the distance of x to the next multiple of q) and
 // -floor(|x| / q) - 1 for a negative one, which is never on the grid.  The number of negative nonzero terms, times q, is added back
 // at the end of the block.  (Truncating the magnitude first and copying the sign back took a multiply-add, two additions and a logic
-// operation per term.  It is fewer instructions, but not time that shows: 2^20 Hopper FP16 dots of length 32 30.8 us before, 30.6 to 31.5
-// since, 4.6 TB/s; 2048 Ampere FP16 dots of length 16, a call, 5.4.)
+// operation per term.  Hopper FP16, 2^20 dots of length 32: 32.8 -> 31.4 us in turn on one B200, 30.8 -> 30.6 on another, 4.6 TB/s: the
+// copies bound it; 2048 Ampere FP16 dots of length 16, a call: 5.4.)
 constexpr double OFFSET = 1.0000000000000002220446049250313;          // 1 + 2^-52
 __device__ __forceinline__ double sum_start(int e_grid) { return __hiloint2double(((1023 + 52 + e_grid) << 20) | 0x80000, 0); }
 __device__ __forceinline__ void add_term(double& sum, double x) { sum = __fma_rd(x, OFFSET, sum); }
