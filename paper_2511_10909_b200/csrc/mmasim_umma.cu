@@ -150,11 +150,11 @@ __device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t* x) {
 
 // The smallest of sixteen E8M0 scale factors (four words, from block `k0` of a row on) by byte position, without those of blocks of zeros:
 // their products have no exponent, and quantisers give such a block the smallest factor there is.  Looked at are only the factors below
-// `small`, which becomes the smallest one that counts: of two that are not below the first `small` neither flags anything, and a row
+// `small`, which comes back as the smallest one that counts: of two that are not below the first `small` neither flags anything, and a row
 // needs its smallest alone.  Eight blocks at a time, their loads in flight together.  (MXFP8 1024 x 4096 x 4096, one block in twenty zero
 // under the smallest factor: 3531 us with every tile flagged, 2870 on the emulation alone.)
 template <int MK>
-__device__ __noinline__ uint32_t without_zero_blocks(const unsigned char* p, int row_bytes, uint32_t magnitude, int k0, uint4 w, uint32_t& small) {
+__device__ __noinline__ uint2 without_zero_blocks(const unsigned char* p, int row_bytes, uint32_t magnitude, int k0, uint4 w, uint32_t small) {
     constexpr int BYTES = MK == MK_MXF4 ? 16 : 32;
     uint32_t least = 0xFFFFFFFFu;
 #pragma unroll 1
@@ -180,7 +180,7 @@ __device__ __noinline__ uint32_t without_zero_blocks(const unsigned char* p, int
             least = __vminu4(least, factor | 0xFFFFFF00u);
         }
     }
-    return least;
+    return make_uint2(least, small);
 }
 
 #define MMASIM_R4(x, i) "r"(x[i]), "r"(x[i + 1]), "r"(x[i + 2]), "r"(x[i + 3])
@@ -384,24 +384,6 @@ __global__ void __launch_bounds__(Layout<MK, BN>::NTHREADS, 1) umma_kernel(const
                 asm volatile("bar.sync 1, 128;" ::: "memory");      // everybody's rows have landed, and everybody has left the slot before
                 fetch(slot == 0 ? LY::SF_RING - 1 : slot - 1);
                 slot = slot + 1 == LY::SF_RING ? 0 : slot + 1;
-                if (MK != MK_NVF4) {
-#pragma unroll
-                    for (int i = 0; i < PER; ++i)
-                        if (inside[i]) {
-                            const uint4 v = lds16(buf + 16 * (me + 128 * i));
-                            uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {           // (bytes beyond the row's are not its exponents)
-                                const int over = 16 * c + 4 * q + 4 - g.nsf;
-                                w[q] |= over <= 0 ? 0u : (over >= 4 ? 0xFFFFFFFFu : ~(0xFFFFFFFFu >> (8 * over)));
-                            }
-                            uint32_t m4 = __vminu4(__vminu4(w[0], w[1]), __vminu4(w[2], w[3]));
-                            if (__vcmpltu4(m4, small[i] * 0x01010101u))
-                                m4 = without_zero_blocks<MK>(i == 0 ? g.codes_l + row_at(t, i) * g.pitch_l : g.codes_q + row_at(t, i) * g.pitch_q, g.row_bytes,
-                                                             i == 0 ? g.magnitude_l : g.magnitude_q, 16 * c, make_uint4(w[0], w[1], w[2], w[3]), small[i]);
-                            least[i] = __vminu4(least[i], m4);
-                        }
-                }
                 uint4 x[NR];
 #pragma unroll
                 for (int j = 0; j < NR; ++j) x[j] = lds16(buf + 16 * (32 * j + lane < LY::SF_ROWS ? 32 * j + lane : 0));
@@ -434,6 +416,27 @@ __global__ void __launch_bounds__(Layout<MK, BN>::NTHREADS, 1) umma_kernel(const
                         if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(bar_sf + 8 * s) : "memory");
                     }
                     if (++s == STAGES) { s = 0; phase ^= 1u; }
+                }
+                if (MK != MK_NVF4) {                    // (behind the stores, which the instructions wait for)
+#pragma unroll
+                    for (int i = 0; i < PER; ++i)
+                        if (inside[i]) {
+                            const uint4 v = lds16(buf + 16 * (me + 128 * i));
+                            uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {           // (bytes beyond the row's are not its exponents)
+                                const int over = 16 * c + 4 * q + 4 - g.nsf;
+                                w[q] |= over <= 0 ? 0u : (over >= 4 ? 0xFFFFFFFFu : ~(0xFFFFFFFFu >> (8 * over)));
+                            }
+                            uint32_t m4 = __vminu4(__vminu4(w[0], w[1]), __vminu4(w[2], w[3]));
+                            if (__vcmpltu4(m4, small[i] * 0x01010101u)) {
+                                const uint2 f = without_zero_blocks<MK>(i == 0 ? g.codes_l + row_at(t, i) * g.pitch_l : g.codes_q + row_at(t, i) * g.pitch_q, g.row_bytes,
+                                                                        i == 0 ? g.magnitude_l : g.magnitude_q, 16 * c, make_uint4(w[0], w[1], w[2], w[3]), small[i]);
+                                m4 = f.x;
+                                small[i] = f.y;
+                            }
+                            least[i] = __vminu4(least[i], m4);
+                        }
                 }
             }
             if (MK != MK_NVF4) {                        // the tile's smallest scale factors of A and of B
