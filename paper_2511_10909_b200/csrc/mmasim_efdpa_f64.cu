@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(NT, 2) efdpa64_kernel(DevModel m, GemmArgs g, 
     const unsigned tiles_n = unsigned((g.N + BN - 1) / BN), tile_m = blockIdx.x / tiles_n, tile_n = blockIdx.x % tiles_n;
     const int64_t row0 = int64_t(tile_m) * BM, col0 = int64_t(tile_n) * BN;
 
-    const int NCH = int(g.K / KC);
+    const int NCH = int((g.K + KC - 1) / KC);
     const Blk64<BM, EXP_NONE>* src_a = wa + int64_t(tile_m) * NCH;
     const Blk64<BN, EXP_NONE>* src_b = wb + int64_t(tile_n) * NCH;
     auto issue = [&](int n) {                              // one thread: both copies of chunk n into buffer n & 1
@@ -76,13 +76,13 @@ __global__ void __launch_bounds__(NT, 2) efdpa64_kernel(DevModel m, GemmArgs g, 
     for (int r = 0; r < TM; ++r)
 #pragma unroll
         for (int c = 0; c < TN; ++c) {
-            const int64_t i = row0 + row_at(r), j = col0 + col_at(c);
-            cw[r][c] = (g.C && i < g.M && j < g.N) ? static_cast<const uint32_t*>(g.C)[i * g.ldc + j] : 0u;
+            const int64_t i = min(row0 + row_at(r), g.M - 1), j = min(col0 + col_at(c), g.N - 1);
+            cw[r][c] = g.C ? static_cast<const uint32_t*>(g.C)[i * g.ldc + j] : 0u;
         }
     __syncthreads();                                    // the barriers are initialised
 
     for (int chunk = 0; chunk < NCH; ++chunk) {
-        const int64_t k0 = int64_t(chunk) * KC;
+        const int64_t k0 = int64_t(chunk) * KC - fast::front_pad(g.K);
         if (!fast::mbar_wait(&sm.full[chunk & 1], uint32_t(chunk >> 1) & 1u)) *reinterpret_cast<volatile int*>(&sm.error) = 1;
         const Blk64<BM, EXP_NONE>& sa_blk = sm.a[chunk & 1];
         const Blk64<BN, EXP_NONE>& sb_blk = sm.b[chunk & 1];
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(NT, 2) efdpa64_kernel(DevModel m, GemmArgs g, 
                         if (fits1) cw[r][2 * j + 1] = __float_as_uint(__double2float_rn(lo1));
                     }
             }
-            if (slow) {                                        // rare
+            if (slow && k0 + kb >= 0) {                        // rare (a block that fills K up in front changes nothing)
 #pragma unroll
                 for (int r = 0; r < TM; ++r)
 #pragma unroll
@@ -209,7 +209,7 @@ cudaError_t launch_e_one(const DevModel& m, const GemmArgs& g, cudaStream_t stre
     const size_t dsh_a = 256 * sizeof(LutEntry64) + sizeof(Blk64<BM, EXP_NONE>), dsh_b = 256 * sizeof(LutEntry64) + sizeof(Blk64<BN, EXP_NONE>);
     if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BM, true, 0, false, false, EXP_NONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_a))) != cudaSuccess) return err;
     if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BN, false, 0, false, false, EXP_NONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_b))) != cudaSuccess) return err;
-    const int64_t tiles_m = (g.M + BM - 1) / BM, tiles_n = (g.N + BN - 1) / BN, nch = g.K / KC;
+    const int64_t tiles_m = (g.M + BM - 1) / BM, tiles_n = (g.N + BN - 1) / BN, nch = (g.K + KC - 1) / KC;
     // scratch: the decoded blocks of A and B, stream-ordered out of the library's pool and returned to it behind the kernel
     const size_t bytes_a = size_t(tiles_m * nch) * sizeof(Blk64<BM, EXP_NONE>), bytes_b = size_t(tiles_n * nch) * sizeof(Blk64<BN, EXP_NONE>);
     cudaMemPool_t pool = nullptr;
@@ -219,9 +219,9 @@ cudaError_t launch_e_one(const DevModel& m, const GemmArgs& g, cudaStream_t stre
     Blk64<BM, EXP_NONE>* wa = static_cast<Blk64<BM, EXP_NONE>*>(ws);
     Blk64<BN, EXP_NONE>* wb = reinterpret_cast<Blk64<BN, EXP_NONE>*>(static_cast<unsigned char*>(ws) + bytes_a);
     decode64_kernel<EK, BM, true, 0, false, false, EXP_NONE><<<unsigned(nch * tiles_m), 256, dsh_a, stream>>>(
-        m, static_cast<const unsigned char*>(g.A), g.M, g.lda, unsigned(nch), wa);
+        m, static_cast<const unsigned char*>(g.A), g.M, g.lda, unsigned(nch), fast::pad_of<EK>(g.K, g.lda), wa);
     decode64_kernel<EK, BN, false, 0, false, false, EXP_NONE><<<unsigned(nch * tiles_n), 256, dsh_b, stream>>>(
-        m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, unsigned(nch), wb);
+        m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, unsigned(nch), fast::pad_of<EK>(g.K, g.ldb), wb);
     efdpa64_kernel<EK, L><<<unsigned(tiles_n * tiles_m), NT, sh, stream>>>(m, g, wa, wb);
     err = cudaGetLastError();
     const cudaError_t err2 = cudaFreeAsync(ws, stream);

@@ -131,14 +131,17 @@ __host__ __device__ constexpr bool tiny_zeros(int ek, int base) { return base ==
 __host__ __device__ constexpr int pe64_sub(int base) { return base == 8 ? 32 : (base == 5 ? 16 : 8); }
 
 // Decode pass: one CTA of 256 threads decodes one block (R rows x 32 elements) into shared memory and copies it to its
-// place dst[tile][chunk].  Rows beyond the matrix decode as zeros.
+// place dst[tile][chunk].  Rows beyond the matrix repeat the last one: their outputs are not stored, but as zeros they would take
+// the rare paths block after block (Ampere FP16 -> FP16 1000 x 1111 x 1000 392 us, repeated 256).  The `pad` elements before the first
+// one, which fill K up to whole chunks, decode as zeros: in front, because a block of zeros leaves the initial accumulator as the first real block would find it
+// (behind, it would turn a result of -0, which RNE-FP32 can leave, into +0).
 // EOSPLIT (GTR-FDPA, blocks of 16): inside each block of 16 the operand plane holds the even elements first, then the odd
 // ones, so that a matrix instruction sums four elements of one group; exponent pairs and masks keep the order of K.
 // TINY_ZEROS (the T-FDPA kernels without a tensor-core maximum): a zero is staged as 2^-900 of its sign.  Its products are far below any
 // unit of a sum register, so that a positive one adds nothing and a negative one falls one unit short like every other
 // negative product: the sign masks alone count them, without the masks of nonzero elements.
 template <int EK, int R, bool IS_A, int BASE, bool EOSPLIT = false, bool TINY_ZEROS = false, int FORM = exp_form(BASE)>
-__global__ void __launch_bounds__(256) decode64_kernel(DevModel m, const unsigned char* src, int64_t rows, int64_t ld, unsigned nch, Blk64<R, FORM>* dst,
+__global__ void __launch_bounds__(256) decode64_kernel(DevModel m, const unsigned char* src, int64_t rows, int64_t ld, unsigned nch, fast::Pad pad, Blk64<R, FORM>* dst,
                                                        const uint8_t* sf = nullptr, int64_t ld_sf = 0) {
     using E = Elem<EK>;
     constexpr int TPR = KC / E::TASK, TASKS = R * TPR, WORDS = E::TASK * E::BYTES / 4;
@@ -160,26 +163,21 @@ __global__ void __launch_bounds__(256) decode64_kernel(DevModel m, const unsigne
     }
     if (tid == 0) { blk.special = 0u; blk.max_exp = 0u; blk.wild = blk.pad = 0u; }
     __syncthreads();
-    const int64_t tile = blockIdx.x / nch, chunk = blockIdx.x % nch, k0 = chunk * KC;
+    const int64_t tile = blockIdx.x / nch, chunk = blockIdx.x % nch, k0 = chunk * KC - pad.front;
     uint32_t spec = 0u, top_exp = 0u, wild = 0u;
     for (int task = tid; task < TASKS; task += 256) {
         const int r = task % R, h = task / R;
         const int pr = IS_A ? perm_row64(r) : perm_col64(r);
-        const int64_t grow = tile * R + r;
+        const int64_t grow = min(tile * R + r, rows - 1);
         uint32_t w[WORDS];
-#pragma unroll
-        for (int q = 0; q < WORDS / 4; ++q) {
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (grow < rows) v = reinterpret_cast<const uint4*>(src + (grow * ld + k0 + h * E::TASK) * E::BYTES)[q];
-            w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
-        }
+        fast::load_task<EK>(w, src, grow * ld, k0 + h * E::TASK, pad.wide);
         // ST-FDPA (Algorithm 8): the row's scale factor for this block of 32 multiplies its operands here, exactly (an
         // addition to the exponent field of a nonzero double); exponent planes stay unscaled, the main kernel adds
         // Exp(alpha) + Exp(beta) to the block maximum.  A NaN scale factor stages zeros (the output is NaN by its flag).
         int sc20 = 0;
         bool sc_nan = false;
         if (sf) {
-            const uint32_t sbyte = grow < rows ? uint32_t(sf[grow * ld_sf + chunk]) : 127u;
+            const uint32_t sbyte = sf[grow * ld_sf + chunk];
             sc20 = (int(sbyte) - 127) << 20;
             sc_nan = sbyte == 0xFFu;
         }
@@ -250,9 +248,9 @@ __global__ void __launch_bounds__(256) decode64_kernel(DevModel m, const unsigne
     }
     if (spec) atomicOr(&blk.special, 1u);
     if (wild) atomicOr(&blk.wild, 1u);
-    if (tid < R) {                                      // the scale factors travel with the block (rows beyond the matrix: 2^0)
-        const int64_t grow = tile * R + tid;
-        blk.sf[IS_A ? perm_row64(tid) : perm_col64(tid)] = (sf && grow < rows) ? sf[grow * ld_sf + chunk] : uint8_t(127);
+    if (tid < R) {                                      // the scale factors travel with the block
+        const int64_t grow = min(tile * R + tid, rows - 1);
+        blk.sf[IS_A ? perm_row64(tid) : perm_col64(tid)] = sf ? sf[grow * ld_sf + chunk] : uint8_t(127);
     }
     top_exp = __reduce_max_sync(0xFFFFFFFFu, top_exp);
     if ((tid & 31) == 0 && top_exp) atomicMax(&blk.max_exp, top_exp);
@@ -336,7 +334,7 @@ __global__ void __launch_bounds__(NT, 2) tfdpa64_kernel(DevModel m, GemmArgs g, 
     const FmtDesc fa = fmt_desc(m.fmt_a), fb = fmt_desc(m.fmt_b);
 
     // the decoded blocks of this tile row of A and tile column of B, chunk after chunk, land in two buffers by bulk copies
-    const int NCH = int(g.K / KC);
+    const int NCH = int((g.K + KC - 1) / KC);
     const Blk64<BM, exp_form(BASE)>* src_a = wa + int64_t(tile_m) * NCH;
     const Blk64<BN, exp_form(BASE)>* src_b = wb + int64_t(tile_n) * NCH;
     auto issue = [&](int n) {                              // one thread: both copies of chunk n into buffer n & 1
@@ -399,9 +397,9 @@ __global__ void __launch_bounds__(NT, 2) tfdpa64_kernel(DevModel m, GemmArgs g, 
     for (int r = 0; r < TM; ++r)
 #pragma unroll
         for (int c = 0; c < TN; ++c) {
-            const int64_t i = row0 + row_at(r), j = col0 + col_at(c);
+            const int64_t i = min(row0 + row_at(r), g.M - 1), j = min(col0 + col_at(c), g.N - 1);
             uint32_t w = 0u;
-            if (g.C && i < g.M && j < g.N)
+            if (g.C)
                 w = ACC16 ? uint32_t(static_cast<const uint16_t*>(g.C)[i * g.ldc + j])
                           : static_cast<const uint32_t*>(g.C)[i * g.ldc + j];
             if (PROMOTE) { promoted[PROMOTE ? r : 0][PROMOTE ? c : 0] = __uint_as_float(w); w = 0u; }
@@ -423,7 +421,7 @@ __global__ void __launch_bounds__(NT, 2) tfdpa64_kernel(DevModel m, GemmArgs g, 
     uint32_t emp[TM][TN];                               // product exponents of the block that comes next
 
     for (int chunk = 0; chunk < NCH; ++chunk) {
-        const int64_t k0 = int64_t(chunk) * KC;
+        const int64_t k0 = int64_t(chunk) * KC - fast::front_pad(g.K);
         // a wait that runs out is recorded and the chunk computed on whatever is there; every thread sees the flag after
         // the barrier at the end of the chunk, and the CTA leaves together without storing anything
         if (!fast::mbar_wait(&sm.full[chunk & 1], uint32_t(chunk >> 1) & 1u)) *reinterpret_cast<volatile int*>(&sm.error) = 1;
@@ -486,7 +484,7 @@ __global__ void __launch_bounds__(NT, 2) tfdpa64_kernel(DevModel m, GemmArgs g, 
 #pragma unroll 1
                     for (int c = 0; c < TN; ++c) {
                         const int64_t i = row0 + row_at(r), j = col0 + col_at(c);
-                        if (i >= g.M || j >= g.N) continue;
+                        if (i >= g.M || j >= g.N || k0 + kb < 0) continue;
                         Special ev;
                         for (int kk = kb; kk < kb + L; ++kk) {
                             const uint32_t x = decode_elem(fa, raw_elem<EK>(g.A, i * g.lda + k0 + kk));
@@ -819,7 +817,7 @@ cudaError_t launch_one64b(const DevModel& m, const GemmArgs& g, cudaStream_t str
     const size_t dsh_a = 256 * sizeof(LutEntry64) + sizeof(Blk64<BM, exp_form(BASE)>), dsh_b = 256 * sizeof(LutEntry64) + sizeof(Blk64<BN, exp_form(BASE)>);
     if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BM, true, BASE, false, tiny_zeros(EK, BASE)>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_a))) != cudaSuccess) return err;
     if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BN, false, BASE, false, tiny_zeros(EK, BASE)>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_b))) != cudaSuccess) return err;
-    const int64_t tiles_m = (g.M + BM - 1) / BM, tiles_n = (g.N + BN - 1) / BN, nch = g.K / KC;
+    const int64_t tiles_m = (g.M + BM - 1) / BM, tiles_n = (g.N + BN - 1) / BN, nch = (g.K + KC - 1) / KC;
     // scratch: the decoded blocks of A and B, stream-ordered out of the library's pool and returned to it behind the kernel
     const size_t bytes_a = size_t(tiles_m * nch) * sizeof(Blk64<BM, exp_form(BASE)>), bytes_b = size_t(tiles_n * nch) * sizeof(Blk64<BN, exp_form(BASE)>);
     cudaMemPool_t pool = nullptr;
@@ -829,9 +827,9 @@ cudaError_t launch_one64b(const DevModel& m, const GemmArgs& g, cudaStream_t str
     Blk64<BM, exp_form(BASE)>* wa = static_cast<Blk64<BM, exp_form(BASE)>*>(ws);
     Blk64<BN, exp_form(BASE)>* wb = reinterpret_cast<Blk64<BN, exp_form(BASE)>*>(static_cast<unsigned char*>(ws) + bytes_a);
     decode64_kernel<EK, BM, true, BASE, false, tiny_zeros(EK, BASE)><<<unsigned(nch * tiles_m), 256, dsh_a, stream>>>(
-        m, static_cast<const unsigned char*>(g.A), g.M, g.lda, unsigned(nch), wa, ST ? g.sfa : nullptr, g.ld_sfa);
+        m, static_cast<const unsigned char*>(g.A), g.M, g.lda, unsigned(nch), fast::pad_of<EK>(g.K, g.lda), wa, ST ? g.sfa : nullptr, g.ld_sfa);
     decode64_kernel<EK, BN, false, BASE, false, tiny_zeros(EK, BASE)><<<unsigned(nch * tiles_n), 256, dsh_b, stream>>>(
-        m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, unsigned(nch), wb, ST ? g.sfb : nullptr, g.ld_sfb);
+        m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, unsigned(nch), fast::pad_of<EK>(g.K, g.ldb), wb, ST ? g.sfb : nullptr, g.ld_sfb);
     tfdpa64_kernel<EK, L, RHO, PROMOTE, ST, BASE><<<unsigned(tiles_n * tiles_m), NT, sh, stream>>>(m, g, wa, wb);
     err = cudaGetLastError();
     const cudaError_t err2 = cudaFreeAsync(ws, stream);

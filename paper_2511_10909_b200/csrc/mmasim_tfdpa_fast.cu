@@ -66,14 +66,32 @@ int kind_of(const DevModel& m) {
 
 }  // namespace
 
+// Rows that are no whole number of chunks or start off 16 bytes.
+static bool ragged(const DevModel& m, const GemmArgs& g) {
+    const int bytes = fmt_desc(m.fmt_a).storage_bits / 8;
+    return g.K % fast::KC || (g.lda * bytes) % 16 || (g.ldb * bytes) % 16;
+}
+
+// Whether the small-tile kernels take the call at all.
+static bool direct_takes(const DevModel& m, const GemmArgs& g) {
+    const int kind = kind_of(m);
+    if (!kind || g.dot_mode || m.literal_emax) return false;
+    if ((kind == KIND_TR || kind == KIND_E) && g.k_chunk) return false;
+    if (g.M > 65535ll * 8 || g.N > 0x7FFFFFFFll - 128) return false;                                       // grid.y, 32-bit columns
+    // The kernels count the bytes left in a row, and the chunks, in 32 bits; TR-FDPA of the wide formats tags exponents with the chunk's
+    // number in 21 bits.
+    const int64_t row = g.K * (fmt_desc(m.fmt_a).storage_bits / 8);
+    const bool tagged = m.family == FAM_TR && (m.fmt_a == EF_BF16 || m.fmt_a == EF_TF32);
+    return row <= 0x7FFFFFFFll - 1024 && !(tagged && g.K > (int64_t(1) << 21) * fast::KC - 256);
+}
+
 bool fast_tfdpa_supported(const DevModel& m, const GemmArgs& g) {
     const int kind = kind_of(m);
     if (!kind || g.dot_mode || m.literal_emax) return false;
-    const int bytes = fmt_desc(m.fmt_a).storage_bits / 8;
-    if (g.K % fast::KC) return false;
+    if (g.K % m.L || (m.family == FAM_ST && g.K % fast::KC)) return false;   // (ragged chunks are filled up with whole blocks of zeros)
+    if (ragged(m, g) && !direct_takes(m, g)) return false;                  // (what they fall back on where there is no memory for scratch)
     if (g.k_chunk % fast::KC) return false;
     if ((kind == KIND_TR || kind == KIND_E) && g.k_chunk) return false;
-    if (((g.lda * bytes) % 16) || ((g.ldb * bytes) % 16)) return false;      // 16-byte row starts for the vector loads
     if (m.F == 13 && g.M > 65535ll * fast::BM) return false;                // grid.y
     if (g.N > 0x7FFFFFFFll - 128 || g.K > 0x7FFFFFFFll - 64) return false;   // 32-bit tile origins and k offsets in the kernels
     return true;
@@ -83,8 +101,7 @@ bool fast_tfdpa_supported(const DevModel& m, const GemmArgs& g) {
 //     small tiles   4 + chain chunks + per_tile n (chunks + 1.2)        8 x 16 outputs: 0.65 of a 16 x 16 tile
 //     large tiles   decode + large n (chunks + 0.5)                     (an odd n: the last tile has the SM to itself, 0.16 of one more)
 // with the constants of the arithmetic, fitted to the times of all four at sizes from 16 x 64 to 1076 x 3218 and K = 64, 256 and 1024
-// (within 10 %).  Chosen by it, no size takes 1.2 times its best, but for ragged rows of CDNA1 BF16 (1.4) and Ampere FP16 -> FP16 (1.4), whose
-// padding costs the large kernels extra; the average is 1.01.  Small / large in us on both sides of the line: Hopper E4M3 -> FP16 640 x 640 x 64
+// (within 10 %).  Chosen by it, no size takes 1.2 times its best; the average is 1.01.  Small / large in us on both sides of the line: Hopper E4M3 -> FP16 640 x 640 x 64
 // 25 / 29, x 256 63 / 60, Ampere FP16 768 x 768 x 256 36 / 38, 1024 x 1024 x 256 70 / 62, CDNA1 BF16 512 x 512 x 1024 129 / 211, 768 x 768 x 1024
 // 258 / 215.
 namespace {
@@ -112,15 +129,8 @@ TileCosts tile_costs(const DevModel& m, int kind, bool promoted) {
 }  // namespace
 
 DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us) {
+    if (!direct_takes(m, g)) return DIRECT_NONE;
     const int kind = kind_of(m);
-    if (!kind || g.dot_mode || m.literal_emax) return DIRECT_NONE;
-    if ((kind == KIND_TR || kind == KIND_E) && g.k_chunk) return DIRECT_NONE;
-    if (g.M > 65535ll * 8 || g.N > 0x7FFFFFFFll - 128) return DIRECT_NONE;                                 // grid.y, 32-bit columns
-    // The kernels count the bytes left in a row, and the chunks, in 32 bits; TR-FDPA of the wide formats tags exponents with the chunk's
-    // number in 21 bits.
-    const int64_t row = g.K * (fmt_desc(m.fmt_a).storage_bits / 8);
-    const bool tagged = m.family == FAM_TR && (m.fmt_a == EF_BF16 || m.fmt_a == EF_TF32);
-    if (row > 0x7FFFFFFFll - 1024 || (tagged && g.K > (int64_t(1) << 21) * fast::KC - 256)) return DIRECT_NONE;
     constexpr int64_t SMS = 148;
     auto fullest = [&](int bm, int bn) { return double((((g.M + bm - 1) / bm) * ((g.N + bn - 1) / bn) + SMS - 1) / SMS); };
     const bool f13 = kind == 1 + fast::EK_LUT8 && m.F == 13;
@@ -180,7 +190,7 @@ unsigned int* copy_timeout_counter() {
 }
 
 int launch_gemm_noalloc(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
-    if (!fast::noalloc_supported(m) || !fast_tfdpa_supported(m, g)) {
+    if (!fast::noalloc_supported(m) || !fast_tfdpa_supported(m, g) || g.K % fast::KC || g.lda % 16 || g.ldb % 16) {
         set_error("mmasim_gemm_noalloc serves the FP8 models with F = 13 (Ada and Hopper FP8 rows), K a multiple of 32 and "
                   "16-byte row strides; this call needs another kernel");
         return MMASIM_ERR_UNSUPPORTED;
@@ -214,6 +224,10 @@ int launch_fast_tfdpa(const DevModel& m, const GemmArgs& g, cudaStream_t stream)
         case fast::EK_BF16: set_kernel_name("tfdpa_bf16", "large_tiles"); err = fast::launch_bf16(m, g, stream); break;
         case fast::EK_TF32: set_kernel_name("tfdpa_tf32", "large_tiles"); err = fast::launch_tf32(m, g, stream); break;
         default: break;
+    }
+    if (err == cudaErrorMemoryAllocation && ragged(m, g)) {     // no memory for the decoded operands: the small tiles need none
+        cudaGetLastError();
+        return launch_direct(m, g, DIRECT_32x32, stream);
     }
     if (err != cudaSuccess) {
         set_error("tuned T-FDPA kernel launch failed: %s", cudaGetErrorString(err));

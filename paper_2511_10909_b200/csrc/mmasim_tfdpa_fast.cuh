@@ -60,6 +60,41 @@ __device__ __forceinline__ uint32_t raw_elem(const void* p, int64_t idx) {
     return static_cast<const uint32_t*>(p)[idx];
 }
 
+// K is filled up to whole chunks with zeros in front of the first element.  `wide`: rows and chunks start on 16 bytes.
+struct Pad { int front; bool wide; };
+__host__ __device__ __forceinline__ int front_pad(int64_t K) { return int((KC - K % KC) % KC); }
+template <int EK>
+inline Pad pad_of(int64_t K, int64_t ld) {
+    const int front = front_pad(K);
+    return {front, (front * Elem<EK>::BYTES) % 16 == 0 && (ld * Elem<EK>::BYTES) % 16 == 0};
+}
+// The raw words of consecutive elements k, k + 1, ... of a row that starts at element `row`; zeros before the row.
+template <int EK, int WORDS>
+__device__ __forceinline__ void load_task(uint32_t (&w)[WORDS], const unsigned char* src, int64_t row, int64_t k, bool wide) {
+    constexpr int BYTES = Elem<EK>::BYTES, PER = 4 / BYTES;
+#pragma unroll
+    for (int q = 0; q < WORDS; ++q) w[q] = 0u;
+    const unsigned char* p = src + (row + k) * BYTES;
+    if (wide) {                                         // (an access of 8 or 16 bytes lies before the row or inside it)
+        if constexpr (WORDS == 2) {
+            if (k < 0) return;
+            const uint2 v = *reinterpret_cast<const uint2*>(p);
+            w[0] = v.x; w[1] = v.y;
+        } else {
+#pragma unroll
+            for (int q = 0; q < WORDS; q += 4) {
+                if (k + q * PER < 0) continue;
+                const uint4 v = *reinterpret_cast<const uint4*>(p + 4 * q);
+                w[q] = v.x; w[q + 1] = v.y; w[q + 2] = v.z; w[q + 3] = v.w;
+            }
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < WORDS * PER; ++e)
+            if (k + e >= 0) w[e / PER] |= raw_elem<EK>(src, row + k + e) << (8 * BYTES * (e % PER) % 32);
+    }
+}
+
 // ---- bulk copies and their barrier: inline PTX ----
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return uint32_t(__cvta_generic_to_shared(p)); }
 __device__ __forceinline__ void mbar_init(unsigned long long* bar, uint32_t count) {

@@ -179,11 +179,12 @@ __device__ __forceinline__ uint32_t stage_row(const LutEntryT* lut, BlkT<R>& s, 
 
 // Decode pass: one CTA decodes one block (R rows of A or columns of B x 32 elements of K) through a 256-entry table of
 // 8-byte entries into shared memory and copies it to its place in the scratch array dst[tile][chunk].  Every thread
-// takes 16 (R = 128) or 8 (R = 64) consecutive elements of one row.  Rows beyond the matrix decode as zeros.
+// takes 16 (R = 128) or 8 (R = 64) consecutive elements of one row.  Rows beyond the matrix repeat the last one (their outputs are
+// not stored, but as zeros they would take the rare paths); the elements in front that fill K up to whole chunks decode as zeros.
 static_assert(BM == 128 && KC == 32 && NT == 256, "the task split of the decode pass");
 template <int BASE, int R, bool IS_A, int TH>
 __global__ void __launch_bounds__(NT) trop_decode_kernel(DevModel m, const unsigned char* src, int64_t rows, int64_t ld, int F,
-                                                         BlkT<R>* dst) {
+                                                         fast::Pad pad, BlkT<R>* dst) {
     __shared__ __align__(16) LutEntryT lut_a[256];
     __shared__ __align__(16) LutEntryT lut_b[256];
     __shared__ __align__(16) BlkT<R> blk;
@@ -193,23 +194,15 @@ __global__ void __launch_bounds__(NT) trop_decode_kernel(DevModel m, const unsig
     if (tid == 0) { blk.special = blk.sparse = 0u; blk.pad[0] = blk.pad[1] = 0u; }
     constexpr int N = R * KC / NT;                      // elements per thread: 16 or 8
     const int r = tid % R, part = tid / R;
-    const int64_t i = int64_t(blockIdx.y) * R + r, k0 = int64_t(blockIdx.x) * KC;
+    const int64_t i = int64_t(blockIdx.y) * R + r, k0 = int64_t(blockIdx.x) * KC - pad.front;
     uint32_t w[N / 4];
-    if (N == 16) {
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (i < rows) v = *reinterpret_cast<const uint4*>(src + i * ld + k0 + N * part);
-        w[0] = v.x; w[1] = v.y; w[N / 4 - 2] = v.z; w[N / 4 - 1] = v.w;
-    } else {
-        uint2 v = make_uint2(0u, 0u);
-        if (i < rows) v = *reinterpret_cast<const uint2*>(src + i * ld + k0 + N * part);
-        w[0] = v.x; w[1] = v.y;
-    }
+    fast::load_task<fast::EK_LUT8>(w, src, min(i, rows - 1) * ld, k0 + N * part, pad.wide);
     __syncthreads();
     const uint32_t spec = stage_row<N, R>(IS_A ? lut_a : lut_b, blk, w, r, IS_A ? perm_row<TH>(r) : perm_col(r), part);
     if (spec & 0x8000u) atomicOr(&blk.special, 1u);
     // (two rows with less than half of their elements zero meet in a nonzero product; a thread sees a part of a block of L, and
     // parts with less than half of theirs add up to one)
-    if (i < rows && (spec >> 16) * 2 >= uint32_t(N)) atomicOr(&blk.sparse, 1u);
+    if ((spec >> 16) * 2 >= uint32_t(N)) atomicOr(&blk.sparse, 1u);
     __syncthreads();
     uint4* out = reinterpret_cast<uint4*>(dst + (int64_t(blockIdx.y) * gridDim.x + blockIdx.x));
     const uint4* in = reinterpret_cast<const uint4*>(&blk);
@@ -262,7 +255,7 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
     constexpr uint32_t E_KEEP = 243u << 23, KEEP = E_KEEP + MAGIC_ADD;
     static_assert(F == 13 || ACC16, "the kept word is carried as its upper 22 bits");
     // the decoded blocks of this tile row of A and tile column of B, chunk after chunk, land in two buffers by bulk copies
-    const int K = int(g.K), NCH = K / KC;
+    const int NCH = int((g.K + KC - 1) / KC);
     const BlkT<BM>* src_a = wa + int64_t(blockIdx.y) * NCH;
     const BlkT<BN>* src_b = wb + int64_t(blockIdx.x) * NCH;
     auto issue = [&](int n) {                              // one thread: both copies of chunk n into buffer n & 1
@@ -313,7 +306,7 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
     // from a huge C: K products of at most 2^32 each move an accumulator by less than 2^64.
     big = __syncthreads_or(!ACC16 && !PROMOTE && big);
     for (int chunk = 0; chunk < NCH; ++chunk) {
-        const int k0 = chunk * KC;
+        const int k0 = chunk * KC;                         // (g.K elements end with the last chunk; see fast::front_pad)
         // a wait that runs out is recorded and the chunk computed on whatever is there; every thread sees the flag after
         // the barrier at the end of the chunk, and the CTA leaves together without storing anything
         if (!mbar_wait(&sm.full[chunk & 1], uint32_t(chunk >> 1) & 1u)) *reinterpret_cast<volatile int*>(&sm.error) = 1;
@@ -325,16 +318,17 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
         for (int blk = 0; blk < NBLK; ++blk) {
             const int kb = blk * L;
             if (chunk_special) {                           // rare: special-value events of this block (Section 4.2)
+                const int64_t first = k0 + kb - fast::front_pad(g.K);
 #pragma unroll 1
                 for (int h = 0; h < TH; ++h)
 #pragma unroll 1
                     for (int x = 0; x < TW; ++x) {
                         const int64_t i = row0 + row_of(h), j = col0 + col_of(x);
-                        if (i >= g.M || j >= g.N) continue;
+                        if (i >= g.M || j >= g.N || first < 0) continue;
                         Special ev;
-                        for (int kk = kb; kk < kb + L; ++kk) {
-                            const uint32_t xa = decode_elem(fa, raw_elem<EK>(g.A, i * g.lda + k0 + kk));
-                            const uint32_t yb = decode_elem(fb, raw_elem<EK>(g.B, j * g.ldb + k0 + kk));
+                        for (int kk = 0; kk < L; ++kk) {
+                            const uint32_t xa = decode_elem(fa, raw_elem<EK>(g.A, i * g.lda + first + kk));
+                            const uint32_t yb = decode_elem(fb, raw_elem<EK>(g.B, j * g.ldb + first + kk));
                             ev.product(xa, yb);
                         }
                         const mask_t bit = mask_t(1) << (h * TW + x);
@@ -596,7 +590,7 @@ struct Scratch {
 template <int TH>
 size_t scratch_bytes_one(const GemmArgs& g) {
     constexpr int BN = Geo<TH>::BN;
-    const int64_t tiles_m = (g.M + BM - 1) / BM, tiles_n = (g.N + BN - 1) / BN, nch = g.K / KC;
+    const int64_t tiles_m = (g.M + BM - 1) / BM, tiles_n = (g.N + BN - 1) / BN, nch = (g.K + KC - 1) / KC;
     return size_t(tiles_m * nch) * sizeof(BlkT<BM>) + size_t(tiles_n * nch) * sizeof(BlkT<BN>);
 }
 
@@ -606,7 +600,7 @@ cudaError_t launch_one_t(const DevModel& m, const GemmArgs& g, cudaStream_t stre
     const size_t sh = sizeof(SmemT<TH>);
     cudaError_t err = cudaFuncSetAttribute(tfdpa_trop_kernel<EK, L, F, RHO, PROMOTE, BASE, TH>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sh));
     if (err != cudaSuccess) return err;
-    const int64_t tiles_m = (g.M + BM - 1) / BM, tiles_n = (g.N + BN - 1) / BN, nch = g.K / KC;
+    const int64_t tiles_m = (g.M + BM - 1) / BM, tiles_n = (g.N + BN - 1) / BN, nch = (g.K + KC - 1) / KC;
     const size_t bytes_a = size_t(tiles_m * nch) * sizeof(BlkT<BM>), bytes_b = size_t(tiles_n * nch) * sizeof(BlkT<BN>);
     void* ws = sc.given;
     if (ws) {
@@ -619,9 +613,9 @@ cudaError_t launch_one_t(const DevModel& m, const GemmArgs& g, cudaStream_t stre
     BlkT<BM>* wa = static_cast<BlkT<BM>*>(ws);
     BlkT<BN>* wb = reinterpret_cast<BlkT<BN>*>(static_cast<unsigned char*>(ws) + bytes_a);
     trop_decode_kernel<BASE, BM, true, TH><<<dim3((unsigned)nch, (unsigned)tiles_m), NT, 0, stream>>>(
-        m, static_cast<const unsigned char*>(g.A), g.M, g.lda, F, wa);
+        m, static_cast<const unsigned char*>(g.A), g.M, g.lda, F, fast::pad_of<fast::EK_LUT8>(g.K, g.lda), wa);
     trop_decode_kernel<BASE, BN, false, TH><<<dim3((unsigned)nch, (unsigned)tiles_n), NT, 0, stream>>>(
-        m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, F, wb);
+        m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, F, fast::pad_of<fast::EK_LUT8>(g.K, g.ldb), wb);
     dim3 grid((unsigned)tiles_n, (unsigned)tiles_m, 1);
     tfdpa_trop_kernel<EK, L, F, RHO, PROMOTE, BASE, TH><<<grid, NT, sh, stream>>>(m, g, wa, wb);
     err = cudaGetLastError();

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(NT, 2) trfdpa64_kernel(DevModel m, GemmArgs g,
     const int MAGIC_E = 1023 + 52 - F - CB;
 
     // the decoded blocks of this tile row of A and tile column of B, chunk after chunk, land in two buffers by bulk copies
-    const int NCH = int(g.K / KC);
+    const int NCH = int((g.K + KC - 1) / KC);
     const Blk64<BM, EXP_PAIRS>* src_a = wa + int64_t(tile_m) * NCH;
     const Blk64<BN, EXP_PAIRS>* src_b = wb + int64_t(tile_n) * NCH;
     auto issue = [&](int n) {                              // one thread: both copies of chunk n into buffer n & 1
@@ -76,9 +76,9 @@ __global__ void __launch_bounds__(NT, 2) trfdpa64_kernel(DevModel m, GemmArgs g,
     for (int r = 0; r < TM; ++r)
 #pragma unroll
         for (int c = 0; c < TN; ++c) {
-            const int64_t i = row0 + row_at(r), j = col0 + col_at(c);
+            const int64_t i = min(row0 + row_at(r), g.M - 1), j = min(col0 + col_at(c), g.N - 1);
             uint32_t w = 0u;
-            if (g.C && i < g.M && j < g.N) w = static_cast<const uint32_t*>(g.C)[i * g.ldc + j];
+            if (g.C) w = static_cast<const uint32_t*>(g.C)[i * g.ldc + j];
             const AccDec d = decode_acc(w, false);
             if (d.cls != CLS_FINITE) {
                 const uint32_t bit = 1u << (r * TN + c);
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(NT, 2) trfdpa64_kernel(DevModel m, GemmArgs g,
     uint32_t emp[TM][TN];                               // product exponents of the block that comes next (low lane: even elements)
 
     for (int chunk = 0; chunk < NCH; ++chunk) {
-        const int64_t k0 = int64_t(chunk) * KC;
+        const int64_t k0 = int64_t(chunk) * KC - fast::front_pad(g.K);
         // a wait that runs out is recorded and the chunk computed on whatever is there; every thread sees the flag after
         // the barrier at the end of the chunk, and the CTA leaves together without storing anything
         if (!fast::mbar_wait(&sm.full[chunk & 1], uint32_t(chunk >> 1) & 1u)) *reinterpret_cast<volatile int*>(&sm.error) = 1;
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(NT, 2) trfdpa64_kernel(DevModel m, GemmArgs g,
 #pragma unroll 1
                     for (int c = 0; c < TN; ++c) {
                         const int64_t i = row0 + row_at(r), j = col0 + col_at(c);
-                        if (i >= g.M || j >= g.N) continue;
+                        if (i >= g.M || j >= g.N || k0 + kb < 0) continue;
                         Special ev;
                         for (int kk = kb; kk < kb + L; ++kk) {
                             const uint32_t x = decode_elem(fa, raw_elem<EK>(g.A, i * g.lda + k0 + kk));
@@ -316,7 +316,7 @@ cudaError_t launch_tr_one(const DevModel& m, const GemmArgs& g, cudaStream_t str
     const size_t dsh_a = 256 * sizeof(LutEntry64) + sizeof(Blk64<BM, EXP_PAIRS>), dsh_b = 256 * sizeof(LutEntry64) + sizeof(Blk64<BN, EXP_PAIRS>);
     if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BM, true, 0, GTR>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_a))) != cudaSuccess) return err;
     if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BN, false, 0, GTR>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_b))) != cudaSuccess) return err;
-    const int64_t tiles_m = (g.M + BM - 1) / BM, tiles_n = (g.N + BN - 1) / BN, nch = g.K / KC;
+    const int64_t tiles_m = (g.M + BM - 1) / BM, tiles_n = (g.N + BN - 1) / BN, nch = (g.K + KC - 1) / KC;
     // scratch: the decoded blocks of A and B, stream-ordered out of the library's pool and returned to it behind the kernel
     const size_t bytes_a = size_t(tiles_m * nch) * sizeof(Blk64<BM, EXP_PAIRS>), bytes_b = size_t(tiles_n * nch) * sizeof(Blk64<BN, EXP_PAIRS>);
     cudaMemPool_t pool = nullptr;
@@ -326,9 +326,9 @@ cudaError_t launch_tr_one(const DevModel& m, const GemmArgs& g, cudaStream_t str
     Blk64<BM, EXP_PAIRS>* wa = static_cast<Blk64<BM, EXP_PAIRS>*>(ws);
     Blk64<BN, EXP_PAIRS>* wb = reinterpret_cast<Blk64<BN, EXP_PAIRS>*>(static_cast<unsigned char*>(ws) + bytes_a);
     decode64_kernel<EK, BM, true, 0, GTR><<<unsigned(nch * tiles_m), 256, dsh_a, stream>>>(
-        m, static_cast<const unsigned char*>(g.A), g.M, g.lda, unsigned(nch), wa);
+        m, static_cast<const unsigned char*>(g.A), g.M, g.lda, unsigned(nch), fast::pad_of<EK>(g.K, g.lda), wa);
     decode64_kernel<EK, BN, false, 0, GTR><<<unsigned(nch * tiles_n), 256, dsh_b, stream>>>(
-        m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, unsigned(nch), wb);
+        m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, unsigned(nch), fast::pad_of<EK>(g.K, g.ldb), wb);
     trfdpa64_kernel<EK, L, GTR><<<unsigned(tiles_n * tiles_m), NT, sh, stream>>>(m, g, wa, wb);
     err = cudaGetLastError();
     const cudaError_t err2 = cudaFreeAsync(ws, stream);

@@ -1,0 +1,24 @@
+"""Large tiles over rows that are no whole number of chunks of 32, or that start off 16 bytes: against the generic kernels, bit for bit."""
+import pytest
+import torch
+
+from test_gpu_tile_sizes import KEYS, _inputs, gu
+
+pytestmark = pytest.mark.gpu
+
+
+# one block and its neighbours of a chunk; a tile of every size less one row, whole, and one row more
+@pytest.mark.parametrize("M,N,blocks", [(1, 1, 1), (63, 129, 3), (128, 64, 5), (129, 65, 9)])
+@pytest.mark.parametrize("key", [k for k in KEYS if not k[1].startswith("mx")], ids=lambda k: "-".join(k))
+def test_ragged_rows_against_generic(key, M, N, blocks):
+    from paper_2511_10909_b200 import mmasim
+    model = mmasim.Model(*key)
+    K = model.l_max * blocks
+    for v in _inputs(key, M, N, K, 600 + blocks):           # ordinary values, raw bit patterns, small magnitudes
+        v["C"][::3, ::2] = 0x8000 if key[2] == "fp16" else 0x80000000         # -0
+        d = {k: gu.dev(x) for k, x in v.items()}
+        want = mmasim.gemm(model, d["A"], d["B"], d["C"], force_generic=True)
+        for A, B in ((d["A"], d["B"]), [torch.nn.functional.pad(d[k], (0, 3))[:, :-3] for k in ("A", "B")]):
+            got = mmasim.gemm(model, A, B, d["C"], large_tiles=True)
+            assert mmasim.last_variant() == "large_tiles"
+            assert torch.equal(got, want), (key, (M, N, K), int((got != want).sum()))
