@@ -117,8 +117,8 @@ TileCosts tile_costs(const DevModel& m, int kind, bool promoted) {
     if (kind == 1 + fast::EK_LUT8) {
         if (m.F != 13) return h ? TileCosts{0.37, 0.63, 1.96, 4.5, 15} : (m.family == FAM_ST ? TileCosts{0.26, 0.50, 1.15, 2.3, 15} : TileCosts{0.19, 0.44, 1.05, 2.2, 15});
         if (h) return m.L == 16 ? TileCosts{0.66, 0.56, 2.13, 6.8, 22} : TileCosts{0.37, 0.63, 1.96, 4.65, 22};
-        const double large = m.L == 16 ? 6.3 : 5.0;     // (promoted sums: tiles of half the size)
-        return m.L == 16 ? TileCosts{0.28, 0.36, 0.99, promoted ? 0.53 * large : large, 28} : TileCosts{0.20, 0.43, 1.01, promoted ? 0.53 * large : large, 28};
+        // (large: times f13_chunk_us; promoted sums only have the smaller tiles)
+        return m.L == 16 ? TileCosts{0.28, 0.36, 0.99, promoted ? 1.38 : 1.3, 22} : TileCosts{0.20, 0.43, 1.01, promoted ? 1.06 : 1.0, 22};
     }
     if (kind == 1 + fast::EK_F16 && h) return m.L == 4 ? TileCosts{0.46, 0.45, 1.83, 6.3, 15} : TileCosts{0.25, 0.36, 1.15, 3.75, 15};
     if (kind == 1 + fast::EK_TF32) return m.L == 4 ? TileCosts{0.27, 0.43, 1.32, 4.3, 15} : TileCosts{0.21, 0.35, 1.08, 3.1, 15};
@@ -139,8 +139,13 @@ DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us) {
     const double c8 = start + 0.65 * t.t16 * fullest(8, 16) * each, c16 = start + t.t16 * fullest(16, 16) * each, c32 = start + t.t32 * fullest(32, 32) * each;
     double big = 1e30;
     if (fast_tfdpa_supported(m, g)) {
-        const double n = f13 ? fullest(fast::BM, m.acc != ACC_F16 && !g.k_chunk ? 128 : fast::BN) : fullest(64, 64);
-        big = t.decode + t.large * (f13 || int64_t(n) % 2 == 0 ? n : n + 0.16 / n) * (f13 ? chunks : chunks + 0.5);
+        if (f13 && m.acc != ACC_F16) {
+            const double low = fast::f13_chunk_us(g, 64), tall = fast::f13_chunk_us(g, 128);
+            big = t.decode + t.large * (g.k_chunk || low < tall ? low : tall) * chunks;
+        } else {
+            const double n = f13 ? fullest(fast::BM, fast::BN) : fullest(64, 64);
+            big = t.decode + t.large * (f13 || int64_t(n) % 2 == 0 ? n : n + 0.16 / n) * (f13 ? chunks : chunks + 0.5);
+        }
     }
     if (us) *us = std::min(std::min(c8, c16), std::min(c32, big));
     if (big <= c8 && big <= c16 && big <= c32) return DIRECT_NONE;

@@ -120,6 +120,14 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t pari
     return false;
 }
 
+// What the fullest SM takes for 32 elements of K in the F = 13 kernels, in us: CTAs of 128 x 128 outputs two at a time 8.55, one alone
+// 4.7; of 128 x 64 4.55 and 2.65.  (Hopper E4M3, K = 2048, 128 x 64 / 128 x 128 in us: 512 x 1024 190 / 330, 640 x 1920 315 / 335,
+// 2048 x 2048 602 / 587, 2304 x 2304 742 / 862, 3072 x 3072 1157 / 1111.)
+inline double f13_chunk_us(const GemmArgs& g, int bn) {
+    const int64_t n = (((g.M + BM - 1) / BM) * ((g.N + bn - 1) / bn) + 147) / 148;
+    return bn == 128 ? double(n / 2) * 8.55 + double(n % 2) * 4.7 : double(n / 2) * 4.55 + double(n % 2) * 2.65;
+}
+
 // A CTA whose bounded wait on a bulk copy ran out (never in a healthy run) stores nothing and counts itself in the
 // library's device counter (GemmArgs::copy_timeouts), which mmasim_copy_timeouts() reads.
 

@@ -76,7 +76,8 @@ constexpr int TW = 8;                   // micro-tile: TH rows x 8 columns
 
 // Geometry by the height TH of the micro-tile.  TH = 4: warps 4 x 2, warp tile 32 x 32, CTA tile 128 x 64.
 // TH = 8: warps 2 x 4, warp tile 64 x 32, CTA tile 128 x 128 - sixteen operand words per 64 multiply-adds instead of
-// twelve per 32, at the price of 64 accumulator registers (used where nothing else has to live across the K loop).
+// twelve per 32, at the price of 64 accumulator registers (where nothing else has to live across the K loop, and the larger tiles
+// fill the SMs as well; see tall_tile).
 template <int TH>
 struct Geo {
     static_assert(TH == 4 || TH == 8, "two or four accumulator fragments stacked");
@@ -110,6 +111,7 @@ struct SmemT {
     BlkT<BM> a[2];
     BlkT<Geo<TH>::BN> b[2];
     unsigned long long full[2];         // mbarriers: the bulk copies of a buffer have landed
+    unsigned long long flags[3][NT];    // per thread: outputs (bit h * TW + x) that have seen a NaN, +infinity, -infinity
     int error;                          // a bounded wait ran out
 };
 
@@ -274,9 +276,15 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
     }
 
     uint32_t cw[TH][TW];
-    mask_t sp_nan = 0, sp_pinf = 0, sp_ninf = 0;        // per output (bit h * TW + x)
+    // The sticky flags wait in shared memory: six registers that only rare events touch (90 bytes of spills with them, 48 without; 4096^3
+    // 3828 -> 3746 us).
+    volatile unsigned long long* const flags = &sm.flags[0][tid];
+    enum { NAN_SEEN = 0, PINF = NT, NINF = 2 * NT };
+    flags[NAN_SEEN] = flags[PINF] = flags[NINF] = 0ull;
+    auto note = [&](int which, int h, int x) { flags[which] = flags[which] | 1ull << (h * TW + x); };
     float promoted[PROMOTE ? TH : 1][PROMOTE ? TW : 1];
     int big = 0;
+#define MMASIM_SP_LOAD const mask_t sp_nan = mask_t(flags[NAN_SEEN]), sp_pinf = mask_t(flags[PINF]), sp_ninf = mask_t(flags[NINF])
 #define MMASIM_SP_GET(h, x) (uint32_t((sp_nan >> ((h) * TW + (x))) & 1u) | (uint32_t((sp_pinf >> ((h) * TW + (x))) & 1u) << 1) | (uint32_t((sp_ninf >> ((h) * TW + (x))) & 1u) << 2))
 #define MMASIM_SP_WORD(h, x, w) (MMASIM_SP_GET(h, x) ? special_word(((MMASIM_SP_GET(h, x) & 1u) || (MMASIM_SP_GET(h, x) & 6u) == 6u) ? 1 : ((MMASIM_SP_GET(h, x) & 2u) ? 2 : 3), ACC16, true) : (w))
 #pragma unroll
@@ -291,8 +299,7 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
             if (PROMOTE) { promoted[PROMOTE ? h : 0][PROMOTE ? x : 0] = __uint_as_float(w); w = 0u; }
             const AccDec d = decode_acc(w, ACC16);
             if (d.cls != CLS_FINITE) {
-                const mask_t bit = mask_t(1) << (h * TW + x);
-                if (d.cls == CLS_NAN) sp_nan |= bit; else if (d.sign) sp_ninf |= bit; else sp_pinf |= bit;
+                note(d.cls == CLS_NAN ? NAN_SEEN : (d.sign ? NINF : PINF), h, x);
                 w = 0u;
             }
             // an FP32 accumulator enters with the bits that its own exponent keeps (units of 2^(Exp(c) - F): the first block's are as
@@ -331,10 +338,9 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
                             const uint32_t yb = decode_elem(fb, raw_elem<EK>(g.B, j * g.ldb + first + kk));
                             ev.product(xa, yb);
                         }
-                        const mask_t bit = mask_t(1) << (h * TW + x);
-                        if (ev.nan) sp_nan |= bit;
-                        if (ev.pinf) sp_pinf |= bit;
-                        if (ev.ninf) sp_ninf |= bit;
+                        if (ev.nan) note(NAN_SEEN, h, x);
+                        if (ev.pinf) note(PINF, h, x);
+                        if (ev.ninf) note(NINF, h, x);
                     }
             }
 
@@ -449,7 +455,10 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
                     }
             }
             // ---- pass 2: one fused multiply-add per term, rounding toward minus infinity onto the grid of S; two
-            // columns of the micro-tile per instruction (fma.rm.f32x2: lanes (a_h, a_h) x (b_x, b_x+1) + (S_h,x, S_h,x+1)) ----
+            // columns of the micro-tile per instruction (fma.rm.f32x2: lanes (a_h, a_h) x (b_x, b_x+1) + (S_h,x, S_h,x+1)).
+            // The columns are walked to and fro: every instruction shares its a or its b with the one before, which saves reads of
+            // the register file, the packed instruction's bound beside its own pipe (five 32-bit reads in two cycles that have four):
+            // 4096^3 3839 -> 3709 us; b kept for all rows instead of a 3735, to and fro that way 3790 ----
             {
                 unsigned long long acc[TH][TW / 2];
 #pragma unroll
@@ -473,8 +482,10 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
                         unsigned long long oav;
                         asm("mov.b64 %0, {%1, %1};" : "=l"(oav) : "f"(oas[h]));
 #pragma unroll
-                        for (int xp = 0; xp < TW / 2; ++xp)
+                        for (int xq = 0; xq < TW / 2; ++xq) {
+                            const int xp = (h & 1) ? TW / 2 - 1 - xq : xq;
                             asm("fma.rm.f32x2 %0, %1, %2, %0;" : "+l"(acc[h][xp]) : "l"(oav), "l"(obv[xp]));
+                        }
                     }
                 }
 #pragma unroll
@@ -525,8 +536,7 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
 #pragma unroll
                     for (int x = 0; x < TW; ++x)
                         if ((cw[h][x] & 0x7FFFu) == 0x7C00u) {
-                            const mask_t bit = mask_t(1) << (h * TW + x);
-                            if (!((sp_nan | sp_pinf | sp_ninf) & bit)) { if (cw[h][x] >> 15) sp_ninf |= bit; else sp_pinf |= bit; }
+                            if (!((flags[NAN_SEEN] | flags[PINF] | flags[NINF]) >> (h * TW + x) & 1ull)) note(cw[h][x] >> 15 ? NINF : PINF, h, x);
                             cw[h][x] = 0u;
                         }
             }
@@ -535,17 +545,25 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
         if (*reinterpret_cast<volatile int*>(&sm.error)) break;
         if (tid == 0 && chunk + 2 < NCH) issue(chunk + 2);
         if (PROMOTE && ((k0 + KC) % int(g.k_chunk)) == 0) {     // FP32 promotion of the partial sum every k_chunk elements
+            MMASIM_SP_LOAD;
+            if (sp_nan | sp_pinf | sp_ninf) {                  // (rare: the flags of 32 outputs one by one cost as much as a block of 32)
+#pragma unroll
+                for (int h = 0; h < TH; ++h)
+#pragma unroll
+                    for (int x = 0; x < TW; ++x) cw[h][x] = MMASIM_SP_WORD(h, x, cw[h][x]);
+            }
 #pragma unroll
             for (int h = 0; h < TH; ++h)
 #pragma unroll
                 for (int x = 0; x < TW; ++x) {
-                    const float part = __uint_as_float(MMASIM_SP_WORD(h, x, positive_zero(cw[h][x] & RHO_MASK, 0x7FFFFFFFu)));
+                    // (a NaN's word may lose low bits: every NaN becomes the same below)
+                    const float part = __uint_as_float(positive_zero(cw[h][x] & RHO_MASK, 0x7FFFFFFFu));
                     float v = __fadd_rn(promoted[PROMOTE ? h : 0][PROMOTE ? x : 0], part);
                     if (v != v) v = __uint_as_float(0x7FFFFFFFu);
                     promoted[PROMOTE ? h : 0][PROMOTE ? x : 0] = v;
                     cw[h][x] = 0u;
                 }
-            sp_nan = sp_pinf = sp_ninf = 0;
+            flags[NAN_SEEN] = flags[PINF] = flags[NINF] = 0ull;
         }
     }
 
@@ -557,6 +575,7 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
         }
         return;
     }
+    MMASIM_SP_LOAD;
 #pragma unroll
     for (int h = 0; h < TH; ++h)
 #pragma unroll
@@ -576,6 +595,7 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
             if (ACC16) static_cast<uint16_t*>(g.D)[i * g.ldd + j] = uint16_t(w);
             else static_cast<uint32_t*>(g.D)[i * g.ldd + j] = w;
         }
+#undef MMASIM_SP_LOAD
 #undef MMASIM_SP_GET
 #undef MMASIM_SP_WORD
 }
@@ -624,10 +644,16 @@ cudaError_t launch_one_t(const DevModel& m, const GemmArgs& g, cudaStream_t stre
     return err != cudaSuccess ? err : err2;
 }
 
-// The tall micro-tile where the registers allow it: FP32 accumulators without promoted partial sums beside them.
-inline bool tall_tile(const DevModel& m, const GemmArgs& g) { return m.rho != RHO_RNE_FP16 && !g.k_chunk; }
+// The tall micro-tile (128 x 128 outputs per CTA) or the short one (128 x 64)?  RNE-FP16 and promoted partial sums: the short one, they
+// need the registers.  Otherwise what the fullest SM does decides; in given memory always the tall one, so that what fits there does
+// not depend on the number of SMs.
+inline bool tall_tile(const DevModel& m, const GemmArgs& g, bool given) {
+    if (m.rho == RHO_RNE_FP16 || g.k_chunk) return false;
+    return given || fast::f13_chunk_us(g, 128) < fast::f13_chunk_us(g, 64);
+}
+// (of a call in given memory)
 inline size_t scratch_bytes(const DevModel& m, const GemmArgs& g) {
-    return tall_tile(m, g) ? scratch_bytes_one<8>(g) : scratch_bytes_one<4>(g);
+    return tall_tile(m, g, true) ? scratch_bytes_one<8>(g) : scratch_bytes_one<4>(g);
 }
 
 template <int EK, int L, int F, int RHO, int BASE>
@@ -636,7 +662,8 @@ cudaError_t launch_variant_t(const DevModel& m, const GemmArgs& g, cudaStream_t 
         return launch_one_t<EK, L, F, RHO, false, BASE, 4>(m, g, stream, sc);
     } else {
         if (g.k_chunk) return launch_one_t<EK, L, F, RHO, true, BASE, 4>(m, g, stream, sc);
-        return launch_one_t<EK, L, F, RHO, false, BASE, 8>(m, g, stream, sc);
+        if (tall_tile(m, g, sc.given != nullptr)) return launch_one_t<EK, L, F, RHO, false, BASE, 8>(m, g, stream, sc);
+        return launch_one_t<EK, L, F, RHO, false, BASE, 4>(m, g, stream, sc);
     }
 }
 
