@@ -770,6 +770,7 @@ __device__ __forceinline__ void direct_tile(const DevModel& m, const GemmArgs& g
 
 template <int FAM, int EK, int L, int RHO, bool PROMOTE, int TM, int CN, int WR, int WC, int PW, int TASK>
 __global__ void __launch_bounds__(32 * (WR * WC + PW), min_ctas(TM * CN, L, WR * WC + PW)) direct_kernel(DevModel m, GemmArgs g, int unit_a, int unit_b) {
+    after_previous();
     direct_tile<FAM, EK, L, RHO, PROMOTE, TM, CN, WR, WC, PW, TASK>(m, g, unit_a, unit_b, int64_t(blockIdx.y) * (8 * TM * WR), int64_t(blockIdx.x) * (8 * CN * WC));
 }
 
@@ -777,6 +778,7 @@ __global__ void __launch_bounds__(32 * (WR * WC + PW), min_ctas(TM * CN, L, WR *
 // none, and every CTA reads the flags and leaves (1024 x 4096: a CTA per tile that looked for itself took 18 us).
 template <int FAM, int EK, int L, int RHO, int TM, int CN, int WR, int WC, int PW, int TASK>
 __global__ void __launch_bounds__(32 * (WR * WC + PW), min_ctas(TM * CN, L, WR * WC + PW)) direct_rest_kernel(DevModel m, GemmArgs g, int unit_a, int unit_b) {
+    after_previous();
     constexpr int BM = 8 * TM * WR, BN = 8 * CN * WC;
     const int64_t flags = (g.N + 127) / 128 * g.redo_across;
     int any = 0;
@@ -809,8 +811,7 @@ cudaError_t launch_tile(const DevModel& m, const GemmArgs& g, cudaStream_t st) {
         if (err != cudaSuccess) return err;
     }
     const dim3 grid((unsigned)((g.N + BN - 1) / BN), (unsigned)((g.M + BM - 1) / BM), 1);
-    kernel<<<grid, NTH, sh, st>>>(m, g, copy_unit<EK, TASK>(g.lda), copy_unit<EK, TASK>(g.ldb));
-    return cudaGetLastError();
+    return enqueue(kernel, grid, NTH, sh, st, m, g, copy_unit<EK, TASK>(g.lda), copy_unit<EK, TASK>(g.ldb));
 }
 
 template <int FAM, int EK, int L, int RHO>
@@ -821,8 +822,7 @@ cudaError_t launch_rest(const DevModel& m, const GemmArgs& g, cudaStream_t st) {
     const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sh));
     if (err != cudaSuccess) return err;
     const int64_t tiles = (g.M + 31) / 32 * ((g.N + 31) / 32);
-    kernel<<<unsigned(tiles < 296 ? tiles : 296), NTH, sh, st>>>(m, g, copy_unit<EK, TASK>(g.lda), copy_unit<EK, TASK>(g.ldb));
-    return cudaGetLastError();
+    return enqueue(kernel, unsigned(tiles < 296 ? tiles : 296), NTH, sh, st, m, g, copy_unit<EK, TASK>(g.lda), copy_unit<EK, TASK>(g.ldb));
 }
 
 // Accumulator tiles per warp, warps and staging warps per CTA for each size (chosen by direct_size in mmasim_tfdpa_fast.cu).

@@ -353,6 +353,7 @@ __device__ __forceinline__ uint32_t tfdpa8_dot(const Rows& rows, int K, uint32_t
 // One dot product per thread through `body(rows, c)`.
 template <int BYTES, bool ACC16, bool STAGED, class Body>
 __device__ __forceinline__ void one_dot(unsigned char* smem, int64_t n, int64_t K, const void* A, const void* B, const void* C, void* D, Body body) {
+    after_previous();
     const int row_bytes = int(K) * BYTES;
     if (STAGED) {
         staged_tile<ACC16>(smem, n, row_bytes, A, B, C, D, [&](const StagedRows& rows, int64_t, uint32_t c) { return body(rows, c); });
@@ -462,8 +463,7 @@ cudaError_t launch_dot(Kernel kernel, bool staged, int64_t n, int64_t row_bytes,
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
         if (e != cudaSuccess) return e;
     }
-    kernel<<<blocks, DOT_THREADS, smem, st>>>(args...);
-    return cudaGetLastError();
+    return enqueue(kernel, blocks, DOT_THREADS, smem, st, args...);
 }
 
 template <int EK, int L, int RHO>

@@ -56,6 +56,7 @@ __global__ void __launch_bounds__(NT, 2) efdpa64_kernel(DevModel m, GemmArgs g, 
     const int NCH = int((g.K + KC - 1) / KC);
     const Blk64<BM, EXP_NONE>* src_a = wa + int64_t(tile_m) * NCH;
     const Blk64<BN, EXP_NONE>* src_b = wb + int64_t(tile_n) * NCH;
+    after_previous();
     auto issue = [&](int n) {                              // one thread: both copies of chunk n into buffer n & 1
         unsigned long long* bar = &sm.full[n & 1];
         fast::mbar_expect_tx(bar, uint32_t(sizeof(Blk64<BM, EXP_NONE>) + sizeof(Blk64<BN, EXP_NONE>)));
@@ -203,29 +204,7 @@ __global__ void __launch_bounds__(NT, 2) efdpa64_kernel(DevModel m, GemmArgs g, 
 
 template <int EK, int L>
 cudaError_t launch_e_one(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
-    const size_t sh = sizeof(SmemMM<EXP_NONE>);
-    cudaError_t err = cudaFuncSetAttribute(efdpa64_kernel<EK, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sh));
-    if (err != cudaSuccess) return err;
-    const size_t dsh_a = 256 * sizeof(LutEntry64) + sizeof(Blk64<BM, EXP_NONE>), dsh_b = 256 * sizeof(LutEntry64) + sizeof(Blk64<BN, EXP_NONE>);
-    if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BM, true, 0, false, false, EXP_NONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_a))) != cudaSuccess) return err;
-    if ((err = cudaFuncSetAttribute(decode64_kernel<EK, BN, false, 0, false, false, EXP_NONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dsh_b))) != cudaSuccess) return err;
-    const int64_t tiles_m = (g.M + BM - 1) / BM, tiles_n = (g.N + BN - 1) / BN, nch = (g.K + KC - 1) / KC;
-    // scratch: the decoded blocks of A and B, stream-ordered out of the library's pool and returned to it behind the kernel
-    const size_t bytes_a = size_t(tiles_m * nch) * sizeof(Blk64<BM, EXP_NONE>), bytes_b = size_t(tiles_n * nch) * sizeof(Blk64<BN, EXP_NONE>);
-    cudaMemPool_t pool = nullptr;
-    if ((err = scratch_pool(&pool)) != cudaSuccess) return err;
-    void* ws = nullptr;
-    if ((err = cudaMallocFromPoolAsync(&ws, bytes_a + bytes_b, pool, stream)) != cudaSuccess) return err;
-    Blk64<BM, EXP_NONE>* wa = static_cast<Blk64<BM, EXP_NONE>*>(ws);
-    Blk64<BN, EXP_NONE>* wb = reinterpret_cast<Blk64<BN, EXP_NONE>*>(static_cast<unsigned char*>(ws) + bytes_a);
-    decode64_kernel<EK, BM, true, 0, false, false, EXP_NONE><<<unsigned(nch * tiles_m), 256, dsh_a, stream>>>(
-        m, static_cast<const unsigned char*>(g.A), g.M, g.lda, unsigned(nch), fast::pad_of<EK>(g.K, g.lda), wa);
-    decode64_kernel<EK, BN, false, 0, false, false, EXP_NONE><<<unsigned(nch * tiles_n), 256, dsh_b, stream>>>(
-        m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, unsigned(nch), fast::pad_of<EK>(g.K, g.ldb), wb);
-    efdpa64_kernel<EK, L><<<unsigned(tiles_n * tiles_m), NT, sh, stream>>>(m, g, wa, wb);
-    err = cudaGetLastError();
-    const cudaError_t err2 = cudaFreeAsync(ws, stream);
-    return err != cudaSuccess ? err : err2;
+    return decode_and_run<EK, 0, false, false, EXP_NONE>(efdpa64_kernel<EK, L>, m, g, false, stream);
 }
 
 }  // namespace

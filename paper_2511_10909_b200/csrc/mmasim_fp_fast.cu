@@ -52,6 +52,7 @@ __device__ __forceinline__ float load_flushed(uint32_t w, bool bf16) {
 enum Rows : int { ROWS_ANY = 0, ROWS_16, ROWS_WHOLE };
 template <int MODE, int P, int TM, int TN, int KC, int ROWS>
 __global__ void __launch_bounds__(NT, TM >= 8 ? 2 : 3) fp_kernel(GemmArgs g) {
+    after_previous();
     using T = ModeTraits<MODE>;
     using in_t = float;
     using acc_t = float;
@@ -226,6 +227,7 @@ struct Stage {
 // multiple of a chunk (the test for it in every chunk cost 2048 x 2048 x 2048 684 instead of 620 us).
 template <int WR, int WC, int TI, int TJ, int UNIT, bool TAIL>
 __global__ void __launch_bounds__(32 * WR * WC, 2) fma64_mma_kernel(GemmArgs g) {
+    after_previous();
     using namespace dm;
     constexpr int BM = 8 * WR * TI, BN = 8 * WC * TJ, DNT = 32 * WR * WC, SEGS = DKC * 8 / UNIT, PER = UNIT / 8;
     using ST = Stage<BM, BN>;
@@ -332,8 +334,7 @@ cudaError_t launch_fma64_tile(const GemmArgs& g, cudaStream_t stream) {
                                             : (g.K % dm::DKC ? fma64_mma_kernel<WR, WC, TI, TJ, 16, true> : fma64_mma_kernel<WR, WC, TI, TJ, 16, false>);
     const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sh));
     if (err != cudaSuccess) return err;
-    kernel<<<dim3(unsigned(up_div(g.N, BN)), unsigned(up_div(g.M, BM))), 32 * WR * WC, sh, stream>>>(g);
-    return cudaGetLastError();
+    return enqueue(kernel, dim3(unsigned(up_div(g.N, BN)), unsigned(up_div(g.M, BM))), 32 * WR * WC, sh, stream, g);
 }
 cudaError_t launch_fma64_mma(const GemmArgs& g, cudaStream_t stream) {
     const bool small = use_small(g, 128, 64, 32, 32, 1.15);
@@ -345,10 +346,9 @@ template <int MODE, int P, int TM, int TN, int KC>
 cudaError_t launch_fp_tile(const GemmArgs& g, cudaStream_t stream) {
     constexpr int B = ModeTraits<MODE>::IN_BYTES;
     const dim3 grid(unsigned(up_div(g.N, 16 * TN)), unsigned(up_div(g.M, 16 * TM)), 1);
-    if ((g.lda * B) % 16 || (g.ldb * B) % 16) fp_kernel<MODE, P, TM, TN, KC, ROWS_ANY><<<grid, NT, 0, stream>>>(g);
-    else if (g.K % KC) fp_kernel<MODE, P, TM, TN, KC, ROWS_16><<<grid, NT, 0, stream>>>(g);
-    else fp_kernel<MODE, P, TM, TN, KC, ROWS_WHOLE><<<grid, NT, 0, stream>>>(g);
-    return cudaGetLastError();
+    if ((g.lda * B) % 16 || (g.ldb * B) % 16) return enqueue(fp_kernel<MODE, P, TM, TN, KC, ROWS_ANY>, grid, NT, 0, stream, g);
+    if (g.K % KC) return enqueue(fp_kernel<MODE, P, TM, TN, KC, ROWS_16>, grid, NT, 0, stream, g);
+    return enqueue(fp_kernel<MODE, P, TM, TN, KC, ROWS_WHOLE>, grid, NT, 0, stream, g);
 }
 template <int MODE, int P>
 cudaError_t launch_fp(const GemmArgs& g, cudaStream_t stream) {

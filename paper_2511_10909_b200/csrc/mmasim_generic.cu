@@ -56,6 +56,7 @@ __device__ __forceinline__ float canonical_nan_nv(float x) { return (x != x) ? _
 __global__ void __launch_bounds__(GEN_THREADS)
 fdpa_generic_kernel(DevModel m, GemmArgs g, int rows, int KC, int L) {
     extern __shared__ uint32_t smem[];
+    after_previous();
     const int stride = KC + 1;
     uint32_t* As = smem;
     uint32_t* Bs = As + rows * stride;
@@ -162,6 +163,7 @@ __device__ __forceinline__ float ftz_load(uint32_t w, bool is_bf16) {
 __global__ void __launch_bounds__(GEN_THREADS)
 ftz_generic_kernel(DevModel m, GemmArgs g, int rows, int KC) {
     extern __shared__ uint32_t smem[];
+    after_previous();
     const int stride = KC + 1;
     float* As = reinterpret_cast<float*>(smem);
     float* Bs = As + rows * stride;
@@ -210,6 +212,7 @@ template <typename T>
 __global__ void __launch_bounds__(GEN_THREADS)
 fma_generic_kernel(GemmArgs g, int rows, int KC) {
     extern __shared__ uint32_t smem[];
+    after_previous();
     const int stride = KC + 1;
     T* As = reinterpret_cast<T*>(smem);
     T* Bs = As + rows * stride;
@@ -259,18 +262,18 @@ int launch_generic(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
         if (m.acc == ACC_F64) {
             const size_t sh = size_t(2) * rows * (KC + 1) * sizeof(double);
             err = cudaFuncSetAttribute(fma_generic_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-            if (err == cudaSuccess) fma_generic_kernel<double><<<grid, GEN_THREADS, sh, stream>>>(g, rows, KC);
+            if (err == cudaSuccess) err = enqueue(fma_generic_kernel<double>, grid, GEN_THREADS, sh, stream, g, rows, KC);
         } else {
             const size_t sh = size_t(2) * rows * (KC + 1) * sizeof(float);
             err = cudaFuncSetAttribute(fma_generic_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-            if (err == cudaSuccess) fma_generic_kernel<float><<<grid, GEN_THREADS, sh, stream>>>(g, rows, KC);
+            if (err == cudaSuccess) err = enqueue(fma_generic_kernel<float>, grid, GEN_THREADS, sh, stream, g, rows, KC);
         }
     } else if (m.family == FAM_FTZ) {
         int KC = int(g.K < kmax ? g.K : kmax);
         KC -= KC % m.P;
         const size_t sh = size_t(2) * rows * (KC + 1) * sizeof(float);
         err = cudaFuncSetAttribute(ftz_generic_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-        if (err == cudaSuccess) ftz_generic_kernel<<<grid, GEN_THREADS, sh, stream>>>(m, g, rows, KC);
+        if (err == cudaSuccess) err = enqueue(ftz_generic_kernel, grid, GEN_THREADS, sh, stream, m, g, rows, KC);
     } else {
         const int L = int(g.K < m.L ? g.K : m.L);
         int KC = L * (kmax / L > 0 ? kmax / L : 1);
@@ -278,9 +281,8 @@ int launch_generic(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
         const int nsf_chunk = m.k_block ? (KC + m.k_block - 1) / m.k_block : 0;
         const size_t sh = (size_t(2) * rows * (KC + 1) + size_t(2) * rows * (nsf_chunk + 1)) * sizeof(uint32_t);
         err = cudaFuncSetAttribute(fdpa_generic_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        if (err == cudaSuccess) fdpa_generic_kernel<<<grid, GEN_THREADS, sh, stream>>>(m, g, rows, KC, L);
+        if (err == cudaSuccess) err = enqueue(fdpa_generic_kernel, grid, GEN_THREADS, sh, stream, m, g, rows, KC, L);
     }
-    if (err == cudaSuccess) err = cudaGetLastError();
     if (err != cudaSuccess) {
         set_error("generic kernel launch failed: %s", cudaGetErrorString(err));
         return MMASIM_ERR_CUDA;

@@ -71,6 +71,7 @@ __device__ __forceinline__ uint32_t nonzero16(uint32_t w0, uint32_t w1) { return
 
 template <bool NVF4>
 __global__ void __launch_bounds__(NT, 2) gst_kernel(DevModel m, GemmArgs g) {
+    after_previous();
     constexpr int F = 35;
     constexpr int FRAC = NVF4 ? 8 : 2;              // fractional bits of p_g * Sig(alpha) * Sig(beta)
     constexpr int SPB = NVF4 ? 4 : 2;               // scale factors per block of 64 and row
@@ -298,10 +299,10 @@ int launch_fast_gst(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
     cudaError_t err;
     if (m.scale_fmt == EF_UE4M3) {
         err = cudaFuncSetAttribute(gst_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sh));
-        if (err == cudaSuccess) { gst_kernel<true><<<grid, NT, sh, stream>>>(m, g); err = cudaGetLastError(); }
+        if (err == cudaSuccess) err = enqueue(gst_kernel<true>, grid, NT, sh, stream, m, g);
     } else {
         err = cudaFuncSetAttribute(gst_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sh));
-        if (err == cudaSuccess) { gst_kernel<false><<<grid, NT, sh, stream>>>(m, g); err = cudaGetLastError(); }
+        if (err == cudaSuccess) err = enqueue(gst_kernel<false>, grid, NT, sh, stream, m, g);
     }
     if (err != cudaSuccess) {
         set_error("GST-FDPA kernel launch failed: %s", cudaGetErrorString(err));

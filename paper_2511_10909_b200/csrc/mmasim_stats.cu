@@ -25,6 +25,7 @@ __device__ __forceinline__ double warp_max(double v) {
 
 template <bool ACC16>
 __global__ void __launch_bounds__(256) stats_kernel(int64_t n, const void* D, const double* ref, double* stats) {
+    after_previous();
     double cnt = 0.0, sum = 0.0, sabs = 0.0, ssq = 0.0, nneg = 0.0, npos = 0.0, mx = 0.0, srel = 0.0;
 #pragma unroll 4
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
@@ -83,6 +84,7 @@ __device__ __forceinline__ double widen_one(int fmt, const void* p, int64_t i) {
     }
 }
 __global__ void __launch_bounds__(256) widen_kernel(Widen a, Widen b, Widen c) {
+    after_previous();
     const Widen w = blockIdx.y == 0 ? a : (blockIdx.y == 1 ? b : c);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -98,9 +100,7 @@ int launch_error_stats(int acc, int64_t n, const void* D, const double* ref, dou
     if (acc != ACC_F32 && acc != ACC_F16) { set_error("mmasim_error_stats: the accumulator format must be FP32 or FP16"); return MMASIM_ERR_INVALID_ARG; }
     const int64_t want = (n + 255) / 256;
     const unsigned blocks = unsigned(want < 148 * 4 ? want : 148 * 4);
-    if (acc == ACC_F16) stats_kernel<true><<<blocks, 256, 0, stream>>>(n, D, ref, stats);
-    else stats_kernel<false><<<blocks, 256, 0, stream>>>(n, D, ref, stats);
-    const cudaError_t err = cudaGetLastError();
+    const cudaError_t err = enqueue(acc == ACC_F16 ? stats_kernel<true> : stats_kernel<false>, blocks, 256, 0, stream, n, D, ref, stats);
     if (err != cudaSuccess) { set_error("mmasim_error_stats launch failed: %s", cudaGetErrorString(err)); return MMASIM_ERR_CUDA; }
     return MMASIM_OK;
 }
@@ -116,8 +116,7 @@ int launch_reference_fp64(int fmt, int acc, int64_t M, int64_t N, int64_t K, con
     if (err == cudaSuccess) {
         const Widen wa = {A, scratch + a_at, na, fmt}, wb = {B, scratch + b_at, nb, fmt}, wc = {C, scratch + c_at, nc, acc == ACC_F16 ? EF_F16 : EF_F32};
         const int64_t most = na > nb ? (na > nc ? na : nc) : (nb > nc ? nb : nc);
-        widen_kernel<<<dim3(unsigned((most + 2047) / 2048), C ? 3 : 2), 256, 0, stream>>>(wa, wb, wc);
-        err = cudaGetLastError();
+        err = enqueue(widen_kernel, dim3(unsigned((most + 2047) / 2048), C ? 3 : 2), 256, 0, stream, wa, wb, wc);
     }
     if (err == cudaSuccess) {
         DevModel m;

@@ -184,21 +184,24 @@ __device__ __forceinline__ uint32_t stage_row(const LutEntryT* lut, BlkT<R>& s, 
 // takes 16 (R = 128) or 8 (R = 64) consecutive elements of one row.  Rows beyond the matrix repeat the last one (their outputs are
 // not stored, but as zeros they would take the rare paths); the elements in front that fill K up to whole chunks decode as zeros.
 static_assert(BM == 128 && KC == 32 && NT == 256, "the task split of the decode pass");
+template <int R>
+struct SideT {
+    const unsigned char* src;
+    int64_t rows, ld;
+    fast::Pad pad;
+    BlkT<R>* dst;
+};
 template <int BASE, int R, bool IS_A, int TH>
-__global__ void __launch_bounds__(NT) trop_decode_kernel(DevModel m, const unsigned char* src, int64_t rows, int64_t ld, int F,
-                                                         fast::Pad pad, BlkT<R>* dst) {
-    __shared__ __align__(16) LutEntryT lut_a[256];
-    __shared__ __align__(16) LutEntryT lut_b[256];
-    __shared__ __align__(16) BlkT<R> blk;
+__device__ __forceinline__ void decode_t(const DevModel& m, const SideT<R>& side, int F, LutEntryT* lut_a, LutEntryT* lut_b, BlkT<R>& blk, unsigned tile) {
     const int tid = threadIdx.x;
     const FmtDesc fa = fmt_desc(m.fmt_a), fb = fmt_desc(m.fmt_b);
     init_lut_t<BASE>(lut_a, lut_b, fa, fb, F - (fa.mbits + fb.mbits), fa.mbits + 1, tid);
     if (tid == 0) { blk.special = blk.sparse = 0u; blk.pad[0] = blk.pad[1] = 0u; }
     constexpr int N = R * KC / NT;                      // elements per thread: 16 or 8
     const int r = tid % R, part = tid / R;
-    const int64_t i = int64_t(blockIdx.y) * R + r, k0 = int64_t(blockIdx.x) * KC - pad.front;
+    const int64_t i = min(int64_t(tile) * R + r, side.rows - 1), k0 = int64_t(blockIdx.x) * KC - side.pad.front;
     uint32_t w[N / 4];
-    fast::load_task<fast::EK_LUT8>(w, src, min(i, rows - 1) * ld, k0 + N * part, pad.wide);
+    fast::load_task<fast::EK_LUT8>(w, side.src, i * side.ld, k0 + N * part, side.pad.wide);
     __syncthreads();
     const uint32_t spec = stage_row<N, R>(IS_A ? lut_a : lut_b, blk, w, r, IS_A ? perm_row<TH>(r) : perm_col(r), part);
     if (spec & 0x8000u) atomicOr(&blk.special, 1u);
@@ -206,9 +209,19 @@ __global__ void __launch_bounds__(NT) trop_decode_kernel(DevModel m, const unsig
     // parts with less than half of theirs add up to one)
     if ((spec >> 16) * 2 >= uint32_t(N)) atomicOr(&blk.sparse, 1u);
     __syncthreads();
-    uint4* out = reinterpret_cast<uint4*>(dst + (int64_t(blockIdx.y) * gridDim.x + blockIdx.x));
+    uint4* out = reinterpret_cast<uint4*>(side.dst + (int64_t(tile) * gridDim.x + blockIdx.x));
     const uint4* in = reinterpret_cast<const uint4*>(&blk);
     for (int q = tid; q < int(sizeof(BlkT<R>) / 16); q += NT) out[q] = in[q];
+}
+// Both operands in one launch: the tile rows of A, then the tile columns of B (blockIdx.y).
+template <int BASE, int TH>
+__global__ void __launch_bounds__(NT) trop_decode_kernel(DevModel m, SideT<BM> a, SideT<Geo<TH>::BN> b, int F, unsigned tiles_a) {
+    __shared__ __align__(16) LutEntryT lut_a[256];
+    __shared__ __align__(16) LutEntryT lut_b[256];
+    __shared__ __align__(16) unsigned char blk[sizeof(BlkT<BM>)];
+    after_previous();
+    if (blockIdx.y < tiles_a) decode_t<BASE, BM, true, TH>(m, a, F, lut_a, lut_b, *reinterpret_cast<BlkT<BM>*>(blk), blockIdx.y);
+    else decode_t<BASE, Geo<TH>::BN, false, TH>(m, b, F, lut_a, lut_b, *reinterpret_cast<BlkT<Geo<TH>::BN>*>(blk), blockIdx.y - tiles_a);
 }
 
 
@@ -260,6 +273,7 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
     const int NCH = int((g.K + KC - 1) / KC);
     const BlkT<BM>* src_a = wa + int64_t(blockIdx.y) * NCH;
     const BlkT<BN>* src_b = wb + int64_t(blockIdx.x) * NCH;
+    after_previous();
     auto issue = [&](int n) {                              // one thread: both copies of chunk n into buffer n & 1
         unsigned long long* bar = &sm.full[n & 1];
         mbar_expect_tx(bar, uint32_t(sizeof(BlkT<BM>) + sizeof(BlkT<BN>)));
@@ -632,13 +646,16 @@ cudaError_t launch_one_t(const DevModel& m, const GemmArgs& g, cudaStream_t stre
     }
     BlkT<BM>* wa = static_cast<BlkT<BM>*>(ws);
     BlkT<BN>* wb = reinterpret_cast<BlkT<BN>*>(static_cast<unsigned char*>(ws) + bytes_a);
-    trop_decode_kernel<BASE, BM, true, TH><<<dim3((unsigned)nch, (unsigned)tiles_m), NT, 0, stream>>>(
-        m, static_cast<const unsigned char*>(g.A), g.M, g.lda, F, fast::pad_of<fast::EK_LUT8>(g.K, g.lda), wa);
-    trop_decode_kernel<BASE, BN, false, TH><<<dim3((unsigned)nch, (unsigned)tiles_n), NT, 0, stream>>>(
-        m, static_cast<const unsigned char*>(g.B), g.N, g.ldb, F, fast::pad_of<fast::EK_LUT8>(g.K, g.ldb), wb);
-    dim3 grid((unsigned)tiles_n, (unsigned)tiles_m, 1);
-    tfdpa_trop_kernel<EK, L, F, RHO, PROMOTE, BASE, TH><<<grid, NT, sh, stream>>>(m, g, wa, wb);
-    err = cudaGetLastError();
+    const SideT<BM> a{static_cast<const unsigned char*>(g.A), g.M, g.lda, fast::pad_of<fast::EK_LUT8>(g.K, g.lda), wa};
+    const SideT<BN> b{static_cast<const unsigned char*>(g.B), g.N, g.ldb, fast::pad_of<fast::EK_LUT8>(g.K, g.ldb), wb};
+    // (blockIdx.y has 65535 values: what does not fit goes in two launches)
+    auto decode = trop_decode_kernel<BASE, TH>;
+    if (tiles_m + tiles_n <= 65535) err = enqueue(decode, dim3((unsigned)nch, (unsigned)(tiles_m + tiles_n)), NT, 0, stream, m, a, b, F, unsigned(tiles_m));
+    else {
+        err = enqueue(decode, dim3((unsigned)nch, (unsigned)tiles_m), NT, 0, stream, m, a, b, F, unsigned(tiles_m));
+        if (err == cudaSuccess) err = enqueue(decode, dim3((unsigned)nch, (unsigned)tiles_n), NT, 0, stream, m, a, b, F, 0u);
+    }
+    if (err == cudaSuccess) err = enqueue(tfdpa_trop_kernel<EK, L, F, RHO, PROMOTE, BASE, TH>, dim3((unsigned)tiles_n, (unsigned)tiles_m, 1), NT, sh, stream, m, g, wa, wb);
     if (sc.given) return err;
     const cudaError_t err2 = cudaFreeAsync(ws, stream);
     return err != cudaSuccess ? err : err2;

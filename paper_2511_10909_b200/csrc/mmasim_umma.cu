@@ -250,6 +250,7 @@ __global__ void __launch_bounds__(Layout<MK, BN>::NTHREADS, 1) umma_kernel(const
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    after_previous();
     const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, tmem_base_s, 0);
     // about a second, and longer for a K whose instructions alone take that long
     const long long budget = 2000000000ll + 4000ll * nst;
@@ -543,6 +544,7 @@ struct Side {
 };
 // One code per byte -> chunks of sixteen codes packed from bit 0 upwards, 16 bytes each; rows of ceil(K / 16) chunks.
 __global__ void __launch_bounds__(256) pack_codes_kernel(Side a, Side b, int K) {
+    after_previous();
     const Side s = blockIdx.y ? b : a;
     const int chunks = (K + 15) / 16;
     const int64_t q = int64_t(blockIdx.x) * 256 + threadIdx.x;
@@ -574,6 +576,7 @@ struct LeastSide {
 // 16-byte starts; `odd`: the last word holds one BF16 element only.
 template <bool BF16>
 __global__ void __launch_bounds__(256) least_exponent_kernel(LeastSide a, LeastSide b, int n, bool odd) {
+    after_previous();
     const LeastSide s = blockIdx.y ? b : a;
     const int64_t r = int64_t(blockIdx.x) * 8 + threadIdx.x / 32;
     if (r >= s.rows) return;
@@ -655,8 +658,7 @@ cudaError_t launch_tile(const CUtensorMap& l, const CUtensorMap& q, const UmmaAr
     auto kernel = umma_kernel<MK, BN, ACC16>;
     const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Layout<MK, BN>::SMEM);
     if (err != cudaSuccess) return err;
-    kernel<<<unsigned(a.tiles < SMS ? a.tiles : SMS), Layout<MK, BN>::NTHREADS, Layout<MK, BN>::SMEM, st>>>(l, q, a);
-    return cudaGetLastError();
+    return enqueue(kernel, unsigned(a.tiles < SMS ? a.tiles : SMS), Layout<MK, BN>::NTHREADS, Layout<MK, BN>::SMEM, st, l, q, a);
 }
 template <int MK, bool ACC16>
 cudaError_t launch_bn(int bn, const CUtensorMap& l, const CUtensorMap& q, const UmmaArgs& a, cudaStream_t st) {
@@ -769,17 +771,15 @@ int launch_umma(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
     const int64_t rows = g.M > g.N ? g.M : g.N;
     if (err == cudaSuccess && pa + pb) {
         const Side s[2] = {{A, pa ? scratch : nullptr, g.M, pitch_a, bits_a}, {B, pb ? scratch + pa : nullptr, g.N, pitch_b, bits_b}};
-        pack_codes_kernel<<<dim3(unsigned((rows * (pk / 16) + 255) / 256), 2), 256, 0, stream>>>(s[0], s[1], int(g.K));
-        err = cudaGetLastError();
+        err = enqueue(pack_codes_kernel, dim3(unsigned((rows * (pk / 16) + 255) / 256), 2), 256, 0, stream, s[0], s[1], int(g.K));
         if (pa) { A = s[0].dst; pitch_a = kb_a = pk; }
         if (pb) { B = s[1].dst; pitch_b = kb_b = pk; }
     }
     if (err == cudaSuccess && le) {
         const LeastSide sa{A, least, g.M, pitch_a}, sb{B, least + g.M, g.N, pitch_b};
         const dim3 grid(unsigned((rows + 7) / 8), 2);
-        if (mk == MK_TF32) least_exponent_kernel<false><<<grid, 256, 0, stream>>>(sa, sb, int(g.K), false);
-        else least_exponent_kernel<true><<<grid, 256, 0, stream>>>(sa, sb, int((g.K + 1) / 2), g.K % 2 != 0);
-        err = cudaGetLastError();
+        if (mk == MK_TF32) err = enqueue(least_exponent_kernel<false>, grid, 256, 0, stream, sa, sb, int(g.K), false);
+        else err = enqueue(least_exponent_kernel<true>, grid, 256, 0, stream, sa, sb, int((g.K + 1) / 2), g.K % 2 != 0);
     }
     if (err == cudaSuccess) {
         CUtensorMap ml, mq;
