@@ -122,6 +122,9 @@ int launch_gemm_noalloc(const DevModel& m, const GemmArgs& g, cudaStream_t strea
 // mmasim_umma.cu: the rows that the B200's own matrix instruction computes
 bool umma_supported(const DevModel& m, const GemmArgs& g);
 int launch_umma(const DevModel& m, const GemmArgs& g, cudaStream_t stream);
+// mmasim_warp_mma.cu: FP16 products of few rows (of those that umma_supported takes) on the warp-level instruction
+bool warp_mma_supported(const DevModel& m, const GemmArgs& g);
+cudaError_t launch_warp_mma(const DevModel& m, const GemmArgs& g, cudaStream_t stream);
 // mmasim_fp_fast.cu
 bool fast_fp_supported(const DevModel& m, const GemmArgs& g);
 int launch_fast_fp(const DevModel& m, const GemmArgs& g, cudaStream_t stream);

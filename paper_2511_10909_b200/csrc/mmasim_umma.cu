@@ -24,14 +24,13 @@
 //
 // Every wait is bounded: a role whose wait runs out raises a flag that ends the others' waits, the copies in flight are waited
 // for, nothing more is stored, and the CTA counts itself in the library's counter of given-up waits.
-#include <cuda.h>
 #include <type_traits>
-#include "mmasim_device.cuh"
+#include "mmasim_tma.cuh"
 
 namespace mmasim {
 namespace {
 
-constexpr int KBYTES = 128;             // bytes of K per row and stage: one swizzle atom, four instructions
+using namespace tma;
 constexpr int LANES = 128;
 constexpr int EPI_WARPS = 8;            // warps 0 - 7: C in, D out; 8: copies; 9: instructions; scaled kinds: 10 - 13: scale factors
 constexpr int SMS = 148;
@@ -83,32 +82,6 @@ struct UmmaArgs {
     unsigned int* timeouts;
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return uint32_t(__cvta_generic_to_shared(p)); }
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0u;
-}
-// A whole warp waits until the phase has completed; false when the clock budget ran out or another role gave up.
-__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* gave_up, long long budget) {
-    bool ok = mbar_try(bar, parity);
-    if (!ok) {
-        const long long t0 = clock64();
-        while (!(ok = mbar_try(bar, parity))) {
-            if (*gave_up) break;
-            if (clock64() - t0 > budget) { *gave_up = 1; break; }
-        }
-    }
-    return __all_sync(0xFFFFFFFFu, ok);
-}
-__device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                 :: "r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar) : "memory");
-}
 // K-major operand in the 128-byte swizzle: groups of eight rows 1024 bytes apart.
 __device__ __forceinline__ uint64_t operand_desc(uint32_t addr) {
     return uint64_t((addr & 0x3FFFFu) >> 4) | (uint64_t(1) << 16) | (uint64_t(1024 >> 4) << 32) | (uint64_t(1) << 46) | (uint64_t(2) << 61);
@@ -133,12 +106,6 @@ __device__ __forceinline__ void issue(uint32_t lead, uint32_t d, uint64_t ld, ui
 __device__ __forceinline__ void commit(uint32_t lead, uint32_t bar) {
     asm volatile("{\n\t.reg .pred l;\n\tsetp.ne.b32 l, %1, 0;\n\t@l tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" :: "r"(bar), "r"(lead) : "memory");
 }
-__device__ __forceinline__ uint32_t elect_one() {
-    uint32_t x;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(x));
-    return x;
-}
-
 #define MMASIM_R16(x) "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(x[4]), "r"(x[5]), "r"(x[6]), "r"(x[7]), "r"(x[8]), "r"(x[9]), "r"(x[10]), "r"(x[11]), "r"(x[12]), "r"(x[13]), "r"(x[14]), "r"(x[15])
 #define MMASIM_W16(x) "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]), "=r"(x[7]), "=r"(x[8]), "=r"(x[9]), "=r"(x[10]), "=r"(x[11]), "=r"(x[12]), "=r"(x[13]), "=r"(x[14]), "=r"(x[15])
 __device__ __forceinline__ void tmem_st16(uint32_t addr, const uint32_t* x) {
@@ -601,25 +568,6 @@ __global__ void __launch_bounds__(256) least_exponent_kernel(LeastSide a, LeastS
     if (threadIdx.x % 32 == 0) s.least[r] = least == 0xFFFFFFFFu ? 1 << 20 : int(max(field, 1u)) - 127;
 }
 
-using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
-                              CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeFn encode_fn() {
-    static const EncodeFn fn = [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult res;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &res) != cudaSuccess || res != cudaDriverEntryPointSuccess) p = nullptr;
-        return reinterpret_cast<EncodeFn>(p);
-    }();
-    return fn;
-}
-// rows x row_bytes, rows `pitch` bytes apart, in boxes of KBYTES x box_rows.
-bool encode(CUtensorMap* map, const void* base, int64_t row_bytes, int64_t rows, int64_t pitch, int box_rows) {
-    const cuuint64_t dims[2] = {cuuint64_t(row_bytes), cuuint64_t(rows)}, strides[1] = {cuuint64_t(pitch)};
-    const cuuint32_t box[2] = {KBYTES, cuuint32_t(box_rows)}, unit[2] = {1, 1};
-    return encode_fn()(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, unit, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                       CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 int code_bits(int fmt) { return fmt == EF_E2M1 ? 4 : (fmt == EF_E2M3 || fmt == EF_E3M2 ? 6 : 8); }
 bool is8(int f) { return f == EF_E4M3 || f == EF_E5M2 || f == EF_E3M2 || f == EF_E2M3 || f == EF_E2M1; }
 
@@ -720,6 +668,15 @@ bool umma_supported(const DevModel& m, const GemmArgs& g) {
 
 int launch_umma(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
     const int mk = kind_of(m);
+    if (warp_mma_supported(m, g)) {
+        set_kernel_name("tfdpa_f16", "matrix_instruction");
+        const cudaError_t err = launch_warp_mma(m, g, stream);
+        if (err != cudaSuccess) {
+            set_error("matrix-instruction kernel launch failed: %s", cudaGetErrorString(err));
+            return MMASIM_ERR_CUDA;
+        }
+        return MMASIM_OK;
+    }
     const int64_t kb = row_bytes(m, g.K);
     UmmaArgs a;
     a.steps = int((kb + 31) / 32);
