@@ -547,9 +547,9 @@ bool has_reference(const DevModel& m) {
 }
 }  // namespace
 
-// One call for the pipeline that was five (reference, product, zeroed statistics, statistics, copy): one allocation of kept memory, the
-// eight doubles into pinned memory, and the next launch is queued long before the last kernel ends.  CDNA3 FP16, 1024 x 1024 x 256:
-// 169 us as five calls from Python, 149 us as one; about 125 us of it are the kernels.
+// One call, kernels one behind the other and nothing else in the stream: the operands widened, the product, and the FP64 reference, which
+// is compared where it is computed (see launch_deviation_end).  CDNA3 FP16, 1024 x 1024 x 256: 169 us as five calls from Python, 149 us
+// as one of five kernels, a memset and a copy, now 138.
 int mmasim_deviation_stats(const mmasim_model* model, int64_t M, int64_t N, int64_t K, const void* A, const void* B, const void* C,
                            double* stats, void* stream) {
     GemmArgs g;
@@ -569,19 +569,16 @@ int mmasim_deviation_stats(const mmasim_model* model, int64_t M, int64_t N, int6
     cudaError_t err = take_lane(&lane);
     cudaMemPool_t pool = nullptr;
     if (err == cudaSuccess) err = scratch_pool(&pool);
-    const size_t words = size_t(M) * size_t(N), d_at = 64, ref_at = d_at + (words * model->info.acc_bytes + 255) / 256 * 256;
+    const size_t d_bytes = (size_t(M) * size_t(N) * model->info.acc_bytes + 255) / 256 * 256;
     unsigned char* base = nullptr;
-    if (err == cudaSuccess) err = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&base), ref_at + words * 8, pool, s);
-    double *dev_stats = reinterpret_cast<double*>(base), *ref = reinterpret_cast<double*>(base + ref_at);
-    if (err == cudaSuccess) err = cudaMemsetAsync(dev_stats, 0, 64, s);
+    if (err == cudaSuccess) err = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&base), d_bytes + deviation_scratch(M, N, K), pool, s);
     if (err == cudaSuccess) {
         *lane.gave_up = 0u;
         g.copy_timeouts = lane.gave_up_dev;
-        st = launch_reference_fp64(m.fmt_a, m.acc, M, N, K, A, B, C, ref, s);
-        g.D = base + d_at;
+        st = launch_deviation_start(m.fmt_a, M, N, K, A, B, base + d_bytes, s);
+        g.D = base;
         if (st == MMASIM_OK) st = run_gemm(model, g, 0, s);
-        if (st == MMASIM_OK) st = launch_error_stats(m.acc, int64_t(words), g.D, ref, dev_stats, s);
-        if (st == MMASIM_OK) err = cudaMemcpyAsync(lane.stats, dev_stats, 64, cudaMemcpyDeviceToHost, s);
+        if (st == MMASIM_OK) st = launch_deviation_end(m.acc, M, N, K, C, g.D, base + d_bytes, reinterpret_cast<double*>(lane.gave_up_dev) + 8, s);
     }
     if (st == MMASIM_ERR_CUDA) cudaGetLastError();
     if (base) cudaFreeAsync(base, s);

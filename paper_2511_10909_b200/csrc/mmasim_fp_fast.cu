@@ -16,7 +16,7 @@
 // (a -0 too) takes without a change.  Tiles in two sizes; see use_small.
 #include <cuda_fp16.h>
 #include <algorithm>
-#include "mmasim_internal.h"
+#include "mmasim_stats.cuh"
 
 namespace mmasim {
 namespace {
@@ -225,8 +225,10 @@ struct Stage {
 
 // WR x WC warps of TI x TJ accumulator tiles; UNIT: bytes per asynchronous copy (16, or 8 where a row stride or K is odd); TAIL: K is no
 // multiple of a chunk (the test for it in every chunk cost 2048 x 2048 x 2048 684 instead of 620 us).
-template <int WR, int WC, int TI, int TJ, int UNIT, bool TAIL>
-__global__ void __launch_bounds__(32 * WR * WC, 2) fma64_mma_kernel(GemmArgs g) {
+// OUT_STATS_*: C and the outputs compared with are FP32 or FP16 words, and what leaves are the sums of the deviations (see launch_deviation_end).
+enum Out : int { OUT_WORDS = 0, OUT_STATS_32, OUT_STATS_16 };
+template <int WR, int WC, int TI, int TJ, int UNIT, bool TAIL, int OUT>
+__global__ void __launch_bounds__(32 * WR * WC, 2) fma64_mma_kernel(GemmArgs g, DeviationArgs s_out) {
     after_previous();
     using namespace dm;
     constexpr int BM = 8 * WR * TI, BN = 8 * WC * TJ, DNT = 32 * WR * WC, SEGS = DKC * 8 / UNIT, PER = UNIT / 8;
@@ -246,7 +248,9 @@ __global__ void __launch_bounds__(32 * WR * WC, 2) fma64_mma_kernel(GemmArgs g) 
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 const int64_t r = row0 + 8 * (wr * TI + i) + gq, c = col0 + 8 * (wc * TJ + j) + 2 * tq + e;
-                acc[i][j][e] = (g.C && r < g.M && c < g.N) ? static_cast<const double*>(g.C)[r * g.ldc + c] : 0.0;
+                acc[i][j][e] = 0.0;
+                if (g.C && r < g.M && c < g.N)
+                    acc[i][j][e] = OUT == OUT_WORDS ? static_cast<const double*>(g.C)[r * g.ldc + c] : stats::output_value<OUT == OUT_STATS_16>(g.C, r * g.ldc + c);
             }
 
     // one chunk: consecutive threads on consecutive segments of a row; rows and K beyond the matrix are filled with zeros (a
@@ -300,6 +304,31 @@ __global__ void __launch_bounds__(32 * WR * WC, 2) fma64_mma_kernel(GemmArgs g) 
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 
+    if constexpr (OUT != OUT_WORDS) {
+        stats::Deviations s;
+#pragma unroll
+        for (int i = 0; i < TI; ++i)
+#pragma unroll
+            for (int j = 0; j < TJ; ++j)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int64_t r = row0 + 8 * (wr * TI + i) + gq, c = col0 + 8 * (wc * TJ + j) + 2 * tq + e;
+                    if (r < g.M && c < g.N) s.add(stats::output_value<OUT == OUT_STATS_16>(s_out.D, r * g.ldd + c), acc[i][j][e]);
+                }
+        s.reduce_to<WR * WC>(s_out.sums);
+        if (tid < 32) {                                 // the CTA that finishes last writes the sums out
+            __threadfence();
+            __syncwarp();
+            unsigned int before = 0u;
+            if (lane == 0) before = atomicAdd(s_out.finished, 1u);
+            before = __shfl_sync(0xFFFFFFFFu, before, 0);
+            if (before + 1u == gridDim.x * gridDim.y && lane < stats::NSTAT) {
+                __threadfence();
+                s_out.host[lane] = __ldcg(s_out.sums + lane);
+            }
+        }
+        return;
+    }
 #pragma unroll
     for (int i = 0; i < TI; ++i)
 #pragma unroll
@@ -326,20 +355,24 @@ bool use_small(const GemmArgs& g, int bm, int bn, int sm, int sn, double overhea
     return std::max(n * share * overhead, 0.35) < large;
 }
 
-template <int WR, int WC, int TI, int TJ>
-cudaError_t launch_fma64_tile(const GemmArgs& g, cudaStream_t stream) {
+template <int WR, int WC, int TI, int TJ, int OUT>
+cudaError_t launch_fma64_tile(const GemmArgs& g, const DeviationArgs& s, cudaStream_t stream) {
     constexpr int BM = 8 * WR * TI, BN = 8 * WC * TJ;
     constexpr size_t sh = sizeof(dm::Stage<BM, BN>) * dm::STAGES;
-    auto kernel = (g.lda | g.ldb | g.K) & 1 ? fma64_mma_kernel<WR, WC, TI, TJ, 8, true>
-                                            : (g.K % dm::DKC ? fma64_mma_kernel<WR, WC, TI, TJ, 16, true> : fma64_mma_kernel<WR, WC, TI, TJ, 16, false>);
+    auto kernel = (g.lda | g.ldb | g.K) & 1 ? fma64_mma_kernel<WR, WC, TI, TJ, 8, true, OUT>
+                                            : (g.K % dm::DKC ? fma64_mma_kernel<WR, WC, TI, TJ, 16, true, OUT> : fma64_mma_kernel<WR, WC, TI, TJ, 16, false, OUT>);
     const cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sh));
     if (err != cudaSuccess) return err;
-    return enqueue(kernel, dim3(unsigned(up_div(g.N, BN)), unsigned(up_div(g.M, BM))), 32 * WR * WC, sh, stream, g);
+    return enqueue(kernel, dim3(unsigned(up_div(g.N, BN)), unsigned(up_div(g.M, BM))), 32 * WR * WC, sh, stream, g, s);
 }
 cudaError_t launch_fma64_mma(const GemmArgs& g, cudaStream_t stream) {
     const bool small = use_small(g, 128, 64, 32, 32, 1.15);
     set_kernel_name("fma_f64", small ? "small_tiles" : "large_tiles");
-    return small ? launch_fma64_tile<2, 2, 2, 2>(g, stream) : launch_fma64_tile<4, 2, 4, 4>(g, stream);
+    return small ? launch_fma64_tile<2, 2, 2, 2, OUT_WORDS>(g, DeviationArgs{}, stream) : launch_fma64_tile<4, 2, 4, 4, OUT_WORDS>(g, DeviationArgs{}, stream);
+}
+template <int OUT>
+cudaError_t launch_deviations(const GemmArgs& g, const DeviationArgs& s, cudaStream_t stream) {
+    return use_small(g, 128, 64, 32, 32, 1.15) ? launch_fma64_tile<2, 2, 2, 2, OUT>(g, s, stream) : launch_fma64_tile<4, 2, 4, 4, OUT>(g, s, stream);
 }
 
 template <int MODE, int P, int TM, int TN, int KC>
@@ -375,6 +408,10 @@ bool fast_fp_supported(const DevModel& m, const GemmArgs& g) {
     const int64_t per_sm = up_div(up_div(g.M, 16) * up_div(g.N, 16), 148);
     const int generic_up_to = m.family == FAM_FMA ? (on16 ? 2 : 3) : (on16 ? (m.P == 4 ? 1 : 0) : 2);
     return per_sm > generic_up_to;
+}
+
+cudaError_t launch_fma64_deviations(int acc, const GemmArgs& g, const DeviationArgs& s, cudaStream_t stream) {
+    return acc == ACC_F16 ? launch_deviations<OUT_STATS_16>(g, s, stream) : launch_deviations<OUT_STATS_32>(g, s, stream);
 }
 
 int launch_fast_fp(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {

@@ -128,6 +128,14 @@ cudaError_t launch_warp_mma(const DevModel& m, const GemmArgs& g, cudaStream_t s
 // mmasim_fp_fast.cu
 bool fast_fp_supported(const DevModel& m, const GemmArgs& g);
 int launch_fast_fp(const DevModel& m, const GemmArgs& g, cudaStream_t stream);
+struct DeviationArgs {
+    const void* D;                      // the model's outputs, M x N
+    double* sums;                       // eight, zeroed
+    unsigned int* finished;             // zeroed
+    double* host;                       // device address of mapped host memory
+};
+// Phi_FMA in FP64 with g.C in the model's accumulator type; nothing is stored but the sums of the deviations of s.D from it
+cudaError_t launch_fma64_deviations(int acc, const GemmArgs& g, const DeviationArgs& s, cudaStream_t stream);
 // mmasim_gst_fast.cu
 bool fast_gst_supported(const DevModel& m, const GemmArgs& g);
 int launch_fast_gst(const DevModel& m, const GemmArgs& g, cudaStream_t stream);
@@ -141,6 +149,10 @@ int launch_hw_umma(int kind, int64_t M, int64_t K, const void* A, const void* B,
                    const void* sfb, int32_t* status, cudaStream_t stream);
 // mmasim_stats.cu
 int launch_error_stats(int acc, int64_t n, const void* D, const double* ref, double* stats, cudaStream_t stream);
+constexpr size_t DEVIATION_SUMS = 128;          // bytes in front of the widened operands: eight sums, the number of CTAs that have finished
+size_t deviation_scratch(int64_t M, int64_t N, int64_t K);
+int launch_deviation_start(int fmt, int64_t M, int64_t N, int64_t K, const void* A, const void* B, void* scratch, cudaStream_t stream);
+int launch_deviation_end(int acc, int64_t M, int64_t N, int64_t K, const void* C, const void* D, void* scratch, double* host, cudaStream_t stream);
 int launch_reference_fp64(int fmt, int acc, int64_t M, int64_t N, int64_t K, const void* A, const void* B, const void* C, double* ref, cudaStream_t stream);
 // mmasim_peak.cu
 int launch_int_peak(int kind, int64_t blocks, int64_t iters, void* sink, int32_t* ops_per_round, cudaStream_t stream);

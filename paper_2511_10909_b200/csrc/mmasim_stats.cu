@@ -3,62 +3,19 @@
 // reference's operands.  A grid-stride pass over the outputs, four in flight per thread, per-thread partial sums in FP64, reduced
 // over the CTA, one atomic per CTA and statistic (one per warp, 9472 on each of eight addresses, took 85 of the 89 us
 // of a 1024 x 1024 reduction).
-#include <cuda_fp16.h>
 #include <cstring>
-#include "mmasim_internal.h"
+#include "mmasim_stats.cuh"
 
 namespace mmasim {
 namespace {
 
-constexpr int NSTAT = 8;
-
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-    return v;
-}
-__device__ __forceinline__ double warp_max(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-    return v;
-}
-
 template <bool ACC16>
-__global__ void __launch_bounds__(256) stats_kernel(int64_t n, const void* D, const double* ref, double* stats) {
+__global__ void __launch_bounds__(256) stats_kernel(int64_t n, const void* D, const double* ref, double* out) {
     after_previous();
-    double cnt = 0.0, sum = 0.0, sabs = 0.0, ssq = 0.0, nneg = 0.0, npos = 0.0, mx = 0.0, srel = 0.0;
+    stats::Deviations s;
 #pragma unroll 4
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
-        const double d = ACC16 ? double(__half2float(__ushort_as_half(static_cast<const unsigned short*>(D)[i])))
-                               : double(__uint_as_float(static_cast<const uint32_t*>(D)[i]));
-        const double r = ref[i];
-        const double delta = d - r;
-        if (!(fabs(delta) <= 1.7976931348623157e308)) continue;      // NaN or infinite on either side: not counted
-        cnt += 1.0;
-        sum += delta;
-        sabs += fabs(delta);
-        ssq += delta * delta;
-        nneg += delta < 0.0 ? 1.0 : 0.0;
-        npos += delta > 0.0 ? 1.0 : 0.0;
-        mx = fmax(mx, fabs(delta));
-        if (r != 0.0) srel += fabs(delta) / fabs(r);
-    }
-    const double v[NSTAT] = {warp_sum(cnt), warp_sum(sum), warp_sum(sabs), warp_sum(ssq), warp_sum(nneg), warp_sum(npos),
-                             warp_max(mx), warp_sum(srel)};
-    __shared__ double part[NSTAT][8];
-    if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-        for (int s = 0; s < NSTAT; ++s) part[s][threadIdx.x >> 5] = v[s];
-    }
-    __syncthreads();
-    if (threadIdx.x < NSTAT) {
-        const int s = threadIdx.x;
-        double t = part[s][0];
-#pragma unroll
-        for (int w = 1; w < 8; ++w) t = s == 6 ? fmax(t, part[s][w]) : t + part[s][w];
-        if (s == 6) atomicMax(reinterpret_cast<unsigned long long*>(stats + s), (unsigned long long)__double_as_longlong(t));   // non-negative doubles order like their bit patterns
-        else atomicAdd(stats + s, t);
-    }
+    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) s.add(stats::output_value<ACC16>(D, i), ref[i]);
+    s.reduce_to<8>(out);
 }
 
 // An operand widened exactly to FP64, two elements per thread and step: 16-byte stores, consecutive threads side by side.
@@ -83,8 +40,10 @@ __device__ __forceinline__ double widen_one(int fmt, const void* p, int64_t i) {
         }
     }
 }
-__global__ void __launch_bounds__(256) widen_kernel(Widen a, Widen b, Widen c) {
+// (`zero`: NULL, or memory of that many bytes to be zeroed beside)
+__global__ void __launch_bounds__(256) widen_kernel(Widen a, Widen b, Widen c, unsigned char* zero, int zero_bytes) {
     after_previous();
+    if (zero && blockIdx.x == 0 && blockIdx.y == 0 && int(threadIdx.x) < zero_bytes) zero[threadIdx.x] = 0;
     const Widen w = blockIdx.y == 0 ? a : (blockIdx.y == 1 ? b : c);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -116,7 +75,7 @@ int launch_reference_fp64(int fmt, int acc, int64_t M, int64_t N, int64_t K, con
     if (err == cudaSuccess) {
         const Widen wa = {A, scratch + a_at, na, fmt}, wb = {B, scratch + b_at, nb, fmt}, wc = {C, scratch + c_at, nc, acc == ACC_F16 ? EF_F16 : EF_F32};
         const int64_t most = na > nb ? (na > nc ? na : nc) : (nb > nc ? nb : nc);
-        err = enqueue(widen_kernel, dim3(unsigned((most + 2047) / 2048), C ? 3 : 2), 256, 0, stream, wa, wb, wc);
+        err = enqueue(widen_kernel, dim3(unsigned((most + 2047) / 2048), C ? 3 : 2), 256, 0, stream, wa, wb, wc, nullptr, 0);
     }
     if (err == cudaSuccess) {
         DevModel m;
@@ -135,6 +94,36 @@ int launch_reference_fp64(int fmt, int acc, int64_t M, int64_t N, int64_t K, con
     if (scratch) cudaFreeAsync(scratch, stream);
     if (err != cudaSuccess) { set_error("mmasim_reference_fp64: %s", cudaGetErrorString(err)); return MMASIM_ERR_CUDA; }
     return st;
+}
+
+// The two ends of mmasim_deviation_stats.  Before the product: A and B widened, the sums zeroed.  Behind it: the FP64 kernel, whose CTAs
+// compare their outputs with the model's and add up the deviations in place of storing a reference; the last one to finish writes the
+// eight sums to `host`, mapped host memory.
+size_t deviation_scratch(int64_t M, int64_t N, int64_t K) { return DEVIATION_SUMS + size_t((M * K + 1) / 2 * 2 + N * K) * 8; }
+int launch_deviation_start(int fmt, int64_t M, int64_t N, int64_t K, const void* A, const void* B, void* scratch, cudaStream_t stream) {
+    double* a = reinterpret_cast<double*>(static_cast<unsigned char*>(scratch) + DEVIATION_SUMS);
+    const int64_t na = M * K, nb = N * K, most = na > nb ? na : nb;
+    const Widen wa = {A, a, na, fmt}, wb = {B, a + (na + 1) / 2 * 2, nb, fmt};
+    const cudaError_t err = enqueue(widen_kernel, dim3(unsigned((most + 2047) / 2048), 2), 256, 0, stream, wa, wb, wb, static_cast<unsigned char*>(scratch), int(DEVIATION_SUMS));
+    if (err != cudaSuccess) { set_error("mmasim_deviation_stats: %s", cudaGetErrorString(err)); return MMASIM_ERR_CUDA; }
+    return MMASIM_OK;
+}
+int launch_deviation_end(int acc, int64_t M, int64_t N, int64_t K, const void* C, const void* D, void* scratch, double* host, cudaStream_t stream) {
+    const double* a = reinterpret_cast<const double*>(static_cast<unsigned char*>(scratch) + DEVIATION_SUMS);
+    GemmArgs g;
+    std::memset(&g, 0, sizeof(g));
+    g.M = M; g.N = N; g.K = K;
+    g.A = a; g.B = a + (M * K + 1) / 2 * 2; g.C = C;
+    g.lda = g.ldb = K;
+    g.ldc = g.ldd = N;
+    DeviationArgs s;
+    s.D = D;
+    s.sums = static_cast<double*>(scratch);
+    s.finished = reinterpret_cast<unsigned int*>(s.sums + stats::NSTAT);
+    s.host = host;
+    const cudaError_t err = launch_fma64_deviations(acc, g, s, stream);
+    if (err != cudaSuccess) { set_error("mmasim_deviation_stats: %s", cudaGetErrorString(err)); return MMASIM_ERR_CUDA; }
+    return MMASIM_OK;
 }
 
 }  // namespace mmasim
