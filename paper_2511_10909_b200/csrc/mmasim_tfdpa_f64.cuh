@@ -137,8 +137,8 @@ __host__ __device__ constexpr int pe64_sub(int base) { return base == 8 ? 32 : (
 // (behind, it would turn a result of -0, which RNE-FP32 can leave, into +0).
 // EOSPLIT (GTR-FDPA, blocks of 16): inside each block of 16 the operand plane holds the even elements first, then the odd
 // ones, so that a matrix instruction sums four elements of one group; exponent pairs and masks keep the order of K.
-// TINY_ZEROS (the T-FDPA kernels without a tensor-core maximum): a zero is staged as 2^-900 of its sign.  Its products are far below any
-// unit of a sum register, so that a positive one adds nothing and a negative one falls one unit short like every other
+// TINY_ZEROS (the T-FDPA kernels without a tensor-core maximum, TR- and GTR-FDPA): a zero is staged as 2^-900 of its sign.  Its
+// products are far below any unit of a sum register, so that a positive one adds nothing and a negative one falls one unit short like every other
 // negative product: the sign masks alone count them, without the masks of nonzero elements.
 template <int R, int FORM>
 struct Side64 {
@@ -167,6 +167,7 @@ __device__ __forceinline__ void decode64(const DevModel& m, const Side64<R, FORM
         LutEntry64 e;
         e.op = IS_A ? operand_a(fin ? dec_sign(dd) : 0u, sg, fin ? dec_exp(dd) : 0, f.mbits)
                     : operand_b(fin ? dec_sign(dd) : 0u, sg, fin ? dec_exp(dd) : 0, f.mbits);
+        if (TINY_ZEROS && !sg) e.op = fin && dec_sign(dd) ? -pow2d(-900) : pow2d(-900);
         e.exp = sg ? uint32_t(dec_exp(dd) + EB) : 0u;
         e.bits = (fin ? dec_sign(dd) : 0u) | (fin ? 0u : 2u) | (sg ? 4u : 0u);
         lut[tid] = e;

@@ -191,8 +191,8 @@ __global__ void __launch_bounds__(NT, 2) trfdpa64_kernel(DevModel m, GemmArgs g,
             constexpr uint32_t k_gtr = (53u << 20) + 1u;   // a sum register's field minus Exp(c)'s beyond which c is dropped (GTR)
             float wmax = 0.f;
             auto merge = [&](int r, int c) {
-                const uint32_t sa = sa_blk.sgn[prow + r], nza = sa_blk.nz[prow + r] & kmask;
-                const uint32_t negm = (sa ^ sb_blk.sgn[pcol + c]) & nza & sb_blk.nz[pcol + c];
+                // (zeros are staged as tiny numbers of their sign: the products that fall one short are those of unlike signs)
+                const uint32_t unlike = sa_blk.sgn[prow + r] ^ sb_blk.sgn[pcol + c];
                 double Y;                                   // T * 2^(e_max - F)
                 int m0hi;                                   // high word of the sum register's constant (e_max in place)
                 if (GTR) {
@@ -200,16 +200,16 @@ __global__ void __launch_bounds__(NT, 2) trfdpa64_kernel(DevModel m, GemmArgs g,
                     const double u0 = t0[r][c], u1 = t1[GTR ? r : 0][GTR ? c : 0];
                     const int e_hi = (__double2hiint(u0) & EXPF) | HALF, o_hi = (__double2hiint(u1) & EXPF) | HALF;
                     m0hi = max(e_hi, o_hi);
-                    const double ye = __dsub_rn(__hiloint2double(__double2hiint(u0), __double2loint(u0) + __popc(negm & 0x55555555u)),
+                    const double ye = __dsub_rn(__hiloint2double(__double2hiint(u0), __double2loint(u0) + __popc(unlike & kmask & 0x55555555u)),
                                                 __hiloint2double(e_hi, LOW0));
-                    const double yo = __dsub_rn(__hiloint2double(__double2hiint(u1), __double2loint(u1) + __popc(negm & 0xAAAAAAAAu)),
+                    const double yo = __dsub_rn(__hiloint2double(__double2hiint(u1), __double2loint(u1) + __popc(unlike & kmask & 0xAAAAAAAAu)),
                                                 __hiloint2double(o_hi, LOW0));
                     const double mm = __hiloint2double(m0hi, 0);
                     Y = __dsub_rn(__dadd_rd(yo, __dadd_rd(ye, mm)), mm);
                 } else {
                     const double u0 = t0[r][c];
                     m0hi = KEEP_M0 ? m0k[KEEP_M0 ? r : 0][KEEP_M0 ? c : 0] : (__double2hiint(u0) & EXPF) | HALF;
-                    Y = __dsub_rn(__hiloint2double(__double2hiint(u0), __double2loint(u0) + __popc(negm)), __hiloint2double(m0hi, LOW0));
+                    Y = __dsub_rn(__hiloint2double(__double2hiint(u0), __double2loint(u0) + __popc(unlike & kmask)), __hiloint2double(m0hi, LOW0));
                 }
                 double st = cs[r][c];
                 // the field of Exp(c), minus one: zero wraps to the top and comes back as 0 when the one is added again (inside
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(NT, 2) trfdpa64_kernel(DevModel m, GemmArgs g,
 
 template <int EK, int L, bool GTR>
 cudaError_t launch_tr_one(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
-    return decode_and_run<EK, 0, GTR, false, EXP_PAIRS>(trfdpa64_kernel<EK, L, GTR>, m, g, false, stream);
+    return decode_and_run<EK, 0, GTR, true, EXP_PAIRS>(trfdpa64_kernel<EK, L, GTR>, m, g, false, stream);
 }
 
 }  // namespace
