@@ -116,7 +116,7 @@ TileCosts tile_costs(const DevModel& m, int kind, bool promoted) {
     }
     if (kind == 1 + fast::EK_LUT8) {
         if (m.F != 13) return h ? TileCosts{0.37, 0.63, 1.96, 4.5, 15} : (m.family == FAM_ST ? TileCosts{0.26, 0.50, 1.15, 2.3, 15} : TileCosts{0.19, 0.44, 1.05, 2.2, 15});
-        if (h) return m.L == 16 ? TileCosts{0.66, 0.56, 2.13, 6.8, 22} : TileCosts{0.37, 0.63, 1.96, 4.65, 22};
+        if (h) return m.L == 16 ? TileCosts{0.66, 0.56, 2.13, 5.5, 17} : TileCosts{0.37, 0.63, 1.96, 3.7, 17};
         // (large: times f13_chunk_us; promoted sums only have the smaller tiles)
         return m.L == 16 ? TileCosts{0.28, 0.36, 0.99, promoted ? 1.38 : 1.3, 22} : TileCosts{0.20, 0.43, 1.01, promoted ? 1.06 : 1.0, 22};
     }
