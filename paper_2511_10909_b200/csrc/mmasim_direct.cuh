@@ -45,7 +45,7 @@ using fast64::G_OFF;
 constexpr int KC = 32;
 constexpr int KP = KC + 4;              // doubles per row of an operand plane: fragment loads hit sixteen different bank pairs
 constexpr int EP = KC / 2 + 4;          // exponent words per row: 80 bytes, 16-byte loads of eight rows hit different banks
-constexpr int RING = 4;                 // raw chunks in flight or waiting to be decoded
+constexpr int RING = 4;                 // raw chunks in flight or waiting to be decoded (eight: no gain)
 constexpr int BUF = 3;                  // decoded chunks: one being computed, one whose exponents are looked ahead at, one being decoded
 
 // TASK (4 or 8) raw elements as FP32 words of the same values (exact: every format here has at most 10 significand bits and, but for
@@ -63,20 +63,30 @@ __device__ __forceinline__ void to_fp32(const uint32_t* w, int fmt, uint32_t (&x
 #pragma unroll
         for (int q = 0; q < TASK; ++q) x[q] = half_to_fp32(w[q / 2] >> (16 * (q & 1)));
     } else {
-        uint32_t h[TASK / 2];                           // pairs of FP16 words
+        // Pairs of FP16 words.  One branch for all of them: a choice of the conversion inside the loop made the staging of eight elements
+        // three times that of FP16 ones, and the small tiles of FP8 waited for it (with the blocks left out 20.2 of 21.2 us; Hopper E4M3
+        // 64 x 256 x 1024 21.2 -> 15.3 us, Ada E5M2 32 x 384 x 2816 57.0 -> 42.0, CDNA3 E4M3 64 x 256 x 1024 23.7 -> 18.7).
+        uint32_t h[TASK / 2];
+        auto each = [&](auto convert) {
 #pragma unroll
-        for (int q = 0; q < TASK / 2; ++q) {
-            const unsigned short p = (unsigned short)(w[q / 2] >> (16 * (q & 1)));
-            switch (fmt) {
-                case EF_E4M3: asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(h[q]) : "h"(p)); break;
-                case EF_E5M2: asm("cvt.rn.f16x2.e5m2x2 %0, %1;" : "=r"(h[q]) : "h"(p)); break;
-                case EF_E3M2: asm("cvt.rn.f16x2.e3m2x2 %0, %1;" : "=r"(h[q]) : "h"((unsigned short)(p & 0x3F3Fu))); break;
-                case EF_E2M3: asm("cvt.rn.f16x2.e2m3x2 %0, %1;" : "=r"(h[q]) : "h"((unsigned short)(p & 0x3F3Fu))); break;
-                default: {                              // E2M1, one code per byte: both codes into one byte
-                    const unsigned short b = (unsigned short)((p & 0xFu) | ((p >> 4) & 0xF0u));
-                    asm("{ .reg .b8 lo, hi; mov.b16 {lo, hi}, %1; cvt.rn.f16x2.e2m1x2 %0, lo; }" : "=r"(h[q]) : "h"(b));
-                }
-            }
+            for (int q = 0; q < TASK / 2; ++q) h[q] = convert((unsigned short)(w[q / 2] >> (16 * (q & 1))));
+        };
+        if (fmt == EF_E5M2) {                           // an FP16 word without its low byte
+#pragma unroll
+            for (int q = 0; q < TASK / 2; ++q) h[q] = __byte_perm(w[q / 2], 0u, q & 1 ? 0x3424 : 0x1404);
+        } else if (fmt == EF_E4M3) {
+            each([](unsigned short p) { uint32_t r; asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(r) : "h"(p)); return r; });
+        } else if (fmt == EF_E3M2) {
+            each([](unsigned short p) { uint32_t r; asm("cvt.rn.f16x2.e3m2x2 %0, %1;" : "=r"(r) : "h"((unsigned short)(p & 0x3F3Fu))); return r; });
+        } else if (fmt == EF_E2M3) {
+            each([](unsigned short p) { uint32_t r; asm("cvt.rn.f16x2.e2m3x2 %0, %1;" : "=r"(r) : "h"((unsigned short)(p & 0x3F3Fu))); return r; });
+        } else {
+            each([](unsigned short p) {                 // E2M1, one code per byte: both codes into one byte
+                uint32_t r;
+                const unsigned short b = (unsigned short)((p & 0xFu) | ((p >> 4) & 0xF0u));
+                asm("{ .reg .b8 lo, hi; mov.b16 {lo, hi}, %1; cvt.rn.f16x2.e2m1x2 %0, lo; }" : "=r"(r) : "h"(b));
+                return r;
+            });
         }
 #pragma unroll
         for (int q = 0; q < TASK; ++q) x[q] = half_to_fp32(h[q / 2] >> (16 * (q & 1)));
