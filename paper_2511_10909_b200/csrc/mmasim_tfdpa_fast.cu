@@ -101,16 +101,17 @@ bool fast_tfdpa_supported(const DevModel& m, const GemmArgs& g) {
 //     small tiles   4 + chain chunks + per_tile n (chunks + 1.2)        8 x 16 outputs: 0.65 of a 16 x 16 tile
 //     large tiles   decode + large n (chunks + 0.5)                     (an odd n: the last tile has the SM to itself, 0.16 of one more)
 // with the constants of the arithmetic, fitted to the times of all four at sizes from 16 x 64 to 1076 x 3218 and K = 64, 256 and 1024
-// (within 10 %).  Chosen by it, no size takes 1.2 times its best; the average is 1.01.  Small / large in us on both sides of the line: Hopper E4M3 -> FP16 640 x 640 x 64
-// 25 / 29, x 256 63 / 60, Ampere FP16 768 x 768 x 256 36 / 38, 1024 x 1024 x 256 70 / 62, CDNA1 BF16 512 x 512 x 1024 129 / 211, 768 x 768 x 1024
-// 258 / 215.
+// (within 10 %); those of the FP8 rows again after their staging and the F = 13 tiles had become faster.  Small / large in us on both
+// sides of the line: Hopper E4M3 256 x 1024 x 1024 58 / 96, 768 x 768 x 256 35 / 33, Hopper E4M3 -> FP16 512 x 512 x 256 37 / 43, 256 x
+// 1024 x 1024 130 / 133, Ampere FP16 768 x 768 x 256 36 / 38, 1024 x 1024 x 256 70 / 62, CDNA1 BF16 512 x 512 x 1024 129 / 211, 768 x
+// 768 x 1024 258 / 215.
 namespace {
 struct TileCosts { double chain, t16, t32, large, decode; };
 TileCosts tile_costs(const DevModel& m, int kind, bool promoted) {
     const bool h = m.acc == ACC_F16;
     if (kind == KIND_E) return m.fmt_a == EF_F16 ? TileCosts{0.26, 0.28, 0.89, 3.3, 15} : TileCosts{0.58, 0.50, 1.55, 5.3, 15};
     if (kind == KIND_TR) {
-        if (m.family == FAM_GTR) return {0.27, 0.42, 1.26, 3.7, 15};
+        if (m.family == FAM_GTR) return {0.19, 0.39, 1.17, 3.5, 15};
         if (m.fmt_a == EF_TF32) return {0.35, 0.46, 1.54, 5.8, 15};
         return {0.21, 0.35, 1.13, 3.85, 15};
     }
@@ -118,7 +119,7 @@ TileCosts tile_costs(const DevModel& m, int kind, bool promoted) {
         if (m.F != 13) return h ? TileCosts{0.37, 0.63, 1.96, 4.5, 15} : (m.family == FAM_ST ? TileCosts{0.26, 0.50, 1.15, 2.3, 15} : TileCosts{0.19, 0.44, 1.05, 2.2, 15});
         if (h) return m.L == 16 ? TileCosts{0.66, 0.56, 2.13, 5.5, 17} : TileCosts{0.37, 0.63, 1.96, 3.7, 17};
         // (large: times f13_chunk_us; promoted sums only have the smaller tiles)
-        return m.L == 16 ? TileCosts{0.28, 0.36, 0.99, promoted ? 1.38 : 1.3, 22} : TileCosts{0.20, 0.43, 1.01, promoted ? 1.06 : 1.0, 22};
+        return m.L == 16 ? TileCosts{0.19, 0.32, 0.88, promoted ? 1.38 : 1.3, 22} : TileCosts{0.10, 0.38, 0.90, promoted ? 1.06 : 1.0, 22};
     }
     if (kind == 1 + fast::EK_F16 && h) return m.L == 4 ? TileCosts{0.46, 0.45, 1.83, 6.3, 15} : TileCosts{0.25, 0.36, 1.15, 3.75, 15};
     if (kind == 1 + fast::EK_TF32) return m.L == 4 ? TileCosts{0.27, 0.43, 1.32, 4.3, 15} : TileCosts{0.21, 0.35, 1.08, 3.1, 15};
