@@ -437,14 +437,22 @@ __global__ void __launch_bounds__(NT, 2) tfdpa64_kernel(DevModel m, GemmArgs g, 
     uint32_t cw[TM][TN];                                // the words of C as read (finite ones; the rest become flags)
     uint32_t sp_nan = 0u, sp_pinf = 0u, sp_ninf = 0u;   // per output (bit r * TN + c): NaN / +inf / -inf seen so far
     float promoted[PROMOTE ? TM : 1][PROMOTE ? TN : 1];
+    // The accumulators of rows and columns beyond the matrix (nothing of them is stored): zeros, or those of the last row and column.  It is
+    // a matter of registers, and which of the two makes the faster kernel was measured.  2048 x 2048 x 1024 on large tiles, zeros / last ones
+    // in us: Volta FP16 -> FP16 1303 / 1333, Hopper FP16 488 / 499, Hopper BF16 508 / 523, Ampere FP16 657 / 631, Blackwell E4M3 454 /
+    // 438, -> FP16 591 / 587; sums promoted every 128, 2048^3: Ampere FP16 1343 / 1368 and Hopper TF32 1459 / 1475 (with the division that
+    // to_promotion replaces), Volta FP16 2080 / 2029.
+    constexpr bool C_GUARD = PROMOTE ? L > 4 : (ACC16 && L < 32) || L == 16;
 #define MMASIM_SP_GET(r, c) ((((sp_nan >> ((r) * TN + (c))) & 1u)) | (((sp_pinf >> ((r) * TN + (c))) & 1u) << 1) | (((sp_ninf >> ((r) * TN + (c))) & 1u) << 2))
 #pragma unroll
     for (int r = 0; r < TM; ++r)
 #pragma unroll
         for (int c = 0; c < TN; ++c) {
-            const int64_t i = min(row0 + row_at(r), g.M - 1), j = min(col0 + col_at(c), g.N - 1);
+            int64_t i = row0 + row_at(r), j = col0 + col_at(c);
+            const bool inside = !C_GUARD || (i < g.M && j < g.N);
+            if (!C_GUARD) { i = min(i, g.M - 1); j = min(j, g.N - 1); }
             uint32_t w = 0u;
-            if (g.C)
+            if (g.C && inside)
                 w = ACC16 ? uint32_t(static_cast<const uint16_t*>(g.C)[i * g.ldc + j])
                           : static_cast<const uint32_t*>(g.C)[i * g.ldc + j];
             if (PROMOTE) { promoted[PROMOTE ? r : 0][PROMOTE ? c : 0] = __uint_as_float(w); w = 0u; }
@@ -464,9 +472,10 @@ __global__ void __launch_bounds__(NT, 2) tfdpa64_kernel(DevModel m, GemmArgs g, 
 
     __syncthreads();                                    // the barriers are initialised
     uint32_t emp[TM][TN];                               // product exponents of the block that comes next
+    int to_promotion = PROMOTE ? int(g.k_chunk) : 0;    // elements of K to go (as the remainder of a division per chunk: Ampere FP16 1343, now 1322)
 
     for (int chunk = 0; chunk < NCH; ++chunk) {
-        const int64_t k0 = int64_t(chunk) * KC - fast::front_pad(g.K);
+        const int64_t k0 = int64_t(chunk) * KC - (PROMOTE ? 0 : fast::front_pad(g.K));      // (k_chunk divides K and is whole chunks)
         // a wait that runs out is recorded and the chunk computed on whatever is there; every thread sees the flag after
         // the barrier at the end of the chunk, and the CTA leaves together without storing anything
         if (!fast::mbar_wait(&sm.full[chunk & 1], uint32_t(chunk >> 1) & 1u)) *reinterpret_cast<volatile int*>(&sm.error) = 1;
@@ -529,7 +538,7 @@ __global__ void __launch_bounds__(NT, 2) tfdpa64_kernel(DevModel m, GemmArgs g, 
 #pragma unroll 1
                     for (int c = 0; c < TN; ++c) {
                         const int64_t i = row0 + row_at(r), j = col0 + col_at(c);
-                        if (i >= g.M || j >= g.N || k0 + kb < 0) continue;
+                        if (i >= g.M || j >= g.N || (!PROMOTE && k0 + kb < 0)) continue;
                         Special ev;
                         for (int kk = kb; kk < kb + L; ++kk) {
                             const uint32_t x = decode_elem(fa, raw_elem<EK>(g.A, i * g.lda + k0 + kk));
@@ -803,7 +812,8 @@ __global__ void __launch_bounds__(NT, 2) tfdpa64_kernel(DevModel m, GemmArgs g, 
         if (*reinterpret_cast<volatile int*>(&sm.error)) break;
         if (tid == 0 && chunk + 2 < NCH) issue(chunk + 2);
         // ---- FP32 promotion of the partial sum every k_chunk elements ----
-        if (PROMOTE && ((k0 + KC) % g.k_chunk) == 0) {
+        if (PROMOTE && (to_promotion -= KC) == 0) {
+            to_promotion = int(g.k_chunk);
 #pragma unroll
             for (int r = 0; r < TM; ++r)
 #pragma unroll
