@@ -26,7 +26,9 @@ cudaError_t enqueue(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem
     cfg.stream = stream;
     cfg.attrs = &early;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    if (err != cudaSuccess) cudaGetLastError();         // (it is the caller's now; left in the thread, the next launch of anybody would report it)
+    return err;
 }
 
 // Element formats (device-side ids).  The order is private to the library.
