@@ -129,7 +129,7 @@ TileCosts tile_costs(const DevModel& m, int kind, bool promoted) {
 }
 }  // namespace
 
-DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us) {
+static DirectSize choose_size(const DevModel& m, const GemmArgs& g, bool large_too, double* us) {
     if (!direct_takes(m, g)) return DIRECT_NONE;
     const int kind = kind_of(m);
     constexpr int64_t SMS = 148;
@@ -139,7 +139,7 @@ DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us) {
     const double chunks = double((g.K + fast::KC - 1) / fast::KC), start = 4.0 + t.chain * chunks, each = chunks + 1.2;
     const double c8 = start + 0.65 * t.t16 * fullest(8, 16) * each, c16 = start + t.t16 * fullest(16, 16) * each, c32 = start + t.t32 * fullest(32, 32) * each;
     double big = 1e30;
-    if (fast_tfdpa_supported(m, g)) {
+    if (large_too && fast_tfdpa_supported(m, g)) {
         if (f13 && m.acc != ACC_F16) {
             const double low = fast::f13_chunk_us(g, 64), tall = fast::f13_chunk_us(g, 128);
             big = t.decode + t.large * (g.k_chunk || low < tall ? low : tall) * chunks;
@@ -152,6 +152,8 @@ DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us) {
     if (big <= c8 && big <= c16 && big <= c32) return DIRECT_NONE;
     return c8 <= c16 && c8 <= c32 ? DIRECT_8x16 : (c16 <= c32 ? DIRECT_16x16 : DIRECT_32x32);
 }
+
+DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us) { return choose_size(m, g, true, us); }
 
 int launch_direct(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStream_t stream) {
     cudaError_t err = cudaErrorInvalidValue;
@@ -216,7 +218,17 @@ int launch_gemm_noalloc(const DevModel& m, const GemmArgs& g, cudaStream_t strea
     return MMASIM_OK;
 }
 
+// A stream whose work is being recorded into a graph.
+static bool capturing(cudaStream_t stream) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &status) != cudaSuccess) { cudaGetLastError(); return false; }
+    return status != cudaStreamCaptureStatusNone;
+}
+
 int launch_fast_tfdpa(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
+    // Ragged rows run on the small tiles where the decoded operands get no memory, and in a graph: one with memory nodes in it cannot be
+    // cloned, made part of another one or instantiated twice, and those of ragged calls never had any.  (Whole chunks on large tiles always did.)
+    if (ragged(m, g) && capturing(stream)) return launch_direct(m, g, choose_size(m, g, false, nullptr), stream);
     cudaError_t err = cudaErrorInvalidValue;
     if (kind_of(m) == KIND_TR) {
         set_kernel_name(m.family == FAM_GTR ? "gtrfdpa" : "trfdpa", "large_tiles");
@@ -231,9 +243,9 @@ int launch_fast_tfdpa(const DevModel& m, const GemmArgs& g, cudaStream_t stream)
         case fast::EK_TF32: set_kernel_name("tfdpa_tf32", "large_tiles"); err = fast::launch_tf32(m, g, stream); break;
         default: break;
     }
-    if (err == cudaErrorMemoryAllocation && ragged(m, g)) {     // no memory for the decoded operands: the small tiles need none
+    if (err == cudaErrorMemoryAllocation && ragged(m, g)) {
         cudaGetLastError();
-        return launch_direct(m, g, DIRECT_32x32, stream);
+        return launch_direct(m, g, choose_size(m, g, false, nullptr), stream);
     }
     if (err != cudaSuccess) {
         set_error("tuned T-FDPA kernel launch failed: %s", cudaGetErrorString(err));

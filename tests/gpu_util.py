@@ -51,3 +51,31 @@ def assert_samples_equal(D, want, pairs, what=""):
     bad = np.flatnonzero(got != want)
     assert bad.size == 0, (f"{what}: {bad.size} of {len(want)} sampled outputs differ; first at "
                            f"{tuple(pairs[bad[0]])}: got {int(got[bad[0]]):#x}, oracle {int(want[bad[0]]):#x}")
+
+
+def recorded(call):
+    """Runs `call` while its stream is recorded into a graph; returns the graph (a torch.cuda.CUDAGraph that keeps its nodes), what the call
+    returned, and the nodes: the kernels' names, "alloc" and "free" for memory nodes, "other" for the rest."""
+    from cuda.bindings import driver
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=stream):
+        out = call()
+
+    def ok(result):
+        assert result[0] == driver.CUresult.CUDA_SUCCESS, result[0]
+        return result[1] if len(result) == 2 else result[1:]
+
+    raw = driver.CUgraph(graph.raw_cuda_graph())
+    count = ok(driver.cuGraphGetNodes(raw, 0))[1]
+    names = []
+    for node in ok(driver.cuGraphGetNodes(raw, count))[0]:
+        kind = ok(driver.cuGraphNodeGetType(node))
+        if kind == driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            p = ok(driver.cuGraphKernelNodeGetParams(node))
+            name = ok(driver.cuFuncGetName(p.func)) if int(p.func) else ok(driver.cuKernelGetName(p.kern))
+            names.append(name.decode())
+        else:
+            names.append({driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_MEM_ALLOC: "alloc", driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_MEM_FREE: "free"}.get(kind, "other"))
+    return graph, out, names

@@ -22,3 +22,28 @@ def test_ragged_rows_against_generic(key, M, N, blocks):
             got = mmasim.gemm(model, A, B, d["C"], large_tiles=True)
             assert mmasim.last_variant() == "large_tiles"
             assert torch.equal(got, want), (key, (M, N, K), int((got != want).sum()))
+
+
+@pytest.mark.parametrize("key", [("ampere", "fp16", "fp32"), ("hopper", "e4m3", "fp32"), ("cdna1", "bf16", "fp32")], ids="-".join)
+def test_graphs_of_ragged_calls_hold_no_memory(key):
+    """What is recorded can be cloned and instantiated twice, as a graph with memory nodes cannot."""
+    from cuda.bindings import runtime
+    from paper_2511_10909_b200 import mmasim
+    model = mmasim.Model(*key)
+    M, N, K = 1000, 1111, 96 + model.l_max if model.l_max < 32 else 128
+    v = _inputs(key, M, N, K, 650)[0]
+    A, B, C = (gu.dev(v[k]) for k in ("A", "B", "C"))
+    A = torch.nn.functional.pad(A, (0, 3))[:, :-3]
+    want = mmasim.gemm(model, A, B, C, large_tiles=True)
+    assert mmasim.last_variant() == "large_tiles"
+    graph, out, nodes = gu.recorded(lambda: mmasim.gemm(model, A, B, C, large_tiles=True))
+    assert len(nodes) == 1 and "direct_kernel" in nodes[0], nodes
+    done = lambda r: (r[0] == runtime.cudaError_t.cudaSuccess or pytest.fail(str(r[0]))) and r[-1]
+    raw = runtime.cudaGraph_t(graph.raw_cuda_graph())
+    execs = [done(runtime.cudaGraphInstantiate(g, 0)) for g in (raw, raw, done(runtime.cudaGraphClone(raw)))]
+    for e in execs:
+        out.zero_()
+        done(runtime.cudaGraphLaunch(e, torch.cuda.current_stream().cuda_stream) + (True,))
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
+        done(runtime.cudaGraphExecDestroy(e) + (True,))
