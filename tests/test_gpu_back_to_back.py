@@ -90,3 +90,61 @@ def test_calls_back_to_back():
     for t in threads:
         t.join()
     assert wrong == [0] * 30
+
+
+def _products_only(operands, outs, sync=lambda: None):
+    """Library calls and nothing else in the stream: D of one is C of the next, some in place; scratch of one call is that of the next
+    (the large tiles' decoded operands, the matrix instruction's flags)."""
+    from paper_2511_10909_b200 import mmasim
+    for (model, A, B, C), (D, E) in zip(operands, outs):
+        mmasim.gemm(model, A, B, C, out=D)
+        sync()
+        mmasim.gemm(model, A, B, D, out=E)
+        sync()
+        mmasim.gemm(model, A, B, E, out=E)
+        sync()
+        mmasim.gemm(model, A, B, E, out=D)
+        sync()
+    for (model, A, B, _), (D, E) in zip(reversed(operands), reversed(outs)):
+        mmasim.gemm(model, A, B, D, out=D)
+        sync()
+
+
+def test_products_right_behind_each_other():
+    operands = _operands()
+    make = lambda: [tuple(torch.empty_like(C) for _ in range(2)) for _, _, _, C in operands]
+    want = make()
+    _products_only(operands, want, sync=torch.cuda.synchronize)
+    same = lambda got: all(torch.equal(a, b) for x, y in zip(got, want) for a, b in zip(x, y))
+    got = make()
+    for _ in range(20):
+        _products_only(operands, got)
+        assert same(got)
+    nodes = gu.recorded(lambda: _products_only(operands, got))[2]
+    assert "other" not in nodes and all(x in ("alloc", "free") or "mmasim" in x for x in nodes), nodes
+    stream = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=stream):
+        _products_only(operands, got)
+    for _ in range(5):
+        for x in got:
+            x[0].zero_(), x[1].zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert same(got)
+    wrong = []
+    def run():
+        own, mine = torch.cuda.Stream(), make()
+        with torch.cuda.stream(own):
+            for _ in range(10):
+                _products_only(operands, mine)
+                own.synchronize()
+                wrong.append(not same(mine))
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=run) for _ in range(3)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert wrong == [False] * 30

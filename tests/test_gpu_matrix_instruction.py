@@ -74,6 +74,28 @@ def test_matrix_instruction_against_generic(key):
     assert mmasim.copy_timeouts() == 0
 
 
+@pytest.mark.parametrize("acc", ["fp32", "fp16"])
+def test_fp16_on_either_instruction(acc):
+    """FP16 products of at most 296 tiles of 16 x 32 run on mma.sync, which leaves most of the shapes above to it; larger ones on tcgen05.mma:
+    every width of its tiles, K beyond its ring of stages and off a stage, short blocks, the dequantisation epilogue."""
+    from paper_2511_10909_b200 import mmasim
+    model = mmasim.Model("hopper", "fp16", acc)
+    g = wl.rng(340)
+    for n, (M, N, K) in enumerate([(16, 9472, 48), (16, 9473, 48), (1, 9600, 1040), (17, 5000, 2064), (40, 4000, 144), (70, 3000, 1040), (129, 1100, 528), (300, 1000, 2064),
+                                   (50, 2400, 8)]):
+        tiles = -(-M // 16) * -(-N // 32)
+        kws = [{}] if acc == "fp16" else [{}, dict(row_scale=gu.dev(g.standard_normal(M).astype(np.float32)), col_scale=gu.dev(g.standard_normal(N).astype(np.float32)))]
+        for v in _variants(("hopper", "fp16", acc), M, N, K, 341 + n):
+            for kw in kws:
+                for C in (v["C"], None):
+                    _compare(model, v, K, C, (acc, (M, N, K), list(kw), C is None), **kw)
+        A, B = gu.dev(v["A"]), gu.dev(v["B"])
+        nodes = gu.recorded(lambda: mmasim.gemm(model, A, B))[2]
+        ran = [x for x in nodes if "mma_kernel" in x]
+        assert len(ran) == 1 and ("warp_mma_kernel" in ran[0]) == (tiles <= 296) and ("umma_kernel" in ran[0]) == (tiles > 296), ((M, N, K), nodes)
+    assert mmasim.copy_timeouts() == 0
+
+
 @pytest.mark.parametrize("key", [k for k in KEYS if k[1] in GUARDED], ids=lambda k: "-".join(k))
 def test_few_rows_of_kinds_with_small_products(key):
     """Every width of tile (16 to 256 rows of A) with K long enough that the instruction runs; flags at the edges of such tiles."""

@@ -24,6 +24,24 @@ def test_ragged_rows_against_generic(key, M, N, blocks):
             assert torch.equal(got, want), (key, (M, N, K), int((got != want).sum()))
 
 
+# rows off 16 bytes under scale factors, and with promoted sums and dequantisation scales: every kernel that takes either
+@pytest.mark.parametrize("key", [k for k in KEYS if k[2] == "fp32" and (k[1].startswith("mx") or not k[0].startswith("cdna"))], ids=lambda k: "-".join(k))
+def test_strides_off_16_bytes_with_scales_and_promotion(key):
+    from paper_2511_10909_b200 import mmasim
+    model = mmasim.Model(*key)
+    for M, N, K in ((63, 129, 192), (130, 65, 384)):
+        scales = dict(row_scale=torch.rand(M, device="cuda") * 4, col_scale=torch.rand(N, device="cuda") * 4)
+        for v in _inputs(key, M, N, K, 660 + M):
+            d = {k: gu.dev(x) for k, x in v.items()}
+            sf = {k: d[k] for k in ("sfa", "sfb") if k in d}
+            A, B = (torch.nn.functional.pad(d[k], (0, 3))[:, :-3] for k in ("A", "B"))
+            for kw in ({}, dict(k_chunk=32), dict(k_chunk=64, **scales), dict(k_chunk=K, **scales)):
+                want = mmasim.gemm(model, d["A"], d["B"], d["C"], force_generic=True, **kw, **sf)
+                got = mmasim.gemm(model, A, B, d["C"], large_tiles=True, **kw, **sf)
+                assert mmasim.last_variant() == "large_tiles"
+                assert torch.equal(got, want), (key, (M, N, K), list(kw), int((got != want).sum()))
+
+
 @pytest.mark.parametrize("key", [("ampere", "fp16", "fp32"), ("hopper", "e4m3", "fp32"), ("cdna1", "bf16", "fp32")], ids="-".join)
 def test_graphs_of_ragged_calls_hold_no_memory(key):
     """What is recorded can be cloned and instantiated twice, as a graph with memory nodes cannot."""
