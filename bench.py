@@ -79,11 +79,11 @@ def compute_dtype(kernel: str, model) -> str:
             "efdpa": "f64", "dot_tfdpa": "f64", "dot_ftz": "f32", "ftz_addmul": "f32", "fma_f32": "f32", "fma_f64": "f64", "gstfdpa": "int32"}.get(kernel, "int64")
 
 
-# DRAM bytes per step (the main kernel and the two decode launches before it): dram__bytes_read.sum +
-# dram__bytes_write.sum of a one-pass ncu capture of the same workload at its full size, a STORED CONSTANT, not a figure
+# DRAM bytes per step (the main kernel, and the decode pass before it when A and B had a launch each): dram__bytes_read.sum
+# + dram__bytes_write.sum of a one-pass ncu capture of the same workload at its full size, a STORED CONSTANT, not a figure
 # of this run.  Algorithmic bytes are 168 MB at 4096^3 (operands once, C and D); the rest is the decoded operand blocks
 # (222 MB, larger than the L2) written once and re-read by the tiles of later waves.  The kernels are bound by arithmetic:
-# 1.16 GB in 3.84 ms is 5 % of what the memory could move in that time.
+# 1.16 GB in 3.75 ms is 5 % of what the memory could move in that time.
 NCU_DRAM_BYTES = {"cfg3": (958592768 + 64196608) + (16791552 + 54993920) + (16790528 + 49194752),
                   "cfg3_2k": (73170688 + 6797824) + 4204288 + 4204800}
 NCU_ALGORITHMIC_BYTES = {"cfg3": 2 * 4096 * 4096 + 2 * 4 * 4096 * 4096, "cfg3_2k": 2 * 2048 * 2048 + 2 * 4 * 2048 * 2048}
@@ -92,13 +92,13 @@ DECODING = ("tfdpa_lut8", "tfdpa_f16", "tfdpa_bf16", "tfdpa_tf32", "trfdpa", "gt
 
 
 def kernels_per_call(kernel: str, variant: str, model) -> int:
-    """Kernels one library call launches: the large-tile fused-summation kernels decode A and B into scratch blocks first; in front
+    """Kernels one library call launches: the large-tile fused-summation kernels decode A and B into scratch blocks first, in one launch; in front
     of the matrix instruction FP6 and FP4 codes are packed and the exponents of BF16 and TF32 rows looked at, and behind it the
     emulation looks for tiles that it has to do (not for FP16, unscaled 8-bit and NVFP4 operands)."""
     if variant == "matrix_instruction":
         fmt = model.in_fmt
         return 1 + (fmt.removeprefix("mx") in ("e2m3", "e3m2", "e2m1")) + 2 * (fmt in ("bf16", "tf32")) + fmt.startswith("mx")
-    return 3 if variant == "large_tiles" and kernel in DECODING else 1
+    return 2 if variant == "large_tiles" and kernel in DECODING else 1
 
 
 SMS = 148
@@ -515,7 +515,7 @@ def run_ours(args):
                             "tensor-core product of powers, so this fraction may exceed 1 and bounds nothing")
         roofline = {"bound": "alu", **pipe_view(pipe_key, pipe_ops_per_mac, per_gpu_macs_s, key[1]), "kernel": kernel_name,
                     "traffic": NCU_DRAM_BYTES.get(name),
-                    "traffic_source": "stored constant from a one-pass ncu capture of this workload at full size, main kernel + both decode launches (not measured in this run)" if name in NCU_DRAM_BYTES else None,
+                    "traffic_source": "stored constant from a one-pass ncu capture of this workload at full size, main kernel + decode pass (not measured in this run)" if name in NCU_DRAM_BYTES else None,
                     "algorithmic_bytes": NCU_ALGORITHMIC_BYTES.get(name),
                     "paper_level_integer_count": int_view}
 
