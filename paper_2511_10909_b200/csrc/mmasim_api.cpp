@@ -166,6 +166,17 @@ cudaError_t scratch_pool(cudaMemPool_t* out) {
     return cudaSuccess;
 }
 
+cudaError_t take_scratch(const GemmArgs& g, size_t bytes, cudaStream_t stream, void** out) {
+    *out = g.scratch;
+    if (g.scratch && bytes <= g.scratch_bytes) return cudaSuccess;
+    cudaMemPool_t pool = nullptr;
+    const cudaError_t err = scratch_pool(&pool);
+    return err != cudaSuccess ? err : cudaMallocFromPoolAsync(out, bytes, pool, stream);
+}
+cudaError_t give_scratch(const GemmArgs& g, void* scratch, cudaStream_t stream) {
+    return scratch == g.scratch ? cudaSuccess : cudaFreeAsync(scratch, stream);
+}
+
 namespace {
 // The streams and events of one mmasim_gemm_host call (mmasim_deviation_stats uses only the memory), and a word of mapped host memory
 // that its kernels count given-up waits in (a copy of the device's counter before and after each call cost 15 us).  Creating them took about 100 us of every call, so up to
@@ -389,6 +400,7 @@ int mmasim_gemm_host(const mmasim_model* model, int64_t M, int64_t N, int64_t K,
     // one alone does not fill the SMs.  Large tiles want 512 rows: every one walks all of K, and the last panel's come last.
     // In us, one panel / several: Ampere BF16 1475 x 1214 x 1072 890 / 675, 1477 x 1229 x 144 283 / 256, 1216 x 1306 x 624 604 / 430,
     // Hopper E4M3 2048 x 2048 x 2048 1460 / 1130 (384 rows: 1215).
+    const int flags = opts ? opts->flags : 0;
     const bool large_tiles = fast_tfdpa_supported(model->dev, g) && !umma_supported(model->dev, g) && direct_size(model->dev, g) == DIRECT_NONE;
     int panels = int((a_bytes + c_bytes + d_bytes) / (size_t(3) << 20));
     panels = panels < 1 || M < 512 ? 1 : (panels > HostLane::PANELS ? HostLane::PANELS : panels);
@@ -403,13 +415,30 @@ int mmasim_gemm_host(const mmasim_model* model, int64_t M, int64_t N, int64_t K,
     cudaError_t err = take_lane(&lane);
     cudaMemPool_t pool = nullptr;
     if (err == cudaSuccess) err = scratch_pool(&pool);
-    // one allocation, stream-ordered out of the library's own pool (which keeps up to 1 GiB between calls)
+    // One allocation, stream-ordered out of the library's own pool (which keeps up to 1 GiB between calls), the scratch of the panels in it:
+    // blocks that went back on the panels' streams made every later allocation look at them (a call of 128 x 128 x 64 took 51 us, 68 behind a
+    // product in six panels).
     auto up256 = [](size_t x) { return (x + 255) / 256 * 256; };
     const size_t sizes[8] = {a_bytes, b_bytes, c_bytes, d_bytes, sfa_bytes, sfb_bytes, g.row_scale ? size_t(M) * 4 : 0, g.col_scale ? size_t(N) * 4 : 0};
-    size_t total = 0;
+    size_t total = 0, scratch_at[HostLane::PANELS + 1];
     for (size_t x : sizes) total += up256(x);
+    for (int p = 0; p <= panels; ++p) {
+        scratch_at[p] = total;
+        if (p == panels || (flags & MMASIM_GEMM_FORCE_GENERIC)) continue;
+        GemmArgs q = g;
+        q.M = p + 1 < panels ? panel_rows : M - p * panel_rows;
+        if (!(flags & MMASIM_GEMM_LARGE_TILES) && umma_supported(model->dev, q)) total += up256(umma_scratch(model->dev, q));
+        else if (large_tiles) total += up256(fast_tfdpa_scratch(model->dev, q));
+    }
     unsigned char* base = nullptr;
-    if (err == cudaSuccess) err = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&base), total, pool, lane.in);
+    if (err == cudaSuccess) {
+        err = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&base), total, pool, lane.in);
+        if (err == cudaErrorMemoryAllocation && total > scratch_at[0]) {  // the panels see for themselves, one after the other
+            cudaGetLastError();
+            for (size_t& x : scratch_at) x = scratch_at[0];
+            err = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&base), scratch_at[0], pool, lane.in);
+        }
+    }
     unsigned char* at[8];
     size_t off = 0;
     for (int i = 0; i < 8; ++i) { at[i] = sizes[i] ? base + off : nullptr; off += up256(sizes[i]); }
@@ -469,7 +498,9 @@ int mmasim_gemm_host(const mmasim_model* model, int64_t M, int64_t N, int64_t K,
         q.sfb = dSB;
         q.row_scale = dRS ? reinterpret_cast<const float*>(dRS) + r0 : nullptr;
         q.col_scale = reinterpret_cast<const float*>(dCS);
-        st = run_gemm(model, q, opts ? opts->flags : 0, sk, &host);
+        q.scratch = scratch_at[p + 1] > scratch_at[p] ? base + scratch_at[p] : nullptr;
+        q.scratch_bytes = scratch_at[p + 1] - scratch_at[p];
+        st = run_gemm(model, q, flags, sk, &host);
         if (st != MMASIM_OK) break;
         if (panels > 1) {
             err = cudaEventRecord(lane.ev_k[p], sk);

@@ -98,6 +98,8 @@ struct GemmArgs {
     const unsigned char* redo;
     int redo_rows, redo_across;
     unsigned int* copy_timeouts;  // device counter of CTAs whose bounded wait on a bulk copy ran out (may be NULL)
+    void* scratch;                // memory for the call's scratch (see take_scratch), or NULL
+    size_t scratch_bytes;
 };
 
 }  // namespace mmasim
@@ -115,15 +117,18 @@ bool registry_lookup(int arch, int a_fmt, int b_fmt, int acc_fmt, mmasim_model* 
 int launch_generic(const DevModel& m, const GemmArgs& g, cudaStream_t stream);
 // mmasim_tfdpa_fast.cu
 bool fast_tfdpa_supported(const DevModel& m, const GemmArgs& g);
+size_t fast_tfdpa_scratch(const DevModel& m, const GemmArgs& g);         // bytes that launch_fast_tfdpa takes at most
 int launch_fast_tfdpa(const DevModel& m, const GemmArgs& g, cudaStream_t stream);
 // the small-tile kernels (mmasim_direct.cuh): any K, any row stride; DIRECT_NONE: the large kernel is the better one
 enum DirectSize : int { DIRECT_NONE = 0, DIRECT_8x16, DIRECT_16x16, DIRECT_32x32 };
 DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us = nullptr);       // `us`: about what the emulation takes
+DirectSize small_size(const DevModel& m, const GemmArgs& g);                                // the best of the small tiles (where they take the call)
 int launch_direct(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStream_t stream);
 int launch_gemm_noalloc(const DevModel& m, const GemmArgs& g, cudaStream_t stream);   // status code; sets the error message
 // mmasim_umma.cu: the rows that the B200's own matrix instruction computes
 bool umma_supported(const DevModel& m, const GemmArgs& g);
 int launch_umma(const DevModel& m, const GemmArgs& g, cudaStream_t stream);
+size_t umma_scratch(const DevModel& m, const GemmArgs& g);              // bytes that launch_umma takes
 // mmasim_warp_mma.cu: FP16 products of few rows (of those that umma_supported takes) on the warp-level instruction
 bool warp_mma_supported(const DevModel& m, const GemmArgs& g);
 cudaError_t launch_warp_mma(const DevModel& m, const GemmArgs& g, cudaStream_t stream);
@@ -161,6 +166,9 @@ int launch_int_peak(int kind, int64_t blocks, int64_t iters, void* sink, int32_t
 // mmasim_api.cpp
 unsigned int* copy_timeout_counter();          // the current device's counter (a device variable of the library; NULL on failure)
 cudaError_t scratch_pool(cudaMemPool_t* out);   // the library's own memory pool of the current device (created on first use)
+// Scratch of a call: g.scratch if it is large enough, else out of the pool in the order of the stream, and back behind the call's kernels.
+cudaError_t take_scratch(const GemmArgs& g, size_t bytes, cudaStream_t stream, void** out);
+cudaError_t give_scratch(const GemmArgs& g, void* scratch, cudaStream_t stream);
 // The status of a call that came to `st` and whose kernels counted `count` given-up waits, which join the device's total.
 int given_up_waits(int st, unsigned int count, int device, const char* call);
 void set_error(const char* fmt, ...);

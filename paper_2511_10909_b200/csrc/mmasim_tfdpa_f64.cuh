@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(256) decode64_kernel(DevModel m, Side64<BM, FO
     else decode64<EK, BN, false, BASE, EOSPLIT, TINY_ZEROS, FORM>(m, b, nch, blockIdx.x - blocks_a);
 }
 
-// Scratch (the decoded blocks of A and B, stream-ordered out of the library's pool and returned to it behind the kernel), the decode
+// Scratch (the decoded blocks of A and B), the decode
 // pass and the kernel that reads its blocks.
 template <int EK, int BASE, bool EOSPLIT, bool TINY_ZEROS, int FORM>
 cudaError_t decode_and_run(void (*kernel)(DevModel, GemmArgs, const Blk64<BM, FORM>*, const Blk64<BN, FORM>*), const DevModel& m, const GemmArgs& g, bool scaled,
@@ -290,17 +290,16 @@ cudaError_t decode_and_run(void (*kernel)(DevModel, GemmArgs, const Blk64<BM, FO
     if (err != cudaSuccess) return err;
     const int64_t tiles_m = (g.M + BM - 1) / BM, tiles_n = (g.N + BN - 1) / BN, nch = (g.K + KC - 1) / KC;
     const size_t bytes_a = size_t(tiles_m * nch) * sizeof(Blk64<BM, FORM>), bytes_b = size_t(tiles_n * nch) * sizeof(Blk64<BN, FORM>);
-    cudaMemPool_t pool = nullptr;
-    if ((err = scratch_pool(&pool)) != cudaSuccess) return err;
+    static_assert(sizeof(Blk64<BM, FORM>) <= fast::BLK64_BYTES && BM == 64 && BN == 64, "what fast_tfdpa_scratch counts with");
     void* ws = nullptr;
-    if ((err = cudaMallocFromPoolAsync(&ws, bytes_a + bytes_b, pool, stream)) != cudaSuccess) return err;
+    if ((err = take_scratch(g, bytes_a + bytes_b, stream, &ws)) != cudaSuccess) return err;
     Blk64<BM, FORM>* wa = static_cast<Blk64<BM, FORM>*>(ws);
     Blk64<BN, FORM>* wb = reinterpret_cast<Blk64<BN, FORM>*>(static_cast<unsigned char*>(ws) + bytes_a);
     const Side64<BM, FORM> a{static_cast<const unsigned char*>(g.A), g.M, g.lda, fast::pad_of<EK>(g.K, g.lda), wa, scaled ? g.sfa : nullptr, g.ld_sfa};
     const Side64<BN, FORM> b{static_cast<const unsigned char*>(g.B), g.N, g.ldb, fast::pad_of<EK>(g.K, g.ldb), wb, scaled ? g.sfb : nullptr, g.ld_sfb};
     err = enqueue(decode, unsigned(nch * (tiles_m + tiles_n)), 256, dsh, stream, m, a, b, unsigned(nch), unsigned(nch * tiles_m));
     if (err == cudaSuccess) err = enqueue(kernel, unsigned(tiles_n * tiles_m), NT, sh, stream, m, g, wa, wb);
-    const cudaError_t err2 = cudaFreeAsync(ws, stream);
+    const cudaError_t err2 = give_scratch(g, ws, stream);
     return err != cudaSuccess ? err : err2;
 }
 

@@ -154,6 +154,7 @@ static DirectSize choose_size(const DevModel& m, const GemmArgs& g, bool large_t
 }
 
 DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us) { return choose_size(m, g, true, us); }
+DirectSize small_size(const DevModel& m, const GemmArgs& g) { return choose_size(m, g, false, nullptr); }
 
 int launch_direct(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStream_t stream) {
     cudaError_t err = cudaErrorInvalidValue;
@@ -218,6 +219,13 @@ int launch_gemm_noalloc(const DevModel& m, const GemmArgs& g, cudaStream_t strea
     return MMASIM_OK;
 }
 
+size_t fast_tfdpa_scratch(const DevModel& m, const GemmArgs& g) {
+    auto tiles = [](int64_t rows, int64_t of) { return size_t((rows + of - 1) / of); };
+    const size_t chunks = tiles(g.K, fast::KC);
+    if (m.F != 13 || kind_of(m) != 1 + fast::EK_LUT8) return chunks * fast::BLK64_BYTES * (tiles(g.M, 64) + tiles(g.N, 64));
+    return chunks * (tiles(g.M, fast::BM) * fast::blk_t_bytes(fast::BM) + std::max(tiles(g.N, 64) * fast::blk_t_bytes(64), tiles(g.N, 128) * fast::blk_t_bytes(128)));
+}
+
 // A stream whose work is being recorded into a graph.
 static bool capturing(cudaStream_t stream) {
     cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
@@ -228,7 +236,7 @@ static bool capturing(cudaStream_t stream) {
 int launch_fast_tfdpa(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
     // Ragged rows run on the small tiles where the decoded operands get no memory, and in a graph: one with memory nodes in it cannot be
     // cloned, made part of another one or instantiated twice, and those of ragged calls never had any.  (Whole chunks on large tiles always did.)
-    if (ragged(m, g) && capturing(stream)) return launch_direct(m, g, choose_size(m, g, false, nullptr), stream);
+    if (ragged(m, g) && capturing(stream)) return launch_direct(m, g, small_size(m, g), stream);
     cudaError_t err = cudaErrorInvalidValue;
     if (kind_of(m) == KIND_TR) {
         set_kernel_name(m.family == FAM_GTR ? "gtrfdpa" : "trfdpa", "large_tiles");
@@ -245,7 +253,7 @@ int launch_fast_tfdpa(const DevModel& m, const GemmArgs& g, cudaStream_t stream)
     }
     if (err == cudaErrorMemoryAllocation && ragged(m, g)) {
         cudaGetLastError();
-        return launch_direct(m, g, choose_size(m, g, false, nullptr), stream);
+        return launch_direct(m, g, small_size(m, g), stream);
     }
     if (err != cudaSuccess) {
         set_error("tuned T-FDPA kernel launch failed: %s", cudaGetErrorString(err));

@@ -60,6 +60,10 @@ __device__ __forceinline__ uint32_t raw_elem(const void* p, int64_t idx) {
     return static_cast<const uint32_t*>(p)[idx];
 }
 
+// Bytes of a decoded block: 64 rows (or columns) x 32 elements of the FP64 kernels at most, R of them of the F = 13 kernels.
+constexpr size_t BLK64_BYTES = 64 * ((KC + 4) * 8 + (KC + 8) * 2 + 9) + 16;
+constexpr size_t blk_t_bytes(int R) { return size_t(R) * (KC * 4 + (KC + 8) * 2 + 4) + 16; }
+
 // K is filled up to whole chunks with zeros in front of the first element.  `wide`: rows and chunks start on 16 bytes.
 struct Pad { int front; bool wide; };
 __host__ __device__ __forceinline__ int front_pad(int64_t K) { return int((KC - K % KC) % KC); }

@@ -104,6 +104,7 @@ struct BlkT {
     uint32_t sparse;                    // nonzero: a row (of the matrix) has a block of L with half or more of its elements zero
     uint32_t pad[2];
 };
+static_assert(sizeof(BlkT<128>) == fast::blk_t_bytes(128) && sizeof(BlkT<64>) == fast::blk_t_bytes(64), "what fast_tfdpa_scratch counts with");
 static_assert(sizeof(BlkT<128>) % 16 == 0 && sizeof(BlkT<64>) % 16 == 0, "bulk copies move multiples of 16 bytes");
 
 template <int TH>
@@ -621,8 +622,7 @@ __global__ void __launch_bounds__(NT, 2) tfdpa_trop_kernel(DevModel m, GemmArgs 
 #undef MMASIM_SP_WORD
 }
 
-// Where the decoded blocks go: memory of the caller's (given != nullptr, capacity bytes) or, by default, a stream-ordered
-// allocation out of the library's pool, returned to it behind the kernel.
+// Where the decoded blocks go: a fixed array (given != nullptr, capacity bytes) or, by default, the call's scratch.
 struct Scratch {
     void* given = nullptr;
     size_t capacity = 0;
@@ -647,9 +647,7 @@ cudaError_t launch_one_t(const DevModel& m, const GemmArgs& g, cudaStream_t stre
     if (ws) {
         if (bytes_a + bytes_b > sc.capacity) return cudaErrorInvalidValue;      // the caller checked: never reached
     } else {
-        cudaMemPool_t pool = nullptr;
-        if ((err = scratch_pool(&pool)) != cudaSuccess) return err;
-        if ((err = cudaMallocFromPoolAsync(&ws, bytes_a + bytes_b, pool, stream)) != cudaSuccess) return err;
+        if ((err = take_scratch(g, bytes_a + bytes_b, stream, &ws)) != cudaSuccess) return err;
     }
     BlkT<BM>* wa = static_cast<BlkT<BM>*>(ws);
     BlkT<BN>* wb = reinterpret_cast<BlkT<BN>*>(static_cast<unsigned char*>(ws) + bytes_a);
@@ -664,7 +662,7 @@ cudaError_t launch_one_t(const DevModel& m, const GemmArgs& g, cudaStream_t stre
     }
     if (err == cudaSuccess) err = enqueue(tfdpa_trop_kernel<EK, L, F, RHO, PROMOTE, BASE, TH>, dim3((unsigned)tiles_n, (unsigned)tiles_m, 1), NT, sh, stream, m, g, wa, wb);
     if (sc.given) return err;
-    const cudaError_t err2 = cudaFreeAsync(ws, stream);
+    const cudaError_t err2 = give_scratch(g, ws, stream);
     return err != cudaSuccess ? err : err2;
 }
 

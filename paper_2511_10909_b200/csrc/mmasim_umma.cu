@@ -642,6 +642,23 @@ int pick_columns(const GemmArgs& g, int mk, bool acc16, int steps) {
 
 // Kinds with products below 2^-126 (see the top).
 bool guarded(const DevModel& m, int mk) { return mk == MK_MX8 || mk == MK_MXF4 || mk == MK_TF32 || (mk == MK_F16 && m.fmt_a == EF_BF16); }
+// Scratch of launch_umma: packed codes of A and B, the smallest exponents of their rows, flags of tiles.
+struct UmmaScratch {
+    int bits_a, bits_b;
+    int64_t pk;                         // bytes of a row of packed codes
+    size_t pa, pb, le, fl;
+    UmmaScratch(const DevModel& m, const GemmArgs& g, int mk, int64_t tiles) {
+        const bool narrow = mk == MK_F8 || mk == MK_MX8;
+        bits_a = narrow ? code_bits(m.fmt_a) : 8;
+        bits_b = narrow ? code_bits(m.fmt_b) : 8;
+        pk = up(g.K, 16);
+        pa = bits_a < 8 ? size_t(up(g.M * pk, 256)) : 0;
+        pb = bits_b < 8 ? size_t(up(g.N * pk, 256)) : 0;
+        le = guarded(m, mk) && sf_per_step(mk) == 0 ? size_t(4 * (g.M + g.N)) : 0;
+        fl = guarded(m, mk) ? size_t(tiles) : 0;
+    }
+    size_t bytes() const { return pa + pb + le + fl; }
+};
 bool overlap(const GemmArgs& g) {
     const char *c = static_cast<const char*>(g.C), *d = static_cast<const char*>(g.D);
     return c && c < d + ((g.M - 1) * g.ldd + g.N) * 4 && d < c + ((g.M - 1) * g.ldc + g.N) * 4;
@@ -664,6 +681,11 @@ bool umma_supported(const DevModel& m, const GemmArgs& g) {
     double us = 0.0;
     direct_size(m, g, &us);
     return us > (mk == MK_MX8 && code_bits(m.fmt_a) == 8 && code_bits(m.fmt_b) == 8 ? 11.0 : 15.0);
+}
+
+size_t umma_scratch(const DevModel& m, const GemmArgs& g) {
+    const int mk = kind_of(m), bn = pick_columns(g, mk, m.acc == ACC_F16, int((row_bytes(m, g.K) + 31) / 32));
+    return UmmaScratch(m, g, mk, (g.N + LANES - 1) / LANES * ((g.M + bn - 1) / bn)).bytes();
 }
 
 int launch_umma(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
@@ -695,19 +717,15 @@ int launch_umma(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
     if (scaled) a.idesc |= uint32_t(m.scale_fmt == EF_E8M0) << 23;
     else if (m.acc != ACC_F16) a.idesc |= 1u << 4;
 
-    // scratch: packed codes, smallest exponents, flags of tiles
-    const bool narrow = mk == MK_F8 || mk == MK_MX8, guard = guarded(m, mk);
-    const int bits_a = narrow ? code_bits(m.fmt_a) : 8, bits_b = narrow ? code_bits(m.fmt_b) : 8;
-    const int64_t pk = up(g.K, 16);
-    const size_t pa = bits_a < 8 ? size_t(up(g.M * pk, 256)) : 0, pb = bits_b < 8 ? size_t(up(g.N * pk, 256)) : 0;
-    const size_t le = guard && !scaled ? size_t(4 * (g.M + g.N)) : 0, fl = guard ? size_t(a.tiles) : 0;
+    const bool guard = guarded(m, mk);
+    const UmmaScratch sc(m, g, mk, a.tiles);
+    const int bits_a = sc.bits_a, bits_b = sc.bits_b;
+    const int64_t pk = sc.pk;
+    const size_t pa = sc.pa, pb = sc.pb, le = sc.le, fl = sc.fl;
     cudaError_t err = cudaSuccess;
     unsigned char* scratch = nullptr;
-    if (pa + pb + le + fl) {
-        cudaMemPool_t pool;
-        err = scratch_pool(&pool);
-        if (err == cudaSuccess) err = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&scratch), pa + pb + le + fl, pool, stream);
-    }
+    if (sc.bytes()) err = take_scratch(g, sc.bytes(), stream, reinterpret_cast<void**>(&scratch));
+    if (err != cudaSuccess) scratch = nullptr;
     int* least = reinterpret_cast<int*>(scratch + pa + pb);
     a.least_l = le ? least + g.M : nullptr;
     a.least_q = le ? least : nullptr;
@@ -758,7 +776,7 @@ int launch_umma(const DevModel& m, const GemmArgs& g, cudaStream_t stream) {
         e.redo_across = a.tiles_q;
         st = mk == MK_MXF4 ? launch_fast_gst(m, e, stream) : launch_direct(m, e, DIRECT_32x32, stream);
     }
-    if (scratch) cudaFreeAsync(scratch, stream);
+    if (scratch) give_scratch(g, scratch, stream);
     set_kernel_name(mk >= MK_MXF4 ? "gstfdpa" : (mk == MK_TF32 ? "tfdpa_tf32" : (mk != MK_F16 ? "tfdpa_lut8" : (m.fmt_a == EF_F16 ? "tfdpa_f16" : "tfdpa_bf16"))), "matrix_instruction");
     if (err != cudaSuccess) {
         set_error("matrix-instruction kernel launch failed: %s", cudaGetErrorString(err));
