@@ -63,11 +63,13 @@ int check_k(const DevModel& m, int64_t K) {
     return MMASIM_OK;
 }
 
-// `whole`: the product that g is a row panel of, if it is one: its size decides on the tiles (panels run beside each other).
-int dispatch(const mmasim_model* model, const GemmArgs& g, int flags, cudaStream_t stream, const GemmArgs* whole) {
+// `whole`: the product that g is a row panel of, if it is one: its size decides on the tiles (panels run beside each other).  `small`: on
+// small tiles, whatever direct_size says.
+int dispatch(const mmasim_model* model, const GemmArgs& g, int flags, cudaStream_t stream, const GemmArgs* whole, bool small) {
     const DevModel& m = model->dev;
     if (!(flags & MMASIM_GEMM_FORCE_GENERIC) && !m.literal_emax) {
         if (!(flags & MMASIM_GEMM_LARGE_TILES) && umma_supported(m, g)) return launch_umma(m, g, stream);
+        if (small) return launch_direct(m, g, small_size(m, whole ? *whole : g), stream);
         const DirectSize size = (flags & MMASIM_GEMM_LARGE_TILES) && fast_tfdpa_supported(m, g) ? DIRECT_NONE : direct_size(m, whole ? *whole : g);
         if (size != DIRECT_NONE) return launch_direct(m, g, size, stream);
         if (fast_tfdpa_supported(m, g)) return launch_fast_tfdpa(m, g, stream);
@@ -77,8 +79,8 @@ int dispatch(const mmasim_model* model, const GemmArgs& g, int flags, cudaStream
     set_kernel_name("generic", "generic");
     return launch_generic(m, g, stream);
 }
-int run_gemm(const mmasim_model* model, const GemmArgs& g, int flags, cudaStream_t stream, const GemmArgs* whole = nullptr) {
-    const int st = dispatch(model, g, flags, stream, whole);
+int run_gemm(const mmasim_model* model, const GemmArgs& g, int flags, cudaStream_t stream, const GemmArgs* whole = nullptr, bool small = false) {
+    const int st = dispatch(model, g, flags, stream, whole, small);
     if (st == MMASIM_ERR_CUDA) cudaGetLastError();      // (an allocation that failed is this call's error, not the next launch's)
     return st;
 }
@@ -408,8 +410,14 @@ int mmasim_gemm_host(const mmasim_model* model, int64_t M, int64_t N, int64_t K,
     // D replace its own rows of C.)
     const bool in_place = g.C == g.D && g.ldc == g.ldd;
     if (ranges_meet(D, d_bytes, A, a_bytes) || ranges_meet(D, d_bytes, g.sfa, sfa_bytes) || (!in_place && ranges_meet(D, d_bytes, C, c_bytes))) panels = 1;
-    int64_t panel_rows = panels > 1 ? ((M + panels - 1) / panels + 127) / 128 * 128 : M;
-    if (large_tiles && panels > 1 && panel_rows < 512) panel_rows = 512;
+    const int64_t rows_by_bytes = panels > 1 ? ((M + panels - 1) / panels + 127) / 128 * 128 : M;
+    int64_t panel_rows = large_tiles && panels > 1 && rows_by_bytes < 512 ? 512 : rows_by_bytes;
+    bool small_tiles = false;
+    if (large_tiles && !(flags & (MMASIM_GEMM_LARGE_TILES | MMASIM_GEMM_FORCE_GENERIC))) {
+        const int64_t n = (M + panel_rows - 1) / panel_rows;
+        small_tiles = !panels_on_large_tiles(model->dev, g, n, M - (n - 1) * panel_rows);
+        if (small_tiles) panel_rows = rows_by_bytes;
+    }
     panels = int((M + panel_rows - 1) / panel_rows);
     HostLane lane;
     cudaError_t err = take_lane(&lane);
@@ -428,7 +436,7 @@ int mmasim_gemm_host(const mmasim_model* model, int64_t M, int64_t N, int64_t K,
         GemmArgs q = g;
         q.M = p + 1 < panels ? panel_rows : M - p * panel_rows;
         if (!(flags & MMASIM_GEMM_LARGE_TILES) && umma_supported(model->dev, q)) total += up256(umma_scratch(model->dev, q));
-        else if (large_tiles) total += up256(fast_tfdpa_scratch(model->dev, q));
+        else if (large_tiles && !small_tiles) total += up256(fast_tfdpa_scratch(model->dev, q));
     }
     unsigned char* base = nullptr;
     if (err == cudaSuccess) {
@@ -500,7 +508,7 @@ int mmasim_gemm_host(const mmasim_model* model, int64_t M, int64_t N, int64_t K,
         q.col_scale = reinterpret_cast<const float*>(dCS);
         q.scratch = scratch_at[p + 1] > scratch_at[p] ? base + scratch_at[p] : nullptr;
         q.scratch_bytes = scratch_at[p + 1] - scratch_at[p];
-        st = run_gemm(model, q, flags, sk, &host);
+        st = run_gemm(model, q, flags, sk, &host, small_tiles);
         if (st != MMASIM_OK) break;
         if (panels > 1) {
             err = cudaEventRecord(lane.ev_k[p], sk);

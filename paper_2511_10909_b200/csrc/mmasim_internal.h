@@ -123,6 +123,7 @@ int launch_fast_tfdpa(const DevModel& m, const GemmArgs& g, cudaStream_t stream)
 enum DirectSize : int { DIRECT_NONE = 0, DIRECT_8x16, DIRECT_16x16, DIRECT_32x32 };
 DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us = nullptr);       // `us`: about what the emulation takes
 DirectSize small_size(const DevModel& m, const GemmArgs& g);                                // the best of the small tiles (where they take the call)
+bool panels_on_large_tiles(const DevModel& m, const GemmArgs& g, int64_t panels, int64_t last_rows);     // a product for which direct_size has none
 int launch_direct(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStream_t stream);
 int launch_gemm_noalloc(const DevModel& m, const GemmArgs& g, cudaStream_t stream);   // status code; sets the error message
 // mmasim_umma.cu: the rows that the B200's own matrix instruction computes

@@ -156,6 +156,23 @@ static DirectSize choose_size(const DevModel& m, const GemmArgs& g, bool large_t
 DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us) { return choose_size(m, g, true, us); }
 DirectSize small_size(const DevModel& m, const GemmArgs& g) { return choose_size(m, g, false, nullptr); }
 
+// Row panels whose copies and kernels overlap (mmasim_gemm_host) are not what the costs above were fitted to: large tiles end late where
+// the last panel comes last, above all a short one, and every panel decodes B.  So ragged ones, which the small tiles took before, have to
+// gain by the costs: 1.15 times in several panels, 1.4 with a last one of less than two tiles, hardly in one panel or where they fill
+// the places for tiles (two on each of 148 SMs) one and a half times.  Of 366 ragged products that the costs alone give to the large tiles
+// 38 took over 3 % longer on them, by up to 1.32; of those that are left 13 do, by up to 1.21; and 12 of the others would have been over
+// 3 % faster.  Large / small in us (ratio of the costs): Ampere FP16 1998 x 437 x 2488 (1.10) 878 / 666, Ampere TF32 2690 x 602 x 1444
+// (1.12) 1080 / 939, 1314 x 442 x 1416 (1.07) 534 / 474; kept: Ada E5M2 1726 x 527 x 1712 (1.70) 362 / 469, Ampere FP16 2138 x 2503 x 1016
+// (1360 tiles) 1246 / 1448.
+bool panels_on_large_tiles(const DevModel& m, const GemmArgs& g, int64_t panels, int64_t last_rows) {
+    if (!ragged(m, g)) return true;
+    double small = 0.0, large = 0.0;
+    choose_size(m, g, false, &small);
+    choose_size(m, g, true, &large);                   // (it chose the large ones)
+    const int64_t bm = m.F == 13 ? fast::BM : 64, tiles = ((g.M + bm - 1) / bm) * ((g.N + 63) / 64);
+    return small > large * (tiles > 3 * 148 ? 1.04 : (panels == 1 ? 1.02 : (last_rows < 128 ? 1.4 : 1.15)));
+}
+
 int launch_direct(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStream_t stream) {
     cudaError_t err = cudaErrorInvalidValue;
     const int kind = kind_of(m);

@@ -78,3 +78,15 @@ def test_output_over_an_operand():
     A[:] = inp["A"]
     got = mmasim.gemm_host(model, A, inp["B"], inp["C"], out=flat[half:].view(np.uint32).reshape(M, N))
     assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("key,shape,variant", [(("ampere", "tf32", "fp32"), (1998, 454, 1556), "small_tiles"), (("ampere", "bf16", "fp32"), (1136, 1247, 744), "small_tiles"),
+                                               (("ada", "e5m2", "fp32"), (1726, 527, 1712), "large_tiles")], ids=str)
+def test_panels_of_ragged_rows(key, shape, variant):
+    from paper_2511_10909_b200 import mmasim
+    M, N, K = shape
+    inp = wl.normal_inputs(key[1], key[2], M, N, K, seed=8)
+    want = gu.run_gemm(key, inp)
+    got = mmasim.gemm_host(mmasim.Model(*key), inp["A"], inp["B"], inp["C"])
+    assert mmasim.last_variant() == variant
+    assert np.array_equal(got.view(want.dtype), want)
