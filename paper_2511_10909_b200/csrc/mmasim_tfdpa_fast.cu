@@ -157,20 +157,25 @@ DirectSize direct_size(const DevModel& m, const GemmArgs& g, double* us) { retur
 DirectSize small_size(const DevModel& m, const GemmArgs& g) { return choose_size(m, g, false, nullptr); }
 
 // Row panels whose copies and kernels overlap (mmasim_gemm_host) are not what the costs above were fitted to: large tiles end late where
-// the last panel comes last, above all a short one, and every panel decodes B.  So ragged ones, which the small tiles took before, have to
-// gain by the costs: 1.15 times in several panels, 1.4 with a last one of less than two tiles, hardly in one panel or where they fill
-// the places for tiles (two on each of 148 SMs) one and a half times.  Of 366 ragged products that the costs alone give to the large tiles
-// 38 took over 3 % longer on them, by up to 1.32; of those that are left 13 do, by up to 1.21; and 12 of the others would have been over
-// 3 % faster.  Large / small in us (ratio of the costs): Ampere FP16 1998 x 437 x 2488 (1.10) 878 / 666, Ampere TF32 2690 x 602 x 1444
-// (1.12) 1080 / 939, 1314 x 442 x 1416 (1.07) 534 / 474; kept: Ada E5M2 1726 x 527 x 1712 (1.70) 362 / 469, Ampere FP16 2138 x 2503 x 1016
-// (1360 tiles) 1246 / 1448.
+// the last panel comes last, above all a short one, and where those of all panels do not fill the places for tiles (two on each of 148 SMs)
+// some SMs get two and others none; and every panel decodes B.  So ragged products of the FP64 kernels, which the small tiles took before,
+// have to gain by the costs: 1.15 times in several panels, 1.4 with a last one of less than two tiles or with places left, hardly in one
+// panel or with one and a half times as many tiles as places.  (The F = 13 kernels were never slower than the costs say.)  Of 366 ragged
+// products that the costs alone give to the large tiles 38 took over 3 % longer on them, by up to 1.32; of those that are left 13 do, by up to
+// 1.21; and 12 of the others would have been over 3 % faster.  Large / small in us (ratio of the costs): Ampere FP16 1925 x 441 x 1576 (1.09)
+// 584 / 448, Ampere BF16 1479 x 742 x 1800 (1.30, 288 tiles in three panels) 751 / 618, Ampere TF32 1998 x 454 x 1556 (1.09) 908 / 689; kept:
+// CDNA3 E4M3 2471 x 880 x 688 (1.26, 546 tiles) 460 / 526, Ampere FP16 2138 x 2503 x 1016 (1360 tiles) 1246 / 1448.
 bool panels_on_large_tiles(const DevModel& m, const GemmArgs& g, int64_t panels, int64_t last_rows) {
-    if (!ragged(m, g)) return true;
+    if (!ragged(m, g) || m.F == 13) return true;
     double small = 0.0, large = 0.0;
     choose_size(m, g, false, &small);
     choose_size(m, g, true, &large);                   // (it chose the large ones)
-    const int64_t bm = m.F == 13 ? fast::BM : 64, tiles = ((g.M + bm - 1) / bm) * ((g.N + 63) / 64);
-    return small > large * (tiles > 3 * 148 ? 1.04 : (panels == 1 ? 1.02 : (last_rows < 128 ? 1.4 : 1.15)));
+    constexpr int64_t PLACES = 2 * 148;
+    const int64_t tiles = ((g.M + 63) / 64) * ((g.N + 63) / 64);
+    double gain = last_rows < 128 || tiles <= PLACES ? 1.4 : 1.15;
+    if (panels == 1) gain = 1.02;
+    if (2 * tiles > 3 * PLACES) gain = 1.04;
+    return small > gain * large;
 }
 
 int launch_direct(const DevModel& m, const GemmArgs& g, DirectSize size, cudaStream_t stream) {

@@ -34,6 +34,7 @@ def ask(tmp_path_factory):
 @pytest.mark.parametrize("key,M,N,K,ld,panels,last,large", [
     (("cdna3", "e4m3", "fp32"), 418, 1999, 1552, 1552, 1, 418, 0), (("hopper", "e4m3", "fp32"), 786, 591, 736, 744, 1, 786, 1),          # one panel
     (("ampere", "tf32", "fp32"), 1998, 454, 1556, 1556, 4, 462, 0), (("volta", "fp16", "fp32"), 2459, 3151, 364, 364, 5, 411, 1), (("ampere", "fp16", "fp32"), 2733, 2512, 624, 624, 6, 173, 1),       # several
+    (("ampere", "bf16", "fp32"), 1479, 742, 1800, 1800, 3, 455, 0), (("ada", "e5m2", "fp32"), 1219, 935, 1904, 1904, 2, 579, 1),         # places left
     (("ampere", "bf16", "fp32"), 1136, 1247, 744, 744, 3, 112, 0), (("ampere", "fp16", "fp32"), 624, 3300, 520, 520, 2, 112, 1), (("hopper", "e4m3", "fp32"), 1108, 1702, 1248, 1256, 2, 84, 1),        # a short last one
     (("cdna3", "tf32", "fp32"), 1279, 853, 3072, 3072, 3, 255, 1), (("ampere", "fp16", "fp32"), 624, 3300, 544, 544, 2, 112, 1)], ids=str)   # whole chunks
 def test_panels_of_ragged_rows(ask, key, M, N, K, ld, panels, last, large):
