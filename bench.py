@@ -79,12 +79,11 @@ def compute_dtype(kernel: str, model) -> str:
             "efdpa": "f64", "dot_tfdpa": "f64", "dot_ftz": "f32", "ftz_addmul": "f32", "fma_f32": "f32", "fma_f64": "f64", "gstfdpa": "int32"}.get(kernel, "int64")
 
 
-# DRAM bytes per step (the main kernel, and the decode pass before it when A and B had a launch each): dram__bytes_read.sum
-# + dram__bytes_write.sum of a one-pass ncu capture of the same workload at its full size, a STORED CONSTANT, not a figure
-# of this run.  Algorithmic bytes are 168 MB at 4096^3 (operands once, C and D); the rest is the decoded operand blocks
+# DRAM bytes per step (the main kernel and the decode pass before it): dram__bytes_read.sum + dram__bytes_write.sum of a
+# one-pass ncu capture of the same workload at its full size, a STORED CONSTANT, not a figure of this run.  Algorithmic bytes are 168 MB at 4096^3 (operands once, C and D); the rest is the decoded operand blocks
 # (222 MB, larger than the L2) written once and re-read by the tiles of later waves.  The kernels are bound by arithmetic:
-# 1.16 GB in 3.75 ms is 5 % of what the memory could move in that time.
-NCU_DRAM_BYTES = {"cfg3": (958592768 + 64196608) + (16791552 + 54993920) + (16790528 + 49194752),
+# 1.21 GB in 3.75 ms is 5 % of what the memory could move in that time.
+NCU_DRAM_BYTES = {"cfg3": (952933376 + 59121408) + (33588480 + 162421248),
                   "cfg3_2k": (73170688 + 6797824) + 4204288 + 4204800}
 NCU_ALGORITHMIC_BYTES = {"cfg3": 2 * 4096 * 4096 + 2 * 4 * 4096 * 4096, "cfg3_2k": 2 * 2048 * 2048 + 2 * 4 * 2048 * 2048}
 

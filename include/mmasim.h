@@ -277,8 +277,8 @@ int mmasim_deviation_stats(const mmasim_model* model, int64_t M, int64_t N, int6
 int mmasim_int_peak(int kind, int64_t blocks, int64_t iters, void* sink, int32_t* ops_per_round, void* stream);
 
 /* Whose arithmetic the last mmasim_gemm* call on this thread ran: the kernel family ("tfdpa_f16", "gstfdpa", ...), or "generic"; and
- * which of its kernels: "matrix_instruction" (tcgen05.mma, with the emulation behind it where the two can part), "large_tiles",
- * "small_tiles", "streaming" (mmasim_dot_batch) or "generic". */
+ * which of its kernels: "matrix_instruction" (the B200's own: tcgen05.mma, with the emulation behind it where the two can part, or
+ * mma.sync for FP16 products of at most 296 tiles of 16 x 32 outputs, the same words from either), "large_tiles", "small_tiles", "streaming" (mmasim_dot_batch) or "generic". */
 const char* mmasim_last_kernel(void);
 const char* mmasim_last_variant(void);
 

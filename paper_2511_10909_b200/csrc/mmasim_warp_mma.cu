@@ -4,9 +4,8 @@
 //
 // Why.  Every output is a serial chain of K / 16 instructions.  A link of tcgen05.mma takes 40 ns whatever the width up to 64 columns, a
 // link of mma.sync 10.5 (20.7 clocks; 21 ns here with the loads in between); and a tile of 128 lanes makes 32 CTAs of 4096 rows of
-// B, tiles of 32 make 128.  16 x 4096 x 4096 13.1 us on tcgen05.mma, 9.8 here; 128 x 1024 x 4096 (two CTAs on some SMs) 13.1 / 12.0;
-// three CTAs per SM, 33 x 4096 x 4096, 13.2 / 22.1.  The rows of two tiles of A in one CTA took 14.6: the loads of their fragments
-// stand between the links.  (Fragments fetched between the instructions of the stage before, each into registers that the one
+// B, tiles of 32 make 128.  16 x 4096 x 4096 13.1 us on tcgen05.mma, 8.4 here (launches among others).  The rows of two tiles of A in one
+// CTA took 14.6: the loads of their fragments stand between the links.  (Fragments fetched between the instructions of the stage before, each into registers that the one
 // before it still read: 12.4.)
 //
 // Work decomposition.  A CTA owns 16 rows of A and 32 rows of B.  One warp brings in 128 bytes of K per row and stage (tiled bulk copies,
@@ -207,7 +206,10 @@ cudaError_t launch(const GemmArgs& g, cudaStream_t stream) {
 
 }  // namespace
 
-// While no SM has more than two CTAs (see the figures above).
+// While no SM has more than two CTAs.  tcgen05.mma / here in us, up to the line: 16 x 9472 x 128 2.95 / 2.05, x 1024 5.2 / 4.2, x 4096 13.3 / 11.2,
+// 4736 x 32 x 128 3.6 / 2.0, x 4096 13.4 / 11.1, 128 x 1184 x 64 2.8 / 2.1, 128 x 1024 x 4096 12.9 / 11.1; beyond it: 16 x 9473 x 4096 13.3 / 16.3,
+// 128 x 1700 x 64 2.8 / 3.1, x 512 4.0 / 4.7, 33 x 4096 x 256 3.3 / 3.7, x 4096 13.0 / 16.7.  (Not for rows of A alone: 7000 x 32 x 1024, 438
+// tiles, 8.0 / 6.3, x 4096 13.6 / 16.7; nor for one block: 16 x 9472 x 16 3.1 / 3.9.)
 bool warp_mma_supported(const DevModel& m, const GemmArgs& g) {
     return m.fmt_a == EF_F16 && ((g.N + BN - 1) / BN) * ((g.M + Layout::BM - 1) / Layout::BM) <= 2 * 148;
 }
